@@ -200,6 +200,9 @@ struct BsPlan {
     int64_t* koff = nullptr;
     unsigned long long* counter = nullptr;
     int32_t* klist = nullptr;
+    int32_t* level = nullptr;  // of every row block
+    void* items = nullptr;     // a launch's tiles in work order
+    uint32_t* order = nullptr;  // the order's bins
     T* A = nullptr;
     std::vector<Launch> launches;
     double updates = 0.0;
@@ -207,7 +210,11 @@ struct BsPlan {
         if (klist) cudaFreeAsync(klist, st);
         if (A) cudaFreeAsync(A, st);
         if (scratch) cudaFreeAsync(scratch, st);
+        if (items) cudaFreeAsync(items, st);
+        if (order) cudaFreeAsync(order, st);
         klist = nullptr;
+        items = nullptr;
+        order = nullptr;
         A = nullptr;
         scratch = nullptr;
         ready = false;

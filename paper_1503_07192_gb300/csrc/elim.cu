@@ -18,13 +18,18 @@
 // a 128 x |K(R)| panel (gathered once, before the back-substitution overwrites row R)
 // with |K(R)| gathered rows of the matrix.
 //
-// One persistent launch walks the tiles in that order through an atomic work counter:
-// row blocks from the last to the first, inside a row the tiles right of the diagonal,
-// then the diagonal tile.  Tile (R, J) needs the final tiles (min(k, J), max(k, J)) for
-// the blocks k of K(R); the diagonal needs (R, k).  All of them come earlier in the
-// order, so every tile a CTA waits for is held by a CTA that is already running and
-// waits only for tiles earlier still: the waits always end.  Each wait is bounded
-// anyway (2 s of %globaltimer); past that the launch records kErrWait and stops.
+// One persistent launch walks the tiles through an atomic work counter.  Tile (R, J)
+// needs the final tiles (min(k, J), max(k, J)) for the blocks k of K(R); the diagonal needs
+// (R, k).  The order is by level: level(R) = 1 + the largest level of the blocks of K(R)
+// (0 with none), tiles ascending by level(R) + level(J).  Each k has a smaller level than R,
+// so everything a tile needs comes earlier in the order, is held by a CTA that is already
+// running and waits only for tiles earlier still: the waits always end.  Each wait is
+// bounded anyway (2 s of %globaltimer); past that the launch records kErrWait and stops.
+// Why levels and not row after row: in a dissection order the rows of different pieces do
+// not need one another, but the rows of one chain of separators need the row just before,
+// so a row-by-row order has CTAs wait wherever a row holds fewer tiles than there are CTAs
+// (always on small matrices, the last 300 row blocks of large ones), while a level holds
+// tiles of every piece.
 #include <cuda_runtime.h>
 
 #include <math.h>
@@ -178,11 +183,22 @@ struct BsMat {
     int64_t row0;              // offset of its nR records
 };
 
-// A run of the work order: row block R of matrix mat, its tiles right of the diagonal and
+// A run of the enumeration of a launch's tiles: row block R of matrix mat, its tiles right of the diagonal and
 // then the diagonal tile, as the items [start, start + nR - R).
 struct BsRun {
     int64_t start;
     int32_t mat, R;
+};
+
+// A tile of the work order: row block R and column block J >= R of matrix mat (at most
+// 65,535 matrices of at most 2^20 rows, 2^13 row blocks), whole or one of its BS_STRIPS
+// column strips.  A strip is a quarter of the work on a CTA of its own: where a level holds
+// fewer tiles than the GPU holds CTAs, the chain of levels, not the updates, bounds the
+// launch, and a strip takes a quarter of a tile's time.
+constexpr int BS_STRIPS = 4;
+constexpr uint16_t BS_WHOLE = BS_STRIPS;
+struct BsItem {
+    uint16_t mat, R, J, strip;
 };
 
 // Per row block R of matrix blockIdx.y: the column tiles J > R holding a finite entry of
@@ -240,6 +256,133 @@ __global__ void __launch_bounds__(256) k_colmask(const BsMat<T>* __restrict__ ma
         }
         fcnt[m.row0 + R] = cnt;
         kcnt[m.row0 + R] = kc;
+    }
+}
+
+// Level of every row block of matrix blockIdx.x: 0 without a frontier, else 1 + the
+// largest level among the blocks of K(R) (all of them later rows).  One warp per matrix,
+// from the last row up; the next row's first blocks are fetched a row ahead.
+template <typename T>
+__global__ void __launch_bounds__(32) k_bs_levels(const BsMat<T>* __restrict__ mats, const int32_t* __restrict__ fblk,
+                                                  const int32_t* __restrict__ fcnt, int32_t* __restrict__ level) {
+    extern __shared__ int32_t lev[];  // one word per row block
+    const BsMat<T> m = mats[blockIdx.x];
+    const int lane = threadIdx.x;
+    const int32_t nR = m.nR;
+    const int32_t* fb = fblk + m.pair0;
+    const int32_t* fc = fcnt + m.row0;
+    int32_t cnt = fc[nR - 1];
+    int32_t blk = lane < cnt ? fb[(int64_t)(nR - 1) * nR + lane] : -1;
+    for (int32_t R = nR - 1; R >= 0; --R) {
+        const int32_t c = cnt;
+        const int32_t b = blk;
+        if (R > 0) {
+            cnt = fc[R - 1];
+            blk = lane < cnt ? fb[(int64_t)(R - 1) * nR + lane] : -1;
+        }
+        int32_t x = b >= 0 ? lev[b] + 1 : 0;
+        for (int32_t i = lane + 32; i < c; i += 32) x = max(x, lev[fb[(int64_t)R * nR + i]] + 1);
+        x = __reduce_max_sync(0xffffffffu, x);
+        if (lane == 0) {
+            lev[R] = x;
+            level[m.row0 + R] = x;
+        }
+        __syncwarp();
+    }
+}
+
+// Tile t, of run ru (a matrix of nR row blocks).
+__device__ __forceinline__ BsItem bs_item_of(const BsRun& ru, int32_t nR, int64_t t) {
+    const int64_t p = t - ru.start;
+    const int32_t last = nR - 1 - ru.R;  // tiles right of the diagonal
+    return BsItem{(uint16_t)ru.mat, (uint16_t)ru.R, (uint16_t)(p < last ? ru.R + 1 + (int32_t)p : ru.R), BS_WHOLE};
+}
+
+__device__ __forceinline__ int32_t bs_run_of(const BsRun* __restrict__ runs, int32_t nruns, int64_t t) {
+    int32_t lo = 0, hi = nruns;  // the last run starting at or before t
+    while (hi - lo > 1) {
+        const int32_t mid = (lo + hi) >> 1;
+        if (runs[mid].start <= t) lo = mid; else hi = mid;
+    }
+    return lo;
+}
+
+// The work order by counting: tiles per level sum level(R) + level(J) (the runs enumerate
+// a launch's tiles), the bins' offsets, then every tile to its place.  The order of the
+// tiles inside a bin is arbitrary (they do not need one another).
+template <typename T>
+__device__ __forceinline__ BsItem bs_decode(const BsMat<T>* __restrict__ mats, const BsRun* __restrict__ runs,
+                                            int32_t nruns, int64_t t, const int32_t* __restrict__ level, int32_t& bin) {
+    const BsRun ru = runs[bs_run_of(runs, nruns, t)];
+    const BsMat<T> m = mats[ru.mat];
+    const BsItem it = bs_item_of(ru, m.nR, t);
+    bin = level[m.row0 + it.R] + level[m.row0 + it.J];
+    return it;
+}
+
+template <typename T>
+__global__ void __launch_bounds__(256) k_bs_count(const BsMat<T>* __restrict__ mats, const BsRun* __restrict__ runs,
+                                                  int32_t nruns, int64_t nitems, const int32_t* __restrict__ level,
+                                                  uint32_t* __restrict__ bins) {
+    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < nitems; t += (int64_t)gridDim.x * blockDim.x) {
+        int32_t bin;
+        bs_decode<T>(mats, runs, nruns, t, level, bin);
+        atomicAdd(&bins[bin], 1u);
+    }
+}
+
+// bins[b] (tiles of bin b) -> the bin's first item, with the top bit set where its tiles
+// are split into column strips (fewer tiles than split_below: the CTAs would run short);
+// *nout = items in all.  One block.
+__global__ void __launch_bounds__(1024) k_bs_scan(uint32_t* __restrict__ bins, int32_t nbins, uint32_t split_below,
+                                                  unsigned long long* __restrict__ nout) {
+    __shared__ uint32_t ws[32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    uint32_t carry = 0;
+    for (int32_t base = 0; base < nbins; base += 1024) {
+        const int32_t i = base + tid;
+        const uint32_t c = i < nbins ? bins[i] : 0u;
+        const bool split = c > 0 && c < split_below;
+        const uint32_t x = split ? c * BS_STRIPS : c;
+        uint32_t incl = x;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += y;
+        }
+        if (lane == 31) ws[warp] = incl;
+        __syncthreads();
+        uint32_t before = 0, tot = 0;
+        for (int w = 0; w < 32; ++w) {
+            if (w < warp) before += ws[w];
+            tot += ws[w];
+        }
+        if (i < nbins) bins[i] = (carry + before + incl - x) | (split ? 0x80000000u : 0u);
+        carry += tot;
+        __syncthreads();
+    }
+    if (tid == 0) *nout = carry;
+}
+
+template <typename T>
+__global__ void __launch_bounds__(256) k_bs_place(const BsMat<T>* __restrict__ mats, const BsRun* __restrict__ runs,
+                                                  int32_t nruns, int64_t nitems, const int32_t* __restrict__ level,
+                                                  const uint32_t* __restrict__ bins, uint32_t* __restrict__ used,
+                                                  BsItem* __restrict__ items) {
+    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < nitems; t += (int64_t)gridDim.x * blockDim.x) {
+        int32_t bin;
+        BsItem it = bs_decode<T>(mats, runs, nruns, t, level, bin);
+        const uint32_t b = bins[bin], at = b & 0x7fffffffu;
+        const uint32_t p = atomicAdd(&used[bin], 1u);
+        if (b >> 31) {
+            for (int q = 0; q < BS_STRIPS; ++q) {
+                it.strip = (uint16_t)q;
+                items[at + BS_STRIPS * p + q] = it;
+            }
+        } else {
+            it.strip = BS_WHOLE;
+            items[at + p] = it;
+        }
     }
 }
 
@@ -333,14 +476,124 @@ __device__ __forceinline__ void stage_panel(T (*P)[T_], const T* __restrict__ A,
     }
 }
 
+constexpr int SW = T_ / BS_STRIPS;  // strip width (32 columns: 8 threads x 4)
+
+// acc = min(acc, A (x) B) over a chunk for a strip: 4 x 4 per thread, rows 4sy.., strip
+// columns 4sx..; B rows of SW cells.
+template <typename T>
+__device__ __forceinline__ void strip_chunk(T (&acc)[4][4], const T (*a)[T_], const T* b, int sx, int sy, int kend) {
+#pragma unroll 2
+    for (int kk = 0; kk < kend; kk += 2) {
+        const int4 x = *reinterpret_cast<const int4*>(&a[kk][sy * 4]);
+        const int4 y = *reinterpret_cast<const int4*>(&a[kk + 1][sy * 4]);
+        const int4 z = *reinterpret_cast<const int4*>(b + kk * SW + sx * 4);
+        const int4 w = *reinterpret_cast<const int4*>(b + (kk + 1) * SW + sx * 4);
+        const int xa[4] = {x.x, x.y, x.z, x.w}, ya[4] = {y.x, y.y, y.z, y.w};
+        const int zb[4] = {z.x, z.y, z.z, z.w}, wb[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            if constexpr (std::is_same<T, float>::value) {
+                const float2 p0 = make_float2(__int_as_float(xa[i]), __int_as_float(xa[i]));
+                const float2 p1 = make_float2(__int_as_float(ya[i]), __int_as_float(ya[i]));
+#pragma unroll
+                for (int j = 0; j < 4; j += 2) {
+                    const float2 s0 = __fadd2_rn(p0, make_float2(__int_as_float(zb[j]), __int_as_float(zb[j + 1])));
+                    const float2 s1 = __fadd2_rn(p1, make_float2(__int_as_float(wb[j]), __int_as_float(wb[j + 1])));
+                    acc[i][j] = fmin3(acc[i][j], s0.x, s1.x);
+                    acc[i][j + 1] = fmin3(acc[i][j + 1], s0.y, s1.y);
+                }
+            } else {
+#pragma unroll
+                for (int j = 0; j < 4; ++j) acc[i][j] = MP<T>::upd2(acc[i][j], xa[i], zb[j], ya[i], wb[j]);
+            }
+        }
+    }
+}
+
+// Encoded results of a strip -> stored int32 (as clamp_enc).
+__device__ __forceinline__ bool clamp_enc4(float (&acc)[4][4]) {
+    bool bad = false;
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int b = __float_as_int(acc[i][j]);
+            bad |= b >= (1 << 24) && b < SPQ_INF_I32;
+            acc[i][j] = __int_as_float(b < SPQ_INF_I32 ? b : SPQ_INF_I32);
+        }
+    return bad;
+}
+
+// One column strip of tile (R, J): the same sums and minima as the whole tile's.
+template <typename T, bool CONV>
+__device__ __forceinline__ void backsub_strip(T* __restrict__ M, int64_t N, int64_t r0, int64_t cs, bool diag,
+                                              PanelSmem<T>& sm, const T* __restrict__ Ap,
+                                              const int32_t* __restrict__ rows, int32_t kc, T vinf, int4 fill,
+                                              uint32_t* __restrict__ exact) {
+    const int tid = threadIdx.x, sx = tid & 7, sy = tid >> 3;
+    const int64_t r = r0 + 4 * sy, c = cs + 4 * sx;
+    T acc[4][4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        int4 v = fill;
+        if (diag && r + i < N && c < N) v = *reinterpret_cast<const int4*>(M + (r + i) * N + c);
+        const int va[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            acc[i][j] = diag ? *reinterpret_cast<const T*>(&va[j]) : vinf;
+            if constexpr (CONV)
+                if (diag && r + i < N && c < N) acc[i][j] = enc(acc[i][j]);
+        }
+    }
+    const int32_t nch = (kc + KC - 1) / KC;
+    auto stage = [&](int32_t ch) {
+        stage_panel<T>(sm.a[ch & 1], Ap + (int64_t)ch * KC * T_, tid);
+        T* dst = reinterpret_cast<T*>(sm.b[ch & 1]) + sy * SW + sx * 4;  // (KC = 32 rows x 8 vectors)
+        if (c < N)
+            cp_async16(dst, M + (int64_t)rows[ch * KC + sy] * N + c);
+        else
+            *reinterpret_cast<int4*>(dst) = fill;
+        cp_async_commit();
+    };
+    stage(0);
+#pragma unroll 1
+    for (int32_t ch = 0; ch < nch; ++ch) {
+        if (ch + 1 < nch) {
+            stage(ch + 1);
+            cp_async_wait<1>();
+        } else {
+            cp_async_wait<0>();
+        }
+        __syncthreads();
+        const int kend = ch + 1 < nch ? KC : ((kc - ch * KC) + 1) & ~1;
+        strip_chunk<T>(acc, sm.a[ch & 1], reinterpret_cast<const T*>(sm.b[ch & 1]), sx, sy, kend);
+        __syncthreads();
+    }
+    if constexpr (CONV)
+        if (clamp_enc4(acc)) atomicOr(exact, kErrExact);
+    auto i4 = [](T a, T b, T cc, T d) {
+        return make_int4(*reinterpret_cast<int*>(&a), *reinterpret_cast<int*>(&b), *reinterpret_cast<int*>(&cc),
+                         *reinterpret_cast<int*>(&d));
+    };
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+        if (r + i < N && c < N)
+            *reinterpret_cast<int4*>(M + (r + i) * N + c) = i4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
+    if (!diag)
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            if (c + j < N && r < N)
+                *reinterpret_cast<int4*>(M + (c + j) * N + r) = i4(acc[0][j], acc[1][j], acc[2][j], acc[3][j]);
+}
+
 // CONV (float tables of an int32 graph): every tile is stored as int32 (the final table
 // type) as soon as it is final, and the arithmetic runs on the integer encoding above
 // (tiles read as rows of d need no conversion); a finite value >= 2^24 sets kErrExact.
-// Items [0, nitems) follow the runs (ascending starts); one launch may hold the rows of
-// several independent matrices, interleaved.
+// One launch may hold the tiles of several independent matrices, level by level.
 template <typename T, bool CONV>
 __global__ void __launch_bounds__(NTH, SPQ_FW_MIN_CTAS)
-    k_backsub(const BsMat<T>* __restrict__ mats, const BsRun* __restrict__ runs, int32_t nruns, int64_t nitems,
+    k_backsub(const BsMat<T>* __restrict__ mats, const BsItem* __restrict__ items,
+              const unsigned long long* __restrict__ nitems_p,
               const int64_t* __restrict__ koff, const int32_t* __restrict__ kcnt, const int32_t* __restrict__ klist,
               const T* __restrict__ A, int64_t aoff0, const int32_t* __restrict__ fblk,
               const int32_t* __restrict__ fcnt, uint32_t* __restrict__ tflags,
@@ -349,34 +602,24 @@ __global__ void __launch_bounds__(NTH, SPQ_FW_MIN_CTAS)
     extern __shared__ __align__(16) unsigned char smem_raw[];
     PanelSmem<T>& sm = *reinterpret_cast<PanelSmem<T>*>(smem_raw);
     __shared__ int64_t s_item;
-    __shared__ int32_t s_mat, s_R, s_J;
+    __shared__ BsItem s_it;
     __shared__ int s_fail;
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+    const int64_t nitems = (int64_t)*nitems_p;
     for (;;) {
         if (tid == 0) {
             int64_t t = (int64_t)atomicAdd(counter, 1ull);
             if (*reinterpret_cast<volatile uint32_t*>(err) & kErrWait) t = nitems;
             s_item = t;
             s_fail = 0;
-            if (t < nitems) {
-                int32_t lo = 0, hi = nruns;  // the last run starting at or before t
-                while (hi - lo > 1) {
-                    const int32_t mid = (lo + hi) >> 1;
-                    if (runs[mid].start <= t) lo = mid; else hi = mid;
-                }
-                const BsRun ru = runs[lo];
-                const int64_t p = t - ru.start;
-                const int32_t last = mats[ru.mat].nR - 1 - ru.R;  // tiles right of the diagonal
-                s_mat = ru.mat;
-                s_R = ru.R;
-                s_J = p < last ? ru.R + 1 + (int32_t)p : ru.R;
-            }
+            if (t < nitems) s_it = items[t];
         }
         __syncthreads();
         const int64_t t = s_item;
         if (t >= nitems) break;
-        const BsMat<T> m = mats[s_mat];
-        const int32_t R = s_R, J = s_J, nR = m.nR;
+        const BsItem it = s_it;
+        const BsMat<T> m = mats[it.mat];
+        const int32_t R = it.R, J = it.J, nR = m.nR;
         T* __restrict__ M = m.M;
         const int64_t N = m.N;
         const int32_t kc = kcnt[m.row0 + R];
@@ -392,9 +635,9 @@ __global__ void __launch_bounds__(NTH, SPQ_FW_MIN_CTAS)
                     const int32_t a = (J == R) ? R : (K < J ? K : J);
                     const int32_t b = (J == R) ? K : (K < J ? J : K);
                     const uint32_t* f = tflags + m.pair0 + (int64_t)a * nR + b;
-                    if (ld_acquire(f) == 0u) {
+                    if (ld_acquire(f) < (uint32_t)BS_STRIPS) {
                         const unsigned long long t0 = global_ns();
-                        while (ld_acquire(f) == 0u) {
+                        while (ld_acquire(f) < (uint32_t)BS_STRIPS) {
                             __nanosleep(256);
                             // another CTA gave up (the launch is abandoned), or the bound ran out
                             if (*reinterpret_cast<volatile uint32_t*>(err) & kErrWait) {
@@ -412,6 +655,16 @@ __global__ void __launch_bounds__(NTH, SPQ_FW_MIN_CTAS)
             }
             __syncthreads();
             if (s_fail) break;
+        }
+        uint32_t done = BS_STRIPS;  // strips of the tile this item completes
+        if (kc > 0 && it.strip != BS_WHOLE) {
+            const int64_t kb = koff[m.row0 + R];
+            backsub_strip<T, CONV>(M, N, r0, c0 + it.strip * SW, J == R, sm, A + (kb - aoff0) * T_, klist + kb, kc,
+                                   vinf, fill, exact);
+            done = 1;
+        } else if (kc == 0 && it.strip != BS_WHOLE && it.strip > 0) {
+            done = 0;  // (strip 0 stores the whole tile)
+        } else if (kc > 0) {
             T acc[8][8];
             if (J == R) {
                 load_c<T>(acc, M, N, r0, r0, tx, ty);
@@ -477,9 +730,13 @@ __global__ void __launch_bounds__(NTH, SPQ_FW_MIN_CTAS)
             if (J != R) store_c_transposed<T>(acc, M, N, r0, c0, tx, ty);
         }
         __syncthreads();
-        if (tid == 0 && !withhold) {
+        if (tid == 0 && !withhold && done > 0) {
+            uint32_t* f = tflags + m.pair0 + (int64_t)R * nR + J;  // strips done so far
             __threadfence();
-            st_release(tflags + m.pair0 + (int64_t)R * nR + J, 1u);
+            if (done == (uint32_t)BS_STRIPS)
+                st_release(f, done);
+            else
+                atomicAdd(f, done);
         }
     }
 }
@@ -538,8 +795,10 @@ cudaError_t launch_mark_pairs(const std::vector<int32_t>& blocks, int64_t N, uin
 size_t bg_backsub_scratch_bytes(int64_t N) {
     const int64_t nR = (N + T_ - 1) / T_;
     // masks (16 B), fblk and tile flags (4 B each) per tile pair; per row block: fcnt,
-    // kcnt, koff and a run of the work order; the work counter and the matrix record
-    return (size_t)(nR * nR) * 24 + (size_t)nR * 32 + 256;
+    // kcnt, koff, level and a run of the enumeration; the work counter and the matrix record
+    // (the work order's 8 bytes an item, under 48 MB for the largest matrix that fits the
+    // device, come out of the build's 64 MiB reserve)
+    return (size_t)(nR * nR) * 24 + (size_t)nR * 36 + 256;
 }
 
 // The launches of a back-substitution after its bookkeeping (klist, A panels, work
@@ -553,7 +812,8 @@ cudaError_t bs_enqueue(const BsPlan<T>& p, uint32_t* err, uint32_t* exact, std::
     const uint4* masks = static_cast<const uint4*>(p.masks);
     const BsRun* runs = static_cast<const BsRun*>(p.runs);
     k_klist<T><<<dim3(p.nRmax, p.nmat), T_, 0, st>>>(mats, masks, p.fblk, p.fcnt, p.kcnt, p.koff, p.klist);
-    count_launches(1);
+    k_bs_levels<T><<<p.nmat, 32, (size_t)p.nRmax * 4, st>>>(mats, p.fblk, p.fcnt, p.level);
+    count_launches(2);
     cudaError_t e = cudaGetLastError();
     const size_t psm = sizeof(PanelSmem<T>);
     const int grid = sms_e() * SPQ_FW_MIN_CTAS;
@@ -566,9 +826,22 @@ cudaError_t bs_enqueue(const BsPlan<T>& p, uint32_t* err, uint32_t* exact, std::
                                                                               p.klist, L.aoff0, p.A);
         else
             k_gather_a<T, false><<<gg, 256, 0, st>>>(mats, L.mat0, L.R0, L.R1, p.koff, p.kcnt, p.klist, L.aoff0, p.A);
+        // the launch's tiles in level order
+        BsItem* items = static_cast<BsItem*>(p.items);
+        const BsRun* lr = runs + L.run0;
+        const int32_t nlr = (int32_t)(L.run1 - L.run0), nbins = 2 * p.nRmax;
+        uint32_t* bins = p.order;  // bins | places taken | items in all
+        uint32_t* used = bins + nbins;
+        unsigned long long* nout = reinterpret_cast<unsigned long long*>(used + nbins);
+        const unsigned ig = (unsigned)std::min<int64_t>((L.nit + 255) / 256, 4 * sms_e());
+        cudaMemsetAsync(bins, 0, (size_t)nbins * 8, st);
+        k_bs_count<T><<<ig, 256, 0, st>>>(mats, lr, nlr, L.nit, p.level, bins);
+        k_bs_scan<<<1, 1024, 0, st>>>(bins, nbins, (uint32_t)grid, nout);
+        k_bs_place<T><<<ig, 256, 0, st>>>(mats, lr, nlr, L.nit, p.level, bins, used, items);
+        count_launches(3);
         cudaMemsetAsync(p.counter, 0, 8, st);
         if (ev) cudaEventRecord((*ev)[2 * l], st);
-        kern<<<grid, NTH, psm, st>>>(mats, runs + L.run0, (int32_t)(L.run1 - L.run0), L.nit, p.koff, p.kcnt, p.klist,
+        kern<<<grid, NTH, psm, st>>>(mats, items, nout, p.koff, p.kcnt, p.klist,
                                      p.A, L.aoff0, p.fblk, p.fcnt, p.tflags, p.counter, err, exact, g_wait_ns.load(),
                                      g_withhold.load());
         if (ev) cudaEventRecord((*ev)[2 * l + 1], st);
@@ -625,10 +898,11 @@ cudaError_t bg_backsub_many(const std::vector<BsInput<T>>& in, uint32_t* err, ui
     auto kern = conv ? k_backsub<T, std::is_same<T, float>::value> : k_backsub<T, false>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(PanelSmem<T>));
     if (e != cudaSuccess) return e;
-    // one scratch block: masks | fblk | tflags | koff | fcnt | kcnt | kplan | runs | counter | mats
+    // one scratch block: masks | fblk | tflags | koff | fcnt | kcnt | kplan | level | runs | counter | mats
     const size_t o_fblk = (size_t)P2 * 16, o_tfl = o_fblk + (size_t)P2 * 4, o_koff = o_tfl + (size_t)P2 * 4;
     const size_t o_fcnt = o_koff + (size_t)RR * 8, o_kcnt = o_fcnt + (size_t)RR * 4, o_kpl = o_kcnt + (size_t)RR * 4;
-    const size_t o_runs = (o_kpl + (size_t)RR * 4 + 15) & ~(size_t)15;
+    const size_t o_lev = o_kpl + (size_t)RR * 4;
+    const size_t o_runs = (o_lev + (size_t)RR * 4 + 15) & ~(size_t)15;
     const size_t o_ctr = o_runs + (size_t)RR * sizeof(BsRun);
     const size_t o_mats = (o_ctr + 8 + 15) & ~(size_t)15;
     const size_t bytes = o_mats + (size_t)nmat * sizeof(BsMat<T>);
@@ -641,6 +915,7 @@ cudaError_t bg_backsub_many(const std::vector<BsInput<T>>& in, uint32_t* err, ui
     p.fcnt = reinterpret_cast<int32_t*>(scratch + o_fcnt);
     p.kcnt = reinterpret_cast<int32_t*>(scratch + o_kcnt);
     p.kplan = reinterpret_cast<int32_t*>(scratch + o_kpl);
+    p.level = reinterpret_cast<int32_t*>(scratch + o_lev);
     p.runs = scratch + o_runs;
     p.counter = reinterpret_cast<unsigned long long*>(scratch + o_ctr);
     p.mats = scratch + o_mats;
@@ -728,7 +1003,7 @@ cudaError_t bg_backsub_many(const std::vector<BsInput<T>>& in, uint32_t* err, ui
     }
     // the runs of every launch: row blocks from the last down, the matrices of a launch
     // interleaved (their q-th rows from the end side by side)
-    int64_t maxk = 0;
+    int64_t maxk = 0, maxit = 0;
     for (Launch& L : launches) {
         L.run0 = hruns.size();
         int64_t start = 0;
@@ -743,6 +1018,7 @@ cudaError_t bg_backsub_many(const std::vector<BsInput<T>>& in, uint32_t* err, ui
             }
         L.run1 = hruns.size();
         L.nit = start;
+        maxit = std::max(maxit, start);
         L.aoff0 = hoff[hm[L.mat0].row0 + L.R0];
         const BsMat<T>& z = hm[L.mat0 + L.nm - 1];
         maxk = std::max(maxk, hoff[z.row0 + std::min(z.nR, L.R1)] - L.aoff0);
@@ -752,6 +1028,12 @@ cudaError_t bg_backsub_many(const std::vector<BsInput<T>>& in, uint32_t* err, ui
         return done(e);
     if ((e = scratch_alloc((void**)&p.A, (size_t)(maxk > 0 ? maxk : 1) * row_bytes, st)) != cudaSuccess)
         return done(e);
+    // the work order: at most BS_STRIPS items a tile, in the bins of fewer tiles than CTAs
+    const int64_t nbins = 2 * (int64_t)nRmax;
+    const int64_t most = maxit + (BS_STRIPS - 1) * std::min<int64_t>(maxit, nbins * sms_e() * SPQ_FW_MIN_CTAS);
+    if (most > INT32_MAX) return done(cudaErrorInvalidValue);  // (bin offsets are 31 bits)
+    if ((e = scratch_alloc(&p.items, (size_t)most * sizeof(BsItem), st)) != cudaSuccess) return done(e);
+    if ((e = scratch_alloc((void**)&p.order, (size_t)nbins * 8 + 8, st)) != cudaSuccess) return done(e);
     if (prof) {
         ev.assign(2 * launches.size(), nullptr);
         for (auto& x : ev)
