@@ -18,19 +18,19 @@
 #include <cuda_runtime.h>
 #include <math.h>
 
+#include <algorithm>
+#include <new>
+#include <vector>
+
 #include "common.cuh"
 #include "handle.h"
+#include "walk.cuh"
 
 namespace spq {
 namespace {
 
 constexpr int GTH = 256;
 constexpr int kNoPath = -3, kSame = -2, kDirect = -1;
-
-template <typename T>
-__device__ __forceinline__ bool less_lex(T a, int64_t ai, T b, int64_t bi) {
-    return a < b || (a == b && ai < bi);
-}
 
 // Warp-wide lexicographic argmin of (value, index).
 template <typename T>
@@ -45,25 +45,6 @@ __device__ __forceinline__ void warp_argmin(T& v, int64_t& i) {
         }
     }
 }
-
-template <typename T>
-struct View {
-    int32_t n;
-    const int32_t* comp;
-    const int32_t* local;
-    const MatDesc* descs;
-    const int32_t* nb;
-    const int32_t* bg_off;
-    const int32_t* bgpos;
-    const T* apsp;
-    const T* D;
-    int64_t N;
-    const int64_t* rp;
-    const int32_t* col;
-    const T* w;
-    const int32_t* vorder;
-    const int32_t* vstart;
-};
 
 // Forward with the minimising boundary pair.  dist_out: T[q]; saved: int2[q].
 template <typename T>
@@ -294,6 +275,222 @@ __global__ void __launch_bounds__(GTH) k_query_paths(const View<T> V, const int2
     }
 }
 
+// ---------------- large batches: walks by the records of walk.cuh ----------------
+
+// Part of a backward walk: the moves of pair i through the boundary graph.  A clique edge
+// adds the pair's upstream gradient to its flow, an edge between components to its slot.
+template <typename T>
+__global__ void __launch_bounds__(GTH) k_backward_bg(const View<T> V, const WalkCtx<T> W,
+                                                     const int2* __restrict__ pairs, const int2* __restrict__ saved,
+                                                     int64_t q, const float* __restrict__ gdist,
+                                                     float* __restrict__ grad, uint32_t* __restrict__ err) {
+    const int lane = threadIdx.x & 31;
+    const int64_t nw = ((int64_t)gridDim.x * GTH) >> 5;
+    const int64_t limit = (int64_t)V.n + 1;
+    for (int64_t qi = ((int64_t)blockIdx.x * GTH + threadIdx.x) >> 5; qi < q; qi += nw) {
+        const int2 pr = pairs[qi];
+        const int2 sv = saved[qi];
+        const float g = gdist[qi];
+        if (sv.x == kSame || sv.x == kNoPath || sv.x == kDirect || g == 0.0f) continue;
+        if (pr.x < 0 || pr.x >= V.n || pr.y < 0 || pr.y >= V.n) continue;
+        const int32_t c1 = V.comp[pr.x], c2 = V.comp[pr.y];
+        if (sv.x < 0 || sv.x >= V.nb[c1] || sv.y < 0 || sv.y >= V.nb[c2]) continue;  // (marked by k_backward_ends)
+        const bool ok = walk_bg<T>(
+            V, W, c1, sv.x, c2, sv.y, limit, lane,
+            [&](int32_t c, int32_t b, int32_t y, int32_t nb) {
+                if (lane == 0) atomicAdd(W.flow + W.foff[c] + (int64_t)b * nb + y, g);
+            },
+            [&](int32_t e, int32_t) {
+                if (lane == 0) atomicAdd(grad + e, g);
+            });
+        if (!ok && lane == 0) atomicOr(err, kErrWalk);
+    }
+}
+
+// The rest of it: v1 -> b1* inside C1 (by the hop table) and b2* -> v2 inside C2 (or v1 ->
+// v2 directly), searched slot by slot: v2 is any vertex.  Eight lanes a pair.
+constexpr int ESUB = 8;
+template <typename T>
+__global__ void __launch_bounds__(GTH) k_backward_ends(const View<T> V, const WalkCtx<T> W,
+                                                       const int2* __restrict__ pairs, const int2* __restrict__ saved,
+                                                       int64_t q, const float* __restrict__ gdist,
+                                                       float* __restrict__ grad, uint32_t* __restrict__ err) {
+    const int lane = threadIdx.x & 31, g8 = lane & (ESUB - 1);
+    const unsigned mask = ((1u << ESUB) - 1u) << (lane & ~(ESUB - 1));
+    const int64_t nw = ((int64_t)gridDim.x * GTH) / ESUB;
+    const int64_t limit = (int64_t)V.n + 1;
+    for (int64_t qi = ((int64_t)blockIdx.x * GTH + threadIdx.x) / ESUB; qi < q; qi += nw) {
+        const int2 pr = pairs[qi];
+        const int2 sv = saved[qi];
+        const float g = gdist[qi];
+        if (sv.x == kSame || sv.x == kNoPath || g == 0.0f) continue;
+        if (pr.x < 0 || pr.x >= V.n || pr.y < 0 || pr.y >= V.n) continue;
+        const int32_t c1 = V.comp[pr.x], c2 = V.comp[pr.y], lw = V.local[pr.y];
+        int32_t x = V.local[pr.x];
+        bool ok;
+        if (sv.x == kDirect) {
+            ok = c1 == c2;
+        } else {
+            ok = sv.x >= 0 && sv.x < V.nb[c1] && sv.y >= 0 && sv.y < V.nb[c2];
+            if (ok) {
+                const int32_t vs1 = V.vstart[c1];
+                ok = walk_hops<T, ESUB>(V, W, c1, x, sv.x, limit, g8, mask,
+                                        [&](int32_t from, int64_t slot, int32_t) {
+                                            if (g8 == 0) atomicAdd(grad + V.rp[V.vorder[vs1 + from]] + slot, g);
+                                        });
+                x = sv.y;
+            }
+        }
+        if (ok) {
+            const MatDesc d = V.descs[c2];
+            const T* A = V.apsp + d.off;
+            const int32_t vs = V.vstart[c2];
+            for (int64_t step = 0; x != lw; ++step) {
+                const int64_t e = step < limit ? best_slot<T, ESUB>(V, W, A, d.n, vs, x, lw, g8, mask) : -1;
+                if (e < 0) {
+                    ok = false;
+                    break;
+                }
+                if (g8 == 0) atomicAdd(grad + e, g);
+            }
+        }
+        if (!ok && g8 == 0) atomicOr(err, kErrWalk);
+    }
+}
+
+// Every clique edge's flow onto the slots of its path inside the component, one thread each.
+template <typename T>
+__global__ void __launch_bounds__(GTH) k_backward_flow(const View<T> V, const WalkCtx<T> W, int32_t k, int64_t total,
+                                                       float* __restrict__ grad, uint32_t* __restrict__ err) {
+    const int64_t i = (int64_t)blockIdx.x * GTH + threadIdx.x;
+    if (i >= total) return;
+    const float g = W.flow[i];
+    if (g == 0.0f) return;
+    int32_t lo = 0, hi = k;  // the component whose range holds i
+    while (hi - lo > 1) {
+        const int32_t mid = (lo + hi) >> 1;
+        if (W.foff[mid] <= i) lo = mid; else hi = mid;
+    }
+    const int32_t nb = V.nb[lo], vs = V.vstart[lo];
+    const int32_t r = (int32_t)(i - W.foff[lo]);
+    const bool ok = walk_hops<T, 1>(V, W, lo, r / nb, r % nb, (int64_t)V.n + 1, 0, 1u << (threadIdx.x & 31),
+                                    [&](int32_t from, int64_t slot, int32_t) {
+                                        atomicAdd(grad + V.rp[V.vorder[vs + from]] + slot, g);
+                                    });
+    if (!ok) atomicOr(err, kErrWalk);
+}
+
+// Vertex sequences: as k_query_paths, a warp per pair.  The moves through the boundary graph
+// are collected 32 at a time, and each lane expands one of them: once to count its hops
+// (its place in the row is the sum of the earlier ones'), once to write its vertices.
+template <typename T>
+__global__ void __launch_bounds__(GTH) k_paths_hops(const View<T> V, const WalkCtx<T> W,
+                                                    const int2* __restrict__ pairs, const int2* __restrict__ saved,
+                                                    int64_t q, int32_t max_len, int32_t* __restrict__ verts,
+                                                    int32_t* __restrict__ lens, uint32_t* __restrict__ err) {
+    // collected moves: (component, from, to) or (-1, vertex, 0)
+    __shared__ int32_t sc[GTH / 32][32], sx[GTH / 32][32], st[GTH / 32][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t nw = ((int64_t)gridDim.x * GTH) >> 5;
+    const int64_t limit = (int64_t)V.n + 1;
+    for (int64_t qi = ((int64_t)blockIdx.x * GTH + threadIdx.x) >> 5; qi < q; qi += nw) {
+        const int2 pr = pairs[qi];
+        const int2 sv = saved[qi];
+        int32_t* row = verts + qi * (int64_t)max_len;
+        if (sv.x == kNoPath || pr.x < 0 || pr.x >= V.n || pr.y < 0 || pr.y >= V.n) {
+            if (lane == 0) lens[qi] = -1;
+            continue;
+        }
+        int32_t len = 1;
+        if (lane == 0 && max_len > 0) row[0] = pr.x;
+        bool ok = true;
+        if (sv.x != kSame) {
+            const int32_t c1 = V.comp[pr.x], c2 = V.comp[pr.y], lw = V.local[pr.y];
+            int32_t x = V.local[pr.x];
+            int n = 0;
+            auto flush = [&]() {  // expands the n collected moves; false if one did not arrive
+                __syncwarp();
+                const int32_t c = lane < n ? sc[warp][lane] : -1;
+                const int32_t a = lane < n ? sx[warp][lane] : 0, b = lane < n ? st[warp][lane] : 0;
+                int32_t cnt = lane < n ? 1 : 0;
+                bool good = true;
+                if (c >= 0) {
+                    cnt = 0;
+                    good = walk_hops<T, 1>(V, W, c, a, b, limit, 0, 1u << lane,
+                                           [&](int32_t, int64_t, int32_t) { ++cnt; });
+                }
+                const unsigned bad = __ballot_sync(0xffffffffu, !good);
+                const int last = bad ? __ffs(bad) - 1 : 31;  // the moves after a failed one are not made
+                if (lane > last) cnt = 0;
+                int32_t incl = cnt;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+                    if (lane >= o) incl += y;
+                }
+                int32_t at = len + incl - cnt;
+                if (cnt > 0 && c < 0) {
+                    if (at < max_len) row[at] = a;
+                } else if (cnt > 0) {
+                    const int32_t vs = V.vstart[c];
+                    const int64_t lim = cnt < max_len - at ? cnt : max_len - at;
+                    if (lim > 0)
+                        walk_hops<T, 1>(V, W, c, a, b, lim, 0, 1u << lane, [&](int32_t, int64_t, int32_t y) {
+                            row[at++] = V.vorder[vs + y];
+                        });
+                }
+                len += __shfl_sync(0xffffffffu, incl, 31);
+                n = 0;
+                __syncwarp();
+                return bad == 0;
+            };
+            auto add = [&](int32_t c, int32_t a, int32_t b) {
+                if (lane == 0) {
+                    sc[warp][n] = c;
+                    sx[warp][n] = a;
+                    st[warp][n] = b;
+                }
+                if (++n == 32) ok = flush() && ok;
+            };
+            if (sv.x == kDirect) {
+                ok = c1 == c2;
+            } else if (sv.x < 0 || sv.x >= V.nb[c1] || sv.y < 0 || sv.y >= V.nb[c2]) {
+                ok = false;
+            } else {
+                add(c1, x, sv.x);
+                const bool there = walk_bg<T>(
+                    V, W, c1, sv.x, c2, sv.y, limit, lane,
+                    [&](int32_t c, int32_t b, int32_t y, int32_t) {
+                        if (ok) add(c, b, y);
+                    },
+                    [&](int32_t, int32_t s) {
+                        const int32_t c = W.scomp[s];
+                        if (ok) add(-1, V.vorder[V.vstart[c] + s - V.bg_off[c]], 0);
+                    });
+                if (ok && n > 0) ok = flush();
+                ok = ok && there;
+                x = sv.y;
+            }
+            if (ok) {
+                const MatDesc d = V.descs[c2];
+                const T* A = V.apsp + d.off;
+                const int32_t vs = V.vstart[c2];
+                for (int64_t step = 0; x != lw; ++step) {
+                    const int64_t e = step < limit ? best_slot<T, 32>(V, W, A, d.n, vs, x, lw, lane, 0xffffffffu) : -1;
+                    if (e < 0) {
+                        ok = false;
+                        break;
+                    }
+                    if (lane == 0 && len < max_len) row[len] = V.vorder[vs + x];
+                    ++len;
+                }
+            }
+            if (!ok && lane == 0) atomicOr(err, kErrWalk);
+        }
+        if (lane == 0) lens[qi] = len;
+    }
+}
+
 int grad_sms() {
     static int n = 0;
     if (n == 0) {
@@ -319,6 +516,96 @@ bool on_device(const void* p) {
         return false;
     }
     return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
+}
+
+// The records of walk.cuh for handle h, in one stream-ordered allocation (freed by the caller
+// with cudaFreeAsync(*mem)); false if it does not fit (the caller walks without them).
+template <typename T>
+bool walk_records(const spq_handle* h, bool want_flow, cudaStream_t st, WalkCtx<T>* W, void** mem, int64_t* nflow) {
+    const int32_t k = h->k;
+    std::vector<int64_t> off;
+    try {
+        off.assign(2 * ((size_t)k + 1), 0);
+    } catch (const std::bad_alloc&) {
+        return false;
+    }
+    for (int32_t c = 0; c < k; ++c) {
+        off[c + 1] = off[c] + (int64_t)h->h_csize[c] * h->h_nb[c];
+        off[k + 2 + c] = off[k + 1 + c] + (int64_t)h->h_nb[c] * h->h_nb[c];
+    }
+    const int64_t nt = off[k], nf = want_flow ? off[2 * (size_t)k + 1] : 0;
+    const int64_t o_sr = h->m * 8, o_off = o_sr + h->nbg * 8, o_sc = o_off + (int64_t)off.size() * 8;
+    const int64_t o_hop = o_sc + h->nbg * 4, o_fl = o_hop + nt * 4;
+    unsigned char* p = nullptr;
+    if (scratch_alloc((void**)&p, (size_t)(o_fl + nf * 4), st) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    *mem = p;
+    *nflow = nf;
+    int64_t* d_off = (int64_t*)(p + o_off);
+    *W = WalkCtx<T>{(int2*)p,          (int2*)(p + o_sr), (int32_t*)(p + o_sc),  d_off,
+                    d_off + (k + 1),   (uint32_t*)(p + o_hop), (float*)(p + o_fl)};
+    const View<T> V = view_of<T>(h);
+    cudaMemcpyAsync(d_off, off.data(), off.size() * 8, cudaMemcpyHostToDevice, st);
+    if (nf > 0) cudaMemsetAsync(p + o_fl, 0, (size_t)nf * 4, st);
+    k_walk_slots<T><<<(unsigned)((h->n + 255) / 256), 256, 0, st>>>(V, (int2*)p, (int2*)(p + o_sr), (int32_t*)(p + o_sc));
+    k_walk_hops<T><<<(unsigned)(((int64_t)h->n * 32 + 255) / 256), 256, 0, st>>>(V, *W, (uint32_t*)(p + o_hop));
+    count_launches(2);
+    return true;
+}
+
+// Whether q walks pay for the records: a hop searched on the spot costs about 0.17 ns of the
+// GPU (measured: 1M pairs on 2^18 vertices 86 ms, 100k on 2^14 1.96 ms; the hops of a pair
+// grow with sqrt(n)), the records about 30 us plus 8 ps per table entry.  Never inside a
+// stream capture: a captured call allocates nothing.
+bool walks_pay(const spq_handle* h, int64_t q, cudaStream_t st) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+        cudaGetLastError();
+        return false;
+    }
+    double nt = 0.0;
+    for (int32_t c = 0; c < h->k; ++c) nt += (double)h->h_csize[c] * h->h_nb[c];
+    return 21.0 * (double)q * sqrt((double)h->n) > 3.75e6 + nt;
+}
+
+template <typename T>
+bool backward_by_records(const spq_handle* h, const int32_t* pairs, int64_t q, const int32_t* saved,
+                         const float* grad_dist, float* grad_w, cudaStream_t st) {
+    WalkCtx<T> W;
+    void* mem = nullptr;
+    int64_t nf = 0;
+    if (!walk_records<T>(h, true, st, &W, &mem, &nf)) return false;
+    const View<T> V = view_of<T>(h);
+    const int64_t cap = (int64_t)grad_sms() * 8;
+    const int2 *p2 = (const int2*)pairs, *s2 = (const int2*)saved;
+    k_backward_bg<T><<<(unsigned)std::min<int64_t>((q + 7) / 8, cap), GTH, 0, st>>>(V, W, p2, s2, q, grad_dist, grad_w,
+                                                                                    h->err);
+    k_backward_ends<T><<<(unsigned)std::min<int64_t>((q + GTH / ESUB - 1) / (GTH / ESUB), cap), GTH, 0, st>>>(
+        V, W, p2, s2, q, grad_dist, grad_w, h->err);
+    count_launches(2);
+    if (nf > 0) {
+        k_backward_flow<T><<<(unsigned)((nf + GTH - 1) / GTH), GTH, 0, st>>>(V, W, h->k, nf, grad_w, h->err);
+        count_launches(1);
+    }
+    cudaFreeAsync(mem, st);
+    return true;
+}
+
+template <typename T>
+bool paths_by_records(const spq_handle* h, const int32_t* pairs, int64_t q, const int32_t* saved, int32_t max_len,
+                      int32_t* verts, int32_t* lens, cudaStream_t st) {
+    WalkCtx<T> W;
+    void* mem = nullptr;
+    int64_t nf = 0;
+    if (!walk_records<T>(h, false, st, &W, &mem, &nf)) return false;
+    const int64_t cap = (int64_t)grad_sms() * 8;
+    k_paths_hops<T><<<(unsigned)std::min<int64_t>((q + 7) / 8, cap), GTH, 0, st>>>(
+        view_of<T>(h), W, (const int2*)pairs, (const int2*)saved, q, max_len, verts, lens, h->err);
+    count_launches(1);
+    cudaFreeAsync(mem, st);
+    return true;
 }
 
 }  // namespace
@@ -357,6 +644,10 @@ spq_status spq_query_backward(spq_handle* h, const int32_t* pairs, int64_t q, co
     if (!on_device(pairs) || !on_device(saved) || !on_device(grad_dist) || !on_device(grad_w)) return SPQ_EINVAL;
     if (((uintptr_t)pairs & 7u) || ((uintptr_t)saved & 7u)) return SPQ_EINVAL;
     cudaStream_t st = (cudaStream_t)stream;
+    if (walks_pay(h, q, st) &&
+        (h->f32store ? backward_by_records<float>(h, pairs, q, saved, grad_dist, grad_w, st)
+                     : backward_by_records<int32_t>(h, pairs, q, saved, grad_dist, grad_w, st)))
+        return cudaGetLastError() == cudaSuccess ? SPQ_OK : SPQ_ECUDA;
     int64_t blocks = (q + 7) / 8;
     const int64_t cap = (int64_t)grad_sms() * 16;
     if (blocks > cap) blocks = cap;
@@ -381,6 +672,10 @@ spq_status spq_query_paths(spq_handle* h, const int32_t* pairs, int64_t q, const
         return SPQ_EINVAL;
     if (((uintptr_t)pairs & 7u) || ((uintptr_t)saved & 7u)) return SPQ_EINVAL;
     cudaStream_t st = (cudaStream_t)stream;
+    if (walks_pay(h, q, st) &&
+        (h->f32store ? paths_by_records<float>(h, pairs, q, saved, max_len, verts, lens, st)
+                     : paths_by_records<int32_t>(h, pairs, q, saved, max_len, verts, lens, st)))
+        return cudaGetLastError() == cudaSuccess ? SPQ_OK : SPQ_ECUDA;
     int64_t blocks = (q + 7) / 8;
     const int64_t cap = (int64_t)grad_sms() * 16;
     if (blocks > cap) blocks = cap;

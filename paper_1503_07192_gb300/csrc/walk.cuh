@@ -1,0 +1,308 @@
+// Path walks for large batches (gradients and path retrieval, grad.cu): the same moves as
+// walk_pair's, one by one, from records made once per call.
+//
+// What bounds a walk is latency: a warp that looks at every slot of every vertex on the way
+// waits for five dependent loads a hop (0.2 ns of the whole GPU per hop: 86 ms for a million
+// pairs of 400 hops).  Three records shorten it:
+//   slots   per CSR slot its target's local index (same component) or boundary slot and
+//           matrix position (another component): no comp / local / bgpos look-ups on the way;
+//   hops    per component, vertex x and boundary vertex t: the slot that the walk from x
+//           towards t takes first and the vertex it leads to (4 bytes; sum of |C||B(C)|), so a
+//           hop towards a boundary vertex is one load;
+//   flow    (gradients) per component and pair (b, y) of boundary vertices: the upstream
+//           gradients of all pairs whose walk takes the clique edge b -> y, so that each
+//           clique edge is expanded into its slots once and not once per pair.
+// In the boundary graph a warp holds the distances D(y, b2) of a component's boundary
+// vertices y in registers for as long as the walk stays in the component, and reads them
+// along row b2 of D.  D is symmetric bit for bit outside its diagonal 128 x 128 tiles (the
+// kernels store such a tile and its mirror from the same registers); inside them the walk
+// reads D(y, b2) itself, so that each comparison sees the value it always saw.
+#pragma once
+
+#include <cuda_runtime.h>
+
+#include "common.cuh"
+
+namespace spq {
+namespace {
+
+// Read-only tables of a handle, as the walks use them.
+template <typename T>
+struct View {
+    int32_t n;
+    const int32_t* comp;
+    const int32_t* local;
+    const MatDesc* descs;
+    const int32_t* nb;
+    const int32_t* bg_off;
+    const int32_t* bgpos;
+    const T* apsp;
+    const T* D;
+    int64_t N;
+    const int64_t* rp;
+    const int32_t* col;
+    const T* w;
+    const int32_t* vorder;
+    const int32_t* vstart;
+};
+
+// (value, index) order: ties to the smallest index.
+template <typename T>
+__device__ __forceinline__ bool less_lex(T a, int64_t ai, T b, int64_t bi) {
+    return a < b || (a == b && ai < bi);
+}
+
+constexpr uint32_t kNoHop = 0xffffffffu;  // no entry of the table (searched on the spot)
+
+template <typename T>
+struct WalkCtx {
+    const int2* slots;        // [m]: (local index, 0) inside the component; (~slot, position); (INT_MIN, 0) self-loop
+    const int2* srange;       // [|BG|]: CSR range of a boundary slot's vertex
+    const int32_t* scomp;     // [|BG|]: its component
+    const int64_t* toff;      // [k + 1]: hops of component c at toff[c] + x * |B| + t
+    const int64_t* foff;      // [k + 1]: flow of component c at foff[c] + b * |B| + y
+    const uint32_t* hops;
+    float* flow;
+};
+
+// Values compared as unsigned words: distances are never negative.
+__device__ __forceinline__ uint32_t key_of(int32_t v) { return (uint32_t)v; }
+__device__ __forceinline__ uint32_t key_of(float v) { return (uint32_t)__float_as_int(v + 0.0f); }
+
+template <typename T>
+__global__ void __launch_bounds__(256) k_walk_slots(const View<T> V, int2* __restrict__ slots,
+                                                    int2* __restrict__ srange, int32_t* __restrict__ scomp) {
+    const int32_t u = blockIdx.x * blockDim.x + threadIdx.x;
+    if (u >= V.n) return;
+    const int32_t c = V.comp[u], l = V.local[u];
+    const int64_t e0 = V.rp[u], e1 = V.rp[u + 1];
+    for (int64_t e = e0; e < e1; ++e) {
+        const int32_t v = V.col[e];
+        const int32_t cv = V.comp[v];
+        if (cv == c) {
+            slots[e] = v == u ? make_int2(INT32_MIN, 0) : make_int2(V.local[v], 0);
+        } else {
+            const int32_t s = V.bg_off[cv] + V.local[v];
+            slots[e] = make_int2(~s, V.bgpos[s]);
+        }
+    }
+    if (l < V.nb[c]) {
+        const int32_t s = V.bg_off[c] + l;
+        srange[s] = make_int2((int32_t)e0, (int32_t)e1);
+        scomp[s] = c;
+    }
+}
+
+// The slot a walk inside component c takes at local vertex x towards local vertex t: the one
+// minimising w + dist_C(u, t), ties to the smallest slot.  sub lanes of the warp (lane g of
+// them) share the slots; every one of them returns the slot (-1: none) and, in x, the vertex.
+template <typename T, int SUB>
+__device__ __forceinline__ int64_t best_slot(const View<T>& V, const WalkCtx<T>& W, const T* A, int32_t ld,
+                                             int32_t vs, int32_t& x, int32_t t, int g, unsigned mask) {
+    const int32_t v = V.vorder[vs + x];
+    const int64_t e0 = V.rp[v], e1 = V.rp[v + 1];
+    T best = Inf<T>::value();
+    int64_t be = INT64_MAX;
+    int32_t to = -1;
+    for (int64_t e = e0 + g; e < e1; e += SUB) {
+        const int32_t u = W.slots[e].x;
+        if (u < 0) continue;
+        const T cand = V.w[e] + A[(int64_t)u * ld + t];
+        if (less_lex(cand, e, best, be)) {
+            best = cand;
+            be = e;
+            to = u;
+        }
+    }
+#pragma unroll
+    for (int o = SUB / 2; o > 0; o >>= 1) {
+        const T b2 = __shfl_xor_sync(mask, best, o);
+        const int64_t e2 = __shfl_xor_sync(mask, be, o);
+        const int32_t t2 = __shfl_xor_sync(mask, to, o);
+        if (less_lex(b2, e2, best, be)) {
+            best = b2;
+            be = e2;
+            to = t2;
+        }
+    }
+    if (be == INT64_MAX) return -1;
+    x = to;
+    return be;
+}
+
+// hops: a warp per vertex, lanes over the boundary vertices (consecutive columns of the
+// neighbours' rows of APSP(C)).  An entry is (slot - first slot) << 16 | local target, or
+// kNoHop where either needs more than 16 bits (or no slot leads on).
+template <typename T>
+__global__ void __launch_bounds__(256) k_walk_hops(const View<T> V, const WalkCtx<T> W, uint32_t* __restrict__ hops) {
+    const int lane = threadIdx.x & 31;
+    const int64_t v = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (v >= V.n) return;
+    const int32_t c = V.comp[v], x = V.local[v], nb = V.nb[c];
+    const MatDesc d = V.descs[c];
+    const T* A = V.apsp + d.off;
+    const int64_t e0 = V.rp[v], e1 = V.rp[v + 1];
+    uint32_t* row = hops + W.toff[c] + (int64_t)x * nb;
+    for (int32_t t0 = 0; t0 < nb; t0 += 128) {
+        T best[4];
+        int64_t be[4];
+        int32_t to[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            best[q] = Inf<T>::value();
+            be[q] = INT64_MAX;
+            to[q] = 0;
+        }
+        for (int64_t e = e0; e < e1; ++e) {
+            const int32_t u = W.slots[e].x;
+            if (u < 0) continue;
+            const T we = V.w[e];
+            const T* Au = A + (int64_t)u * d.n;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int32_t t = t0 + 32 * q + lane;
+                if (t < nb) {
+                    const T cand = we + Au[t];
+                    if (less_lex(cand, e, best[q], be[q])) {
+                        best[q] = cand;
+                        be[q] = e;
+                        to[q] = u;
+                    }
+                }
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int32_t t = t0 + 32 * q + lane;
+            if (t < nb) {
+                const bool ok = be[q] != INT64_MAX && be[q] - e0 < 0xffff && to[q] < 0x10000;
+                row[t] = ok ? ((uint32_t)(be[q] - e0) << 16) | (uint32_t)to[q] : kNoHop;
+            }
+        }
+    }
+}
+
+// Walk inside component c from local vertex x to boundary vertex t along the hop table;
+// visit(slot, local vertex) each hop.  SUB lanes walk together (all of them call visit).
+template <typename T, int SUB, typename Visit>
+__device__ __forceinline__ bool walk_hops(const View<T>& V, const WalkCtx<T>& W, int32_t c, int32_t x, int32_t t,
+                                          int64_t limit, int g, unsigned mask, const Visit& visit) {
+    const int32_t nb = V.nb[c], vs = V.vstart[c];
+    const uint32_t* tab = W.hops + W.toff[c] + t;
+    for (int64_t step = 0; x != t; ++step) {
+        if (step >= limit) return false;
+        const uint32_t h = tab[(int64_t)x * nb];
+        if (h != kNoHop) {
+            const int32_t from = x;
+            x = (int32_t)(h & 0xffffu);
+            visit(from, (int64_t)(h >> 16), x);
+        } else {
+            const int32_t from = x;
+            const MatDesc d = V.descs[c];
+            const int64_t e = best_slot<T, SUB>(V, W, V.apsp + d.off, d.n, vs, x, t, g, mask);
+            if (e < 0) return false;
+            visit(from, e - V.rp[V.vorder[vs + from]], x);
+        }
+    }
+    return true;
+}
+
+// Walk through the boundary graph from boundary vertex (c, l) to (c2, l2), the whole warp
+// together: clique(c, l, y, nb) or edge(e) for every move (all lanes call them).  As
+// walk_boundary_graph: the move minimising dist_C(b, y) + D(y, b2) over the component's other
+// boundary vertices y or w(e) + D(u, b2) over the slots into other components, ties to the
+// smallest y, then to the smallest slot.
+template <typename T, typename Clique, typename Edge>
+__device__ __forceinline__ bool walk_bg(const View<T>& V, const WalkCtx<T>& W, int32_t c, int32_t l, int32_t c2,
+                                        int32_t l2, int64_t limit, int lane, const Clique& clique, const Edge& edge) {
+    constexpr int H = 8;  // boundary vertices held per lane: components of up to 256
+    const uint32_t kinf = key_of(Inf<T>::value());
+    const int32_t s2 = V.bg_off[c2] + l2;
+    const int64_t p2 = V.bgpos[s2];
+    const T* Drow = V.D + p2 * V.N;
+    auto dist = [&](int64_t p) {  // D(p, p2)
+        return (p >> 7) == (p2 >> 7) ? V.D[p * V.N + p2] : Drow[p];
+    };
+    int64_t step = 0;
+    bool fresh = true;
+    T dv[H];
+    int32_t nb = 0, off = 0, ld = 0;
+    const T* A = nullptr;
+    for (;;) {
+        if (c == c2 && l == l2) return true;
+        if (step++ >= limit) return false;
+        if (fresh) {  // another component: its slots' distances to b2
+            nb = V.nb[c];
+            off = V.bg_off[c];
+            const MatDesc d = V.descs[c];
+            A = V.apsp + d.off;
+            ld = d.n;
+#pragma unroll
+            for (int q = 0; q < H; ++q) {
+                const int32_t y = lane + 32 * q;
+                dv[q] = y < nb ? dist(V.bgpos[off + y]) : Inf<T>::value();
+            }
+            fresh = false;
+        }
+        const int2 er = W.srange[off + l];
+        const T* Ab = A + (int64_t)l * ld;
+        uint32_t bk = kinf, bi = 0xffffffffu;
+        T av[H];
+#pragma unroll
+        for (int q = 0; q < H; ++q) {
+            const int32_t y = lane + 32 * q;
+            av[q] = y < nb ? Ab[y] : Inf<T>::value();
+        }
+        // the slots into other components (the loads above are in flight meanwhile)
+        uint32_t ek = kinf, ei = 0xffffffffu;
+        for (int32_t e = er.x + lane; e < er.y; e += 32) {
+            const int2 s = W.slots[e];
+            if (s.x >= 0 || s.x == INT32_MIN) continue;
+            const uint32_t k = key_of((T)(V.w[e] + dist(s.y)));
+            if (k < ek) {
+                ek = k;
+                ei = 0x80000000u | (uint32_t)e;
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < H; ++q) {
+            const int32_t y = lane + 32 * q;
+            if (y < nb && y != l) {
+                const uint32_t k = key_of((T)(av[q] + dv[q]));
+                if (k < bk) {
+                    bk = k;
+                    bi = (uint32_t)y;
+                }
+            }
+        }
+        for (int32_t y = lane + 32 * H; y < nb; y += 32) {  // (wider components)
+            if (y == l) continue;
+            const uint32_t k = key_of((T)(Ab[y] + dist(V.bgpos[off + y])));
+            if (k < bk) {
+                bk = k;
+                bi = (uint32_t)y;
+            }
+        }
+        if (ek < bk) {
+            bk = ek;
+            bi = ei;
+        }
+        const uint32_t mk = __reduce_min_sync(0xffffffffu, bk);
+        if (mk >= kinf) return false;
+        const uint32_t mi = __reduce_min_sync(0xffffffffu, bk == mk ? bi : 0xffffffffu);
+        if (mi & 0x80000000u) {
+            const int32_t e = (int32_t)(mi & 0x7fffffffu);
+            const int32_t s = ~W.slots[e].x;
+            edge(e, s);
+            c = W.scomp[s];
+            l = s - V.bg_off[c];
+            fresh = true;
+        } else {
+            clique(c, l, (int32_t)mi, nb);
+            l = (int32_t)mi;
+        }
+    }
+}
+
+}  // namespace
+}  // namespace spq
