@@ -386,6 +386,23 @@ __global__ void __launch_bounds__(256) k_bs_place(const BsMat<T>* __restrict__ m
     }
 }
 
+// The order of a launch with no more tiles than the GPU holds CTAs: every tile is taken at
+// once, so the runs' order (row blocks from the last) serves, in strips; no counting.
+template <typename T>
+__global__ void __launch_bounds__(256) k_bs_few(const BsMat<T>* __restrict__ mats, const BsRun* __restrict__ runs,
+                                                int32_t nruns, int64_t nitems, BsItem* __restrict__ items,
+                                                unsigned long long* __restrict__ nout) {
+    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (t == 0) *nout = (unsigned long long)nitems * BS_STRIPS;
+    if (t >= nitems) return;
+    const BsRun ru = runs[bs_run_of(runs, nruns, t)];
+    BsItem it = bs_item_of(ru, mats[ru.mat].nR, t);
+    for (int q = 0; q < BS_STRIPS; ++q) {
+        it.strip = (uint16_t)q;
+        items[BS_STRIPS * t + q] = it;
+    }
+}
+
 // K(R) of row block blockIdx.x of matrix blockIdx.y as ascending column indices at
 // klist[koff ..), padded to a multiple of KC with copies of its first entry (their panel
 // rows are infinite, so they change nothing).
@@ -812,9 +829,9 @@ cudaError_t bs_enqueue(const BsPlan<T>& p, uint32_t* err, uint32_t* exact, std::
     const uint4* masks = static_cast<const uint4*>(p.masks);
     const BsRun* runs = static_cast<const BsRun*>(p.runs);
     k_klist<T><<<dim3(p.nRmax, p.nmat), T_, 0, st>>>(mats, masks, p.fblk, p.fcnt, p.kcnt, p.koff, p.klist);
-    k_bs_levels<T><<<p.nmat, 32, (size_t)p.nRmax * 4, st>>>(mats, p.fblk, p.fcnt, p.level);
-    count_launches(2);
+    count_launches(1);
     cudaError_t e = cudaGetLastError();
+    bool levels = false;
     const size_t psm = sizeof(PanelSmem<T>);
     const int grid = sms_e() * SPQ_FW_MIN_CTAS;
     for (size_t l = 0; l < p.launches.size() && e == cudaSuccess; ++l) {
@@ -834,11 +851,22 @@ cudaError_t bs_enqueue(const BsPlan<T>& p, uint32_t* err, uint32_t* exact, std::
         uint32_t* used = bins + nbins;
         unsigned long long* nout = reinterpret_cast<unsigned long long*>(used + nbins);
         const unsigned ig = (unsigned)std::min<int64_t>((L.nit + 255) / 256, 4 * sms_e());
-        cudaMemsetAsync(bins, 0, (size_t)nbins * 8, st);
-        k_bs_count<T><<<ig, 256, 0, st>>>(mats, lr, nlr, L.nit, p.level, bins);
-        k_bs_scan<<<1, 1024, 0, st>>>(bins, nbins, (uint32_t)grid, nout);
-        k_bs_place<T><<<ig, 256, 0, st>>>(mats, lr, nlr, L.nit, p.level, bins, used, items);
-        count_launches(3);
+        if (L.nit <= grid) {
+            // (measured on a 1,000-vertex graph: the counting's five launches cost 4% of the
+            //  build, more than the order gives)
+            k_bs_few<T><<<(unsigned)((L.nit + 255) / 256), 256, 0, st>>>(mats, lr, nlr, L.nit, items, nout);
+            count_launches(1);
+        } else {
+            if (!levels) {
+                k_bs_levels<T><<<p.nmat, 32, (size_t)p.nRmax * 4, st>>>(mats, p.fblk, p.fcnt, p.level);
+                levels = true;
+            }
+            cudaMemsetAsync(bins, 0, (size_t)nbins * 8, st);
+            k_bs_count<T><<<ig, 256, 0, st>>>(mats, lr, nlr, L.nit, p.level, bins);
+            k_bs_scan<<<1, 1024, 0, st>>>(bins, nbins, (uint32_t)grid, nout);
+            k_bs_place<T><<<ig, 256, 0, st>>>(mats, lr, nlr, L.nit, p.level, bins, used, items);
+            count_launches(4);
+        }
         cudaMemsetAsync(p.counter, 0, 8, st);
         if (ev) cudaEventRecord((*ev)[2 * l], st);
         kern<<<grid, NTH, psm, st>>>(mats, items, nout, p.koff, p.kcnt, p.klist,
