@@ -339,7 +339,19 @@ template <typename T>
 cudaError_t launch_query(const QueryCtx<T>& ctx, const int32_t* pairs, int64_t q, void* out, bool out_f32,
                          uint32_t k, uint32_t* scratch, cudaStream_t st);
 
+// Distances with their witnesses (spq_query_saved) of a large batch, grouped by ordered
+// component pair; every |B(C)| at most query_blocks_max_nb(), k <= 65535.  T: the tables' type.
+int64_t query_saved_scratch_words(int64_t q);
+template <typename T>
+cudaError_t launch_query_saved_grouped(const QueryCtx<T>& ctx, const int32_t* pairs, int64_t q, T* dist,
+                                       int32_t* saved, uint32_t k, uint32_t* scratch, cudaStream_t st);
+
 // ---- query_blocks.cu ----
+int64_t query_witness_scratch_words(int64_t q);
+template <typename T>
+cudaError_t launch_query_witness(const QueryCtx<T>& ctx, const int32_t* pairs, int64_t q, T* dist, int32_t* saved,
+                                 uint32_t k, const uint32_t* keys, const uint32_t* idx, uint32_t* scratch,
+                                 cudaStream_t st);
 // Largest block side (|B1| or |B2|) the staged grouped kernel handles; larger blocks take
 // the gathering kernel of query.cu.
 int32_t query_blocks_max_nb();

@@ -491,6 +491,15 @@ __global__ void __launch_bounds__(GTH) k_paths_hops(const View<T> V, const WalkC
     }
 }
 
+constexpr int64_t kSavedSlice = 1 << 22;
+
+bool capturing(cudaStream_t st) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cap) == cudaSuccess) return cap != cudaStreamCaptureStatusNone;
+    cudaGetLastError();
+    return true;
+}
+
 int grad_sms() {
     static int n = 0;
     if (n == 0) {
@@ -557,17 +566,13 @@ bool walk_records(const spq_handle* h, bool want_flow, cudaStream_t st, WalkCtx<
 
 // Whether q walks pay for the records: a hop searched on the spot costs about 0.17 ns of the
 // GPU (measured: 1M pairs on 2^18 vertices 86 ms, 100k on 2^14 1.96 ms; the hops of a pair
-// grow with sqrt(n)), the records about 30 us plus 8 ps per table entry.  Never inside a
+// grow with sqrt(n)), the records about 60 us plus 8 ps per table entry.  Never inside a
 // stream capture: a captured call allocates nothing.
 bool walks_pay(const spq_handle* h, int64_t q, cudaStream_t st) {
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
-        cudaGetLastError();
-        return false;
-    }
+    if (capturing(st)) return false;
     double nt = 0.0;
     for (int32_t c = 0; c < h->k; ++c) nt += (double)h->h_csize[c] * h->h_nb[c];
-    return 21.0 * (double)q * sqrt((double)h->n) > 3.75e6 + nt;
+    return 21.0 * (double)q * sqrt((double)h->n) > 7.5e6 + nt;
 }
 
 template <typename T>
@@ -622,6 +627,38 @@ spq_status spq_query_saved(spq_handle* h, const int32_t* pairs, int64_t q, void*
     if (!on_device(pairs) || !on_device(dist_out) || !on_device(saved)) return SPQ_EINVAL;
     if (((uintptr_t)pairs & 7u) || ((uintptr_t)saved & 7u) || ((uintptr_t)dist_out & 3u)) return SPQ_EINVAL;
     cudaStream_t st = (cudaStream_t)stream;
+    // Large batches grouped by component pair, each block of the boundary matrix read once per
+    // group (1M pairs on 2^18 vertices: a warp per pair 29.5 ms, most of it the block's rows
+    // from DRAM again for every pair).  From 4,096 pairs, as spq_query, and 9e7 updates (the
+    // sort's launches take about 60 us, in which a warp per pair does that many); at most
+    // kSavedSlice pairs at a time (39 words of scratch a pair).  Not inside a stream capture: a
+    // captured call allocates nothing.
+    const double nb_mean = (double)h->nbg / h->k;
+    if (q >= 4096 && (double)q * nb_mean * nb_mean >= 9e7 && h->k <= 65535 && h->max_nb <= query_blocks_max_nb() && !capturing(st)) {
+        uint32_t* scratch = nullptr;
+        const int64_t slice = std::min(q, kSavedSlice);
+        if (scratch_alloc((void**)&scratch, (size_t)query_saved_scratch_words(slice) * 4, st) == cudaSuccess) {
+            QueryCtx<int32_t> ci;
+            QueryCtx<float> cf;
+            bool f32store = false, out_f32 = false;
+            int32_t k = 0;
+            const bool ran = h->qprof_ran;  // (the query profile covers spq_query only)
+            handle_query_view(h, &ci, &cf, &f32store, &out_f32, &k);
+            h->qprof_ran = ran;
+            cudaError_t e = cudaSuccess;
+            for (int64_t a = 0; a < q && e == cudaSuccess; a += slice) {
+                const int64_t n = std::min(slice, q - a);
+                e = f32store ? launch_query_saved_grouped<float>(cf, pairs + 2 * a, n, (float*)dist_out + a,
+                                                                 saved + 2 * a, (uint32_t)k, scratch, st)
+                             : launch_query_saved_grouped<int32_t>(ci, pairs + 2 * a, n, (int32_t*)dist_out + a,
+                                                                   saved + 2 * a, (uint32_t)k, scratch, st);
+            }
+            cudaFreeAsync(scratch, st);
+            if (e != cudaSuccess) note_cuda_error(e);
+            return e == cudaSuccess ? SPQ_OK : SPQ_ECUDA;
+        }
+        cudaGetLastError();  // (no room: a warp per pair needs none)
+    }
     int64_t blocks = (q + 7) / 8;
     const int64_t cap = (int64_t)grad_sms() * 16;
     if (blocks > cap) blocks = cap;

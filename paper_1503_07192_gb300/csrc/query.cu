@@ -161,15 +161,16 @@ constexpr int GSEGCAP = 1024;         // longest segment (a power of two)
 // same operations in both.
 constexpr int GCOLS = 256;            // block columns per pass (two groups of 128)
 
+// (ordered: the key of (comp(v1), comp(v2)) as the pair is given, not of the unordered pair)
 __global__ void k_query_keys(const int2* __restrict__ pairs, int64_t q, int32_t n, const int32_t* __restrict__ comp,
-                             uint32_t k, uint32_t* __restrict__ keys, uint32_t* __restrict__ idx) {
+                             uint32_t k, uint32_t* __restrict__ keys, uint32_t* __restrict__ idx, bool ordered) {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= q) return;
     int2 p = pairs[i];
     uint32_t key = k * k;  // sentinel: invalid pair, sorted last
     if (p.x >= 0 && p.x < n && p.y >= 0 && p.y < n) {
         uint32_t a = (uint32_t)comp[p.x], b = (uint32_t)comp[p.y];
-        key = a <= b ? a * k + b : b * k + a;
+        key = a <= b || ordered ? a * k + b : b * k + a;
     }
     keys[i] = key;
     idx[i] = (uint32_t)i;
@@ -520,7 +521,7 @@ cudaError_t launch_query(const QueryCtx<T>& ctx, const int32_t* pairs, int64_t q
         uint32_t* k1 = scratch + 2 * q;
         uint32_t* v1 = scratch + 3 * q;
         uint32_t* hist = scratch + 4 * q;
-        k_query_keys<<<(unsigned)((q + 255) / 256), 256, 0, st>>>(p2, q, ctx.n, ctx.comp, k, keys, vals);
+        k_query_keys<<<(unsigned)((q + 255) / 256), 256, 0, st>>>(p2, q, ctx.n, ctx.comp, k, keys, vals, false);
         count_launches(1);
         int bits = 0;
         const uint64_t mx = (uint64_t)k * k;
@@ -576,6 +577,30 @@ cudaError_t launch_query(const QueryCtx<T>& ctx, const int32_t* pairs, int64_t q
     return cudaGetLastError();
 }
 
+int64_t query_saved_scratch_words(int64_t q) { return 4 * q + radix_hist_words(q) + 4 + query_witness_scratch_words(q); }
+
+template <typename T>
+cudaError_t launch_query_saved_grouped(const QueryCtx<T>& ctx, const int32_t* pairs, int64_t q, T* dist,
+                                       int32_t* saved, uint32_t k, uint32_t* scratch, cudaStream_t st) {
+    uint32_t *keys = scratch, *vals = scratch + q, *k1 = scratch + 2 * q, *v1 = scratch + 3 * q;
+    uint32_t* hist = scratch + 4 * q;
+    k_query_keys<<<(unsigned)((q + 255) / 256), 256, 0, st>>>(reinterpret_cast<const int2*>(pairs), q, ctx.n, ctx.comp,
+                                                              k, keys, vals, true);
+    count_launches(1);
+    int bits = 0;
+    const uint64_t mx = (uint64_t)k * k;
+    while (bits < 32 && (mx >> bits)) ++bits;
+    bool in_k1 = false;
+    const cudaError_t e = radix_sort_pairs(keys, vals, k1, v1, hist, q, bits, &in_k1, st);
+    if (e != cudaSuccess) return e;
+    return launch_query_witness<T>(ctx, pairs, q, dist, saved, k, in_k1 ? k1 : keys, in_k1 ? v1 : vals,
+                                   hist + radix_hist_words(q) + 4, st);
+}
+
+template cudaError_t launch_query_saved_grouped<int32_t>(const QueryCtx<int32_t>&, const int32_t*, int64_t, int32_t*,
+                                                         int32_t*, uint32_t, uint32_t*, cudaStream_t);
+template cudaError_t launch_query_saved_grouped<float>(const QueryCtx<float>&, const int32_t*, int64_t, float*,
+                                                       int32_t*, uint32_t, uint32_t*, cudaStream_t);
 template cudaError_t launch_query<int32_t>(const QueryCtx<int32_t>&, const int32_t*, int64_t, void*, bool, uint32_t,
                                            uint32_t*, cudaStream_t);
 template cudaError_t launch_query<float>(const QueryCtx<float>&, const int32_t*, int64_t, void*, bool, uint32_t,

@@ -39,6 +39,7 @@ constexpr int QB_MAXP = 64;    // pairs per item
 constexpr int QB_UMAX = 2;     // 4 x 4 tiles per thread
 constexpr int QB_CTAS = 3;     // CTAs per SM
 constexpr int QB_PMAX = 512;   // widest block side (rows or columns) staged here
+constexpr int QB_MW = QB_PMAX / 32;  // words of a column mask
 constexpr int QB_PREG = (2 * QB_PMAX) / (2 * QB_TH);  // prefetched positions per thread and side
 
 // One item: its pairs (a run of sorted positions) and the shape of its staged work, set
@@ -198,9 +199,6 @@ __device__ __forceinline__ int32_t res_reset() {
     return std::is_same<T, float>::value ? 0x7f800000 : 0x7fffffff;
 }
 
-__device__ __forceinline__ int32_t qb_addmin(int32_t a, int32_t b, int32_t t) { return __viaddmin_s32(a, b, t); }
-__device__ __forceinline__ float qb_addmin(float a, float b, float t) { return fminf(t, a + b); }
-
 // Queue the asynchronous copies of chunk ch of item p (per-item records in parity pp)
 // into buffer b: the block rows gathered from the matrix (warps over rows, lanes over
 // columns) and the pieces dist_C1(v1, rows) of every pair, spread over all threads.
@@ -259,6 +257,9 @@ __device__ __forceinline__ void qb_issue(QbSmem<T>& sm, int b, int pp, const QbC
 // sum has no term at or above 2^24); an answer at or above it (a long or an unreachable
 // pair) is listed in fb and recomputed exactly in int32 by k_qb_fallback.  No subnormal
 // is flushed: the kernel is built without fast math or .ftz.
+// MODE: 0 int32 answers, 2 float answers, 3 the witness form (spq_query_saved): per sorted
+// position the minimum over (b1, b2) alone (out) and the mask of the columns b2 that attain
+// it (fb, QB_MW words a position).
 template <typename T, int MODE, bool ENC>
 __global__ void __launch_bounds__(QB_TH, QB_CTAS)
     k_qb_blocks(const QbCtx<T> c, const QItem* __restrict__ items, const uint32_t* __restrict__ nitems_p,
@@ -267,6 +268,7 @@ __global__ void __launch_bounds__(QB_TH, QB_CTAS)
     using CT = typename std::conditional<ENC, float, T>::type;  // the arithmetic's type
     extern __shared__ __align__(16) unsigned char qb_raw[];
     QbSmem<T>& sm = *reinterpret_cast<QbSmem<T>*>(qb_raw);
+    __shared__ uint32_t mask[MODE == 3 ? QB_MAXP : 1][MODE == 3 ? QB_MW : 1];
     const int tid = threadIdx.x;
     const uint32_t nitems = *nitems_p;
     const uint32_t G = gridDim.x;
@@ -346,7 +348,7 @@ __global__ void __launch_bounds__(QB_TH, QB_CTAS)
                 const T* sp = sm.s[b] + 4 * h;
 #pragma unroll 1
                 for (int32_t qq = r; qq < nq; qq += Rs) {
-                    if constexpr (ENC) {
+                    if constexpr (std::is_same<CT, float>::value) {
                         float4 av[4], sv[4];
 #pragma unroll
                         for (int i = 0; i < 4; ++i) av[i] = *reinterpret_cast<const float4*>(ap + i * chr + 4 * qq);
@@ -394,7 +396,7 @@ __global__ void __launch_bounds__(QB_TH, QB_CTAS)
                             for (int j = 0; j < 4; ++j)
 #pragma unroll
                                 for (int e = 0; e < 4; ++e)
-                                    acc[k][i][e] = qb_addmin(av[i][j], sv[j][e], acc[k][i][e]);
+                                    acc[k][i][e] = __viaddmin_s32(av[i][j], sv[j][e], acc[k][i][e]);
                     }
                 }
             }
@@ -402,6 +404,16 @@ __global__ void __launch_bounds__(QB_TH, QB_CTAS)
         if (!next_same) {
             // ---- the item's end: + dist_C2(b2, v2), min over the columns, per pair ----
             const int32_t count = cur.count, nb2 = cur.nb2;
+            if constexpr (MODE == 3)
+                for (int32_t x = tid; x < count * QB_MW; x += QB_TH) mask[x / QB_MW][x % QB_MW] = 0u;
+            // (padding columns past |B2| hold no distance: skipped)
+            auto row2 = [&](int32_t u, int32_t h, CT (&c4)[4]) {
+                const int4 cv = __ldg(reinterpret_cast<const int4*>(c.apsp + sm.a2off[par][u] + 4 * h));
+                c4[0] = *reinterpret_cast<const CT*>(&cv.x);
+                c4[1] = *reinterpret_cast<const CT*>(&cv.y);
+                c4[2] = *reinterpret_cast<const CT*>(&cv.z);
+                c4[3] = *reinterpret_cast<const CT*>(&cv.w);
+            };
 #pragma unroll
             for (int k = 0; k < QB_UMAX; ++k) {
                 if (unit[k] >= 0) {
@@ -410,10 +422,8 @@ __global__ void __launch_bounds__(QB_TH, QB_CTAS)
                     for (int i = 0; i < 4; ++i) {
                         const int32_t u = 4 * g + i;
                         if (u < count) {
-                            const int4 cv = __ldg(reinterpret_cast<const int4*>(c.apsp + sm.a2off[par][u] + 4 * h));
-                            const CT c4[4] = {*reinterpret_cast<const CT*>(&cv.x), *reinterpret_cast<const CT*>(&cv.y),
-                                              *reinterpret_cast<const CT*>(&cv.z), *reinterpret_cast<const CT*>(&cv.w)};
-                            // (padding columns past |B2| hold no distance: skipped)
+                            CT c4[4];
+                            row2(u, h, c4);
                             CT v = acc[k][i][0] + c4[0];
 #pragma unroll
                             for (int e = 1; e < 4; ++e) {
@@ -425,8 +435,41 @@ __global__ void __launch_bounds__(QB_TH, QB_CTAS)
                     }
                 }
             }
+            if constexpr (MODE == 3) {
+                // the columns whose sum is the minimum.  (A row split's sum equal to it belongs
+                // to a column whose full sum is: minimum <= full sum <= the split's sum.)
+                __syncthreads();
+#pragma unroll
+                for (int k = 0; k < QB_UMAX; ++k) {
+                    if (unit[k] >= 0) {
+                        const int32_t g = (unit[k] >> 20) & 0xff, h = unit[k] & 0xfffff;
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            const int32_t u = 4 * g + i;
+                            if (u < count) {
+                                const int32_t best = sm.res[par][u];
+                                CT c4[4];
+                                row2(u, h, c4);
+                                uint32_t bits = 0u;
+#pragma unroll
+                                for (int e = 0; e < 4; ++e)
+                                    if (4 * h + e < nb2 && enc_min<CT>(acc[k][i][e] + c4[e]) == best) bits |= 1u << e;
+                                if (bits) atomicOr(&mask[u][h >> 3], bits << (4 * (h & 7)));
+                            }
+                        }
+                    }
+                }
+            }
             __syncthreads();
-            if (tid < count) {
+            if constexpr (MODE == 3) {
+                if (tid < count) {
+                    ((T*)out)[cur.start + tid] = dec_min<T>(sm.res[par][tid]);
+                    sm.res[par][tid] = res_reset<CT>();
+                }
+                const int32_t nw = (nb2 + 31) >> 5;
+                for (int32_t x = tid; x < count * QB_MW; x += QB_TH)
+                    if (x % QB_MW < nw) fb[(int64_t)cur.start * QB_MW + x] = mask[x / QB_MW][x % QB_MW];
+            } else if (tid < count) {
                 const uint32_t qi = sm.qidx[par][tid];
                 const T z = sm.init[par][tid];
                 if constexpr (ENC) {
@@ -522,6 +565,92 @@ __global__ void __launch_bounds__(256) k_qb_fallback(const QueryCtx<int32_t> ctx
     }
 }
 
+// The witness form's last step, a warp per sorted position: of the columns attaining the
+// minimum, each with its first row b1 that attains t(b2) (read again from the matrix: a few
+// of the block's columns), the smallest (b1, b2); then the same-component distance, equal
+// and out-of-range pairs, as k_query_saved answers them.
+template <typename T>
+__global__ void __launch_bounds__(256) k_qb_witness(const QueryCtx<T> ctx, const int2* __restrict__ pairs,
+                                                    const uint32_t* __restrict__ keys,
+                                                    const uint32_t* __restrict__ idx, int64_t q, uint32_t k,
+                                                    const T* __restrict__ best_in, const uint32_t* __restrict__ masks,
+                                                    T* __restrict__ dist, int2* __restrict__ saved) {
+    const int lane = threadIdx.x & 31;
+    const T inf = Inf<T>::value();
+    for (int64_t p = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; p < q;
+         p += ((int64_t)gridDim.x * blockDim.x) >> 5) {
+        const uint32_t key = keys[p], qi = idx[p];
+        if (key >= k * k) {
+            if (lane == 0) {
+                dist[qi] = (T)-1;
+                saved[qi] = make_int2(-3, -3);
+                atomicOr(ctx.err, kErrPair);
+            }
+            continue;
+        }
+        const int2 pr = pairs[qi];
+        if (pr.x == pr.y) {
+            if (lane == 0) {
+                dist[qi] = T(0);
+                saved[qi] = make_int2(-2, -2);
+            }
+            continue;
+        }
+        const int32_t c1 = (int32_t)(key / k), c2 = (int32_t)(key % k);
+        const int32_t nb1 = ctx.nb[c1], nb2 = ctx.nb[c2];
+        const MatDesc d1 = ctx.descs[c1];
+        const T* A1 = ctx.apsp + d1.off + (int64_t)ctx.local[pr.x] * d1.n;
+        const int32_t* pos1 = ctx.bgpos + ctx.bg_off[c1];
+        const int32_t* pos2 = ctx.bgpos + ctx.bg_off[c2];
+        T best = inf;
+        unsigned long long sel = ~0ull;  // (b1 << 32) + b2
+        if (nb1 > 0 && nb2 > 0) {
+            const T b = best_in[p];
+            best = b < inf ? b : inf;
+        }
+        if (best < inf) {
+            const int32_t nw = (nb2 + 31) >> 5;
+            const uint32_t mw = lane < nw ? masks[p * QB_MW + lane] : 0u;
+            for (int32_t w = 0; w < nw; ++w) {
+                for (uint32_t bits = __shfl_sync(0xffffffffu, mw, w); bits; bits &= bits - 1u) {
+                    const int32_t j = 32 * w + __ffs(bits) - 1;
+                    const int64_t cp = pos2[j];
+                    const T* drow = ctx.D + cp * ctx.N;
+                    T t = inf;
+                    uint32_t ti = 0xffffffffu;
+                    for (int32_t i = lane; i < nb1; i += 32) {
+                        // (D is symmetric bit for bit outside its diagonal tiles: read along
+                        //  row b2 there)
+                        const int64_t rp = pos1[i];
+                        const T cand = A1[i] + ((rp / kTile == cp / kTile) ? ctx.D[rp * ctx.N + cp] : drow[rp]);
+                        if (cand < t) {
+                            t = cand;
+                            ti = (uint32_t)i;
+                        }
+                    }
+                    const int32_t tb = enc_min<T>(t);
+                    const int32_t mt = __reduce_min_sync(0xffffffffu, tb);
+                    const uint32_t mi = __reduce_min_sync(0xffffffffu, tb == mt ? ti : 0xffffffffu);
+                    const unsigned long long x = ((unsigned long long)mi << 32) | (uint32_t)j;
+                    if (x < sel) sel = x;
+                }
+            }
+        }
+        if (lane == 0) {
+            int2 sv = best < inf ? make_int2((int32_t)(sel >> 32), (int32_t)(sel & 0xffffffffull)) : make_int2(-3, -3);
+            if (c1 == c2) {
+                const T direct = A1[ctx.local[pr.y]];
+                if (direct <= best && direct < inf) {
+                    best = direct;
+                    sv = make_int2(-1, -1);
+                }
+            }
+            dist[qi] = best;
+            saved[qi] = sv;
+        }
+    }
+}
+
 // Per sorted position: the pair oriented so that v1 lies in the lower component, the
 // table rows of dist_C1(v1, .) and dist_C2(., v2), and the starting value of its answer:
 // 0 if v1 = v2, dist_C1(v1, v2) if both lie in one component, else infinity.  Pairs with
@@ -536,6 +665,7 @@ __global__ void k_qb_prep(const QueryCtx<T> ctx, const int2* __restrict__ pairs,
     if (p >= q) return;
     const uint32_t key = keys[p], qi = idx[p];
     if (key >= k * k) {
+        if (MODE == 3) return;  // (k_qb_witness answers it)
         if (MODE == 2)
             ((float*)out)[qi] = __int_as_float(0x7fc00000);
         else
@@ -556,7 +686,7 @@ __global__ void k_qb_prep(const QueryCtx<T> ctx, const int2* __restrict__ pairs,
     else if (c1 == c2)
         z = ctx.apsp[a1 + ctx.local[pr.y]];
     init[p] = z;
-    if (ctx.nb[c1] == 0 || ctx.nb[c2] == 0) {
+    if (MODE != 3 && (ctx.nb[c1] == 0 || ctx.nb[c2] == 0)) {
         if (MODE == 2)
             ((float*)out)[qi] = (float)z;
         else
@@ -733,6 +863,46 @@ cudaError_t launch_query_blocks(const QueryCtx<T>& ctx, const int32_t* pairs, in
     }
     return e;
 }
+
+int64_t query_witness_scratch_words(int64_t q) {
+    // the blocks kernel's records, the minima (1 word a pair) and the column masks
+    return query_blocks_scratch_words(q) + (1 + QB_MW) * q;
+}
+
+template <typename T>
+cudaError_t launch_query_witness(const QueryCtx<T>& ctx, const int32_t* pairs, int64_t q, T* dist, int32_t* saved,
+                                 uint32_t k, const uint32_t* keys, const uint32_t* idx, uint32_t* scratch,
+                                 cudaStream_t st) {
+    uint32_t* base = (uint32_t*)(((uintptr_t)scratch + 15) & ~(uintptr_t)15);
+    longlong2* rows = reinterpret_cast<longlong2*>(base);
+    T* init = reinterpret_cast<T*>(base + 4 * q);
+    const int64_t o_items = (5 * q + 3) & ~(int64_t)3;
+    QItem* items = reinterpret_cast<QItem*>(base + o_items);
+    uint32_t* nitems = base + o_items + 12 * q;
+    T* best = reinterpret_cast<T*>(nitems + 2);
+    uint32_t* masks = nitems + 2 + q;
+    const int2* p2 = reinterpret_cast<const int2*>(pairs);
+    cudaError_t e = cudaMemsetAsync(nitems, 0, 8, st);
+    if (e != cudaSuccess) return e;
+    const unsigned g = (unsigned)((q + 255) / 256);
+    k_qb_prep<T, 3><<<g, 256, 0, st>>>(ctx, p2, keys, idx, q, k, rows, init, nullptr);
+    k_qb_items<<<g, 256, 0, st>>>(keys, q, k, ctx.nb, items, nitems, nullptr);
+    count_launches(3);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    const QbCtx<T> c{ctx.apsp, ctx.D, ctx.N, ctx.bgpos, ctx.bg_off};
+    if ((e = launch_blocks_kernel<T, 3, false>(c, items, nitems, rows, init, idx, best, masks, nullptr, q, st)) !=
+        cudaSuccess)
+        return e;
+    const int64_t wb = std::min<int64_t>((q + 7) / 8, (int64_t)qb_sms() * 8);
+    k_qb_witness<T><<<(unsigned)wb, 256, 0, st>>>(ctx, p2, keys, idx, q, k, best, masks, dist, (int2*)saved);
+    return cudaGetLastError();
+}
+
+template cudaError_t launch_query_witness<int32_t>(const QueryCtx<int32_t>&, const int32_t*, int64_t, int32_t*,
+                                                   int32_t*, uint32_t, const uint32_t*, const uint32_t*, uint32_t*,
+                                                   cudaStream_t);
+template cudaError_t launch_query_witness<float>(const QueryCtx<float>&, const int32_t*, int64_t, float*, int32_t*,
+                                                 uint32_t, const uint32_t*, const uint32_t*, uint32_t*, cudaStream_t);
 
 template cudaError_t launch_query_blocks<int32_t>(const QueryCtx<int32_t>&, const int32_t*, int64_t, void*, bool,
                                                   uint32_t, const uint32_t*, const uint32_t*, uint32_t*, cudaStream_t);
