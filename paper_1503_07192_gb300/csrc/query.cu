@@ -127,6 +127,90 @@ __global__ void __launch_bounds__(QTH) k_query(const QueryCtx<T> ctx, const int2
     }
 }
 
+// One CTA per pair, for small batches: the eight warps share the block's rows, four columns a
+// lane and four rows of loads in flight, so a pair waits for its block once and not row after
+// row (a warp per pair: 256 pairs of 2^18 vertices 79 us, one pair alone about as long).  The
+// same sums and minima as k_query's.
+template <typename T, int MODE>
+__global__ void __launch_bounds__(QTH) k_query_cta(const QueryCtx<T> ctx, const int2* __restrict__ pairs,
+                                                   void* __restrict__ out) {
+    __shared__ T part[QTH / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const T inf = Inf<T>::value();
+    const int64_t qi = blockIdx.x;
+    const int2 pr = pairs[qi];
+    int32_t v = pr.x, w = pr.y;
+    if (v < 0 || v >= ctx.n || w < 0 || w >= ctx.n) {
+        if (threadIdx.x == 0) {
+            if (MODE == kOutF32)
+                ((float*)out)[qi] = __int_as_float(0x7fc00000);
+            else
+                ((int32_t*)out)[qi] = -1;
+            atomicOr(ctx.err, kErrPair);
+        }
+        return;
+    }
+    if (v == w) {
+        if (threadIdx.x == 0) {
+            if (MODE == kOutF32)
+                ((float*)out)[qi] = 0.0f;
+            else
+                ((int32_t*)out)[qi] = 0;
+        }
+        return;
+    }
+    int32_t c1 = ctx.comp[v], c2 = ctx.comp[w];
+    if (c1 > c2) {  // (from the lower-numbered component's side, as k_query)
+        const int32_t tv = v, tc = c1;
+        v = w;
+        w = tv;
+        c1 = c2;
+        c2 = tc;
+    }
+    const int32_t l2 = ctx.local[w];
+    const MatDesc d1 = ctx.descs[c1], d2 = ctx.descs[c2];
+    const int32_t nb1 = ctx.nb[c1], nb2 = ctx.nb[c2];
+    const T* A1 = ctx.apsp + d1.off + (int64_t)ctx.local[v] * d1.n;
+    const T* A2 = ctx.apsp + d2.off + (int64_t)l2 * d2.n;
+    const int32_t* pos1 = ctx.bgpos + ctx.bg_off[c1];
+    const int32_t* pos2 = ctx.bgpos + ctx.bg_off[c2];
+    T r = inf;
+    for (int32_t jb = 0; jb < nb2; jb += 128) {
+        T t[4], cj[4];
+        int32_t col[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int32_t j = jb + 32 * q + lane;
+            t[q] = inf;
+            cj[q] = j < nb2 ? A2[j] : inf;
+            col[q] = j < nb2 ? pos2[j] : 0;  // (past |B2|: a cell of the row, its sum infinite)
+        }
+#pragma unroll 4
+        for (int32_t i = warp; i < nb1; i += QTH / 32) {
+            const T a = A1[i];
+            const T* row = ctx.D + (int64_t)pos1[i] * ctx.N;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) t[q] = tmin(t[q], a + row[col[q]]);
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) r = tmin(r, t[q] + cj[q]);
+    }
+    r = warp_min(r);
+    if (lane == 0) part[warp] = r;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int x = 1; x < QTH / 32; ++x) r = tmin(r, part[x]);
+        if (c1 == c2) r = tmin(r, A1[l2]);
+        if (MODE == kOutI32)
+            ((int32_t*)out)[qi] = (int32_t)tmin<int32_t>((int32_t)r, SPQ_INF_I32);
+        else
+            ((float*)out)[qi] = (float)r;
+    }
+}
+
+// Largest batch answered a CTA per pair (a larger one fills the GPU with a warp per pair).
+constexpr int64_t kCtaQueries = 4096;
+
 int query_sms() {
     static int n = 0;
     if (n == 0) {
@@ -565,6 +649,14 @@ cudaError_t launch_query(const QueryCtx<T>& ctx, const int32_t* pairs, int64_t q
             for (auto& x : ev)
                 if (x) cudaEventDestroy(x);
         return e;
+    }
+    if (q <= kCtaQueries) {
+        if (!mode_f32 && !out_f32)
+            k_query_cta<T, kOutI32><<<(unsigned)q, QTH, 0, st>>>(ctx, p2, out);
+        else
+            k_query_cta<T, kOutF32><<<(unsigned)q, QTH, 0, st>>>(ctx, p2, out);
+        count_launches(1);
+        return cudaGetLastError();
     }
     int64_t blocks = (q + (QTH / 32) - 1) / (QTH / 32);
     int64_t cap = (int64_t)query_sms() * 16;
