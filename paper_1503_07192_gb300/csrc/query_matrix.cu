@@ -6,27 +6,37 @@
 // and then for every target v2 in C2
 //   dist = min over b2 of t(b2) + dist_C2(b2, v2), and dist_C1(v1, v2) if C1 = C2,
 // so a (source, target component) pair costs |B1||B2| updates once plus |B2| per target
-// instead of |B1||B2| per pair.  Sources and targets are sorted by component; one CTA
-// takes a target component and a group of eight sources: each warp computes t for its
-// source from the rows of dist_BG(B(C1), B(C2)) (read in place: the block of a source
-// component is shared by its sources through L2), the eight t rows stay in shared
-// memory, and every target of C2 is reduced against all of them, one target per lane, so
-// a target's row of APSP(C2) is read once per eight sources.
+// instead of |B1||B2| per pair.
+//
+// Stage 1 (k_matrix_t) is bound by the sources' rows of the boundary matrix (64 sources on
+// 2^18 vertices: 1.2 GB): a warp per source and target component, four rows x four columns
+// of loads in flight, t written once.  Stage 2 (k_matrix_out) is a min-plus matrix product
+// per target component, (sources x |B2|) by (|B2| x targets): tiles of 64 sources x 128
+// targets, both operands in rows along b2 staged by 16-byte asynchronous copies, so the
+// targets' rows of APSP(C2) are read once per 64 sources and in whole lines (one target per
+// lane, walking its own row, read a sector per value: 1.39 ms for 64 x 2^18 where the two
+// stages take 0.4); the tile goes out through shared memory, so that runs of neighbouring
+// targets are written together.  The targets are sorted by component; the tiles are listed
+// on the device, and nothing waits on the host.
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <type_traits>
 #include <vector>
 
 #include "common.cuh"
+#include "fw_tile.cuh"
 #include "handle.h"
 
 namespace spq {
 
 namespace {
 
-constexpr int MTH = 256;           // 8 warps
-constexpr int MSRC = MTH / 32;     // sources per batch: one per warp
-constexpr int MCOLS = 256;         // block columns per pass (8 per lane)
+constexpr int MTH = 256;
+constexpr int MT = 128;      // targets per tile: 16 groups of 8
+constexpr int MS = 64;       // sources per tile: 16 groups of 4
+constexpr int MK = 32;       // boundary vertices per staged chunk
+constexpr int MLD = MK + 4;  // row stride in shared memory: 16-byte rows on different banks
 
 template <typename T>
 __device__ __forceinline__ T tmin2(T a, T b) {
@@ -34,11 +44,11 @@ __device__ __forceinline__ T tmin2(T a, T b) {
 }
 __device__ __forceinline__ int32_t add_min(int32_t a, int32_t b, int32_t t) { return __viaddmin_s32(a, b, t); }
 __device__ __forceinline__ float add_min(float a, float b, float t) { return fminf(t, a + b); }
-template <typename T>
-__device__ __forceinline__ T warp_min2(T x) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) x = tmin2(x, __shfl_xor_sync(0xffffffffu, x, o));
-    return x;
+
+// Column of t where component c's values start: a multiple of 4, the components apart
+// (f(x) = x rounded up to 4 is at most x + 3).
+__device__ __forceinline__ int64_t t_off(const int32_t* __restrict__ bg_off, int32_t c) {
+    return ((int64_t)bg_off[c] + 3 * (int64_t)c + 3) & ~(int64_t)3;
 }
 
 // key = component of the vertex (k for an id out of range: sorted last), val = position
@@ -51,162 +61,226 @@ __global__ void k_comp_keys(const int32_t* __restrict__ ids, int64_t n, int32_t 
     vals[i] = (uint32_t)i;
 }
 
-// flags[i] = 1 where a run of equal sorted keys starts (flags[n] = 0)
-__global__ void k_run_heads(const uint32_t* __restrict__ keys, int64_t n, uint32_t* __restrict__ flags) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i > n) return;
-    flags[i] = (i < n && (i == 0 || keys[i] != keys[i - 1])) ? 1u : 0u;
+// A tile of the sorted targets: positions [start, start + count) of component c (k: ids out
+// of range).
+struct MTile {
+    uint32_t c, start, count, pad_;
+};
+
+// The tiles of every component (thread c): its run of the sorted keys by two binary
+// searches, cut into pieces of MT; cnt[c] = the run's length.
+__global__ void k_matrix_tiles(const uint32_t* __restrict__ keys, int64_t n, uint32_t k, MTile* __restrict__ tiles,
+                               uint32_t* __restrict__ ntiles, uint32_t* __restrict__ cnt) {
+    const uint32_t c = blockIdx.x * blockDim.x + threadIdx.x;
+    if (c > k) return;
+    auto lower = [&](uint32_t x) {  // first position with keys >= x
+        int64_t lo = 0, hi = n;
+        while (lo < hi) {
+            const int64_t mid = (lo + hi) >> 1;
+            if (keys[mid] < x) lo = mid + 1; else hi = mid;
+        }
+        return lo;
+    };
+    const int64_t a = lower(c), b = lower(c + 1);
+    cnt[c] = (uint32_t)(b - a);
+    if (a == b) return;
+    const uint32_t m = (uint32_t)((b - a + MT - 1) / MT), at = atomicAdd(ntiles, m);
+    for (uint32_t i = 0; i < m; ++i)
+        tiles[at + i] = MTile{c, (uint32_t)(a + (int64_t)i * MT), (uint32_t)std::min<int64_t>(MT, b - a - (int64_t)i * MT), 0u};
 }
 
-// after the exclusive scan of flags: run r starts at start[r], has key rkey[r]; start[nrun] = n
-__global__ void k_run_starts(const uint32_t* __restrict__ keys, const uint32_t* __restrict__ scanned, int64_t n,
-                             uint32_t* __restrict__ start, uint32_t* __restrict__ rkey) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i > n) return;
-    if (i == n) {
-        start[scanned[n]] = (uint32_t)n;
-    } else if (i == 0 || keys[i] != keys[i - 1]) {
-        start[scanned[i]] = (uint32_t)i;
-        rkey[scanned[i]] = keys[i];
+// Stage 1: t of the sources sid[s0 .. s0 + ns) for the components with targets, a warp per
+// (source, component); values past |B2| up to a multiple of 4 are infinite.
+template <typename T>
+__global__ void __launch_bounds__(MTH) k_matrix_t(const QueryCtx<T> ctx, uint32_t k, const int32_t* __restrict__ sid,
+                                                  int64_t s0, int64_t ns, const uint32_t* __restrict__ cnt,
+                                                  int64_t ldt, T* __restrict__ t) {
+    const int lane = threadIdx.x & 31;
+    const T inf = Inf<T>::value();
+    const int64_t nw = ((int64_t)gridDim.x * MTH) >> 5;
+    for (int64_t x = ((int64_t)blockIdx.x * MTH + threadIdx.x) >> 5; x < ns * k; x += nw) {
+        const int64_t s = x / k;
+        const int32_t c2 = (int32_t)(x - s * k);
+        if (cnt[c2] == 0) continue;
+        const int32_t v1 = sid[s0 + s];
+        if (v1 < 0 || v1 >= ctx.n) continue;
+        const int32_t c1 = ctx.comp[v1];
+        const MatDesc d1 = ctx.descs[c1];
+        const int32_t nb1 = ctx.nb[c1], nb2 = ctx.nb[c2], nb4 = (nb2 + 3) & ~3;
+        const int32_t* pos1 = ctx.bgpos + ctx.bg_off[c1];
+        const int32_t* pos2 = ctx.bgpos + ctx.bg_off[c2];
+        const T* a1 = ctx.apsp + d1.off + (int64_t)ctx.local[v1] * d1.n;
+        T* tr = t + s * ldt + t_off(ctx.bg_off, c2);
+        for (int32_t jb = 0; jb < nb4; jb += 128) {
+            int32_t col[4];
+            T y[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int32_t j = jb + 32 * q + lane;
+                col[q] = j < nb2 ? pos2[j] : -1;
+                y[q] = inf;
+            }
+            for (int32_t ib = 0; ib < nb1; ib += 32) {
+                const T areg = ib + lane < nb1 ? a1[ib + lane] : inf;
+                const int32_t preg = ib + lane < nb1 ? pos1[ib + lane] : 0;
+                const int iend = (nb1 - ib) < 32 ? (nb1 - ib) : 32;
+#pragma unroll 4
+                for (int ii = 0; ii < iend; ++ii) {
+                    const T a = __shfl_sync(0xffffffffu, areg, ii);
+                    const T* drow = ctx.D + (int64_t)__shfl_sync(0xffffffffu, preg, ii) * ctx.N;
+#pragma unroll
+                    for (int q = 0; q < 4; ++q)
+                        if (col[q] >= 0) y[q] = add_min(a, drow[col[q]], y[q]);
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int32_t j = jb + 32 * q + lane;
+                if (j < nb4) tr[j] = y[q];
+            }
+        }
     }
 }
 
-template <typename T, bool OUT_F32>
-__device__ __forceinline__ void put(void* out, int64_t at, T v) {
-    if (OUT_F32)
-        ((float*)out)[at] = (float)v;
-    else
-        ((int32_t*)out)[at] = (int32_t)tmin2<int32_t>((int32_t)v, SPQ_INF_I32);
-}
+template <typename T>
+struct MSmem {
+    union {
+        struct {
+            T a[2][MT][MLD];  // the targets' rows of APSP(C2)
+            T t[2][MS][MLD];  // the sources' rows of t
+        };
+        T out[MS][MT + 1];
+    };
+    int32_t tv[MT];        // the targets' vertices
+    uint32_t tp[MT];       // and positions in the caller's list
+    int32_t sv[MS];        // the sources' vertices (-1: out of range)
+    int64_t arow[MT];
+};
 
-// Item (target run jr, group of MSRC consecutive sources in component order).
+// Stage 2: items (target tile, group of MS sources), persistent.
 template <typename T, bool OUT_F32>
-__global__ void __launch_bounds__(MTH)
-    k_query_matrix(const QueryCtx<T> ctx, uint32_t k, const int32_t* __restrict__ sid,
-                   const uint32_t* __restrict__ sval, int64_t ns, const int32_t* __restrict__ tid_,
-                   const uint32_t* __restrict__ tval, const uint32_t* __restrict__ tstart,
-                   const uint32_t* __restrict__ tkey, uint32_t ntrun, int64_t nt, int32_t ldt,
-                   void* __restrict__ out) {
+__global__ void __launch_bounds__(MTH, 2)
+    k_matrix_out(const QueryCtx<T> ctx, uint32_t k, const int32_t* __restrict__ sid, int64_t s0, int64_t ns,
+                 const int32_t* __restrict__ tid_, const uint32_t* __restrict__ tval, const MTile* __restrict__ tiles,
+                 const uint32_t* __restrict__ ntiles_p, int64_t nt, int64_t ldt, const T* __restrict__ t,
+                 void* __restrict__ out) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    T* tb = reinterpret_cast<T*>(smem_raw);  // t of the group's sources: [MSRC][ldt]
-    __shared__ int32_t srcv[MSRC];           // the group's source vertices (-1: out of range)
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    MSmem<T>& sm = *reinterpret_cast<MSmem<T>*>(smem_raw);
+    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
     const T inf = Inf<T>::value();
-    const int64_t ngroups = (ns + MSRC - 1) / MSRC;
-    for (int64_t item = blockIdx.x; item < ngroups * ntrun; item += gridDim.x) {
-        const uint32_t jr = (uint32_t)(item % ntrun);
-        const int64_t sb = (item / ntrun) * MSRC;
-        const int nsrc = (int)((ns - sb) < MSRC ? (ns - sb) : MSRC);
-        const uint32_t c2 = tkey[jr];
-        const uint32_t w0 = tstart[jr], w1 = tstart[jr + 1];
-        // ---- stage 1: warp w computes t for source sb + w, reading its block rows of D
-        // (lanes over the columns B(C2), through the slot positions) ----
-        int32_t v1 = -1;
-        if (warp < nsrc) {
-            const int32_t v = sid[sval[sb + warp]];
-            v1 = (v >= 0 && v < ctx.n) ? v : -1;
+    const int64_t ntiles = *ntiles_p, nsg = (ns + MS - 1) / MS;
+    for (int64_t item = blockIdx.x; item < ntiles * nsg; item += gridDim.x) {
+        const MTile tl = tiles[item % ntiles];
+        const int64_t sb = (item / ntiles) * MS;
+        const int nsrc = (int)((ns - sb) < MS ? (ns - sb) : MS);
+        const int nt_ = (int)tl.count;
+        const bool valid = tl.c < k;
+        MatDesc d2{0, 0, 0};
+        int32_t nb4 = 0;
+        int64_t to = 0;
+        if (valid) {
+            d2 = ctx.descs[tl.c];
+            nb4 = (ctx.nb[tl.c] + 3) & ~3;
+            to = t_off(ctx.bg_off, (int32_t)tl.c);
         }
-        if (lane == 0) srcv[warp] = v1;
-        if (c2 < k && v1 >= 0) {
-            const uint32_t c1 = (uint32_t)ctx.comp[v1];
-            const MatDesc d1 = ctx.descs[c1];
-            const int32_t nb1 = ctx.nb[c1], nb2 = ctx.nb[c2];
-            const int32_t* pos1 = ctx.bgpos + ctx.bg_off[c1];
-            const int32_t* pos2 = ctx.bgpos + ctx.bg_off[c2];
-            const T* a1 = ctx.apsp + d1.off + (int64_t)ctx.local[v1] * d1.n;
-            for (int32_t jb = 0; jb < nb2; jb += MCOLS) {
-                const int cols = (nb2 - jb) < MCOLS ? (nb2 - jb) : MCOLS;
-                const int jmax = (cols + 31) >> 5;
-                int32_t colpos[8];
-#pragma unroll
-                for (int jj = 0; jj < 8; ++jj) {
-                    const int j = jj * 32 + lane;
-                    colpos[jj] = j < cols ? pos2[jb + j] : 0;
-                }
-                T t[8];
-#pragma unroll
-                for (int jj = 0; jj < 8; ++jj) t[jj] = inf;
-                for (int32_t ib = 0; ib < nb1; ib += 32) {
-                    const T areg = ib + lane < nb1 ? a1[ib + lane] : inf;
-                    const int32_t preg = ib + lane < nb1 ? pos1[ib + lane] : 0;
-                    const int iend = (nb1 - ib) < 32 ? (nb1 - ib) : 32;
-#pragma unroll 2
-                    for (int ii = 0; ii < iend; ++ii) {
-                        const T a = __shfl_sync(0xffffffffu, areg, ii);
-                        const T* drow = ctx.D + (int64_t)__shfl_sync(0xffffffffu, preg, ii) * ctx.N;
-#pragma unroll
-                        for (int jj = 0; jj < 8; ++jj)
-                            if (jj < jmax && jj * 32 + lane < cols) t[jj] = add_min(a, drow[colpos[jj]], t[jj]);
-                    }
-                }
-#pragma unroll
-                for (int jj = 0; jj < 8; ++jj) {
-                    const int j = jj * 32 + lane;
-                    if (jj < jmax && j < cols) tb[warp * ldt + jb + j] = t[jj];
-                }
-            }
+        if (tid < MT) {
+            const uint32_t p = tid < nt_ ? tval[tl.start + tid] : 0u;
+            const int32_t v = tid < nt_ ? tid_[p] : -1;
+            sm.tv[tid] = v;
+            sm.tp[tid] = p;
+            sm.arow[tid] = valid && tid < nt_ ? d2.off + (int64_t)ctx.local[v] * d2.n : d2.off;
+        } else if (tid < MT + MS) {
+            const int s = tid - MT;
+            const int32_t v = s < nsrc ? sid[s0 + sb + s] : -1;
+            sm.sv[s] = v >= 0 && v < ctx.n ? v : -1;
         }
         __syncthreads();
-        // ---- stage 2: one target per lane against the group's t (broadcast from shared
-        // memory), walking the target's row of APSP(C2) ----
-        if (c2 >= k) {  // targets out of range
-            for (uint32_t b = w0 + tid; b < w1; b += MTH)
-                for (int s = 0; s < nsrc; ++s) {
-                    const int64_t at = (int64_t)sval[sb + s] * nt + tval[b];
+        // (rows past the tile's targets repeat a row of the table, sources past the group's a
+        //  row of t: neither is written out)
+        auto stage = [&](int32_t k0) {
+            const int b = (k0 / MK) & 1;
+            const int q = tid & 7;
+            if (k0 + 4 * q < nb4) {
+                for (int r = tid >> 3; r < MT; r += MTH / 8) cp_async16(&sm.a[b][r][4 * q], ctx.apsp + sm.arow[r] + k0 + 4 * q);
+                for (int r = tid >> 3; r < MS; r += MTH / 8)
+                    cp_async16(&sm.t[b][r][4 * q], t + (sb + (r < nsrc ? r : 0)) * ldt + to + k0 + 4 * q);
+            }
+            cp_async_commit();
+        };
+        T acc[8][4];
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) acc[i][j] = inf;
+        if (nb4 > 0) stage(0);
+        for (int32_t k0 = 0; k0 < nb4; k0 += MK) {
+            if (k0 + MK < nb4) {
+                stage(k0 + MK);
+                cp_async_wait<1>();
+            } else {
+                cp_async_wait<0>();
+            }
+            __syncthreads();
+            const int b = (k0 / MK) & 1;
+            const int kend = nb4 - k0 < MK ? nb4 - k0 : MK;
+#pragma unroll 1
+            for (int kk = 0; kk < kend; kk += 4) {
+                int4 tv[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) tv[j] = *reinterpret_cast<const int4*>(&sm.t[b][tx + 16 * j][kk]);
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const int4 av = *reinterpret_cast<const int4*>(&sm.a[b][ty + 16 * i][kk]);
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        if constexpr (std::is_same<T, float>::value) {
+                            const float2 x = __fadd2_rn(make_float2(__int_as_float(av.x), __int_as_float(av.y)),
+                                                        make_float2(__int_as_float(tv[j].x), __int_as_float(tv[j].y)));
+                            const float2 y = __fadd2_rn(make_float2(__int_as_float(av.z), __int_as_float(av.w)),
+                                                        make_float2(__int_as_float(tv[j].z), __int_as_float(tv[j].w)));
+                            acc[i][j] = fmin3(fmin3(acc[i][j], x.x, x.y), y.x, y.y);
+                        } else {
+                            acc[i][j] = __viaddmin_s32(av.x, tv[j].x, acc[i][j]);
+                            acc[i][j] = __viaddmin_s32(av.y, tv[j].y, acc[i][j]);
+                            acc[i][j] = __viaddmin_s32(av.z, tv[j].z, acc[i][j]);
+                            acc[i][j] = __viaddmin_s32(av.w, tv[j].w, acc[i][j]);
+                        }
+                    }
+                }
+            }
+            __syncthreads();  // (the buffer's next chunk; after the last one, `out` below)
+        }
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) sm.out[tx + 16 * j][ty + 16 * i] = acc[i][j];
+        __syncthreads();
+        const int tt = tid & (MT - 1);
+        if (tt < nt_) {
+            const int32_t v2 = sm.tv[tt];
+            const int32_t l2 = valid ? ctx.local[v2] : 0;
+            for (int s = tid / MT; s < nsrc; s += MTH / MT) {
+                const int32_t v1 = sm.sv[s];
+                const int64_t at = (s0 + sb + s) * nt + sm.tp[tt];
+                if (!valid || v1 < 0) {
                     if (OUT_F32)
                         ((float*)out)[at] = __int_as_float(0x7fc00000);
                     else
                         ((int32_t*)out)[at] = -1;
+                    continue;
                 }
-            if (tid == 0) atomicOr(ctx.err, kErrPair);
-        } else {
-            const MatDesc d2 = ctx.descs[c2];
-            const int32_t nb2 = ctx.nb[c2];
-            for (uint32_t b0 = w0 + (uint32_t)warp * 32; b0 < w1; b0 += MSRC * 32) {
-                const uint32_t b = b0 + lane;
-                const bool tv = b < w1;
-                const int32_t v2 = tv ? tid_[tval[b]] : 0;
-                const int32_t l2 = tv ? ctx.local[v2] : 0;
-                const T* a2 = ctx.apsp + d2.off + (int64_t)l2 * d2.n;
-                T acc[MSRC];
-#pragma unroll
-                for (int s = 0; s < MSRC; ++s) acc[s] = inf;
-#pragma unroll 4
-                for (int32_t c = 0; c < nb2; ++c) {
-                    const T x = tv ? a2[c] : inf;
-#pragma unroll
-                    for (int s = 0; s < MSRC; ++s)
-                        if (s < nsrc) acc[s] = add_min(x, tb[s * ldt + c], acc[s]);
-                }
-                if (tv) {
-#pragma unroll
-                    for (int s = 0; s < MSRC; ++s) {
-                        if (s >= nsrc) break;
-                        const int64_t at = (int64_t)sval[sb + s] * nt + tval[b];
-                        const int32_t v1s = srcv[s];
-                        if (v1s < 0) {
-                            if (OUT_F32)
-                                ((float*)out)[at] = __int_as_float(0x7fc00000);
-                            else
-                                ((int32_t*)out)[at] = -1;
-                            continue;
-                        }
-                        T y = acc[s];
-                        const uint32_t c1s = (uint32_t)ctx.comp[v1s];
-                        if (c1s == c2) {
-                            const MatDesc d1s = ctx.descs[c1s];
-                            y = tmin2(y, ctx.apsp[d1s.off + (int64_t)ctx.local[v1s] * d1s.n + l2]);
-                        }
-                        if (v1s == v2) y = T(0);
-                        put<T, OUT_F32>(out, at, y);
-                    }
-                }
+                T y = sm.out[s][tt];
+                if (ctx.comp[v1] == (int32_t)tl.c)
+                    y = tmin2(y, ctx.apsp[d2.off + (int64_t)ctx.local[v1] * d2.n + l2]);
+                if (v1 == v2) y = T(0);
+                if (OUT_F32)
+                    ((float*)out)[at] = (float)y;
+                else
+                    ((int32_t*)out)[at] = (int32_t)tmin2<int32_t>((int32_t)y, SPQ_INF_I32);
             }
-            if (tid == 0)
-                for (int s = 0; s < nsrc; ++s)
-                    if (srcv[s] < 0) atomicOr(ctx.err, kErrPair);
         }
-        __syncthreads();  // tb and srcv are rewritten by the next item
+        if ((!valid && tid == 0) || (tid < nsrc && sm.sv[tid] < 0)) atomicOr(ctx.err, kErrPair);
+        __syncthreads();  // the tile's records are rewritten by the next item
     }
 }
 
@@ -221,39 +295,28 @@ int msms() {
     return g_msms;
 }
 
-// Sort ids by component and find the runs; returns the run count (host).
-cudaError_t runs_by_component(const int32_t* ids, int64_t n, int32_t nv, const int32_t* comp, uint32_t k,
-                              uint32_t* buf, uint32_t** vals, uint32_t** start, uint32_t** rkey, uint32_t* nrun,
-                              cudaStream_t st) {
-    uint32_t* k0 = buf;
-    uint32_t* v0 = k0 + n;
-    uint32_t* k1 = v0 + n;
-    uint32_t* v1 = k1 + n;
-    uint32_t* fl = v1 + n;  // n + 1
-    uint32_t* sta = fl + n + 1;
-    uint32_t* rk = sta + n + 1;
-    uint32_t* hist = rk + n + 1;
-    const unsigned g = (unsigned)((n + 256) / 256);
-    k_comp_keys<<<g, 256, 0, st>>>(ids, n, nv, comp, k, k0, v0);
-    count_launches(1);
-    int bits = 0;
-    while (bits < 32 && ((uint64_t)k >> bits)) ++bits;
-    bool in_k1 = false;
-    cudaError_t e = radix_sort_pairs(k0, v0, k1, v1, hist, n, bits, &in_k1, st);
-    if (e != cudaSuccess) return e;
-    const uint32_t* ks = in_k1 ? k1 : k0;
-    *vals = in_k1 ? v1 : v0;
-    k_run_heads<<<g, 256, 0, st>>>(ks, n, fl);
-    if ((e = launch_scan_excl(fl, n + 1, st)) != cudaSuccess) return e;
-    k_run_starts<<<g, 256, 0, st>>>(ks, fl, n, sta, rk);
-    count_launches(3);
-    *start = sta;
-    *rkey = rk;
-    if ((e = cudaMemcpyAsync(nrun, fl + n, sizeof(uint32_t), cudaMemcpyDeviceToHost, st)) != cudaSuccess) return e;
-    return cudaStreamSynchronize(st);
-}
+constexpr int64_t kTElems = 1 << 24;  // most values of t at a time (64 MB), at least MS rows
 
-int64_t runs_words(int64_t n) { return 4 * n + 3 * (n + 1) + radix_hist_words(n); }
+template <typename T, bool OUT_F32>
+cudaError_t matrix_launch(const QueryCtx<T>& ctx, uint32_t k, const int32_t* src, int64_t ns,
+                          const int32_t* tgt, const uint32_t* tval, const MTile* tiles, const uint32_t* ntiles,
+                          const uint32_t* cnt, int64_t nt, int64_t ldt, int64_t rows, T* t, void* out,
+                          cudaStream_t st) {
+    auto kern = k_matrix_out<T, OUT_F32>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(MSmem<T>));
+    for (int64_t s0 = 0; s0 < ns && e == cudaSuccess; s0 += rows) {
+        const int64_t n = std::min(rows, ns - s0);
+        const int64_t warps = n * (int64_t)k;
+        k_matrix_t<T><<<(unsigned)std::min<int64_t>((warps + 7) / 8, (int64_t)msms() * 32), MTH, 0, st>>>(
+            ctx, k, src, s0, n, cnt, ldt, t);
+        const int64_t items = ((nt + MT - 1) / MT + k + 1) * ((n + MS - 1) / MS);
+        kern<<<(unsigned)std::min<int64_t>(items, (int64_t)msms() * 2), MTH, sizeof(MSmem<T>), st>>>(
+            ctx, k, src, s0, n, tgt, tval, tiles, ntiles, nt, ldt, t, out);
+        count_launches(2);
+        e = cudaGetLastError();
+    }
+    return e;
+}
 
 }  // namespace
 }  // namespace spq
@@ -285,9 +348,8 @@ extern "C" spq_status spq_query_matrix(spq_handle* h, const int32_t* sources, in
     handle_query_view(h, &ci, &cf, &f32store, &out_f32, &k);
     int32_t nbmax = 0;
     for (int32_t c = 0; c < k; ++c) nbmax = std::max(nbmax, h->h_nb[c]);
-    const int32_t ldt = ((nbmax > 0 ? nbmax : 1) + 31) & ~31;
-    const size_t smem = (size_t)(MSRC * ldt) * 4;
-    if (smem > 200 * 1024) return SPQ_EUNSUPPORTED;  // a component with more than ~6,000 boundary vertices
+    // (a component with more than about 6,000 boundary vertices)
+    if ((size_t)(8 * (((nbmax > 0 ? nbmax : 1) + 31) & ~31)) * 4 > 200 * 1024) return SPQ_EUNSUPPORTED;
     std::vector<void*> tmp;
     auto alloc = [&](void** p, size_t bytes) {
         cudaError_t e = scratch_alloc(p, bytes ? bytes : 4, st);
@@ -316,34 +378,42 @@ extern "C" spq_status spq_query_matrix(spq_handle* h, const int32_t* sources, in
         d_t = (const int32_t*)p2;
         d_out = p3;
     }
-    void *bs, *bt;
-    if ((e = alloc(&bs, (size_t)runs_words(ns) * 4)) != cudaSuccess ||
-        (e = alloc(&bt, (size_t)runs_words(nt) * 4)) != cudaSuccess)
+    // the targets sorted by component, their tiles, t of a batch of sources
+    const int64_t ldt = round_up(h->nbg + 3 * (int64_t)k, 4) + 4;
+    const int64_t rows = std::min(round_up(ns, MS), std::max<int64_t>(MS, kTElems / ldt / MS * MS));
+    const int64_t max_tiles = (nt + MT - 1) / MT + k + 1;
+    uint32_t *buf, *cnt;
+    MTile* tiles;
+    void* t;
+    if ((e = alloc((void**)&buf, (size_t)(4 * nt + radix_hist_words(nt)) * 4)) != cudaSuccess ||
+        (e = alloc((void**)&cnt, ((size_t)k + 2) * 4)) != cudaSuccess ||
+        (e = alloc((void**)&tiles, (size_t)max_tiles * sizeof(MTile))) != cudaSuccess ||
+        (e = alloc(&t, (size_t)(rows * ldt) * 4)) != cudaSuccess)
         return fail(e);
-    uint32_t *sval, *sstart, *skey, *tval, *tstart, *tkey, nsrun = 0, ntrun = 0;
-    if ((e = runs_by_component(d_s, ns, h->n, h->comp, (uint32_t)k, (uint32_t*)bs, &sval, &sstart, &skey, &nsrun, st)) !=
+    uint32_t* ntiles = cnt + k + 1;
+    k_comp_keys<<<(unsigned)((nt + 255) / 256), 256, 0, st>>>(d_t, nt, h->n, h->comp, (uint32_t)k, buf, buf + nt);
+    int bits = 0;
+    while (bits < 32 && ((uint64_t)k >> bits)) ++bits;
+    bool in_k1 = false;
+    if ((e = radix_sort_pairs(buf, buf + nt, buf + 2 * nt, buf + 3 * nt, buf + 4 * nt, nt, bits, &in_k1, st)) !=
             cudaSuccess ||
-        (e = runs_by_component(d_t, nt, h->n, h->comp, (uint32_t)k, (uint32_t*)bt, &tval, &tstart, &tkey, &ntrun, st)) !=
-            cudaSuccess)
+        (e = cudaMemsetAsync(ntiles, 0, 4, st)) != cudaSuccess)
         return fail(e);
-    const int64_t items = ((ns + MSRC - 1) / MSRC) * (int64_t)ntrun;
-    const unsigned grid = (unsigned)std::min<int64_t>(items, (int64_t)msms() * 16);
-    (void)nsrun;
-    (void)sstart;
-    (void)skey;
-    if (f32store) {
-        auto kern = out_f32 ? k_query_matrix<float, true> : k_query_matrix<float, false>;
-        if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
-            return fail(e);
-        kern<<<grid, MTH, smem, st>>>(cf, (uint32_t)k, d_s, sval, ns, d_t, tval, tstart, tkey, ntrun, nt, ldt, d_out);
-    } else {
-        auto kern = out_f32 ? k_query_matrix<int32_t, true> : k_query_matrix<int32_t, false>;
-        if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
-            return fail(e);
-        kern<<<grid, MTH, smem, st>>>(ci, (uint32_t)k, d_s, sval, ns, d_t, tval, tstart, tkey, ntrun, nt, ldt, d_out);
-    }
-    count_launches(1);
-    if ((e = cudaGetLastError()) != cudaSuccess) return fail(e);
+    k_matrix_tiles<<<(unsigned)((k + 1 + 127) / 128), 128, 0, st>>>(in_k1 ? buf + 2 * nt : buf, nt, (uint32_t)k, tiles,
+                                                                    ntiles, cnt);
+    count_launches(2);
+    const uint32_t* tval = in_k1 ? buf + 3 * nt : buf + nt;
+    if (f32store)
+        e = out_f32 ? matrix_launch<float, true>(cf, (uint32_t)k, d_s, ns, d_t, tval, tiles, ntiles, cnt, nt,
+                                                 ldt, rows, (float*)t, d_out, st)
+                    : matrix_launch<float, false>(cf, (uint32_t)k, d_s, ns, d_t, tval, tiles, ntiles, cnt, nt,
+                                                  ldt, rows, (float*)t, d_out, st);
+    else
+        e = out_f32 ? matrix_launch<int32_t, true>(ci, (uint32_t)k, d_s, ns, d_t, tval, tiles, ntiles, cnt, nt,
+                                                   ldt, rows, (int32_t*)t, d_out, st)
+                    : matrix_launch<int32_t, false>(ci, (uint32_t)k, d_s, ns, d_t, tval, tiles, ntiles, cnt,
+                                                    nt, ldt, rows, (int32_t*)t, d_out, st);
+    if (e != cudaSuccess) return fail(e);
     if (!ds) {
         if ((e = cudaMemcpyAsync(dist_out, d_out, (size_t)(ns * nt) * 4, cudaMemcpyDeviceToHost, st)) != cudaSuccess)
             return fail(e);
