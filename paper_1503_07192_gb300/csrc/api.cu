@@ -354,7 +354,14 @@ cudaError_t build_bg_tables(spq_handle* h, const BuildInputs& in, bool check_exa
             for (const ElimTask& tk : plan.layout.tasks)
                 if (!tk.deps.empty())
                     for (int32_t b = tk.lo; b < tk.hi; ++b) shared.push_back(b);
-            if ((e = launch_mark_pairs(shared, h->N, plan.rowflags, st)) != cudaSuccess) return e;
+            if (!shared.empty()) {
+                int32_t* d = nullptr;
+                if ((e = scratch_alloc((void**)&d, shared.size() * 4, st)) != cudaSuccess) return e;
+                e = cudaMemcpyAsync(d, shared.data(), shared.size() * 4, cudaMemcpyHostToDevice, st);
+                if (e == cudaSuccess) e = launch_mark_pairs(d, (int32_t)shared.size(), h->N, plan.rowflags, st);
+                cudaFreeAsync(d, st);  // (pageable upload: staged before it returned)
+                if (e != cudaSuccess) return e;
+            }
         }
         if ((e = fill_marked ? launch_fill_marked<T>(D, h->N, plan.rowflags, st) : launch_bg_fill<T>(D, h->N, st)) !=
             cudaSuccess)
@@ -370,13 +377,13 @@ cudaError_t build_bg_tables(spq_handle* h, const BuildInputs& in, bool check_exa
     // the elimination stores the float32 boundary-graph table as int32 itself (checked)
     const bool d_converted = plan.elim && check_exact && h->N > 0;
     if (h->N > 0 && !plan.elim) {
-        if ((e = fw_single<T>(D, h->N, skip_inf, fw_scratch, nullptr, &h->bg_updates, profile ? &h->fwprof : nullptr,
-                              st)) != cudaSuccess)
+        if ((e = fw_single<T>(D, h->N, skip_inf, fw_scratch, &h->bg_updates, profile ? &h->fwprof : nullptr, st)) !=
+            cudaSuccess)
             return e;
     } else if (h->N > 0) {
         double fwd = 0.0, bs = 0.0;
-        if ((e = fw_single<T>(D, h->N, skip_inf, fw_scratch, plan.rowflags, &fwd, profile ? &h->fwprof : nullptr,
-                              st, plan.layout.tasks.empty() ? nullptr : &plan.layout.tasks)) != cudaSuccess)
+        const std::vector<ElimMat<T>> mats{ElimMat<T>{D, h->N, plan.rowflags, &plan.layout.tasks}};
+        if ((e = elim_forward<T>(mats, skip_inf, &fwd, profile ? &h->fwprof : nullptr, st)) != cudaSuccess)
             return e;
         if ((e = bg_backsub<T>(D, h->N, plan.rowflags, h->err, d_converted ? d_flag : nullptr, plan.apanel_budget, &bs,
                                profile ? &h->fwprof : nullptr, st)) != cudaSuccess)
@@ -515,7 +522,7 @@ spq_status build_impl(int32_t n, const int64_t* row_ptr, const int32_t* col, con
     // elimination scratch: per-round row flags, back-substitution bookkeeping, A panels,
     // and per-run compaction lists
     const size_t elim_bytes = may_elim ? 4 * (size_t)(nR * nR) + bg_backsub_scratch_bytes(n_max) + apanel_budget +
-                                             (size_t)max_runs * 4 * (size_t)(6 * nR + 10)
+                                             (size_t)max_runs * 4 * (size_t)(10 * nR + 13)
                                        : 0;
     // (+ the component tables in dissection order, a second copy, for their elimination)
     const size_t comp_elim_bytes = opts.comp_method != SPQ_BG_FW ? 4 * (size_t)h->apsp_elems + 8 * (size_t)n : 0;

@@ -148,18 +148,49 @@ cudaError_t fw_batched(T* base, const MatDesc* d_descs, const MatDesc* h_descs, 
                        cudaStream_t st, int32_t** keep_buf = nullptr);
 // One matrix of size N, optionally skipping tiles whose pivot panel is all infinite.
 // *updates receives the number of min-plus updates issued (host-side count).
-// rowflags == NULL: the full Floyd-Warshall.  rowflags = R x R words (R = ceil(N/128)),
-// zeroed: the elimination (forward) form: round r updates only tiles right of and below
-// the pivot (I, J > r), and rowflags[r][J] marks the row tiles (r, J > r) that hold a
-// finite entry; bg_backsub then completes the matrix.
-// tasks (elimination form only, may be NULL): runs of rounds to do side by side where
-// they do not depend on each other (see ElimTask in order.h); NULL: one run in order.
+template <typename T>
+cudaError_t fw_single(T* M, int64_t N, bool skip_inf, uint32_t* scratch, double* updates, FwProfile* prof,
+                      cudaStream_t st);
+int64_t fw_single_scratch_words(int64_t N);
+// The elimination (forward) form: round r updates only tiles right of and below the pivot
+// (I, J > r).  rowflags: R x R words (R = ceil(N / 128)), marking the tiles I < J that may
+// hold a finite entry (only those and the diagonal tiles need to be initialised; without
+// skip_inf, all of them); afterwards they mark the tiles that do.  tasks: runs of rounds to
+// do side by side where they do not depend on each other (see ElimTask in order.h), or null:
+// one run in order.  bg_backsub_many then completes the matrices.  Reads the update count on
+// the host, but not with keep (build plans) ready: the same launches again, no host step and
+// no allocation.
 struct ElimTask;
 template <typename T>
-cudaError_t fw_single(T* M, int64_t N, bool skip_inf, uint32_t* scratch_flags, uint32_t* rowflags, double* updates,
-                      FwProfile* prof, cudaStream_t st, const std::vector<ElimTask>* tasks = nullptr);
-int64_t fw_single_scratch_words(int64_t N);
-// ---- elim.cu: back-substitution after the forward form of fw_single ----
+struct ElimMat {
+    T* M;
+    int64_t N;
+    uint32_t* rowflags;
+    const std::vector<ElimTask>* tasks;
+};
+struct ElimPlan {
+    struct Step {
+        size_t first;         // of its entries
+        int32_t count, most;  // runs with a round in it, most row tiles right of a pivot
+    };
+    bool ready = false;
+    unsigned char* mem = nullptr;  // runs' scratch | counter offsets | sums | entries
+    int64_t words = 0;
+    int32_t nrun = 0;
+    size_t o_off = 0, o_out = 0, o_ent = 0;
+    double diag = 0.0, updates = 0.0;
+    std::vector<Step> steps;
+    void release(cudaStream_t st) {
+        if (mem) cudaFreeAsync(mem, st);
+        mem = nullptr;
+        ready = false;
+        steps.clear();
+    }
+};
+template <typename T>
+cudaError_t elim_forward(const std::vector<ElimMat<T>>& mats, bool skip_inf, double* updates, FwProfile* prof,
+                         cudaStream_t st, ElimPlan* keep = nullptr);
+// ---- elim.cu: back-substitution after elim_forward ----
 // Completes M (N x N, symmetric storage) to all-pairs distances.  err: device status
 // word (kErrWait if a bounded wait gave up).  *updates: min-plus updates issued.
 // Needs bg_backsub_scratch_bytes(N) bytes of device scratch plus its A panels, which it
@@ -224,8 +255,8 @@ struct BsPlan {
 template <typename T>
 cudaError_t bg_backsub_many(const std::vector<BsInput<T>>& in, uint32_t* err, uint32_t* exact, size_t apanel_budget,
                             double* updates, FwProfile* prof, cudaStream_t st, BsPlan<T>* keep = nullptr);
-// Marks of every pair of the given tiles (host list).
-cudaError_t launch_mark_pairs(const std::vector<int32_t>& blocks, int64_t N, uint32_t* flags, cudaStream_t st);
+// Marks of every pair of the nb given tiles (device list).
+cudaError_t launch_mark_pairs(const int32_t* blocks, int32_t nb, int64_t N, uint32_t* flags, cudaStream_t st);
 // Infinity (0 on the diagonal) in the marked tiles, their mirrors and the diagonal tiles.
 template <typename T>
 cudaError_t launch_fill_marked(T* M, int64_t N, const uint32_t* flags, cudaStream_t st);

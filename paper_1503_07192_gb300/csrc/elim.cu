@@ -195,7 +195,7 @@ struct BsRun {
 // column strips.  A strip is a quarter of the work on a CTA of its own: where a level holds
 // fewer tiles than the GPU holds CTAs, the chain of levels, not the updates, bounds the
 // launch, and a strip takes a quarter of a tile's time.
-constexpr int BS_STRIPS = 4;
+constexpr int BS_STRIPS = kStrips;
 constexpr uint16_t BS_WHOLE = BS_STRIPS;
 struct BsItem {
     uint16_t mat, R, J, strip;
@@ -493,40 +493,6 @@ __device__ __forceinline__ void stage_panel(T (*P)[T_], const T* __restrict__ A,
     }
 }
 
-constexpr int SW = T_ / BS_STRIPS;  // strip width (32 columns: 8 threads x 4)
-
-// acc = min(acc, A (x) B) over a chunk for a strip: 4 x 4 per thread, rows 4sy.., strip
-// columns 4sx..; B rows of SW cells.
-template <typename T>
-__device__ __forceinline__ void strip_chunk(T (&acc)[4][4], const T (*a)[T_], const T* b, int sx, int sy, int kend) {
-#pragma unroll 2
-    for (int kk = 0; kk < kend; kk += 2) {
-        const int4 x = *reinterpret_cast<const int4*>(&a[kk][sy * 4]);
-        const int4 y = *reinterpret_cast<const int4*>(&a[kk + 1][sy * 4]);
-        const int4 z = *reinterpret_cast<const int4*>(b + kk * SW + sx * 4);
-        const int4 w = *reinterpret_cast<const int4*>(b + (kk + 1) * SW + sx * 4);
-        const int xa[4] = {x.x, x.y, x.z, x.w}, ya[4] = {y.x, y.y, y.z, y.w};
-        const int zb[4] = {z.x, z.y, z.z, z.w}, wb[4] = {w.x, w.y, w.z, w.w};
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            if constexpr (std::is_same<T, float>::value) {
-                const float2 p0 = make_float2(__int_as_float(xa[i]), __int_as_float(xa[i]));
-                const float2 p1 = make_float2(__int_as_float(ya[i]), __int_as_float(ya[i]));
-#pragma unroll
-                for (int j = 0; j < 4; j += 2) {
-                    const float2 s0 = __fadd2_rn(p0, make_float2(__int_as_float(zb[j]), __int_as_float(zb[j + 1])));
-                    const float2 s1 = __fadd2_rn(p1, make_float2(__int_as_float(wb[j]), __int_as_float(wb[j + 1])));
-                    acc[i][j] = fmin3(acc[i][j], s0.x, s1.x);
-                    acc[i][j + 1] = fmin3(acc[i][j + 1], s0.y, s1.y);
-                }
-            } else {
-#pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] = MP<T>::upd2(acc[i][j], xa[i], zb[j], ya[i], wb[j]);
-            }
-        }
-    }
-}
-
 // Encoded results of a strip -> stored int32 (as clamp_enc).
 __device__ __forceinline__ bool clamp_enc4(float (&acc)[4][4]) {
     bool bad = false;
@@ -588,19 +554,8 @@ __device__ __forceinline__ void backsub_strip(T* __restrict__ M, int64_t N, int6
     }
     if constexpr (CONV)
         if (clamp_enc4(acc)) atomicOr(exact, kErrExact);
-    auto i4 = [](T a, T b, T cc, T d) {
-        return make_int4(*reinterpret_cast<int*>(&a), *reinterpret_cast<int*>(&b), *reinterpret_cast<int*>(&cc),
-                         *reinterpret_cast<int*>(&d));
-    };
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-        if (r + i < N && c < N)
-            *reinterpret_cast<int4*>(M + (r + i) * N + c) = i4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
-    if (!diag)
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-            if (c + j < N && r < N)
-                *reinterpret_cast<int4*>(M + (c + j) * N + r) = i4(acc[0][j], acc[1][j], acc[2][j], acc[3][j]);
+    store_strip<T>(acc, M, N, r0, cs, sx, sy);
+    if (!diag) store_strip_transposed<T>(acc, M, N, r0, cs, sx, sy);
 }
 
 // CONV (float tables of an int32 graph): every tile is stored as int32 (the final table
@@ -791,22 +746,13 @@ cudaError_t launch_fill_marked(T* M, int64_t N, const uint32_t* flags, cudaStrea
     return cudaGetLastError();
 }
 
-cudaError_t launch_mark_pairs(const std::vector<int32_t>& blocks, int64_t N, uint32_t* flags, cudaStream_t st) {
-    if (blocks.empty() || N <= 0) return cudaSuccess;
+cudaError_t launch_mark_pairs(const int32_t* blocks, int32_t nb, int64_t N, uint32_t* flags, cudaStream_t st) {
+    if (nb <= 0 || N <= 0) return cudaSuccess;
     const int32_t nR = (int32_t)((N + T_ - 1) / T_);
-    int32_t* d = nullptr;
-    cudaError_t e = scratch_alloc((void**)&d, blocks.size() * sizeof(int32_t), st);
-    if (e != cudaSuccess) return e;
-    e = cudaMemcpyAsync(d, blocks.data(), blocks.size() * sizeof(int32_t), cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess) {
-        const int32_t nb = (int32_t)blocks.size();
-        k_mark_pairs<<<(nb * nb + 255) / 256 < 1024 ? (nb * nb + 255) / 256 : 1024, 256, 0, st>>>(d, nb, nR, flags);
-        count_launches(1);
-        e = cudaGetLastError();
-    }
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);  // (the host list may go away)
-    cudaFreeAsync(d, st);
-    return e;
+    const int64_t g = ((int64_t)nb * nb + 255) / 256;
+    k_mark_pairs<<<(unsigned)std::min<int64_t>(g, 1024), 256, 0, st>>>(blocks, nb, nR, flags);
+    count_launches(1);
+    return cudaGetLastError();
 }
 
 size_t bg_backsub_scratch_bytes(int64_t N) {

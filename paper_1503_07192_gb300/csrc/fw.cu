@@ -130,90 +130,6 @@ __global__ void __launch_bounds__(NTH) k_phase1(T* __restrict__ base, const MatD
     }
 }
 
-// Phase 1 of round r of one matrix with 1,024 threads, each owning a 4 x 4 block (rows
-// 4ty.., columns 4tx..): the same two pivot steps per barrier as k_phase1, with four
-// times the warps to hide each step's latency, and the sums formed two at a time by
-// packed f32x2 adds.  For the elimination rounds of one boundary graph, where the closure
-// of the diagonal tile lies on the critical path of every round.  Every step is the
-// same rounded float operation as in k_phase1, so the results are identical.
-__global__ void __launch_bounds__(1024, 1) k_phase1_wide(float* __restrict__ M, int64_t n, int32_t r) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    float(*S)[T_] = reinterpret_cast<float(*)[T_]>(smem_raw);
-    const int tid = threadIdx.x, tx = tid & 31, ty = tid >> 5;
-    const int64_t o = (int64_t)r * T_;
-    for (int idx = tid; idx < T_ * T_ / 4; idx += 1024) {
-        const int i = idx >> 5, c4 = idx & 31;
-        const int64_t gr = o + i, gc = o + c4 * 4;
-        int4 v = (gr < n && gc < n) ? *reinterpret_cast<const int4*>(M + gr * n + gc) : inf4<float>();
-        *reinterpret_cast<int4*>(&S[i][c4 * 4]) = v;
-    }
-    __syncthreads();
-    float acc[4][4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const float4 v = *reinterpret_cast<const float4*>(&S[4 * ty + i][4 * tx]);
-        acc[i][0] = v.x;
-        acc[i][1] = v.y;
-        acc[i][2] = v.z;
-        acc[i][3] = v.w;
-    }
-    const int K = (int)((n - o) < T_ ? (n - o) : T_);
-    int k = 0;
-    // rows k and k + 1 are current (by symmetry also columns k and k + 1); row k + 1
-    // after step k is min(D(k+1, x), D(k+1, k) + D(k, x)), formed on the fly
-    for (; k + 1 < K; k += 2) {
-        const float4 p = *reinterpret_cast<const float4*>(&S[k][4 * ty]);
-        const float4 q = *reinterpret_cast<const float4*>(&S[k][4 * tx]);
-        const float4 u = *reinterpret_cast<const float4*>(&S[k + 1][4 * ty]);
-        const float4 v = *reinterpret_cast<const float4*>(&S[k + 1][4 * tx]);
-        const float skk = S[k][k + 1];
-        const float a0[4] = {p.x, p.y, p.z, p.w};
-        const float a1[4] = {fminf(u.x, skk + p.x), fminf(u.y, skk + p.y), fminf(u.z, skk + p.z),
-                             fminf(u.w, skk + p.w)};
-        const float2 b0l = make_float2(q.x, q.y), b0h = make_float2(q.z, q.w);
-        const float2 b1l = make_float2(fminf(v.x, skk + q.x), fminf(v.y, skk + q.y));
-        const float2 b1h = make_float2(fminf(v.z, skk + q.z), fminf(v.w, skk + q.w));
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const float2 x0 = make_float2(a0[i], a0[i]), x1 = make_float2(a1[i], a1[i]);
-            const float2 s0l = __fadd2_rn(x0, b0l), s0h = __fadd2_rn(x0, b0h);
-            const float2 s1l = __fadd2_rn(x1, b1l), s1h = __fadd2_rn(x1, b1h);
-            acc[i][0] = fmin3(acc[i][0], s0l.x, s1l.x);
-            acc[i][1] = fmin3(acc[i][1], s0l.y, s1l.y);
-            acc[i][2] = fmin3(acc[i][2], s0h.x, s1h.x);
-            acc[i][3] = fmin3(acc[i][3], s0h.y, s1h.y);
-        }
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int row = 4 * ty + i;
-            if (row == k + 2 || row == k + 3)
-                *reinterpret_cast<float4*>(&S[row][4 * tx]) = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
-        }
-        __syncthreads();
-    }
-    for (; k < K; ++k) {
-        const float4 p = *reinterpret_cast<const float4*>(&S[k][4 * ty]);
-        const float4 q = *reinterpret_cast<const float4*>(&S[k][4 * tx]);
-        const float a[4] = {p.x, p.y, p.z, p.w}, b[4] = {q.x, q.y, q.z, q.w};
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-            for (int j = 0; j < 4; ++j) acc[i][j] = fminf(acc[i][j], a[i] + b[j]);
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-            if (4 * ty + i == k + 1)
-                *reinterpret_cast<float4*>(&S[k + 1][4 * tx]) =
-                    make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
-        __syncthreads();
-    }
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int64_t gr = o + 4 * ty + i, gc = o + 4 * tx;
-        if (gr < n && gc < n)
-            *reinterpret_cast<float4*>(M + gr * n + gc) = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
-    }
-}
-
 // ---------------- phase 2: pivot row tiles (and their transposes) ----------------
 template <typename T>
 __global__ void __launch_bounds__(NTH, SPQ_FW_MIN_CTAS) k_phase2(T* __restrict__ base, const MatDesc* __restrict__ descs,
@@ -289,111 +205,6 @@ __device__ void compact_row(const uint32_t* __restrict__ f, int32_t lo, int32_t 
     }
     if (threadIdx.x == 0) out[0] = cnt;
     __syncthreads();
-}
-
-// Elimination form, after phase 2 of round r (r = -1: before round 0):
-//   list = the finite row tiles J > r of round r (phase 3 updates list x list);
-//   marks every pair of the list as a tile that may hold a finite entry from now on
-//   (2 where it was unmarked: only the marked tiles were initialised);
-//   cand = the marked tiles J > r + 1 of row r + 1 (phase 2 of the next round).
-__device__ void compact_trail(uint32_t* __restrict__ rowflags, int32_t R, int32_t r, uint32_t* __restrict__ list,
-                              uint32_t* __restrict__ cand, unsigned long long* __restrict__ tiles, int32_t do_list) {
-    if (r >= 0 && do_list) {
-        compact_row(rowflags + (int64_t)r * R, r + 1, R, list);
-        const uint32_t c = list[0];
-        for (uint32_t t = threadIdx.x; t < c * c; t += blockDim.x) {
-            const uint32_t x = t / c, y = t % c;
-            if (y > x) {
-                // 2: newly marked, its cells are not initialised yet (phase 3 starts it
-                // from infinity and then marks it 1)
-                uint32_t* f = rowflags + (int64_t)list[1 + x] * R + list[1 + y];
-                if (__ldcg(f) == 0u) *f = 2u;
-            }
-        }
-        if (threadIdx.x == 0) {
-            tiles[0] += (unsigned long long)c * (c + 1) / 2;  // phase-3 tiles of this round
-            tiles[1] += (unsigned long long)c;                // phase-2 tiles computed (finite)
-        }
-        __syncthreads();
-    }
-    if (r + 1 < R) compact_row(rowflags + (int64_t)(r + 1) * R, r + 2, R, cand);
-}
-
-__global__ void k_compact_trail(uint32_t* __restrict__ rowflags, int32_t R, int32_t r, uint32_t* __restrict__ list,
-                                uint32_t* __restrict__ cand, unsigned long long* __restrict__ tiles, int32_t do_list) {
-    compact_trail(rowflags, R, r, list, cand, tiles, do_list);
-}
-
-// ---------------- phase 2, elimination form: candidate row tiles only ----------------
-// cand[0] = count, cand[1..] = the tiles J > r of row r that may hold a finite entry (the
-// assembly's and earlier rounds' marks).  A candidate that is all-infinite is unmarked
-// (it stays infinite); the others are updated, with their transposes.
-// With counter != NULL the last CTA to finish (counted there; the counter is left at 0)
-// also does the round's compaction (compact_trail; with mark_all, after marking every
-// tile J > r of row r): no separate launch on the round's critical path.
-template <typename T>
-__global__ void __launch_bounds__(NTH, SPQ_FW_MIN_CTAS) k_phase2_cand(T* __restrict__ M, int64_t n, int32_t r,
-                                                                      int32_t R, uint32_t* __restrict__ cand,
-                                                                      uint32_t* __restrict__ rowflags,
-                                                                      uint32_t* __restrict__ list,
-                                                                      unsigned long long* __restrict__ tiles,
-                                                                      uint32_t* __restrict__ counter,
-                                                                      int32_t mark_all,
-                                                                      uint32_t* __restrict__ kmask) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    PanelSmem<T>& sm = *reinterpret_cast<PanelSmem<T>*>(smem_raw);
-    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-    const int64_t o = (int64_t)r * T_;
-    const uint32_t c = cand[0];
-    const T inf = Inf<T>::value();
-    for (uint32_t ci = blockIdx.x; ci < c; ci += gridDim.x) {
-        const int32_t J = (int32_t)cand[1 + ci];
-        const int64_t cj = (int64_t)J * T_;
-        T acc[8][8];
-        load_c<T>(acc, M, n, o, cj, tx, ty);
-        bool fin = false;
-#pragma unroll
-        for (int i = 0; i < 8; ++i)
-#pragma unroll
-            for (int j = 0; j < 8; ++j) fin |= acc[i][j] < inf;
-        if (!__syncthreads_or(fin)) {
-            if (tid == 0) rowflags[(int64_t)r * R + J] = 0u;
-            continue;
-        }
-        if (kmask) {
-            // the B panel is this tile's own rows: skip the chunks of rows that are all
-            // infinite; then record the updated tile's finite rows for phase 3
-            __shared__ uint32_t rm[4];
-            tile_row_mask<T>(acc, rm, tid, tx, ty);
-            uint32_t cm = 0u;
-#pragma unroll
-            for (int c = 0; c < NCHUNK; ++c) cm |= rm[c] ? (1u << c) : 0u;
-            minplus_panels_masked<T>(acc, M, n, o, o, cj, sm, tid, tx, ty, cm);
-            tile_row_mask<T>(acc, rm, tid, tx, ty);
-            if (tid < 4) kmask[(int64_t)J * 4 + tid] = rm[tid];
-        } else {
-            minplus_panels<T>(acc, M, n, o, o, cj, sm, tid, tx, ty);
-        }
-        store_c<T>(acc, M, n, o, cj, tx, ty);
-        store_c_transposed<T>(acc, M, n, o, cj, tx, ty);
-    }
-    if (counter == nullptr) return;
-    __shared__ uint32_t last;
-    __threadfence();  // (this CTA's tiles and flags, before its ticket)
-    __syncthreads();
-    if (tid == 0) last = atomicAdd(counter, 1u) == gridDim.x - 1u ? 1u : 0u;
-    __syncthreads();
-    if (!last) return;
-    __threadfence();  // (every other CTA's writes, after their tickets)
-    if (mark_all)
-        for (int32_t J = r + 1 + tid; J < R; J += blockDim.x) rowflags[(int64_t)r * R + J] = 0xffffffffu;
-    __syncthreads();
-    compact_trail(rowflags, R, r, list, cand, tiles, 1);
-    if (tid == 0) *counter = 0u;
-}
-
-__global__ void k_add_u64(unsigned long long* __restrict__ dst, const unsigned long long* __restrict__ src, int n) {
-    if ((int)threadIdx.x < n) dst[threadIdx.x] += src[threadIdx.x];
 }
 
 // Upper-triangle task t (0 <= t < c(c+1)/2) -> pair (x, y), 0 <= x <= y < c, row-major.
@@ -475,75 +286,17 @@ __global__ void __launch_bounds__(NTH, SPQ_FW_MIN_CTAS) k_phase3_sel(T* __restri
 // holds a finite entry; every (I, J) in list x list is updated, the pairs I < J once
 // for both triangles.  Tiles outside list x list keep their values: their pivot panel
 // is entirely infinite, so min(D, inf + x) = D.
-// With rowflags (elimination form), a target marked 2 was never initialised: it starts
-// from infinity instead of being loaded, and is marked 1 afterwards.  Targets (I, J) with
-// I >= shared_from may be updated by concurrent runs of rounds: stored with atomicMin.
 template <typename T>
 __global__ void __launch_bounds__(NTH, SPQ_FW_MIN_CTAS) k_phase3_list(T* __restrict__ M, int64_t n, int32_t r,
-                                                        const uint32_t* __restrict__ list,
-                                                        uint32_t* __restrict__ rowflags, int32_t R,
-                                                        int32_t shared_from,
-                                                        const uint32_t* __restrict__ kmask = nullptr) {
+                                                                      const uint32_t* __restrict__ list) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     PanelSmem<T>& sm = *reinterpret_cast<PanelSmem<T>*>(smem_raw);
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
     const int64_t c = list[0];
-    const int64_t o = (int64_t)r * T_;
     for (int64_t t = blockIdx.x; t < c * (c + 1) / 2; t += gridDim.x) {
         int64_t x, y;
         tri_pair(t, c, x, y);
-        const int64_t I = list[1 + x], J = list[1 + y];
-        uint32_t* f = (rowflags && I < J) ? rowflags + I * R + J : nullptr;
-        if (!kmask) {
-            if (f && *f == 2u) {
-                const int64_t ci = I * T_, cj = J * T_;
-                T acc[8][8];
-#pragma unroll
-                for (int i = 0; i < 8; ++i)
-#pragma unroll
-                    for (int j = 0; j < 8; ++j) acc[i][j] = Inf<T>::value();
-                minplus_panels<T>(acc, M, n, o, ci, cj, sm, tid, tx, ty);
-                store_c<T>(acc, M, n, ci, cj, tx, ty);
-                store_c_transposed<T>(acc, M, n, ci, cj, tx, ty);
-                if (tid == 0) *f = 1u;  // (every thread read the flag before the panel barriers)
-            } else if (I >= shared_from) {
-                const int64_t ci = I * T_, cj = J * T_;
-                T acc[8][8];
-                load_c<T>(acc, M, n, ci, cj, tx, ty);
-                minplus_panels<T>(acc, M, n, o, ci, cj, sm, tid, tx, ty);
-                store_c_min<T>(acc, M, n, ci, cj, tx, ty);
-                if (I != J) store_c_transposed_min<T>(acc, M, n, ci, cj, tx, ty);
-            } else {
-                phase3_tile<T>(M, n, o, I, J, sm, tid, tx, ty);
-            }
-            continue;
-        }
-        // with the row masks of this round's row tiles (kmask: 4 words per tile, set by
-        // phase 2): only the chunks of pivot rows finite in both panels
-        uint32_t cm = 0u;
-#pragma unroll
-        for (int q = 0; q < NCHUNK; ++q) cm |= (kmask[I * 4 + q] & kmask[J * 4 + q]) ? (1u << q) : 0u;
-        const bool fresh = f && *f == 2u;
-        __syncthreads();  // (every thread has read the mark before thread 0 may change it)
-        const int64_t ci = I * T_, cj = J * T_;
-        T acc[8][8];
-        if (fresh) {
-#pragma unroll
-            for (int i = 0; i < 8; ++i)
-#pragma unroll
-                for (int j = 0; j < 8; ++j) acc[i][j] = Inf<T>::value();
-        } else {
-            load_c<T>(acc, M, n, ci, cj, tx, ty);
-        }
-        minplus_panels_masked<T>(acc, M, n, o, ci, cj, sm, tid, tx, ty, cm);
-        if (!fresh && I >= shared_from) {
-            store_c_min<T>(acc, M, n, ci, cj, tx, ty);
-            if (I != J) store_c_transposed_min<T>(acc, M, n, ci, cj, tx, ty);
-        } else {
-            store_c<T>(acc, M, n, ci, cj, tx, ty);
-            if (I != J) store_c_transposed<T>(acc, M, n, ci, cj, tx, ty);
-        }
-        if (fresh && tid == 0) *f = 1u;
+        phase3_tile<T>(M, n, (int64_t)r * T_, list[1 + x], list[1 + y], sm, tid, tx, ty);
     }
 }
 
@@ -672,6 +425,329 @@ __global__ void __launch_bounds__(NTH, SPQ_FW_MIN_CTAS) k_phase3_many(T* __restr
     }
 }
 
+// ---------------- elimination form (forward rounds) ----------------
+// A step holds one round of every run of rounds that is active in it, of one matrix or of
+// many (ents[o ..], one per blockIdx.y): runs do not depend on one another and touch
+// disjoint tiles except those with both indices >= shared_from, which they update with
+// atomicMin.  Three launches a step: phase 1, phase 2 over the candidates of the round's row
+// with the compaction in each run's last CTA, phase 3 over its list.  (One stream per run
+// took three launches a round of every run: on 2^20 vertices 3,000 launches and as many
+// hardware queues as runs, on 2^16 vertices 18.0 of 30 ms serialised device time in rounds of
+// a few tiles.)  What bounds a step of few tiles is the time of one tile on one CTA, so
+// tiles are split into column strips where a step's tiles would leave CTAs idle.
+template <typename T>
+struct ElimEnt {
+    T* M;
+    int64_t N;
+    uint32_t* rowflags;  // R x R marks (see ElimScratch)
+    uint32_t* scratch;   // of the run
+    int32_t r, R, shared_from, first;  // the round; first: the first of its run
+};
+
+// A run's scratch.  list / cand: count, then ascending tile indices J > r: the finite row
+// tiles of round r (phase 3 updates list x list), the marked tiles of row r (phase 2's
+// candidates).  kmask: 4 words per tile J, the finite rows of row tile (r, J) after phase 2
+// (phase 3 multiplies only the 32-row chunks finite in both panels); kacc: the same while
+// phase 2's CTAs collect it, zero otherwise.
+// Marks: 1 a tile that may hold a finite entry, 2 one marked in this round, whose cells are
+// not initialised yet (phase 3 starts it from infinity; 1 from the next compaction on).
+struct ElimScratch {
+    uint32_t *list, *cand, *counter, *kmask, *kacc;
+    unsigned long long* tiles;  // phase-3 tiles, finite phase-2 tiles
+    __device__ ElimScratch(uint32_t* p, int32_t R)
+        : list(p),
+          cand(p + R + 2),
+          counter(p + 2 * R + 8),
+          kmask(p + ((2 * R + 13) & ~3)),  // (16-byte words; the run's scratch is 16-byte aligned)
+          kacc(kmask + 4 * R),
+          tiles(reinterpret_cast<unsigned long long*>(p + 2 * R + 4)) {}
+    static int64_t words(int32_t R) { return 10 * (int64_t)R + 13; }
+};
+
+// Phase 1: closure of the diagonal tile, 1,024 threads, each owning a 4 x 4 block (rows
+// 4ty.., columns 4tx..); two pivot steps per barrier as in k_phase1, the sums two at a time
+// by packed adds.  blockIdx.x = 1: the candidates of a run's first round, meanwhile.
+template <typename T>
+__global__ void __launch_bounds__(1024, 1) k_elim_phase1(const ElimEnt<T>* __restrict__ ents) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const ElimEnt<T> en = ents[blockIdx.y];
+    if (blockIdx.x == 1) {
+        if (en.first)
+            compact_row(en.rowflags + (int64_t)en.r * en.R, en.r + 1, en.R, ElimScratch(en.scratch, en.R).cand);
+        return;
+    }
+    T* __restrict__ M = en.M;
+    const int64_t n = en.N;
+    T(*S)[T_] = reinterpret_cast<T(*)[T_]>(smem_raw);
+    const int tid = threadIdx.x, tx = tid & 31, ty = tid >> 5;
+    const int64_t o = (int64_t)en.r * T_;
+    for (int idx = tid; idx < T_ * T_ / 4; idx += 1024) {
+        const int i = idx >> 5, c4 = idx & 31;
+        const int64_t gr = o + i, gc = o + c4 * 4;
+        int4 v = (gr < n && gc < n) ? *reinterpret_cast<const int4*>(M + gr * n + gc) : inf4<T>();
+        *reinterpret_cast<int4*>(&S[i][c4 * 4]) = v;
+    }
+    __syncthreads();
+    auto row4 = [&](int k, int at, T (&v)[4]) {
+        const int4 x = *reinterpret_cast<const int4*>(&S[k][at]);
+        const int y[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) v[i] = *reinterpret_cast<const T*>(&y[i]);
+    };
+    T acc[4][4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) row4(4 * ty + i, 4 * tx, acc[i]);
+    const int K = (int)((n - o) < T_ ? (n - o) : T_);
+    int k = 0;
+    // rows k and k + 1 are current (by symmetry also columns k and k + 1); row k + 1
+    // after step k is min(D(k+1, x), D(k+1, k) + D(k, x)), formed on the fly
+    for (; k + 1 < K; k += 2) {
+        T a0[4], b0[4], a1[4], b1[4];
+        row4(k, 4 * ty, a0);
+        row4(k, 4 * tx, b0);
+        row4(k + 1, 4 * ty, a1);
+        row4(k + 1, 4 * tx, b1);
+        const T skk = S[k][k + 1];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            a1[i] = MP<T>::upd1(a1[i], skk, a0[i]);
+            b1[i] = MP<T>::upd1(b1[i], skk, b0[i]);
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            if constexpr (std::is_same<T, float>::value) {
+                const float2 x0 = make_float2(a0[i], a0[i]), x1 = make_float2(a1[i], a1[i]);
+#pragma unroll
+                for (int j = 0; j < 4; j += 2) {
+                    const float2 s0 = __fadd2_rn(x0, make_float2(b0[j], b0[j + 1]));
+                    const float2 s1 = __fadd2_rn(x1, make_float2(b1[j], b1[j + 1]));
+                    acc[i][j] = fmin3(acc[i][j], s0.x, s1.x);
+                    acc[i][j + 1] = fmin3(acc[i][j + 1], s0.y, s1.y);
+                }
+            } else {
+#pragma unroll
+                for (int j = 0; j < 4; ++j) acc[i][j] = MP<T>::upd2(acc[i][j], a0[i], b0[j], a1[i], b1[j]);
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int row = 4 * ty + i;
+            if (row == k + 2 || row == k + 3)
+                *reinterpret_cast<int4*>(&S[row][4 * tx]) = as_int4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
+        }
+        __syncthreads();
+    }
+    for (; k < K; ++k) {
+        T a[4], b[4];
+        row4(k, 4 * ty, a);
+        row4(k, 4 * tx, b);
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) acc[i][j] = MP<T>::upd1(acc[i][j], a[i], b[j]);
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            if (4 * ty + i == k + 1)
+                *reinterpret_cast<int4*>(&S[k + 1][4 * tx]) = as_int4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
+        __syncthreads();
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int64_t gr = o + 4 * ty + i, gc = o + 4 * tx;
+        if (gr < n && gc < n)
+            *reinterpret_cast<int4*>(M + gr * n + gc) = as_int4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
+    }
+}
+
+// A step's tiles are split into strips when fewer than this many would be at work.
+constexpr int64_t kStripTiles = 152;
+
+// Phase 2: the candidate row tiles (r, J) <- D*(r, r) (x) D(r, J) and their transposes.  A
+// candidate that is all infinite stays so and is unmarked.  The last CTA of the run to finish
+// (counted; the counter is left at 0) does the compaction.
+template <typename T>
+__global__ void __launch_bounds__(NTH, SPQ_FW_MIN_CTAS) k_elim_phase2(const ElimEnt<T>* __restrict__ ents,
+                                                                      int32_t skip_inf) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    PanelSmem<T>& sm = *reinterpret_cast<PanelSmem<T>*>(smem_raw);
+    __shared__ uint32_t rm[4];
+    const ElimEnt<T> en = ents[blockIdx.y];
+    const ElimScratch sc(en.scratch, en.R);
+    T* __restrict__ M = en.M;
+    const int64_t n = en.N;
+    const int32_t r = en.r, R = en.R;
+    const int tid = threadIdx.x;
+    const int64_t o = (int64_t)r * T_;
+    const uint32_t c = sc.cand[0];
+    // the B panel is the tile's own rows: the chunks of rows that are all infinite are
+    // skipped; then the updated tile's finite rows are recorded for phase 3
+    if ((int64_t)c * gridDim.y <= kStripTiles) {
+        const int sx = tid & 7, sy = tid >> 3;
+        for (uint32_t ci = blockIdx.x; ci < c * kStrips; ci += gridDim.x) {
+            const int32_t J = (int32_t)sc.cand[1 + ci / kStrips];
+            const int64_t cs = (int64_t)J * T_ + (ci % kStrips) * SW;
+            T acc[4][4];
+            load_strip<T>(acc, M, n, o, cs, sx, sy);
+            strip_row_mask<T>(acc, rm, tid, sy);
+            uint32_t cm = 0u;
+#pragma unroll
+            for (int q = 0; q < NCHUNK; ++q) cm |= rm[q] ? (1u << q) : 0u;
+            if (cm == 0u) continue;
+            minplus_strip_masked<T>(acc, M, n, o, o, cs, sm, tid, sx, sy, cm);
+            strip_row_mask<T>(acc, rm, tid, sy);
+            if (tid < 4 && rm[tid]) atomicOr(&sc.kacc[(int64_t)J * 4 + tid], rm[tid]);
+            store_strip<T>(acc, M, n, o, cs, sx, sy);
+            store_strip_transposed<T>(acc, M, n, o, cs, sx, sy);
+        }
+    } else {
+        const int tx = tid & 15, ty = tid >> 4;
+        for (uint32_t ci = blockIdx.x; ci < c; ci += gridDim.x) {
+            const int32_t J = (int32_t)sc.cand[1 + ci];
+            const int64_t cj = (int64_t)J * T_;
+            T acc[8][8];
+            load_c<T>(acc, M, n, o, cj, tx, ty);
+            tile_row_mask<T>(acc, rm, tid, tx, ty);
+            uint32_t cm = 0u;
+#pragma unroll
+            for (int q = 0; q < NCHUNK; ++q) cm |= rm[q] ? (1u << q) : 0u;
+            if (cm == 0u) continue;
+            minplus_panels_masked<T>(acc, M, n, o, o, cj, sm, tid, tx, ty, cm);
+            tile_row_mask<T>(acc, rm, tid, tx, ty);
+            if (tid < 4) sc.kacc[(int64_t)J * 4 + tid] = rm[tid];
+            store_c<T>(acc, M, n, o, cj, tx, ty);
+            store_c_transposed<T>(acc, M, n, o, cj, tx, ty);
+        }
+    }
+    __shared__ uint32_t last;
+    __threadfence();  // (this CTA's tiles and masks, before its ticket)
+    __syncthreads();
+    if (tid == 0) last = atomicAdd(sc.counter, 1u) == gridDim.x - 1u ? 1u : 0u;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();  // (every other CTA's writes, after their tickets)
+    // the previous round's new tiles are initialised now
+    const uint32_t pc = sc.list[0];
+    for (uint32_t t = tid; t < pc * pc; t += blockDim.x) {
+        const uint32_t x = t / pc, y = t % pc;
+        if (y > x) {
+            uint32_t* f = en.rowflags + (int64_t)sc.list[1 + x] * R + sc.list[1 + y];
+            if (__ldcg(f) == 2u) *f = 1u;
+        }
+    }
+    for (uint32_t ci = tid; ci < c; ci += blockDim.x) {
+        const int64_t J = sc.cand[1 + ci];
+        uint4* ka = reinterpret_cast<uint4*>(sc.kacc + J * 4);
+        uint4* km = reinterpret_cast<uint4*>(sc.kmask + J * 4);
+        const uint4 m = __ldcg(ka);
+        *km = m;
+        *ka = make_uint4(0u, 0u, 0u, 0u);
+        if (!(m.x | m.y | m.z | m.w)) en.rowflags[(int64_t)r * R + J] = 0u;
+    }
+    __syncthreads();
+    if (!skip_inf)  // (no skipping: every tile of the row takes part)
+        for (int32_t J = r + 1 + tid; J < R; J += blockDim.x) en.rowflags[(int64_t)r * R + J] = 0xffffffffu;
+    __syncthreads();
+    compact_row(en.rowflags + (int64_t)r * R, r + 1, R, sc.list);
+    const uint32_t lc = sc.list[0];
+    for (uint32_t t = tid; t < lc * lc; t += blockDim.x) {
+        const uint32_t x = t / lc, y = t % lc;
+        if (y > x) {
+            uint32_t* f = en.rowflags + (int64_t)sc.list[1 + x] * R + sc.list[1 + y];
+            if (__ldcg(f) == 0u) *f = 2u;
+        }
+    }
+    if (tid == 0) {
+        sc.tiles[0] += (unsigned long long)lc * (lc + 1) / 2;
+        sc.tiles[1] += (unsigned long long)lc;
+        *sc.counter = 0u;
+    }
+    __syncthreads();
+    if (r + 1 < R) compact_row(en.rowflags + (int64_t)(r + 1) * R, r + 2, R, sc.cand);
+}
+
+// Phase 3: tiles (I, J), I <= J of the run's list, <- min(D(I, J), D(r, I)^T (x) D(r, J)).
+template <typename T>
+__global__ void __launch_bounds__(NTH, SPQ_FW_MIN_CTAS) k_elim_phase3(const ElimEnt<T>* __restrict__ ents,
+                                                                      int32_t skip_inf) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    PanelSmem<T>& sm = *reinterpret_cast<PanelSmem<T>*>(smem_raw);
+    const ElimEnt<T> en = ents[blockIdx.y];
+    const ElimScratch sc(en.scratch, en.R);
+    T* __restrict__ M = en.M;
+    const int64_t n = en.N;
+    const int tid = threadIdx.x;
+    const int64_t c = sc.list[0], tiles = c * (c + 1) / 2;
+    const int64_t o = (int64_t)en.r * T_;
+    const bool strips = tiles * gridDim.y <= kStripTiles;
+    for (int64_t t = blockIdx.x; t < (strips ? tiles * kStrips : tiles); t += gridDim.x) {
+        int64_t x, y;
+        tri_pair(strips ? t / kStrips : t, c, x, y);
+        const int64_t I = sc.list[1 + x], J = sc.list[1 + y];
+        uint32_t cm = (1u << NCHUNK) - 1u;
+        if (skip_inf) {  // only the chunks of pivot rows finite in both panels
+            cm = 0u;
+#pragma unroll
+            for (int q = 0; q < NCHUNK; ++q) cm |= (sc.kmask[I * 4 + q] & sc.kmask[J * 4 + q]) ? (1u << q) : 0u;
+        }
+        const bool fresh = I < J && en.rowflags[I * en.R + J] == 2u;
+        const bool shared = !fresh && I >= en.shared_from;
+        const int64_t ci = I * T_, cj = J * T_;
+        if (strips) {
+            const int sx = tid & 7, sy = tid >> 3;
+            const int64_t cs = cj + (t % kStrips) * SW;
+            T acc[4][4];
+            if (fresh) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) acc[i][j] = Inf<T>::value();
+            } else {
+                load_strip<T>(acc, M, n, ci, cs, sx, sy);
+            }
+            minplus_strip_masked<T>(acc, M, n, o, ci, cs, sm, tid, sx, sy, cm);
+            if (shared) {
+                store_strip_min<T>(acc, M, n, ci, cs, sx, sy, false);
+                if (I != J) store_strip_min<T>(acc, M, n, ci, cs, sx, sy, true);
+            } else {
+                store_strip<T>(acc, M, n, ci, cs, sx, sy);
+                if (I != J) store_strip_transposed<T>(acc, M, n, ci, cs, sx, sy);
+            }
+        } else {
+            const int tx = tid & 15, ty = tid >> 4;
+            T acc[8][8];
+            if (fresh) {
+#pragma unroll
+                for (int i = 0; i < 8; ++i)
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) acc[i][j] = Inf<T>::value();
+            } else {
+                load_c<T>(acc, M, n, ci, cj, tx, ty);
+            }
+            minplus_panels_masked<T>(acc, M, n, o, ci, cj, sm, tid, tx, ty, cm);
+            if (shared) {
+                store_c_min<T>(acc, M, n, ci, cj, tx, ty);
+                if (I != J) store_c_transposed_min<T>(acc, M, n, ci, cj, tx, ty);
+            } else {
+                store_c<T>(acc, M, n, ci, cj, tx, ty);
+                if (I != J) store_c_transposed<T>(acc, M, n, ci, cj, tx, ty);
+            }
+        }
+    }
+}
+
+// Sum of the runs' tile counters (run i's at base + off[i]).
+__global__ void k_elim_tiles(const uint32_t* __restrict__ base, const int64_t* __restrict__ off, int32_t nrun,
+                             unsigned long long* __restrict__ out) {
+    unsigned long long a = 0, b = 0;
+    for (int32_t i = threadIdx.x; i < nrun; i += blockDim.x) {
+        const unsigned long long* t = reinterpret_cast<const unsigned long long*>(base + off[i]);
+        a += t[0];
+        b += t[1];
+    }
+    atomicAdd(&out[0], a);
+    atomicAdd(&out[1], b);
+}
+
 int g_sms = 0;
 int sms() {
     if (g_sms == 0) {
@@ -690,7 +766,7 @@ cudaError_t set_smem_attrs() {
     cudaError_t e;
     e = cudaFuncSetAttribute(k_phase1<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, T_ * T_ * (int)sizeof(T));
     if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_phase1_wide, cudaFuncAttributeMaxDynamicSharedMemorySize, T_ * T_ * (int)sizeof(float));
+    e = cudaFuncSetAttribute(k_elim_phase1<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, T_ * T_ * (int)sizeof(T));
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(k_phase2<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(PanelSmem<T>));
     if (e != cudaSuccess) return e;
@@ -699,8 +775,9 @@ cudaError_t set_smem_attrs() {
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(k_phase3_list<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(PanelSmem<T>));
     if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_phase2_cand<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(PanelSmem<T>));
-
+    e = cudaFuncSetAttribute(k_elim_phase2<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(PanelSmem<T>));
+    if (e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(k_elim_phase3<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(PanelSmem<T>));
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(k_phase3_many<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(PanelSmem<T>));
     if (e != cudaSuccess) return e;
@@ -712,34 +789,147 @@ cudaError_t set_smem_attrs() {
 
 }  // namespace
 
-// One round r of the elimination form: phase 1, phase 2 over the candidates of row r,
-// the compaction (phase-3 list, marks, next candidates), phase 3 over the list.
+// The forward rounds of every matrix (see common.cuh).
 template <typename T>
-cudaError_t elim_round(T* M, const MatDesc* dd, int64_t N, int32_t r, int32_t R, uint32_t* rowflags, uint32_t* cand,
-                       uint32_t* list, bool skip_inf, unsigned long long* tiles, uint32_t* counter,
-                       uint32_t* kmask, int32_t shared_from, cudaEvent_t ev0, cudaEvent_t ev1, cudaStream_t st) {
-    const size_t psm = sizeof(PanelSmem<T>);
-    const int grid = sms() * 2;
-    if constexpr (std::is_same<T, float>::value)
-        k_phase1_wide<<<1, 1024, T_ * T_ * sizeof(float), st>>>(M, N, r);
-    else
-        k_phase1<T><<<dim3(1, 1), NTH, T_ * T_ * sizeof(T), st>>>(M, dd, 1, r, nullptr);
-    count_launches(1);
-    const int32_t np2 = R - 1 - r;
-    if (np2 > 0) {
-        // phase 2, and the compaction in its last CTA (without skipping: every tile J > r
-        // marked, so the compaction lists them all)
-        // (with skipping, phase 2 records the row masks of the row tiles it computed and
-        //  phase 3 skips the pivot-row chunks that are infinite in either panel)
-        uint32_t* km = skip_inf ? kmask : nullptr;
-        k_phase2_cand<T><<<np2 < grid ? np2 : grid, NTH, psm, st>>>(M, N, r, R, cand, rowflags, list, tiles,
-                                                                     counter, skip_inf ? 0 : 1, km);
-        if (ev0) cudaEventRecord(ev0, st);
-        k_phase3_list<T><<<grid, NTH, psm, st>>>(M, N, r, list, rowflags, R, shared_from, km);
-        if (ev1) cudaEventRecord(ev1, st);
-        count_launches(2);
+cudaError_t elim_forward(const std::vector<ElimMat<T>>& mats, bool skip_inf, double* updates, FwProfile* prof,
+                         cudaStream_t st, ElimPlan* keep) {
+    if (updates) *updates = 0.0;
+    cudaError_t e = set_smem_attrs<T>();
+    if (e != cudaSuccess || mats.empty()) {
+        if (keep) keep->ready = true;
+        return e;
     }
-    return cudaGetLastError();
+    const size_t psm = sizeof(PanelSmem<T>);
+    const bool replay = keep && keep->ready;
+    ElimPlan local;
+    ElimPlan& p = replay ? *keep : local;
+    if (!replay) {
+        // the runs of every matrix, each from the step after the last of its dependencies'
+        struct Run {
+            int32_t mat, lo, hi, shared_from, start;
+            int64_t scratch;
+        };
+        std::vector<Run> runs;
+        int64_t words = 0;
+        int32_t nstep = 0;
+        double diag = 0.0;
+        for (size_t m = 0; m < mats.size(); ++m) {
+            const int32_t R = (int32_t)((mats[m].N + T_ - 1) / T_);
+            diag += R;
+            std::vector<ElimTask> one(1);
+            one[0].hi = one[0].shared_from = R;
+            const std::vector<ElimTask>& tasks = mats[m].tasks && !mats[m].tasks->empty() ? *mats[m].tasks : one;
+            const size_t base = runs.size();
+            for (const ElimTask& tk : tasks) {
+                int32_t start = 0;
+                for (int32_t d : tk.deps) start = std::max(start, runs[base + d].start + runs[base + d].hi - runs[base + d].lo);
+                runs.push_back(Run{(int32_t)m, tk.lo, tk.hi, tk.shared_from, start, words});
+                words += round_up(ElimScratch::words(R), 4);
+                nstep = std::max(nstep, start + tk.hi - tk.lo);
+            }
+        }
+        std::vector<std::vector<ElimEnt<T>>> steps(nstep);
+        const size_t o_off = ((size_t)words * 4 + 15) & ~(size_t)15, o_out = o_off + runs.size() * 8;
+        size_t total = 0;
+        for (const Run& ru : runs) total += (size_t)std::max(ru.hi - ru.lo, 0);
+        const size_t o_ent = (o_out + 16 + 15) & ~(size_t)15;
+        if ((e = scratch_alloc((void**)&p.mem, o_ent + total * sizeof(ElimEnt<T>), st)) != cudaSuccess) return e;
+        std::vector<int64_t> off;
+        for (const Run& ru : runs) {
+            const ElimMat<T>& m = mats[ru.mat];
+            const int32_t R = (int32_t)((m.N + T_ - 1) / T_);
+            off.push_back(ru.scratch + 2 * R + 4);
+            for (int32_t r = ru.lo; r < ru.hi; ++r)
+                steps[ru.start + r - ru.lo].push_back(ElimEnt<T>{m.M, m.N, m.rowflags,
+                                                                 reinterpret_cast<uint32_t*>(p.mem) + ru.scratch, r, R,
+                                                                 ru.shared_from, r == ru.lo ? 1 : 0});
+        }
+        std::vector<ElimEnt<T>> ents;
+        ents.reserve(total);
+        for (const auto& s : steps) {
+            int32_t most = 0;  // row tiles right of a pivot
+            for (const ElimEnt<T>& x : s) most = std::max(most, x.R - 1 - x.r);
+            p.steps.push_back(ElimPlan::Step{ents.size(), (int32_t)s.size(), most});
+            ents.insert(ents.end(), s.begin(), s.end());
+        }
+        p.words = words;
+        p.nrun = (int32_t)runs.size();
+        p.o_off = o_off;
+        p.o_out = o_out;
+        p.o_ent = o_ent;
+        p.diag = diag;
+        if ((e = cudaMemcpyAsync(p.mem + o_off, off.data(), off.size() * 8, cudaMemcpyHostToDevice, st)) == cudaSuccess)
+            e = cudaMemcpyAsync(p.mem + o_ent, ents.data(), ents.size() * sizeof(ElimEnt<T>), cudaMemcpyHostToDevice, st);
+        if (e != cudaSuccess) {
+            p.release(st);
+            return e;
+        }
+    }
+    const ElimEnt<T>* d_ents = reinterpret_cast<const ElimEnt<T>*>(p.mem + p.o_ent);
+    unsigned long long* out = reinterpret_cast<unsigned long long*>(p.mem + p.o_out);
+    if ((e = cudaMemsetAsync(p.mem, 0, (size_t)p.words * 4, st)) == cudaSuccess) e = cudaMemsetAsync(out, 0, 16, st);
+    std::vector<cudaEvent_t> evs;  // around every phase 3 (profiling only)
+    if (prof && e == cudaSuccess) {
+        evs.resize(2 * p.steps.size(), nullptr);
+        for (auto& ev : evs)
+            if (e == cudaSuccess) e = cudaEventCreate(&ev);
+    }
+    for (size_t i = 0; i < p.steps.size() && e == cudaSuccess; ++i) {
+        const ElimPlan::Step& s = p.steps[i];
+        const ElimEnt<T>* en = d_ents + s.first;
+        // CTAs per run: two per SM side by side, or as many as its strips could use; a list
+        // is much shorter than the row (about 10 tiles on planar boundary graphs)
+        for (int32_t y0 = 0; y0 < s.count; y0 += 65535) {
+            const unsigned gy = (unsigned)std::min(s.count - y0, 65535);
+            const int64_t share = std::max<int64_t>(8, (4 * (int64_t)sms() + gy - 1) / gy);
+            const unsigned g2 = (unsigned)std::min<int64_t>(std::max<int64_t>(1, (int64_t)kStrips * s.most), std::min<int64_t>(share, 2 * sms()));
+            const unsigned g3 = (unsigned)std::min<int64_t>(2 * share, 2 * sms());
+            k_elim_phase1<T><<<dim3(2, gy), 1024, T_ * T_ * sizeof(T), st>>>(en + y0);
+            count_launches(1);
+            if (s.most > 0) {
+                k_elim_phase2<T><<<dim3(g2, gy), NTH, psm, st>>>(en + y0, skip_inf ? 1 : 0);
+                if (!evs.empty() && y0 == 0) cudaEventRecord(evs[2 * i], st);
+                k_elim_phase3<T><<<dim3(g3, gy), NTH, psm, st>>>(en + y0, skip_inf ? 1 : 0);
+                count_launches(2);
+            }
+        }
+        if (!evs.empty()) cudaEventRecord(evs[2 * i + 1], st);
+        e = cudaGetLastError();
+    }
+    if (!replay && e == cudaSuccess) {
+        k_elim_tiles<<<1, 256, 0, st>>>(reinterpret_cast<const uint32_t*>(p.mem),
+                                        reinterpret_cast<const int64_t*>(p.mem + p.o_off), p.nrun, out);
+        count_launches(1);
+        unsigned long long htv[2] = {0, 0};
+        e = cudaMemcpyAsync(htv, out, sizeof(htv), cudaMemcpyDeviceToHost, st);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+        const double t3 = (double)T_ * T_ * T_;
+        p.updates = ((double)htv[0] + (double)htv[1] + p.diag) * t3;  // phase 3, phase 2, phase 1 tiles
+        if (prof) {
+            prof->p3_ms = 0.0;
+            prof->p3_launches = 0;
+            for (size_t i = 0; e == cudaSuccess && i < p.steps.size(); ++i) {
+                float t = 0.f;
+                if (p.steps[i].most > 0 && cudaEventElapsedTime(&t, evs[2 * i], evs[2 * i + 1]) == cudaSuccess) {
+                    prof->p3_ms += t;
+                    prof->p3_launches += 1;
+                }
+            }
+            prof->p3_updates = (double)htv[0] * t3;
+        }
+    }
+    for (auto& ev : evs)
+        if (ev) cudaEventDestroy(ev);
+    if (updates) *updates = p.updates;
+    if (!replay) {
+        if (keep && e == cudaSuccess) {
+            p.ready = true;
+            *keep = std::move(p);
+        } else {
+            p.release(st);
+        }
+    }
+    return e;
 }
 
 template <typename T>
@@ -804,12 +994,12 @@ cudaError_t fw_batched(T* base, const MatDesc* d_descs, const MatDesc* h_descs, 
 
 int64_t fw_single_scratch_words(int64_t N) {
     int64_t R = (N + T_ - 1) / T_;
-    return 3 * R + 8;  // flags[R], list[1 + R] (+1 pad), two tile counters (u64), cand[1 + R] (+1)
+    return 2 * R + 8;  // flags[R], list[1 + R] (+1 pad), two tile counters (u64)
 }
 
 template <typename T>
-cudaError_t fw_single(T* M, int64_t N, bool skip_inf, uint32_t* scratch, uint32_t* rowflags, double* updates,
-                      FwProfile* prof, cudaStream_t st, const std::vector<ElimTask>* tasks) {
+cudaError_t fw_single(T* M, int64_t N, bool skip_inf, uint32_t* scratch, double* updates, FwProfile* prof,
+                      cudaStream_t st) {
     if (updates) *updates = 0.0;
     if (N <= 0) return cudaSuccess;
     cudaError_t e = set_smem_attrs<T>();
@@ -834,76 +1024,7 @@ cudaError_t fw_single(T* M, int64_t N, bool skip_inf, uint32_t* scratch, uint32_
         for (auto& ev : evs)
             if (e == cudaSuccess) e = cudaEventCreate(&ev);
     }
-    // runs of elimination rounds: one run over every block row, or the caller's runs (side
-    // by side on their own streams where they do not depend on each other)
-    std::vector<ElimTask> one(1);
-    one[0].lo = 0;
-    one[0].hi = R;
-    one[0].shared_from = R;
-    const std::vector<ElimTask>& runs = (rowflags && tasks && !tasks->empty()) ? *tasks : one;
-    const size_t nrun = rowflags ? runs.size() : 0;
-    // per run: list[R + 2], cand[R + 2], tiles (2 x u64), the phase-2 CTA counter (+ pad),
-    // the row masks of the round's row tiles (4 words per tile)
-    const int64_t rw = 6 * (int64_t)R + 10;
-    uint32_t* run_scratch = nullptr;
-    std::vector<cudaStream_t> rs(nrun, nullptr);
-    std::vector<cudaEvent_t> done(nrun, nullptr);
-    cudaEvent_t start_ev = nullptr;
-    if (nrun > 0) {
-        if (e == cudaSuccess) e = scratch_alloc((void**)&run_scratch, nrun * rw * sizeof(uint32_t), st);
-        if (e == cudaSuccess) e = cudaMemsetAsync(run_scratch, 0, nrun * rw * sizeof(uint32_t), st);
-        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&start_ev, cudaEventDisableTiming);
-        if (e == cudaSuccess) e = cudaEventRecord(start_ev, st);
-        for (size_t i = 0; i < nrun && e == cudaSuccess; ++i) {
-            e = cudaStreamCreateWithFlags(&rs[i], cudaStreamNonBlocking);
-            if (e == cudaSuccess) e = cudaEventCreateWithFlags(&done[i], cudaEventDisableTiming);
-            if (e == cudaSuccess) e = cudaStreamWaitEvent(rs[i], start_ev, 0);
-        }
-        // issue the rounds of every startable run in turn, one round at a time
-        std::vector<int32_t> next(nrun, 0), state(nrun, 0);  // 0 waiting, 1 issuing, 2 issued
-        size_t finished = 0;
-        while (finished < nrun && e == cudaSuccess) {
-            for (size_t i = 0; i < nrun && e == cudaSuccess; ++i) {
-                const ElimTask& tk = runs[i];
-                uint32_t* rl = run_scratch + i * rw;
-                uint32_t* rc = rl + R + 2;
-                unsigned long long* rt = reinterpret_cast<unsigned long long*>(rl + 2 * R + 4);
-                if (state[i] == 0) {
-                    bool ready = true;
-                    for (int32_t d : tk.deps) ready = ready && state[d] == 2;
-                    if (!ready) continue;
-                    for (int32_t d : tk.deps) cudaStreamWaitEvent(rs[i], done[d], 0);
-                    if (tk.lo < tk.hi) {  // candidates of the run's first round
-                        k_compact_trail<<<1, 1024, 0, rs[i]>>>(rowflags, R, tk.lo - 1, rl, rc, rt, 0);
-                        count_launches(1);
-                    }
-                    next[i] = tk.lo;
-                    state[i] = 1;
-                }
-                if (state[i] == 1) {
-                    if (next[i] < tk.hi) {
-                        const int32_t r = next[i]++;
-                        e = elim_round<T>(M, dd, N, r, R, rowflags, rc, rl, skip_inf, rt, rl + 2 * R + 8,
-                                          rl + 2 * R + 10, tk.shared_from,
-                                          evs.empty() ? nullptr : evs[2 * r], evs.empty() ? nullptr : evs[2 * r + 1],
-                                          rs[i]);
-                    } else {
-                        e = cudaEventRecord(done[i], rs[i]);
-                        state[i] = 2;
-                        ++finished;
-                    }
-                }
-            }
-        }
-        for (size_t i = 0; i < nrun && e == cudaSuccess; ++i) e = cudaStreamWaitEvent(st, done[i], 0);
-        // tile counters of every run, summed
-        for (size_t i = 0; i < nrun && e == cudaSuccess; ++i) {
-            k_add_u64<<<1, 32, 0, st>>>(tiles, reinterpret_cast<unsigned long long*>(run_scratch + i * rw + 2 * R + 4),
-                                        2);
-            count_launches(1);
-        }
-    }
-    for (int32_t r = 0; r < R && e == cudaSuccess && !rowflags; ++r) {
+    for (int32_t r = 0; r < R && e == cudaSuccess; ++r) {
         k_phase1<T><<<dim3(1, 1), NTH, T_ * T_ * sizeof(T), st>>>(M, dd, 1, r, nullptr);
         count_launches(1);
         if (R > 1) {
@@ -914,7 +1035,7 @@ cudaError_t fw_single(T* M, int64_t N, bool skip_inf, uint32_t* scratch, uint32_
             }
             k_compact<<<1, 1024, 0, st>>>(flags, R, r, list, tiles);
             if (!evs.empty()) cudaEventRecord(evs[2 * r], st);
-            k_phase3_list<T><<<p3_grid, NTH, psm, st>>>(M, N, r, list, nullptr, 0, (int32_t)R);
+            k_phase3_list<T><<<p3_grid, NTH, psm, st>>>(M, N, r, list);
             if (!evs.empty()) cudaEventRecord(evs[2 * r + 1], st);
             count_launches(3);
         }
@@ -924,17 +1045,10 @@ cudaError_t fw_single(T* M, int64_t N, bool skip_inf, uint32_t* scratch, uint32_
     if (e == cudaSuccess) e = cudaMemcpyAsync(htv, tiles, sizeof(htv), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     cudaFreeAsync(dd, st);
-    if (run_scratch) cudaFreeAsync(run_scratch, st);
-    for (auto& x : rs)
-        if (x) cudaStreamDestroy(x);
-    for (auto& x : done)
-        if (x) cudaEventDestroy(x);
-    if (start_ev) cudaEventDestroy(start_ev);
     if (prof) {
         prof->p3_ms = 0.0;
         prof->p3_launches = 0;
         for (size_t r = 0; e == cudaSuccess && 2 * r + 1 < evs.size(); ++r) {
-            if (rowflags && (int32_t)r + 1 >= R) break;  // no phase 3 in the last round
             float t = 0.f;
             if (cudaEventElapsedTime(&t, evs[2 * r], evs[2 * r + 1]) == cudaSuccess) {
                 prof->p3_ms += t;
@@ -1017,9 +1131,11 @@ template cudaError_t fw_batched<int32_t>(int32_t*, const MatDesc*, const MatDesc
                                          int32_t**);
 template cudaError_t fw_batched<float>(float*, const MatDesc*, const MatDesc*, int32_t, int32_t, cudaStream_t,
                                        int32_t**);
-template cudaError_t fw_single<int32_t>(int32_t*, int64_t, bool, uint32_t*, uint32_t*, double*, FwProfile*,
-                                        cudaStream_t, const std::vector<ElimTask>*);
-template cudaError_t fw_single<float>(float*, int64_t, bool, uint32_t*, uint32_t*, double*, FwProfile*, cudaStream_t,
-                                      const std::vector<ElimTask>*);
+template cudaError_t fw_single<int32_t>(int32_t*, int64_t, bool, uint32_t*, double*, FwProfile*, cudaStream_t);
+template cudaError_t fw_single<float>(float*, int64_t, bool, uint32_t*, double*, FwProfile*, cudaStream_t);
+template cudaError_t elim_forward<int32_t>(const std::vector<ElimMat<int32_t>>&, bool, double*, FwProfile*, cudaStream_t,
+                                           ElimPlan*);
+template cudaError_t elim_forward<float>(const std::vector<ElimMat<float>>&, bool, double*, FwProfile*, cudaStream_t,
+                                         ElimPlan*);
 
 }  // namespace spq

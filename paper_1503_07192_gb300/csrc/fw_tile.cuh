@@ -342,5 +342,149 @@ __device__ __forceinline__ void tile_row_mask(const T (&acc)[8][8], uint32_t* wo
     __syncthreads();
 }
 
+// ---------------- column strips ----------------
+// A quarter of a tile (128 rows x 32 columns) on a CTA of its own, 4 x 4 cells a thread: the
+// same sums and minima in a quarter of a tile's time, for launches with fewer tiles than the
+// GPU holds CTAs.
+constexpr int kStrips = 4;
+constexpr int SW = T_ / kStrips;  // strip width (32 columns: 8 threads x 4)
+
+// acc = min(acc, A (x) B) over a chunk for a strip: 4 x 4 per thread, rows 4sy.., strip
+// columns 4sx..; B rows of SW cells.
+template <typename T>
+__device__ __forceinline__ void strip_chunk(T (&acc)[4][4], const T (*a)[T_], const T* b, int sx, int sy, int kend) {
+#pragma unroll 2
+    for (int kk = 0; kk < kend; kk += 2) {
+        const int4 x = *reinterpret_cast<const int4*>(&a[kk][sy * 4]);
+        const int4 y = *reinterpret_cast<const int4*>(&a[kk + 1][sy * 4]);
+        const int4 z = *reinterpret_cast<const int4*>(b + kk * SW + sx * 4);
+        const int4 w = *reinterpret_cast<const int4*>(b + (kk + 1) * SW + sx * 4);
+        const int xa[4] = {x.x, x.y, x.z, x.w}, ya[4] = {y.x, y.y, y.z, y.w};
+        const int zb[4] = {z.x, z.y, z.z, z.w}, wb[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            if constexpr (std::is_same<T, float>::value) {
+                const float2 p0 = make_float2(__int_as_float(xa[i]), __int_as_float(xa[i]));
+                const float2 p1 = make_float2(__int_as_float(ya[i]), __int_as_float(ya[i]));
+#pragma unroll
+                for (int j = 0; j < 4; j += 2) {
+                    const float2 s0 = __fadd2_rn(p0, make_float2(__int_as_float(zb[j]), __int_as_float(zb[j + 1])));
+                    const float2 s1 = __fadd2_rn(p1, make_float2(__int_as_float(wb[j]), __int_as_float(wb[j + 1])));
+                    acc[i][j] = fmin3(acc[i][j], s0.x, s1.x);
+                    acc[i][j + 1] = fmin3(acc[i][j + 1], s0.y, s1.y);
+                }
+            } else {
+#pragma unroll
+                for (int j = 0; j < 4; ++j) acc[i][j] = MP<T>::upd2(acc[i][j], xa[i], zb[j], ya[i], wb[j]);
+            }
+        }
+    }
+}
+
+
+template <typename T>
+__device__ __forceinline__ int4 as_int4(T a, T b, T c, T d) {
+    return make_int4(*reinterpret_cast<int*>(&a), *reinterpret_cast<int*>(&b), *reinterpret_cast<int*>(&c),
+                     *reinterpret_cast<int*>(&d));
+}
+
+// Loads and stores of a strip: rows r0 + 4sy.., columns cs + 4sx..; cells outside the matrix
+// read as infinity.
+template <typename T>
+__device__ __forceinline__ void load_strip(T (&acc)[4][4], const T* __restrict__ M, int64_t n, int64_t r0, int64_t cs,
+                                           int sx, int sy) {
+    const int64_t r = r0 + 4 * sy, c = cs + 4 * sx;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int4 v = (r + i < n && c < n) ? *reinterpret_cast<const int4*>(M + (r + i) * n + c) : inf4<T>();
+        const int va[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = *reinterpret_cast<const T*>(&va[j]);
+    }
+}
+template <typename T>
+__device__ __forceinline__ void store_strip(const T (&acc)[4][4], T* __restrict__ M, int64_t n, int64_t r0,
+                                            int64_t cs, int sx, int sy) {
+    const int64_t r = r0 + 4 * sy, c = cs + 4 * sx;
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+        if (r + i < n && c < n)
+            *reinterpret_cast<int4*>(M + (r + i) * n + c) = as_int4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
+}
+template <typename T>
+__device__ __forceinline__ void store_strip_transposed(const T (&acc)[4][4], T* __restrict__ M, int64_t n, int64_t r0,
+                                                       int64_t cs, int sx, int sy) {
+    const int64_t r = r0 + 4 * sy, c = cs + 4 * sx;
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+        if (c + j < n && r < n)
+            *reinterpret_cast<int4*>(M + (c + j) * n + r) = as_int4(acc[0][j], acc[1][j], acc[2][j], acc[3][j]);
+}
+// (concurrent writers: the min of every contribution, as store_c_min)
+template <typename T>
+__device__ __forceinline__ void store_strip_min(const T (&acc)[4][4], T* __restrict__ M, int64_t n, int64_t r0,
+                                                int64_t cs, int sx, int sy, bool transposed) {
+    const int64_t r = r0 + 4 * sy, c = cs + 4 * sx;
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            if (r + i < n && c + j < n) {
+                T* p = transposed ? M + (c + j) * n + r + i : M + (r + i) * n + c + j;
+                atomicMin(reinterpret_cast<int*>(p), *reinterpret_cast<const int*>(&acc[i][j]));
+            }
+}
+
+// minplus_panels_masked for a strip: acc = min(acc, A (x) B) with A[i][k] = M[prow0 + k][acol0
+// + i], B[k][j] = M[prow0 + k][cs + j], over the chunks of the mask.
+template <typename T>
+__device__ __forceinline__ void minplus_strip_masked(T (&acc)[4][4], const T* __restrict__ M, int64_t n,
+                                                     int64_t prow0, int64_t acol0, int64_t cs, PanelSmem<T>& sm,
+                                                     int tid, int sx, int sy, uint32_t cmask) {
+    auto stage = [&](int c, int s) {
+        stage_chunk<T>(sm.a[s], M, n, prow0 + c * KC, acol0, tid);
+        T* dst = reinterpret_cast<T*>(sm.b[s]) + sy * SW + sx * 4;  // (32 rows x 8 vectors)
+        const int64_t r = prow0 + c * KC + sy, col = cs + sx * 4;
+        if (r < n && col < n)
+            cp_async16(dst, M + r * n + col);
+        else
+            *reinterpret_cast<int4*>(dst) = inf4<T>();
+        cp_async_commit();
+    };
+    int c = __ffs(cmask) - 1;
+    if (c < 0) return;
+    stage(c, 0);
+#pragma unroll 1
+    for (int s = 0; c >= 0; s ^= 1) {
+        cmask &= cmask - 1u;
+        const int next = __ffs(cmask) - 1;
+        if (next >= 0) {
+            stage(next, s ^ 1);
+            cp_async_wait<1>();
+        } else {
+            cp_async_wait<0>();
+        }
+        __syncthreads();
+        strip_chunk<T>(acc, sm.a[s], reinterpret_cast<const T*>(sm.b[s]), sx, sy, KC);
+        __syncthreads();
+        c = next;
+    }
+}
+
+// Rows of the CTA's strip with a finite cell, as tile_row_mask.
+template <typename T>
+__device__ __forceinline__ void strip_row_mask(const T (&acc)[4][4], uint32_t* words, int tid, int sy) {
+    __syncthreads();
+    if (tid < 4) words[tid] = 0u;
+    __syncthreads();
+    uint32_t f = 0u;
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) f |= acc[i][j] < Inf<T>::value() ? 1u << i : 0u;
+    if (f) atomicOr(&words[sy >> 3], f << (4 * (sy & 7)));
+    __syncthreads();
+}
+
 }  // namespace
 }  // namespace spq
