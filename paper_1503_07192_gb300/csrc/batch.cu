@@ -124,6 +124,8 @@ struct Inst {
     int64_t apsp_off = 0, apsp_elems = 0, d_off = 0, N = 0, nbg = 0;
     int32_t max_ld = 0;
     bool elim = false;  // boundary graph by elimination + back-substitution
+    int64_t marks = 0;  // ... its R x R marks in the batch's
+    BgLayout layout;    // aligned pieces of its order and their runs of rounds
     std::vector<int32_t> csize, nb, bgoff;
     std::vector<MatDesc> descs;  // relative to the instance's own APSP base
 };
@@ -142,14 +144,15 @@ struct BatchPtrs {
     int64_t table_elems = 0;
 };
 
-// The instances whose boundary graph takes the elimination form: their matrices'
-// descriptors (device), the forward rounds' scratch, the A-panel budget of the
-// back-substitution and its status word.
+// The instances whose boundary graph takes the elimination form: their matrices' marks
+// (the assembly's, kept, and the working copy that the rounds extend), the A-panel budget of
+// the back-substitution and its status word.
 struct BatchElim {
     int dev = 0;
-    int32_t n = 0, max_N = 0;
-    MatDesc* descs = nullptr;
-    uint32_t* scratch = nullptr;
+    int32_t n = 0;
+    uint32_t* marks0 = nullptr;
+    uint32_t* marks = nullptr;
+    int64_t mark_words = 0;
     uint32_t* err = nullptr;
     size_t panel_cap = 0;
 };
@@ -184,11 +187,13 @@ struct StageKeep {
     bool ready = false;
     CompElimPlan<T> ce;
     int32_t* fwb = nullptr;
+    ElimPlan fwd;
     BsPlan<T> bg;
     cudaStream_t s2 = nullptr;
     cudaEvent_t fork = nullptr, join = nullptr;
     void release(cudaStream_t st) {
         ce.release(st);
+        fwd.release(st);
         bg.release(st);
         if (fwb) cudaFreeAsync(fwb, st);
         fwb = nullptr;
@@ -264,10 +269,17 @@ cudaError_t batch_bg_tables(std::vector<Inst>& I, const BatchPtrs& P, const MatD
     const bool replay = keep && keep->ready;
     T* base = reinterpret_cast<T*>(P.tables);
     cudaError_t e;
+    if (be.n > 0 && (e = cudaMemcpyAsync(be.marks, be.marks0, (size_t)be.mark_words * 4, cudaMemcpyDeviceToDevice,
+                                         st)) != cudaSuccess)
+        return e;
     for (auto& x : I) {
         if (x.N == 0) continue;
         T* D = base + x.d_off;
-        if ((e = launch_bg_fill<T>(D, x.N, st)) != cudaSuccess) return e;
+        // (elimination: only the marked tiles and the diagonal are read before the
+        //  back-substitution writes every tile)
+        if ((e = x.elim ? launch_fill_marked<T>(D, x.N, be.marks + x.marks, st) : launch_bg_fill<T>(D, x.N, st)) !=
+            cudaSuccess)
+            return e;
         e = launch_bg_clique<T>(base + x.apsp_off, P.descs + x.kbase, P.nb + x.kbase, P.bgoff + x.kbase,
                                 P.bgpos + x.slotbase, x.k, D, x.N, st);
         if (e != cudaSuccess) return e;
@@ -314,11 +326,15 @@ cudaError_t batch_bg_tables(std::vector<Inst>& I, const BatchPtrs& P, const MatD
     double el_upd = 0.0;
     if (be.n > 0) {
         double fwd = 0.0, bs = 0.0;
-        e = fw_many_skip<T>(base, be.descs, be.n, be.max_N, be.scratch, &fwd, st, true, !replay);
+        std::vector<ElimMat<T>> mats;
+        std::vector<BsInput<T>> bin;
+        for (auto& x : I)
+            if (x.elim) {
+                mats.push_back(ElimMat<T>{base + x.d_off, x.N, be.marks + x.marks, &x.layout.tasks});
+                bin.push_back(BsInput<T>{base + x.d_off, x.N, be.marks + x.marks});
+            }
+        e = elim_forward<T>(mats, true, &fwd, nullptr, st, keep ? &keep->fwd : nullptr);
         if (e == cudaSuccess) {
-            std::vector<BsInput<T>> bin;
-            for (auto& x : I)
-                if (x.elim) bin.push_back(BsInput<T>{base + x.d_off, x.N, nullptr});
             e = bg_backsub_many<T>(bin, be.err, nullptr, be.panel_cap, &bs, nullptr, st, keep ? &keep->bg : nullptr);
         }
         el_upd = fwd + bs;
@@ -533,16 +549,32 @@ spq_status build_many_impl(int32_t G, const spq_graph* gs, const spq_opts& o, cu
         slot_tot += bo;
         max_ld = std::max(max_ld, x.max_ld);
     }
-    int64_t d_tot = 0;
     int32_t max_N = 0, nbmat = 0;
-    for (auto& x : I) {
-        x.d_off = apsp_tot + d_tot;
-        d_tot += x.N * x.N;
+    for (auto& x : I)
         if (x.N > 0) {
             ++nbmat;
             max_N = std::max(max_N, (int32_t)x.N);
         }
-    }
+    // The elimination's matrices may be ordered in aligned pieces whose rounds run side by
+    // side (a matrix of 146 row blocks alone was 146 rounds one after another, two fifths of a
+    // batch of 48): as many levels as leave pieces of 16 row blocks, each boundary padded to
+    // the tile edge.  Sized here for the most padding, placed once the order is known; without
+    // the pieces where that does not fit.
+    auto run_depth = [](int64_t nbg) {
+        int d = 0;
+        while (d < kMaxRunDepth && (nbg >> (d + 1)) >= 16 * kTile) ++d;
+        return d;
+    };
+    auto reserve = [&](bool pieces) {  // elements of every boundary-graph matrix
+        int64_t tot = 0;
+        for (auto& x : I) {
+            x.layout.depth = pieces && o.bg_method != SPQ_BG_FW && x.nbg >= kBatchElimMin ? run_depth(x.nbg) : 0;
+            const int64_t N = round_up(x.nbg + (((int64_t)2 << x.layout.depth) - 2) * (kTile - 1), 4);
+            tot += x.nbg > 0 ? N * N : 0;
+        }
+        return tot;
+    };
+    int64_t d_tot = reserve(true);
     // arena: metadata arrays, then the tables (16-byte aligned)
     size_t off = 0;
     auto take = [&](size_t bytes) {
@@ -554,9 +586,8 @@ spq_status build_many_impl(int32_t G, const spq_graph* gs, const spq_opts& o, cu
     const size_t o_descs = take(sizeof(MatDesc) * (size_t)ktot), o_nb = take(4 * (size_t)ktot);
     const size_t o_bgoff = take(4 * (size_t)ktot), o_csize = take(4 * (size_t)ktot);
     const size_t o_bgpos = take(4 * (size_t)slot_tot), o_err = take(16 * (size_t)G);
-    const int64_t table_elems = apsp_tot + d_tot;
-    const size_t o_tables = take(4 * (size_t)table_elems);
-    const size_t arena_bytes = off;
+    const size_t o_tables = off;
+    size_t arena_bytes = align256(o_tables + 4 * (size_t)(apsp_tot + d_tot));
     const int64_t fw_words = nbmat > 0 ? fw_many_scratch_words(nbmat, max_N) : 1;
     const bool comp_elim = o.comp_method != SPQ_BG_FW;
     const size_t temp_bytes = 16 * (size_t)ntot + 4 * (size_t)radix_hist_words(ntot) + 12 * (size_t)mtot +
@@ -565,6 +596,10 @@ spq_status build_many_impl(int32_t G, const spq_graph* gs, const spq_opts& o, cu
     size_t free_b = 0, total_b = 0;
     BCK(cudaMemGetInfo(&free_b, &total_b));
     free_b += pool_cached_bytes_current();
+    if (arena_bytes + temp_bytes > free_b) {
+        d_tot = reserve(false);
+        arena_bytes = align256(o_tables + 4 * (size_t)(apsp_tot + d_tot));
+    }
     if (arena_bytes + temp_bytes > free_b) return SPQ_ENOMEM;
     void* arena_base = nullptr;
     {
@@ -593,7 +628,6 @@ spq_status build_many_impl(int32_t G, const spq_graph* gs, const spq_opts& o, cu
     P.bgpos = reinterpret_cast<int32_t*>(ab + o_bgpos);
     P.err = reinterpret_cast<uint32_t*>(ab + o_err);
     P.tables = reinterpret_cast<uint32_t*>(ab + o_tables);
-    P.table_elems = table_elems;
     {
         std::vector<MatDesc> hd;
         std::vector<int32_t> hnb, hbo, hcs;
@@ -711,7 +745,8 @@ spq_status build_many_impl(int32_t G, const spq_graph* gs, const spq_opts& o, cu
                 if (hk[g].empty()) continue;
                 std::vector<int32_t> bp;
                 int32_t meth = 0;
-                if (boundary_order_host(x.k, x.nb, std::move(hk[g]), hs[g], hcm[g], order, &bp, &meth) != SPQ_OK ||
+                if (boundary_order_host(x.k, x.nb, std::move(hk[g]), hs[g], hcm[g], order, &bp, &meth,
+                                        x.layout.depth > 0 ? &x.layout : nullptr) != SPQ_OK ||
                     (int64_t)bp.size() != x.nbg) {
                     bad = 1;
                     continue;
@@ -729,7 +764,7 @@ spq_status build_many_impl(int32_t G, const spq_graph* gs, const spq_opts& o, cu
     }
 
     // ---- component tables of every instance (while the host orders the slots) ----
-    std::vector<MatDesc> cd, bd, ed;
+    std::vector<MatDesc> cd, bd;
     cd.reserve(ktot);
     // components by elimination (selected), the others by Floyd-Warshall (cd_fw: n = 0
     // for the selected ones)
@@ -820,22 +855,54 @@ spq_status build_many_impl(int32_t G, const spq_graph* gs, const spq_opts& o, cu
         x.elim = x.nbg > 0 && (o.bg_method == SPQ_BG_ELIM ||
                                (o.bg_method == SPQ_BG_AUTO && x.nbg >= kBatchElimMin && methods[g] != 0));
     }
-    for (auto& x : I)
-        if (x.N > 0) (x.elim ? ed : bd).push_back(MatDesc{x.d_off, (int32_t)x.N, 0});
-    int32_t max_N_fw = 0, max_N_el = 0;
-    for (const MatDesc& d : bd) max_N_fw = std::max(max_N_fw, d.n);
-    for (const MatDesc& d : ed) max_N_el = std::max(max_N_el, d.n);
+    // the matrices' places
     BatchElim be;
     BCK(cudaGetDevice(&be.dev));
-    be.n = (int32_t)ed.size();
-    be.max_N = max_N_el;
     be.panel_cap = o.bg_panel_mib > 0 ? ((size_t)o.bg_panel_mib << 20) : ((size_t)2 << 30);
+    int64_t at = apsp_tot;
+    int32_t max_N_fw = 0;
+    std::vector<int32_t> shared;  // the separators' blocks of every matrix (see launch_mark_pairs)
+    std::vector<size_t> shared_at(G + 1, 0);
+    for (int32_t g = 0; g < G; ++g) {
+        Inst& x = I[g];
+        if (x.layout.npad > 0) x.N = round_up(x.layout.npad, 4);
+        x.d_off = at;
+        at += x.N * x.N;
+        if (x.N > 0 && !x.elim) {
+            bd.push_back(MatDesc{x.d_off, (int32_t)x.N, 0});
+            max_N_fw = std::max(max_N_fw, (int32_t)x.N);
+        }
+        if (x.elim) {
+            const int64_t R = (x.N + kTile - 1) / kTile;
+            ++be.n;
+            x.marks = be.mark_words;
+            be.mark_words += R * R;
+            for (const ElimTask& tk : x.layout.tasks)
+                if (!tk.deps.empty())
+                    for (int32_t b = tk.lo; b < tk.hi; ++b) shared.push_back(b);
+        }
+        shared_at[g + 1] = shared.size();
+    }
+    P.table_elems = at;
     if (be.n > 0) {
-        BCK(tmp.alloc(&be.descs, ed.size()));
-        BCK(tmp.alloc(&be.scratch, (size_t)fw_many_scratch_words(be.n, be.max_N)));
+        int32_t* d_shared = nullptr;
+        BCK(tmp.alloc(&be.marks0, (size_t)be.mark_words));
+        BCK(tmp.alloc(&be.marks, (size_t)be.mark_words));
         BCK(tmp.alloc(&be.err, 1));
-        BCK(cudaMemcpyAsync(be.descs, ed.data(), ed.size() * sizeof(MatDesc), cudaMemcpyHostToDevice, st));
         BCK(cudaMemsetAsync(be.err, 0, 4, st));
+        BCK(cudaMemsetAsync(be.marks0, 0, (size_t)be.mark_words * 4, st));
+        if (!shared.empty()) {
+            BCK(tmp.alloc(&d_shared, shared.size()));
+            BCK(cudaMemcpyAsync(d_shared, shared.data(), shared.size() * 4, cudaMemcpyHostToDevice, st));
+        }
+        for (int32_t g = 0; g < G; ++g) {
+            const Inst& x = I[g];
+            if (!x.elim) continue;
+            BCK(launch_mark_bg_tiles(x.n, x.rp, x.col, x.part, P.local + x.vbase, P.nb + x.kbase, P.bgoff + x.kbase,
+                                     P.bgpos + x.slotbase, x.k, x.N, be.marks0 + x.marks, st));
+            BCK(launch_mark_pairs(d_shared + shared_at[g], (int32_t)(shared_at[g + 1] - shared_at[g]), x.N,
+                                  be.marks0 + x.marks, st));
+        }
     }
     BCK(tmp.alloc(&d_bd, bd.size()));
     BCK(tmp.alloc(&fw_scratch, (size_t)fw_words));

@@ -39,3 +39,24 @@ def test_elimination_equals_floyd_warshall(kind, side, leaf, panel, arith):
         assert np.array_equal(a.apsp(c), b.apsp(c))
     a.free()
     b.free()
+
+
+def test_batched_pieces_equal_floyd_warshall():
+    """Batched instances whose boundary graphs are ordered in aligned pieces (from 4,096 slots,
+    2 to 8 leaf runs side by side), beside smaller ones and one with pockets, against
+    Floyd-Warshall of each alone."""
+    graphs = []
+    for side, leaf, holes in [(40, 60, 0.0), (150, 24, 0.0), (230, 24, 0.0), (170, 20, 0.25)]:
+        if holes:
+            g = gen.graphs.grid_holes(side * side, holes, wmax=100, seed=side)
+        else:
+            g = gen.graphs.grid4(side, side, wmax=100, seed=side)
+        graphs.append((g, *gen.partition.kdtree(g.xy, leaf)))
+    hs = spq.spq_build_many([(g.n, g.row_ptr, g.col, g.w, part, k) for g, part, k in graphs])
+    assert max(h.stats()["n_bg"] for h in hs) >= 16384
+    for h, (g, part, k) in zip(hs, graphs):
+        b = spq.spq_build(g.n, g.row_ptr, g.col, g.w, part, k, _opts(spq.SPQ_BG_FW, spq.SPQ_ARITH_F32, 0))
+        assert np.array_equal(h.bg(), b.bg())
+        b.free()
+    for h in hs:
+        h.free()
