@@ -226,25 +226,28 @@ __global__ void __launch_bounds__(256) k_unpermute(T* __restrict__ A, const T* _
     for (int32_t s = blockIdx.y; s < nsel; s += gridDim.y) {
         const int32_t c = sel[s];
         const MatDesc d = descs[c];
-        const int32_t a = blockIdx.x;
-        if (a >= d.n) continue;  // (the same for the whole block)
         const int32_t nc = csize[c];
         const int32_t* pos = ndpos + vstart[c];
-        const int32_t pa = a < nc ? pos[a] : a;
-        const int4* prow = reinterpret_cast<const int4*>(P + d.off + (int64_t)pa * d.n);
-        for (int32_t b4 = threadIdx.x; b4 < d.n / 4; b4 += blockDim.x) reinterpret_cast<int4*>(row)[b4] = prow[b4];
-        __syncthreads();
-        int4* arow = reinterpret_cast<int4*>(A + d.off + (int64_t)a * d.n);
-        for (int32_t b4 = threadIdx.x; b4 < d.n / 4; b4 += blockDim.x) {
-            T v[4];
+        // (a block takes rows in a stride: a block per row of the largest component is mostly
+        //  blocks without a row where the sizes are uneven, 2.2 ms for 48 graphs in
+        //  components of 128 to 2,048)
+        for (int32_t a = blockIdx.x; a < d.n; a += gridDim.x) {
+            const int32_t pa = a < nc ? pos[a] : a;
+            const int4* prow = reinterpret_cast<const int4*>(P + d.off + (int64_t)pa * d.n);
+            for (int32_t b4 = threadIdx.x; b4 < d.n / 4; b4 += blockDim.x) reinterpret_cast<int4*>(row)[b4] = prow[b4];
+            __syncthreads();
+            int4* arow = reinterpret_cast<int4*>(A + d.off + (int64_t)a * d.n);
+            for (int32_t b4 = threadIdx.x; b4 < d.n / 4; b4 += blockDim.x) {
+                T v[4];
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const int32_t bb = 4 * b4 + e;
-                v[e] = row[bb < nc ? pos[bb] : bb];
+                for (int e = 0; e < 4; ++e) {
+                    const int32_t bb = 4 * b4 + e;
+                    v[e] = row[bb < nc ? pos[bb] : bb];
+                }
+                arow[b4] = *reinterpret_cast<const int4*>(v);
             }
-            arow[b4] = *reinterpret_cast<const int4*>(v);
+            __syncthreads();
         }
-        __syncthreads();
     }
 }
 
@@ -318,7 +321,7 @@ cudaError_t comp_elim_finish(T* apsp, T* P, const MatDesc* d_descs, const std::v
         cudaSuccess)
         return done(e);
     // back to the local order
-    const dim3 g((unsigned)max_el, (unsigned)std::min<size_t>(ed.size(), 65535));
+    const dim3 g((unsigned)std::min(max_el, 64), (unsigned)std::min<size_t>(ed.size(), 65535));
     k_unpermute<T><<<g, 256, 0, st>>>(apsp, P, d_descs, d_sel, (int32_t)ed.size(), d_csize, d_vstart, ndpos);
     count_launches(1);
     if ((e = cudaGetLastError()) != cudaSuccess) return done(e);
