@@ -1025,6 +1025,87 @@ spq_status build_many_impl(int32_t G, const spq_graph* gs, const spq_opts& o, cu
     return SPQ_OK;
 }
 
+// Streams beside st for the queries of many instances, which do not depend on one another:
+// an instance's dozen launches (keys, sort passes, items, blocks) are mostly too small to
+// fill the GPU (50,000 pairs: 0.2 ms, 70 us of it the blocks kernel), so up to four instances
+// are in flight.  fork() makes them wait for st's work so far, join() makes st wait for
+// theirs; both may be part of a stream capture, the streams outliving it.
+struct QueryLanes {
+    static constexpr int kMax = 4;
+    int n = 1;
+    cudaStream_t s[kMax] = {};
+    cudaEvent_t ev[kMax] = {};
+    // One lane for few instances, and for profiled handles (their events and counts are one
+    // launch's).
+    QueryLanes(int32_t count, spq_handle* const* hs, cudaStream_t st) {
+        s[0] = st;
+        if (count < kMax) return;
+        for (int32_t i = 0; i < count; ++i)
+            if (hs[i] && hs[i]->qstats) return;
+        bool ok = true;
+        for (int i = 0; i < kMax && ok; ++i) {
+            ok = cudaEventCreateWithFlags(&ev[i], cudaEventDisableTiming) == cudaSuccess;
+            if (ok && i > 0) ok = cudaStreamCreateWithFlags(&s[i], cudaStreamNonBlocking) == cudaSuccess;
+        }
+        if (ok) n = kMax;
+        cudaGetLastError();
+    }
+    ~QueryLanes() {
+        for (int i = 0; i < kMax; ++i) {
+            if (ev[i]) cudaEventDestroy(ev[i]);
+            if (i > 0 && s[i]) cudaStreamDestroy(s[i]);
+        }
+    }
+    cudaError_t fork() {
+        if (n == 1) return cudaSuccess;
+        cudaError_t e = cudaEventRecord(ev[0], s[0]);
+        for (int i = 1; i < n && e == cudaSuccess; ++i) e = cudaStreamWaitEvent(s[i], ev[0], 0);
+        return e;
+    }
+    cudaError_t join() {
+        cudaError_t e = cudaSuccess;
+        for (int i = 1; i < n && e == cudaSuccess; ++i) {
+            e = cudaEventRecord(ev[i], s[i]);
+            if (e == cudaSuccess) e = cudaStreamWaitEvent(s[0], ev[i], 0);
+        }
+        return e;
+    }
+};
+
+// The launches of one batch (device buffers) over the lanes; scratch: `words` per lane.
+cudaError_t issue_queries(int32_t count, spq_handle* const* hs, const int32_t* const* pairs, const int64_t* q,
+                          void* const* dist_out, uint32_t* scratch, int64_t words, QueryLanes& lanes) {
+    cudaError_t e = lanes.fork();
+    int lane = 0;
+    for (int32_t i = 0; i < count && e == cudaSuccess; ++i) {
+        if (q[i] == 0) continue;
+        QueryCtx<int32_t> ci;
+        QueryCtx<float> cf;
+        bool f32store = false, out_f32 = false;
+        int32_t k = 0;
+        handle_query_view(hs[i], &ci, &cf, &f32store, &out_f32, &k);
+        uint32_t* sc = hs[i]->query_grouped ? scratch + lane * words : nullptr;
+        cudaStream_t st = lanes.s[lane];
+        e = f32store ? launch_query<float>(cf, pairs[i], q[i], dist_out[i], out_f32, (uint32_t)k, sc, st)
+                     : launch_query<int32_t>(ci, pairs[i], q[i], dist_out[i], out_f32, (uint32_t)k, sc, st);
+        lane = (lane + 1) % lanes.n;
+    }
+    const cudaError_t j = lanes.join();  // (also after a failed launch: the scratch is freed in st's order)
+    return e != cudaSuccess ? e : j;
+}
+
+// Scratch words of one lane, and the lanes' scratch (fewer lanes where it does not fit).
+int64_t lane_words(int64_t qmax) { return round_up(query_scratch_words(std::max<int64_t>(qmax, 1)), 4); }
+cudaError_t lane_scratch(uint32_t** p, int64_t words, QueryLanes& lanes, cudaStream_t st) {
+    cudaError_t e = scratch_alloc((void**)p, (size_t)(words * lanes.n) * 4, st);
+    if (e != cudaSuccess && lanes.n > 1) {
+        cudaGetLastError();
+        lanes.n = 1;
+        e = scratch_alloc((void**)p, (size_t)words * 4, st);
+    }
+    return e;
+}
+
 }  // namespace
 
 extern "C" {
@@ -1064,26 +1145,30 @@ spq_status spq_query_many(int32_t count, spq_handle* const* hs, const int32_t* c
     }
     if (qtot == 0) return SPQ_OK;
     if (any_dev && any_host) return SPQ_EINVAL;
+    if (any_dev) {
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        cudaStreamIsCapturing(st, &cap);
+        QueryLanes lanes(cap == cudaStreamCaptureStatusNone ? count : 1, hs, st);
+        const int64_t words = lane_words(qmax);
+        uint32_t* scratch = nullptr;
+        BCK(lane_scratch(&scratch, words, lanes, st));
+        const cudaError_t e = issue_queries(count, hs, pairs, q, dist_out, scratch, words, lanes);
+        cudaFreeAsync(scratch, st);
+        return e == cudaSuccess ? SPQ_OK : batch_cuda_fail(e);
+    }
     TempList tmp(st);
     // one scratch for every instance's grouped form, reused in stream order
     uint32_t* scratch;
     BCK(tmp.alloc(&scratch, (size_t)query_scratch_words(qmax)));
-    int32_t* dpairs = nullptr;
-    int32_t* dout = nullptr;
-    if (any_host) {
-        BCK(tmp.alloc(&dpairs, 2 * (size_t)qtot));
-        BCK(tmp.alloc(&dout, (size_t)qtot));
-    }
+    int32_t *dpairs, *dout;
+    BCK(tmp.alloc(&dpairs, 2 * (size_t)qtot));
+    BCK(tmp.alloc(&dout, (size_t)qtot));
     int64_t base = 0;
     for (int32_t i = 0; i < count; ++i) {
         if (q[i] == 0) continue;
-        const int32_t* p = pairs[i];
-        void* o = dist_out[i];
-        if (any_host) {
-            BCK(cudaMemcpyAsync(dpairs + 2 * base, pairs[i], 2 * (size_t)q[i] * 4, cudaMemcpyHostToDevice, st));
-            p = dpairs + 2 * base;
-            o = dout + base;
-        }
+        BCK(cudaMemcpyAsync(dpairs + 2 * base, pairs[i], 2 * (size_t)q[i] * 4, cudaMemcpyHostToDevice, st));
+        const int32_t* p = dpairs + 2 * base;
+        void* o = dout + base;
         QueryCtx<int32_t> ci;
         QueryCtx<float> cf;
         bool f32store = false, out_f32 = false;
@@ -1092,25 +1177,21 @@ spq_status spq_query_many(int32_t count, spq_handle* const* hs, const int32_t* c
         uint32_t* sc = hs[i]->query_grouped ? scratch : nullptr;
         BCK(f32store ? launch_query<float>(cf, p, q[i], o, out_f32, (uint32_t)k, sc, st)
                      : launch_query<int32_t>(ci, p, q[i], o, out_f32, (uint32_t)k, sc, st));
-        if (any_host)
-            BCK(cudaMemcpyAsync(dist_out[i], dout + base, (size_t)q[i] * 4, cudaMemcpyDeviceToHost, st));
+        BCK(cudaMemcpyAsync(dist_out[i], dout + base, (size_t)q[i] * 4, cudaMemcpyDeviceToHost, st));
         base += q[i];
     }
-    if (any_host) {
-        BCK(cudaStreamSynchronize(st));
-        bool bad = false;
-        for (int32_t i = 0; i < count; ++i) {
-            if (q[i] == 0) continue;
-            uint32_t f = 0;
-            BCK(cudaMemcpy(&f, hs[i]->err, sizeof(f), cudaMemcpyDeviceToHost));
-            if (f & kErrPair) {
-                bad = true;
-                BCK(cudaMemset(hs[i]->err, 0, sizeof(uint32_t)));
-            }
+    BCK(cudaStreamSynchronize(st));
+    bool bad = false;
+    for (int32_t i = 0; i < count; ++i) {
+        if (q[i] == 0) continue;
+        uint32_t f = 0;
+        BCK(cudaMemcpy(&f, hs[i]->err, sizeof(f), cudaMemcpyDeviceToHost));
+        if (f & kErrPair) {
+            bad = true;
+            BCK(cudaMemset(hs[i]->err, 0, sizeof(uint32_t)));
         }
-        if (bad) return SPQ_EINVAL;
     }
-    return SPQ_OK;
+    return bad ? SPQ_EINVAL : SPQ_OK;
 }
 
 // A batched query plan: the launches of spq_query_many for fixed handles, device buffers
@@ -1135,26 +1216,6 @@ void plan_destroy(spq_query_plan* p) {
     delete p;
 }
 
-// The launches of one batch on stream st (device buffers; the grouped form's scratch is
-// shared in stream order).
-cudaError_t issue_queries(int32_t count, spq_handle* const* hs, const int32_t* const* pairs, const int64_t* q,
-                          void* const* dist_out, uint32_t* scratch, cudaStream_t st) {
-    for (int32_t i = 0; i < count; ++i) {
-        if (q[i] == 0) continue;
-        QueryCtx<int32_t> ci;
-        QueryCtx<float> cf;
-        bool f32store = false, out_f32 = false;
-        int32_t k = 0;
-        handle_query_view(hs[i], &ci, &cf, &f32store, &out_f32, &k);
-        uint32_t* sc = hs[i]->query_grouped ? scratch : nullptr;
-        const cudaError_t e = f32store ? launch_query<float>(cf, pairs[i], q[i], dist_out[i], out_f32, (uint32_t)k, sc, st)
-                                       : launch_query<int32_t>(ci, pairs[i], q[i], dist_out[i], out_f32, (uint32_t)k,
-                                                               sc, st);
-        if (e != cudaSuccess) return e;
-    }
-    return cudaSuccess;
-}
-
 }  // namespace
 
 spq_status spq_query_plan_create(int32_t count, spq_handle* const* hs, const int32_t* const* pairs, const int64_t* q,
@@ -1175,14 +1236,17 @@ spq_status spq_query_plan_create(int32_t count, spq_handle* const* hs, const int
     if (!p) return SPQ_ENOMEM;
     cudaStream_t st = (cudaStream_t)stream;
     cudaStream_t cs = nullptr;
-    cudaError_t e = scratch_alloc((void**)&p->scratch, (size_t)query_scratch_words(std::max<int64_t>(qmax, 1)) * 4, st);
+    const int64_t words = lane_words(qmax);
+    QueryLanes lanes(count, hs, st);
+    cudaError_t e = lane_scratch(&p->scratch, words, lanes, st);
     // one eager pass first (every kernel attribute set, the batch checked), then the capture
-    if (e == cudaSuccess) e = issue_queries(count, hs, pairs, q, dist_out, p->scratch, st);
+    if (e == cudaSuccess) e = issue_queries(count, hs, pairs, q, dist_out, p->scratch, words, lanes);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
-        const cudaError_t e1 = issue_queries(count, hs, pairs, q, dist_out, p->scratch, cs);
+        lanes.s[0] = cs;
+        const cudaError_t e1 = issue_queries(count, hs, pairs, q, dist_out, p->scratch, words, lanes);
         const cudaError_t e2 = cudaStreamEndCapture(cs, &p->graph);
         e = e1 != cudaSuccess ? e1 : e2;
     }
