@@ -208,7 +208,7 @@ spq_status spq_query(spq_handle* h, const int32_t* pairs, int64_t q, void* dist_
  *   - q <= SPQ_NOALLOC_MAX_PAIRS (a larger q returns SPQ_EINVAL and queues nothing);
  *   - pairs and dist_out must be device memory (else SPQ_EINVAL); the call returns once
  *     the work is queued, and spq_query_status reports out-of-range pairs;
- *   - its scratch is one fixed array of about 23.1 MB in the library's device memory,
+ *   - its scratch is one fixed array of about 23.2 MB in the library's device memory,
  *     present on every GPU that loads the library until the process exits.  The first
  *     call on a device looks up that array's address (cudaGetSymbolAddress, once per
  *     device); make that first call before any stream capture.  All calls share the

@@ -102,7 +102,21 @@ cudaError_t launch_validate_many(bool f32, const ValGraph* gs, const int64_t* vb
 // Stable LSD radix sort of (key, val) by the low key_bits bits.  Buffers: k0/v0 hold
 // the input, k1/v1 are scratch of the same size; hist needs radix_hist_words(n) words.
 // Returns (via *in_k1) whether the sorted result ended in k1/v1.
-int64_t radix_hist_words(int64_t n);
+// Keys per thread: 16 in long sorts; 4 in short ones (up to kRsShort keys), where a tile's
+// serial passes are what a launch takes and the tiles do not fill the GPU (10,000 keys: the
+// scatter 16 us with 3 tiles of 16 keys a thread).
+constexpr int kRsThreads = 256, kRsItems = 16, kRsItemsShort = 4;
+constexpr int64_t kRsShort = 1 << 17;
+constexpr int rs_items(int64_t n) { return n <= kRsShort ? kRsItemsShort : kRsItems; }
+constexpr int64_t rs_tiles(int64_t n) {
+    return (n + kRsThreads * rs_items(n) - 1) / (kRsThreads * rs_items(n));
+}
+// Histogram words for n keys or any fewer (a short sort has smaller tiles): per digit and
+// tile, then per digit.
+constexpr int64_t radix_hist_words(int64_t n) {
+    const int64_t a = rs_tiles(n), b = rs_tiles(n < kRsShort ? n : kRsShort), t = a > b ? a : b;
+    return 256 * (t > 0 ? t : 1) + 256;
+}
 // In-place exclusive prefix sum of len words (one CTA; for short arrays).
 cudaError_t launch_scan_excl(uint32_t* a, int64_t len, cudaStream_t st);
 cudaError_t radix_sort_pairs(uint32_t* k0, uint32_t* v0, uint32_t* k1, uint32_t* v1, uint32_t* hist, int64_t n,

@@ -5,6 +5,8 @@
 //    vertices first inside each component (each class in ascending vertex id), done
 //    with a stable LSD radix sort on the key 2 * part + (interior ? 1 : 0).
 #include <cuda_runtime.h>
+
+#include <algorithm>
 #include <math.h>
 
 #include "common.cuh"
@@ -132,19 +134,18 @@ __global__ void k_assign_local(int32_t n, const uint32_t* __restrict__ sorted_va
 }
 
 // ---------------- stable LSD radix sort, 8-bit digits ----------------
-constexpr int kRsThreads = 256;
-constexpr int kRsItems = 16;
-constexpr int kRsTile = kRsThreads * kRsItems;
 constexpr int kRsWarps = kRsThreads / 32;
 
 // hist[d * ntiles + t] = number of keys of tile t whose digit is d.
+template <int ITEMS>
 __global__ void __launch_bounds__(kRsThreads) k_rs_hist(const uint32_t* __restrict__ keys, int64_t n, int shift,
                                                         uint32_t* __restrict__ hist, int64_t ntiles) {
     __shared__ uint32_t h[256];
     h[threadIdx.x] = 0;
     __syncthreads();
-    int64_t base = (int64_t)blockIdx.x * kRsTile;
-    for (int it = 0; it < kRsItems; ++it) {
+    int64_t base = (int64_t)blockIdx.x * (kRsThreads * ITEMS);
+#pragma unroll
+    for (int it = 0; it < ITEMS; ++it) {
         int64_t i = base + it * kRsThreads + threadIdx.x;
         if (i < n) atomicAdd(&h[(keys[i] >> shift) & 255u], 1u);
     }
@@ -218,6 +219,7 @@ __global__ void __launch_bounds__(1024) k_scan_digits(uint32_t* __restrict__ his
 // Stable scatter of one tile: element it*256 + tid of the tile goes after every earlier
 // element of the tile with the same digit (earlier rounds, then lower warps, then lower
 // lanes of the same warp).
+template <int ITEMS>
 __global__ void __launch_bounds__(kRsThreads) k_rs_scatter(const uint32_t* __restrict__ kin,
                                                            const uint32_t* __restrict__ vin,
                                                            uint32_t* __restrict__ kout, uint32_t* __restrict__ vout,
@@ -247,8 +249,8 @@ __global__ void __launch_bounds__(kRsThreads) k_rs_scatter(const uint32_t* __res
     run[tid] = 0;
     for (int w = 0; w < kRsWarps; ++w) wcnt[w][tid] = 0;
     __syncthreads();
-    const int64_t base = (int64_t)blockIdx.x * kRsTile;
-    for (int it = 0; it < kRsItems; ++it) {
+    const int64_t base = (int64_t)blockIdx.x * (kRsThreads * ITEMS);
+    for (int it = 0; it < ITEMS; ++it) {
         int64_t i = base + it * kRsThreads + tid;
         bool valid = i < n;
         uint32_t key = valid ? kin[i] : 0u;
@@ -324,25 +326,27 @@ cudaError_t launch_scan_excl(uint32_t* a, int64_t len, cudaStream_t st) {
     return cudaGetLastError();
 }
 
-int64_t radix_hist_words(int64_t n) {
-    int64_t ntiles = (n + kRsTile - 1) / kRsTile;
-    return 256 * (ntiles > 0 ? ntiles : 1) + 256;  // per digit and tile, then per digit
-}
-
 cudaError_t radix_sort_pairs(uint32_t* k0, uint32_t* v0, uint32_t* k1, uint32_t* v1, uint32_t* hist, int64_t n,
                              int key_bits, bool* in_k1, cudaStream_t st) {
     *in_k1 = false;
     if (n <= 0) return cudaSuccess;
-    int64_t ntiles = (n + kRsTile - 1) / kRsTile;
+    const int64_t ntiles = rs_tiles(n);
+    const bool shrt = rs_items(n) == kRsItemsShort;
     bool flip = false;
     for (int shift = 0; shift < key_bits; shift += 8) {
         const uint32_t* ki = flip ? k1 : k0;
         const uint32_t* vi = flip ? v1 : v0;
         uint32_t* ko = flip ? k0 : k1;
         uint32_t* vo = flip ? v0 : v1;
-        k_rs_hist<<<(unsigned)ntiles, kRsThreads, 0, st>>>(ki, n, shift, hist, ntiles);
+        if (shrt)
+            k_rs_hist<kRsItemsShort><<<(unsigned)ntiles, kRsThreads, 0, st>>>(ki, n, shift, hist, ntiles);
+        else
+            k_rs_hist<kRsItems><<<(unsigned)ntiles, kRsThreads, 0, st>>>(ki, n, shift, hist, ntiles);
         k_scan_digits<<<256, 1024, 0, st>>>(hist, ntiles, hist + 256 * ntiles);
-        k_rs_scatter<<<(unsigned)ntiles, kRsThreads, 0, st>>>(ki, vi, ko, vo, n, shift, hist, ntiles);
+        if (shrt)
+            k_rs_scatter<kRsItemsShort><<<(unsigned)ntiles, kRsThreads, 0, st>>>(ki, vi, ko, vo, n, shift, hist, ntiles);
+        else
+            k_rs_scatter<kRsItems><<<(unsigned)ntiles, kRsThreads, 0, st>>>(ki, vi, ko, vo, n, shift, hist, ntiles);
         count_launches(3);
         flip = !flip;
     }

@@ -29,11 +29,11 @@ namespace spq {
 namespace {
 
 constexpr int64_t kMaxPairs = SPQ_NOALLOC_MAX_PAIRS;
-// 4 words per pair (keys, values and their sort copies) + one radix histogram of 256
-// words per 4,096-pair tile + 4 spare words, then the grouped kernel's records (18 words
+// 4 words per pair (keys, values and their sort copies) + the radix sort's histogram + 4
+// spare words, then the grouped kernel's records (18 words
 // per pair: table rows, starting values, item records, fallback list; + 8):
-// query_scratch_words(kMaxPairs), about 23.1 MB.
-constexpr int64_t kWords = 4 * kMaxPairs + (256 * ((kMaxPairs + 4095) / 4096) + 256) + 4 + 18 * kMaxPairs + 8;
+// query_scratch_words(kMaxPairs), about 23.2 MB.
+constexpr int64_t kWords = 4 * kMaxPairs + radix_hist_words(kMaxPairs) + 4 + 18 * kMaxPairs + 8;
 
 static __device__ __align__(256) uint32_t g_noalloc_scratch[kWords];
 
