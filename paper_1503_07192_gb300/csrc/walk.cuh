@@ -57,7 +57,7 @@ constexpr uint32_t kNoHop = 0xffffffffu;  // no entry of the table (searched on 
 template <typename T>
 struct WalkCtx {
     const int2* slots;        // [m]: (local index, 0) inside the component; (~slot, position); (INT_MIN, 0) self-loop
-    const int2* srange;       // [|BG|]: CSR range of a boundary slot's vertex
+    const int2* vrange;       // [n]: CSR range of the vertex at vstart[c] + local index
     const int32_t* scomp;     // [|BG|]: its component
     const int64_t* toff;      // [k + 1]: hops of component c at toff[c] + x * |B| + t
     const int64_t* foff;      // [k + 1]: flow of component c at foff[c] + b * |B| + y
@@ -65,13 +65,15 @@ struct WalkCtx {
     float* flow;
 };
 
-// Values compared as unsigned words: distances are never negative.
+// Values compared as unsigned words: distances are never negative (word_of: nor -0).
 __device__ __forceinline__ uint32_t key_of(int32_t v) { return (uint32_t)v; }
 __device__ __forceinline__ uint32_t key_of(float v) { return (uint32_t)__float_as_int(v + 0.0f); }
+__device__ __forceinline__ uint32_t word_of(int32_t v) { return (uint32_t)v; }
+__device__ __forceinline__ uint32_t word_of(float v) { return (uint32_t)__float_as_int(v); }
 
 template <typename T>
 __global__ void __launch_bounds__(256) k_walk_slots(const View<T> V, int2* __restrict__ slots,
-                                                    int2* __restrict__ srange, int32_t* __restrict__ scomp) {
+                                                    int2* __restrict__ vrange, int32_t* __restrict__ scomp) {
     const int32_t u = blockIdx.x * blockDim.x + threadIdx.x;
     if (u >= V.n) return;
     const int32_t c = V.comp[u], l = V.local[u];
@@ -86,25 +88,20 @@ __global__ void __launch_bounds__(256) k_walk_slots(const View<T> V, int2* __res
             slots[e] = make_int2(~s, V.bgpos[s]);
         }
     }
-    if (l < V.nb[c]) {
-        const int32_t s = V.bg_off[c] + l;
-        srange[s] = make_int2((int32_t)e0, (int32_t)e1);
-        scomp[s] = c;
-    }
+    vrange[V.vstart[c] + l] = make_int2((int32_t)e0, (int32_t)e1);
+    if (l < V.nb[c]) scomp[V.bg_off[c] + l] = c;
 }
 
 // The slot a walk inside component c takes at local vertex x towards local vertex t: the one
 // minimising w + dist_C(u, t), ties to the smallest slot.  sub lanes of the warp (lane g of
 // them) share the slots; every one of them returns the slot (-1: none) and, in x, the vertex.
 template <typename T, int SUB>
-__device__ __forceinline__ int64_t best_slot(const View<T>& V, const WalkCtx<T>& W, const T* A, int32_t ld,
+__device__ __forceinline__ int32_t best_slot(const View<T>& V, const WalkCtx<T>& W, const T* A, int32_t ld,
                                              int32_t vs, int32_t& x, int32_t t, int g, unsigned mask) {
-    const int32_t v = V.vorder[vs + x];
-    const int64_t e0 = V.rp[v], e1 = V.rp[v + 1];
+    const int2 er = W.vrange[vs + x];
     T best = Inf<T>::value();
-    int64_t be = INT64_MAX;
-    int32_t to = -1;
-    for (int64_t e = e0 + g; e < e1; e += SUB) {
+    int32_t be = INT32_MAX, to = -1;  // (a graph has fewer than INT32_MAX slots)
+    for (int32_t e = er.x + g; e < er.y; e += SUB) {
         const int32_t u = W.slots[e].x;
         if (u < 0) continue;
         const T cand = V.w[e] + A[(int64_t)u * ld + t];
@@ -117,7 +114,7 @@ __device__ __forceinline__ int64_t best_slot(const View<T>& V, const WalkCtx<T>&
 #pragma unroll
     for (int o = SUB / 2; o > 0; o >>= 1) {
         const T b2 = __shfl_xor_sync(mask, best, o);
-        const int64_t e2 = __shfl_xor_sync(mask, be, o);
+        const int32_t e2 = __shfl_xor_sync(mask, be, o);
         const int32_t t2 = __shfl_xor_sync(mask, to, o);
         if (less_lex(b2, e2, best, be)) {
             best = b2;
@@ -125,7 +122,7 @@ __device__ __forceinline__ int64_t best_slot(const View<T>& V, const WalkCtx<T>&
             to = t2;
         }
     }
-    if (be == INT64_MAX) return -1;
+    if (be == INT32_MAX) return -1;
     x = to;
     return be;
 }
@@ -183,7 +180,7 @@ __global__ void __launch_bounds__(256) k_walk_hops(const View<T> V, const WalkCt
 }
 
 // Walk inside component c from local vertex x to boundary vertex t along the hop table;
-// visit(slot, local vertex) each hop.  SUB lanes walk together (all of them call visit).
+// visit(from, slot - first slot of from, to) each hop.  SUB lanes walk together (all of them call visit).
 template <typename T, int SUB, typename Visit>
 __device__ __forceinline__ bool walk_hops(const View<T>& V, const WalkCtx<T>& W, int32_t c, int32_t x, int32_t t,
                                           int64_t limit, int g, unsigned mask, const Visit& visit) {
@@ -195,13 +192,13 @@ __device__ __forceinline__ bool walk_hops(const View<T>& V, const WalkCtx<T>& W,
         if (h != kNoHop) {
             const int32_t from = x;
             x = (int32_t)(h & 0xffffu);
-            visit(from, (int64_t)(h >> 16), x);
+            visit(from, (int32_t)(h >> 16), x);
         } else {
             const int32_t from = x;
             const MatDesc d = V.descs[c];
-            const int64_t e = best_slot<T, SUB>(V, W, V.apsp + d.off, d.n, vs, x, t, g, mask);
+            const int32_t e = best_slot<T, SUB>(V, W, V.apsp + d.off, d.n, vs, x, t, g, mask);
             if (e < 0) return false;
-            visit(from, e - V.rp[V.vorder[vs + from]], x);
+            visit(from, e - W.vrange[vs + from].x, x);
         }
     }
     return true;
@@ -212,10 +209,10 @@ __device__ __forceinline__ bool walk_hops(const View<T>& V, const WalkCtx<T>& W,
 // walk_boundary_graph: the move minimising dist_C(b, y) + D(y, b2) over the component's other
 // boundary vertices y or w(e) + D(u, b2) over the slots into other components, ties to the
 // smallest y, then to the smallest slot.
-template <typename T, typename Clique, typename Edge>
+// H: boundary vertices held per lane (components of up to 32 H; wider ones look the rest up).
+template <typename T, int H, typename Clique, typename Edge>
 __device__ __forceinline__ bool walk_bg(const View<T>& V, const WalkCtx<T>& W, int32_t c, int32_t l, int32_t c2,
                                         int32_t l2, int64_t limit, int lane, const Clique& clique, const Edge& edge) {
-    constexpr int H = 8;  // boundary vertices held per lane: components of up to 256
     const uint32_t kinf = key_of(Inf<T>::value());
     const int32_t s2 = V.bg_off[c2] + l2;
     const int64_t p2 = V.bgpos[s2];
@@ -226,7 +223,7 @@ __device__ __forceinline__ bool walk_bg(const View<T>& V, const WalkCtx<T>& W, i
     int64_t step = 0;
     bool fresh = true;
     T dv[H];
-    int32_t nb = 0, off = 0, ld = 0;
+    int32_t nb = 0, off = 0, ld = 0, vs = 0;
     const T* A = nullptr;
     for (;;) {
         if (c == c2 && l == l2) return true;
@@ -234,72 +231,73 @@ __device__ __forceinline__ bool walk_bg(const View<T>& V, const WalkCtx<T>& W, i
         if (fresh) {  // another component: its slots' distances to b2
             nb = V.nb[c];
             off = V.bg_off[c];
+            vs = V.vstart[c];
             const MatDesc d = V.descs[c];
             A = V.apsp + d.off;
             ld = d.n;
 #pragma unroll
             for (int q = 0; q < H; ++q) {
                 const int32_t y = lane + 32 * q;
-                dv[q] = y < nb ? dist(V.bgpos[off + y]) : Inf<T>::value();
+                // (+ 0: a sum with it is never -0, whose pattern is the largest)
+                dv[q] = y < nb ? dist(V.bgpos[off + y]) + T(0) : Inf<T>::value();
             }
             fresh = false;
         }
-        const int2 er = W.srange[off + l];
+        const int2 er = W.vrange[vs + l];
         const T* Ab = A + (int64_t)l * ld;
-        uint32_t bk = kinf, bi = 0xffffffffu;
+        // the sums over the component's other boundary vertices, as words that order like them
+        uint32_t key[H], bk = kinf;
         T av[H];
 #pragma unroll
         for (int q = 0; q < H; ++q) {
             const int32_t y = lane + 32 * q;
-            av[q] = y < nb ? Ab[y] : Inf<T>::value();
+            av[q] = y < nb && y != l ? Ab[y] : Inf<T>::value();
         }
-        // the slots into other components (the loads above are in flight meanwhile)
-        uint32_t ek = kinf, ei = 0xffffffffu;
+        // ... and over the slots into other components
+        uint32_t ek = kinf;
+        int32_t ei = 0;
         for (int32_t e = er.x + lane; e < er.y; e += 32) {
             const int2 s = W.slots[e];
             if (s.x >= 0 || s.x == INT32_MIN) continue;
-            const uint32_t k = key_of((T)(V.w[e] + dist(s.y)));
+            const uint32_t k = word_of((T)(V.w[e] + (dist(s.y) + T(0))));
             if (k < ek) {
                 ek = k;
-                ei = 0x80000000u | (uint32_t)e;
+                ei = e;
             }
         }
 #pragma unroll
         for (int q = 0; q < H; ++q) {
-            const int32_t y = lane + 32 * q;
-            if (y < nb && y != l) {
-                const uint32_t k = key_of((T)(av[q] + dv[q]));
-                if (k < bk) {
-                    bk = k;
-                    bi = (uint32_t)y;
-                }
-            }
+            key[q] = word_of((T)(av[q] + dv[q]));
+            bk = min(bk, key[q]);
         }
-        for (int32_t y = lane + 32 * H; y < nb; y += 32) {  // (wider components)
+        uint32_t wk = kinf;
+        int32_t wi = 0;
+        for (int32_t y = lane + 32 * H; y < nb; y += 32) {
             if (y == l) continue;
-            const uint32_t k = key_of((T)(Ab[y] + dist(V.bgpos[off + y])));
-            if (k < bk) {
-                bk = k;
-                bi = (uint32_t)y;
+            const uint32_t k = word_of((T)(Ab[y] + (dist(V.bgpos[off + y]) + T(0))));
+            if (k < wk) {
+                wk = k;
+                wi = y;
             }
         }
-        if (ek < bk) {
-            bk = ek;
-            bi = ei;
-        }
-        const uint32_t mk = __reduce_min_sync(0xffffffffu, bk);
+        const uint32_t mk = __reduce_min_sync(0xffffffffu, min(min(bk, wk), ek));
         if (mk >= kinf) return false;
-        const uint32_t mi = __reduce_min_sync(0xffffffffu, bk == mk ? bi : 0xffffffffu);
-        if (mi & 0x80000000u) {
-            const int32_t e = (int32_t)(mi & 0x7fffffffu);
+        // the smallest y attaining it, else the smallest slot
+        uint32_t yi = wk == mk ? (uint32_t)wi : 0xffffffffu;
+#pragma unroll
+        for (int q = H - 1; q >= 0; --q)
+            if (key[q] == mk) yi = (uint32_t)(lane + 32 * q);
+        const int32_t y = (int32_t)__reduce_min_sync(0xffffffffu, yi);
+        if (y >= 0) {
+            clique(c, l, y, nb);
+            l = y;
+        } else {
+            const int32_t e = (int32_t)__reduce_min_sync(0xffffffffu, ek == mk ? (uint32_t)ei : 0xffffffffu);
             const int32_t s = ~W.slots[e].x;
             edge(e, s);
             c = W.scomp[s];
             l = s - V.bg_off[c];
             fresh = true;
-        } else {
-            clique(c, l, (int32_t)mi, nb);
-            l = (int32_t)mi;
         }
     }
 }
