@@ -280,7 +280,7 @@ __global__ void __launch_bounds__(GTH) k_query_paths(const View<T> V, const int2
 // Part of a backward walk: the moves of pair i through the boundary graph.  A clique edge
 // adds the pair's upstream gradient to its flow, an edge between components to its slot.
 template <typename T, int H>
-__global__ void __launch_bounds__(GTH) k_backward_bg(const View<T> V, const WalkCtx<T> W,
+__global__ void __launch_bounds__(GTH, 5) k_backward_bg(const View<T> V, const WalkCtx<T> W,
                                                      const uint32_t* __restrict__ order, const int2* __restrict__ pairs, const int2* __restrict__ saved,
                                                      int64_t q, const float* __restrict__ gdist,
                                                      float* __restrict__ grad, uint32_t* __restrict__ err) {
@@ -312,7 +312,7 @@ __global__ void __launch_bounds__(GTH) k_backward_bg(const View<T> V, const Walk
 // v2 directly), searched slot by slot: v2 is any vertex.  Eight lanes a pair.
 constexpr int ESUB = 8;
 template <typename T>
-__global__ void __launch_bounds__(GTH) k_backward_ends(const View<T> V, const WalkCtx<T> W,
+__global__ void __launch_bounds__(GTH, 6) k_backward_ends(const View<T> V, const WalkCtx<T> W,
                                                        const uint32_t* __restrict__ order, const int2* __restrict__ pairs, const int2* __restrict__ saved,
                                                        int64_t q, const float* __restrict__ gdist,
                                                        float* __restrict__ grad, uint32_t* __restrict__ err) {
@@ -386,7 +386,7 @@ __global__ void __launch_bounds__(GTH) k_backward_flow(const View<T> V, const Wa
 // are collected 32 at a time, and each lane expands one of them: once to count its hops
 // (its place in the row is the sum of the earlier ones'), once to write its vertices.
 template <typename T, int H>
-__global__ void __launch_bounds__(GTH) k_paths_hops(const View<T> V, const WalkCtx<T> W,
+__global__ void __launch_bounds__(GTH, 4) k_paths_hops(const View<T> V, const WalkCtx<T> W,
                                                     const uint32_t* __restrict__ order, const int2* __restrict__ pairs, const int2* __restrict__ saved,
                                                     int64_t q, int32_t max_len, int32_t* __restrict__ verts,
                                                     int32_t* __restrict__ lens, uint32_t* __restrict__ err) {
