@@ -466,9 +466,8 @@ __global__ void __launch_bounds__(GTH, 4) k_paths_hops(const View<T> V, const Wa
                     [&](int32_t c, int32_t b, int32_t y, int32_t) {
                         if (ok) add(c, b, y);
                     },
-                    [&](int32_t, int32_t s) {
-                        const int32_t c = W.scomp[s];
-                        if (ok) add(-1, V.vorder[V.vstart[c] + s - V.bg_off[c]], 0);
+                    [&](int32_t, int32_t at) {
+                        if (ok) add(-1, V.vorder[at], 0);
                     });
                 if (ok && n > 0) ok = flush();
                 ok = ok && there;
@@ -546,7 +545,9 @@ bool walk_records(const spq_handle* h, bool want_flow, cudaStream_t st, WalkCtx<
         off[k + 2 + c] = off[k + 1 + c] + (int64_t)h->h_nb[c] * h->h_nb[c];
     }
     const int64_t nt = off[k], nf = want_flow ? off[2 * (size_t)k + 1] : 0;
-    const int64_t o_sr = h->m * 8, o_off = o_sr + (int64_t)h->n * 8, o_sc = o_off + (int64_t)off.size() * 8;
+    const int64_t o_out = h->nbg * (2 * kOut * 16);
+    const int64_t o_sl = o_out, o_sr = o_sl + h->m * 8, o_off = o_sr + (int64_t)h->n * 8;
+    const int64_t o_sc = o_off + (int64_t)off.size() * 8;
     const int64_t o_hop = o_sc + h->nbg * 4, o_fl = o_hop + nt * 4;
     unsigned char* p = nullptr;
     if (scratch_alloc((void**)&p, (size_t)(o_fl + nf * 4), st) != cudaSuccess) {
@@ -556,12 +557,13 @@ bool walk_records(const spq_handle* h, bool want_flow, cudaStream_t st, WalkCtx<
     *mem = p;
     *nflow = nf;
     int64_t* d_off = (int64_t*)(p + o_off);
-    *W = WalkCtx<T>{(int2*)p,          (int2*)(p + o_sr), (int32_t*)(p + o_sc),  d_off,
-                    d_off + (k + 1),   (uint32_t*)(p + o_hop), (float*)(p + o_fl)};
+    *W = WalkCtx<T>{(int2*)(p + o_sl), (int2*)(p + o_sr), (int32_t*)(p + o_sc),    (int4*)p,
+                    d_off,             d_off + (k + 1),   (uint32_t*)(p + o_hop), (float*)(p + o_fl)};
     const View<T> V = view_of<T>(h);
     cudaMemcpyAsync(d_off, off.data(), off.size() * 8, cudaMemcpyHostToDevice, st);
     if (nf > 0) cudaMemsetAsync(p + o_fl, 0, (size_t)nf * 4, st);
-    k_walk_slots<T><<<(unsigned)((h->n + 255) / 256), 256, 0, st>>>(V, (int2*)p, (int2*)(p + o_sr), (int32_t*)(p + o_sc));
+    k_walk_slots<T><<<(unsigned)((h->n + 255) / 256), 256, 0, st>>>(V, (int2*)(p + o_sl), (int2*)(p + o_sr),
+                                                                       (int32_t*)(p + o_sc), (int4*)p);
     k_walk_hops<T><<<(unsigned)(((int64_t)h->n * 32 + 255) / 256), 256, 0, st>>>(V, *W, (uint32_t*)(p + o_hop));
     count_launches(2);
     return true;

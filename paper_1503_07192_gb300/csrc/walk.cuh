@@ -3,9 +3,13 @@
 //
 // What bounds a walk is latency: a warp that looks at every slot of every vertex on the way
 // waits for five dependent loads a hop (0.2 ns of the whole GPU per hop: 86 ms for a million
-// pairs of 400 hops).  Three records shorten it:
+// pairs of 400 hops).  Four records shorten it:
 //   slots   per CSR slot its target's local index (same component) or boundary slot and
 //           matrix position (another component): no comp / local / bgpos look-ups on the way;
+//   out     per boundary slot its slots into other components with all that a move needs
+//           (slot, target, position, weight; the target's component, |B|, first slot, first
+//           vertex): one load where the CSR is three deep, and none of the look-ups by
+//           component after the move;
 //   hops    per component, vertex x and boundary vertex t: the slot that the walk from x
 //           towards t takes first and the vertex it leads to (4 bytes; sum of |C||B(C)|), so a
 //           hop towards a boundary vertex is one load;
@@ -52,13 +56,15 @@ __device__ __forceinline__ bool less_lex(T a, int64_t ai, T b, int64_t bi) {
     return a < b || (a == b && ai < bi);
 }
 
+constexpr int kOut = 4;  // slots into other components in a boundary slot's record
 constexpr uint32_t kNoHop = 0xffffffffu;  // no entry of the table (searched on the spot)
 
 template <typename T>
 struct WalkCtx {
     const int2* slots;        // [m]: (local index, 0) inside the component; (~slot, position); (INT_MIN, 0) self-loop
     const int2* vrange;       // [n]: CSR range of the vertex at vstart[c] + local index
-    const int32_t* scomp;     // [|BG|]: its component
+    const int32_t* scomp;     // [|BG|]: a boundary slot's component
+    const int4* out;          // [|BG| x kOut x 2]: a boundary slot's slots into other components
     const int64_t* toff;      // [k + 1]: hops of component c at toff[c] + x * |B| + t
     const int64_t* foff;      // [k + 1]: flow of component c at foff[c] + b * |B| + y
     const uint32_t* hops;
@@ -73,14 +79,27 @@ __device__ __forceinline__ uint32_t word_of(float v) { return (uint32_t)__float_
 
 template <typename T>
 __global__ void __launch_bounds__(256) k_walk_slots(const View<T> V, int2* __restrict__ slots,
-                                                    int2* __restrict__ vrange, int32_t* __restrict__ scomp) {
+                                                    int2* __restrict__ vrange, int32_t* __restrict__ scomp,
+                                                    int4* __restrict__ out) {
     const int32_t u = blockIdx.x * blockDim.x + threadIdx.x;
     if (u >= V.n) return;
     const int32_t c = V.comp[u], l = V.local[u];
     const int64_t e0 = V.rp[u], e1 = V.rp[u + 1];
+    const bool bnd = l < V.nb[c];
+    int4* o = out + (int64_t)(bnd ? V.bg_off[c] + l : 0) * (2 * kOut);
+    int n = 0;
     for (int64_t e = e0; e < e1; ++e) {
         const int32_t v = V.col[e];
         const int32_t cv = V.comp[v];
+        if (cv != c && bnd) {
+            if (n < kOut) {
+                const int32_t s = V.bg_off[cv] + V.local[v];
+                const T w = V.w[e];
+                o[2 * n] = make_int4((int32_t)e, s, V.bgpos[s], *reinterpret_cast<const int32_t*>(&w));
+                o[2 * n + 1] = make_int4(cv, V.nb[cv], V.bg_off[cv], V.vstart[cv]);
+            }
+            ++n;
+        }
         if (cv == c) {
             slots[e] = v == u ? make_int2(INT32_MIN, 0) : make_int2(V.local[v], 0);
         } else {
@@ -89,7 +108,11 @@ __global__ void __launch_bounds__(256) k_walk_slots(const View<T> V, int2* __res
         }
     }
     vrange[V.vstart[c] + l] = make_int2((int32_t)e0, (int32_t)e1);
-    if (l < V.nb[c]) scomp[V.bg_off[c] + l] = c;
+    if (bnd) {
+        scomp[V.bg_off[c] + l] = c;
+        // (unused places: position -1; too many slots: -2 in all, the CSR is searched)
+        for (int i = n > kOut ? 0 : n; i < kOut; ++i) o[2 * i] = make_int4(0, 0, n > kOut ? -2 : -1, 0);
+    }
 }
 
 // The slot a walk inside component c takes at local vertex x towards local vertex t: the one
@@ -205,7 +228,8 @@ __device__ __forceinline__ bool walk_hops(const View<T>& V, const WalkCtx<T>& W,
 }
 
 // Walk through the boundary graph from boundary vertex (c, l) to (c2, l2), the whole warp
-// together: clique(c, l, y, nb) or edge(e) for every move (all lanes call them).  As
+// together: clique(c, l, y, nb) or edge(e, the target's place in vorder) for every move (all
+// lanes call them).  As
 // walk_boundary_graph: the move minimising dist_C(b, y) + D(y, b2) over the component's other
 // boundary vertices y or w(e) + D(u, b2) over the slots into other components, ties to the
 // smallest y, then to the smallest slot.
@@ -223,15 +247,12 @@ __device__ __forceinline__ bool walk_bg(const View<T>& V, const WalkCtx<T>& W, i
     int64_t step = 0;
     bool fresh = true;
     T dv[H];
-    int32_t nb = 0, off = 0, ld = 0, vs = 0;
+    int32_t nb = V.nb[c], off = V.bg_off[c], vs = V.vstart[c], ld = 0;
     const T* A = nullptr;
     for (;;) {
         if (c == c2 && l == l2) return true;
         if (step++ >= limit) return false;
         if (fresh) {  // another component: its slots' distances to b2
-            nb = V.nb[c];
-            off = V.bg_off[c];
-            vs = V.vstart[c];
             const MatDesc d = V.descs[c];
             A = V.apsp + d.off;
             ld = d.n;
@@ -243,7 +264,9 @@ __device__ __forceinline__ bool walk_bg(const View<T>& V, const WalkCtx<T>& W, i
             }
             fresh = false;
         }
-        const int2 er = W.vrange[vs + l];
+        const int4* o = W.out + (int64_t)(off + l) * (2 * kOut);
+        const int4 oa = lane < kOut ? o[2 * lane] : make_int4(0, 0, -1, 0);
+        const int4 ob = lane < kOut ? o[2 * lane + 1] : make_int4(0, 0, 0, 0);
         const T* Ab = A + (int64_t)l * ld;
         // the sums over the component's other boundary vertices, as words that order like them
         uint32_t key[H], bk = kinf;
@@ -256,13 +279,22 @@ __device__ __forceinline__ bool walk_bg(const View<T>& V, const WalkCtx<T>& W, i
         // ... and over the slots into other components
         uint32_t ek = kinf;
         int32_t ei = 0;
-        for (int32_t e = er.x + lane; e < er.y; e += 32) {
-            const int2 s = W.slots[e];
-            if (s.x >= 0 || s.x == INT32_MIN) continue;
-            const uint32_t k = word_of((T)(V.w[e] + (dist(s.y) + T(0))));
-            if (k < ek) {
-                ek = k;
-                ei = e;
+        if (oa.z >= 0) {
+            const T w = *reinterpret_cast<const T*>(&oa.w);
+            ek = word_of((T)(w + (dist(oa.z) + T(0))));
+            ei = oa.x;
+        }
+        const bool many = __any_sync(0xffffffffu, oa.z == -2);
+        if (many) {
+            const int2 er = W.vrange[vs + l];
+            for (int32_t e = er.x + lane; e < er.y; e += 32) {
+                const int2 s = W.slots[e];
+                if (s.x >= 0 || s.x == INT32_MIN) continue;
+                const uint32_t k = word_of((T)(V.w[e] + (dist(s.y) + T(0))));
+                if (k < ek) {
+                    ek = k;
+                    ei = e;
+                }
             }
         }
 #pragma unroll
@@ -293,10 +325,23 @@ __device__ __forceinline__ bool walk_bg(const View<T>& V, const WalkCtx<T>& W, i
             l = y;
         } else {
             const int32_t e = (int32_t)__reduce_min_sync(0xffffffffu, ek == mk ? (uint32_t)ei : 0xffffffffu);
-            const int32_t s = ~W.slots[e].x;
-            edge(e, s);
-            c = W.scomp[s];
-            l = s - V.bg_off[c];
+            int32_t s;
+            if (many) {
+                s = ~W.slots[e].x;
+                c = W.scomp[s];
+                nb = V.nb[c];
+                off = V.bg_off[c];
+                vs = V.vstart[c];
+            } else {
+                const int src = __ffs(__ballot_sync(0xffffffffu, oa.z >= 0 && oa.x == e)) - 1;
+                s = __shfl_sync(0xffffffffu, oa.y, src);
+                c = __shfl_sync(0xffffffffu, ob.x, src);
+                nb = __shfl_sync(0xffffffffu, ob.y, src);
+                off = __shfl_sync(0xffffffffu, ob.z, src);
+                vs = __shfl_sync(0xffffffffu, ob.w, src);
+            }
+            edge(e, vs + s - off);
+            l = s - off;
             fresh = true;
         }
     }
