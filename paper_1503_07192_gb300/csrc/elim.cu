@@ -210,28 +210,40 @@ __global__ void __launch_bounds__(256) k_colmask(const BsMat<T>* __restrict__ ma
                                                  int32_t* __restrict__ fblk, int32_t* __restrict__ fcnt,
                                                  int32_t* __restrict__ kcnt, const int32_t* __restrict__ kplan,
                                                  uint32_t* __restrict__ err) {
-    __shared__ uint32_t colf[2][T_];
+    __shared__ uint32_t colf[8][32];
     __shared__ uint32_t wm[4];
     const BsMat<T> m = mats[blockIdx.y];
     const int32_t R = blockIdx.x, nR = m.nR;
     if (R >= nR) return;
     const int64_t N = m.N;
-    const int tid = threadIdx.x, c = tid & (T_ - 1), h = tid >> 7;
+    const int tid = threadIdx.x, c4 = tid & 31, h = tid >> 5;  // four columns, every eighth row
     const T inf = Inf<T>::value();
     const int64_t r0 = (int64_t)R * T_;
-    const int64_t nrows = (N - r0) < T_ ? (N - r0) : T_;
+    const int nrows = (int)((N - r0) < T_ ? (N - r0) : T_);
     int32_t cnt = 0, kc = 0;
     for (int32_t J = R + 1; J < nR; ++J) {
         if (m.rowflags && m.rowflags[(int64_t)R * nR + J] == 0u) continue;
-        const int64_t col = (int64_t)J * T_ + c;
+        const int64_t col = (int64_t)J * T_ + 4 * c4;
         uint32_t f = 0;
         if (col < N)
-            for (int64_t i = h; i < nrows; i += 2) f |= (m.M[(r0 + i) * N + col] < inf) ? 1u : 0u;
-        colf[h][c] = f;
+#pragma unroll
+            for (int i = 0; i < T_ / 8; ++i)
+                if (h + 8 * i < nrows) {
+                    const int4 v = *reinterpret_cast<const int4*>(m.M + (r0 + h + 8 * i) * N + col);
+                    const int va[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) f |= *reinterpret_cast<const T*>(&va[e]) < inf ? 1u << e : 0u;
+                }
+        colf[h][c4] = f;
         __syncthreads();
-        if (tid < T_) {
-            const unsigned b = __ballot_sync(0xffffffffu, (colf[0][tid] | colf[1][tid]) != 0u);
-            if ((tid & 31) == 0) wm[tid >> 5] = b;
+        if (tid < 32) {
+            for (int q = 1; q < 8; ++q) f |= colf[q][tid];
+            // eight lanes' four columns make a word
+            f <<= 4 * (tid & 7);
+            f |= __shfl_xor_sync(0xffffffffu, f, 1);
+            f |= __shfl_xor_sync(0xffffffffu, f, 2);
+            f |= __shfl_xor_sync(0xffffffffu, f, 4);
+            if ((tid & 7) == 0) wm[tid >> 3] = f;
         }
         __syncthreads();
         const uint4 mk = make_uint4(wm[0], wm[1], wm[2], wm[3]);
@@ -452,7 +464,9 @@ __global__ void __launch_bounds__(256) k_gather_a(const BsMat<T>* __restrict__ m
     const int32_t kc = kcnt[m.row0 + R];
     const int32_t kp = (kc + KC - 1) / KC * KC;
     const int64_t col0 = (int64_t)R * T_;
-    for (int64_t idx = threadIdx.x; idx < (int64_t)kp * (T_ / 4); idx += blockDim.x) {
+    // (a row block's panel is spread over gridDim.z blocks)
+    for (int64_t idx = blockIdx.z * blockDim.x + threadIdx.x; idx < (int64_t)kp * (T_ / 4);
+         idx += gridDim.z * blockDim.x) {
         const int32_t k = (int32_t)(idx >> 5), c4 = (int32_t)(idx & 31);
         int4 v = inf4<T>();
         if (k < kc && col0 + c4 * 4 < N)
@@ -782,7 +796,10 @@ cudaError_t bs_enqueue(const BsPlan<T>& p, uint32_t* err, uint32_t* exact, std::
     const int grid = sms_e() * SPQ_FW_MIN_CTAS;
     for (size_t l = 0; l < p.launches.size() && e == cudaSuccess; ++l) {
         const typename BsPlan<T>::Launch& L = p.launches[l];
-        const dim3 gg((unsigned)(std::min(L.R1, p.nRmax) - L.R0), (unsigned)L.nm);
+        // (few row blocks: more blocks each)
+        const int64_t gb = (int64_t)(std::min(L.R1, p.nRmax) - L.R0) * L.nm;
+        const dim3 gg((unsigned)(std::min(L.R1, p.nRmax) - L.R0), (unsigned)L.nm,
+                      (unsigned)std::max<int64_t>(1, std::min<int64_t>(8, 8 * sms_e() / gb)));
         // A panels of the launch's rows: read before the launch overwrites those rows
         if (conv)
             k_gather_a<T, std::is_same<T, float>::value><<<gg, 256, 0, st>>>(mats, L.mat0, L.R0, L.R1, p.koff, p.kcnt,
