@@ -312,10 +312,29 @@ def spq_query_many(handles, pairs_list, outs=None, stream=None) -> list:
     return outs_k
 
 
+def _raw_stream():
+    """The current CUDA stream's handle, without building a torch.cuda.Stream object."""
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    if raw is None:
+        return torch.cuda.current_stream().cuda_stream
+    return raw(torch.cuda.current_device())
+
+
 def spq_query(h: SpqHandle, pairs, out=None, stream=None):
     """dist(v1, v2) for each row of pairs (int32[q, 2]); returns int32[q] (float32 for
     float-weight graphs) in the same memory space as pairs."""
     lib = _lib.load()
+    # The usual call (a contiguous int32 CUDA tensor, no output given) without the general
+    # marshalling, which takes longer than a small batch does on the GPU (256 pairs: 14 us a
+    # call, about 6 of them the kernel).
+    if (out is None and stream is None and torch is not None and type(pairs) is torch.Tensor and pairs.is_cuda
+            and pairs.dtype is torch.int32 and pairs.dim() == 2 and pairs.is_contiguous()):
+        q = pairs.shape[0]
+        out = torch.empty(q, dtype=torch.float32 if h.wt == SPQ_F32 else torch.int32, device=pairs.device)
+        st = lib.spq_query(h.ptr, pairs.data_ptr(), q, out.data_ptr(), _raw_stream())
+        if st:
+            raise SpqError(st, "spq_query")
+        return out
     p_p, p_k, p_dev = _ptr(pairs, np.int32)
     q = int(p_k.shape[0]) if p_k.ndim > 1 else int(p_k.shape[0]) // 2
     odt = np.float32 if h.wt == SPQ_F32 else np.int32
