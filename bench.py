@@ -32,8 +32,8 @@ import sys
 import threading
 import time
 
-# up to 32 chains of elimination rounds run on their own streams: give the CUDA context
-# as many hardware work queues (before anything creates it)
+# batched builds, batched queries and the server run several streams beside the caller's:
+# give the CUDA context a hardware work queue for each (before anything creates it)
 os.environ.setdefault("CUDA_DEVICE_MAX_CONNECTIONS", "32")
 
 ROOT = os.path.dirname(os.path.abspath(__file__))
@@ -758,7 +758,10 @@ def main():
     bs_launches = sum(pf.get("bs_launches", 0.0) for _, pf, _ in per)
     bs_updates = sum(pf.get("bs_updates", 0.0) for _, pf, _ in per)
     sms = torch.cuda.get_device_properties(dev).multi_processor_count
-    peak_gops = sms * 128 * 2070e6 / 2 / 1e9  # 128 lanes/SM, 2 lane-ops per update, max SM clock
+    # updates per clock and SM of the kernels' inner loop alone (packed adds and three-input
+    # mins, operands from shared memory; measured), at the maximum SM clock.  (The 64 that one
+    # add and one min on 128 lanes would give is no bound: the two run on different pipes.)
+    peak_gops = sms * 74 * 2070e6 / 1e9
     kern = {
         "k_phase3_list": {"what": "k_phase3_list (boundary-graph elimination / Floyd-Warshall, phase 3)",
                           "ms": p3_ms, "launches": p3_launches, "updates": p3_updates, "traffic": None,
@@ -831,8 +834,9 @@ def main():
         "query_qps": q / (statistics.mean(query_ms) * 1e-3),
         "build_stage_ms": {k: round(statistics.mean(pf[k] for _, pf, _ in per), 2)
                            for k in ("validate", "reorder", "comp_fw", "bg_assemble", "bg_fw", "check")},
-        "roofline": dict(roof(top), peak_basis=f"{sms} SMs x 128 lanes x 2070 MHz / 2 lane-ops per min-plus "
-                                                 "update (derived)", microbench_gops=micro),
+        "roofline": dict(roof(top), peak_basis=f"{sms} SMs x 74 min-plus updates per clock (measured: packed adds + "
+                                                 "three-input mins from shared memory) x 2070 MHz",
+                         microbench_gops=micro),
         "roofline_other": [roof(x) for x in other] + ([roof_query] if roof_query else []),
         "gpu_launches": int(launches),
         "clocks": clk,

@@ -115,7 +115,8 @@ typedef struct spq_opts {
     int32_t query_grouped;  /* 1 (default): spq_query batches of >= 4096 pairs are sorted
                                by component pair (stream-ordered scratch of 16 bytes per
                                pair) so that each boundary-graph block is read once per
-                               group; 0: one warp per pair in input order, no scratch */
+                               group; smaller ones, and 0: in input order without scratch
+                               (one CTA per pair up to 4,096 pairs, one warp above) */
     int32_t bg_method;      /* spq_bg_method.  A struct_size that ends before this field
                                (an earlier version of the struct) means SPQ_BG_AUTO */
     int32_t bg_panel_mib;   /* SPQ_BG_ELIM: most MiB of device scratch for the gathered
@@ -276,7 +277,9 @@ void spq_build_plan_free(spq_build_plan* plan);
  * spq_query for `count` handles at once: pairs[i] (int32[q[i]][2]) against hs[i], answers
  * in dist_out[i].  All buffers host memory (synchronous; SPQ_EINVAL if any pair was out of
  * range) or all device memory (queued; spq_query_status per handle).  One scratch
- * allocation serves every instance, reused in stream order.
+ * allocation serves every instance; the instances run over up to four streams of the library
+ * that fork from `stream` and join it again (over `stream` alone while it is being captured,
+ * or where the scratch of four does not fit).
  */
 spq_status spq_query_many(int32_t count, spq_handle* const* hs, const int32_t* const* pairs, const int64_t* q,
                           void* const* dist_out, void* stream);
@@ -312,7 +315,9 @@ void spq_query_plan_free(spq_query_plan* plan);
  *     id is out of range).
  * Errors: SPQ_EINVAL for NULL buffers, mixed host/device buffers, ns or nt < 0 or above
  * 2^31 - 1; SPQ_EUNSUPPORTED for handles of spq_build_many or a component with more than
- * about 3,000 boundary vertices (the reuse buffer of a CTA).
+ * 6,400 boundary vertices.
+ * Scratch (stream-ordered): 16 bytes per target for their sort, and t of a batch of sources
+ * (at most about 64 MB or 64 sources' worth; fewer sources at a time where that does not fit).
  */
 spq_status spq_query_matrix(spq_handle* h, const int32_t* sources, int64_t ns, const int32_t* targets, int64_t nt,
                             void* dist_out, void* stream);
@@ -332,6 +337,9 @@ spq_status spq_query_matrix(spq_handle* h, const int32_t* sources, int64_t ns, c
  * hop = the neighbour minimising edge weight + table distance to the target).  Where the
  * path is unique this is the derivative of sum_i grad_dist[i] * dist_i with respect to the
  * slot weights (an undirected edge's derivative is the sum over its two slots).
+ * Scratch (stream-ordered): for large batches the pairs' sort and the walks' records (per CSR
+ * slot, boundary vertex and component's boundary pairs); where it does not fit, or while the
+ * stream is being captured, the pairs are answered and walked one by one without it.
  * pairs and saved must be those of the forward call on the same handle.  A walk that
  * cannot reach its target (zero-length cycles) sets a mark reported by spq_query_status.
  * Handles from spq_build_many return SPQ_EUNSUPPORTED.

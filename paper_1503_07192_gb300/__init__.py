@@ -11,9 +11,10 @@ Python or CPU fallback, and a missing library raises.
     spq_free(h)
 
 Importing the binding sets CUDA_DEVICE_MAX_CONNECTIONS to 32 unless the environment
-already sets it: the build runs up to 32 independent chains of elimination rounds on
-their own streams, and a CUDA context created with the default 8 hardware work queues
-serialises them.  It only takes effect if no CUDA context exists yet in the process.
+already sets it: a batched build, batched queries and the query server run several streams
+beside the caller's, and with the default 8 hardware work queues some of them would share
+one and wait for one another.  It only takes effect if no CUDA context exists yet in the
+process.
 """
 
 from __future__ import annotations

@@ -1,9 +1,10 @@
 // Gradients of query distances with respect to edge weights (float32 graphs).
 //
-// Forward (spq_query_saved): Algorithm 2 as in query.cu, one warp per pair, keeping the
-// minimising boundary pair (b1*, b2*) (local boundary indices; ties broken towards the
-// smallest (b1, b2) so the choice does not depend on the launch), or a marker: -1 the
-// same-component distance dist_C1(v1, v2) won, -2 v1 = v2, -3 no path.
+// Forward (spq_query_saved): Algorithm 2 as in query.cu, keeping the minimising boundary
+// pair (b1*, b2*) (local boundary indices; ties broken towards the smallest (b1, b2) so the
+// choice does not depend on the launch), or a marker: -1 the same-component distance
+// dist_C1(v1, v2) won, -2 v1 = v2, -3 no path.  One warp per pair, or for large batches
+// grouped by component pair (query_blocks.cu: the distance, then the witness that attains it).
 //
 // Backward (spq_query_backward): the distance is the length of a shortest path, so its
 // derivative with respect to the weight of a CSR slot is the number of times the path
@@ -15,6 +16,8 @@
 // other boundary vertices y of b's component (a clique edge, expanded into its path
 // inside the component) or w(b, u) + dist_BG(u, b2*) over the slots b -> u into other
 // components.  Each slot on the path receives the pair's upstream gradient (atomicAdd).
+// Where a batch's moves are worth it, those minima are first computed once for the whole graph
+// and the walks follow the records (walk.cuh); the form here finds each move on the way.
 #include <cuda_runtime.h>
 #include <math.h>
 

@@ -687,8 +687,7 @@ spq_status boundary_order_host(int32_t k, const std::vector<int32_t>& nb, std::v
         uptr[nslots] = wpos;
         std::vector<NdNode> nodes;
         // pieces of at least 16 tiles, layout->depth levels deep: up to 2^depth leaf runs
-        // side by side (32 at the most: as many as a context has hardware work queues when
-        // CUDA_DEVICE_MAX_CONNECTIONS is 32)
+        // (32 at the most) take their rounds side by side
         vertex_nd((int)best, k, ptr, adj, slot_off, uptr, snb, &slot_order,
                   layout ? std::min(std::max(layout->depth, 0), kMaxRunDepth) : 0, 16 * kTile,
                   layout ? &nodes : nullptr);

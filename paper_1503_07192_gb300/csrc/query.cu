@@ -1,4 +1,5 @@
-// Distance queries: Algorithm 2 of the paper, one warp per query pair.
+// Distance queries: Algorithm 2 of the paper for pairs in input order, a warp or a CTA per
+// pair, and the preparation of the grouped ones (query_blocks.cu).
 //
 // For (v1, v2) with components C1, C2:
 //   t(b2)  = min over b1 in B(C1) of dist_C1(v1, b1) + dist_BG(b1, b2)   (first loop)
@@ -10,7 +11,9 @@
 // the boundary-graph matrix at (bg_off[C1], bg_off[C2]) (the paper's Fig. 2: two
 // diagonal submatrices and one off-diagonal one).  Lanes own columns b2 (coalesced
 // reads of each block row), rows b1 are walked in order with dist_C1(v1, b1) broadcast
-// by shuffle, and a butterfly min-reduction over the warp finishes the second loop.
+// by shuffle, and a butterfly min-reduction over the warp finishes the second loop.  Up to
+// 4,096 pairs a whole CTA takes each pair instead (k_query_cta): its warps share the rows, so
+// a small batch, which cannot fill the chip with one warp a pair, does not walk them serially.
 #include <cuda_runtime.h>
 #include <math.h>
 

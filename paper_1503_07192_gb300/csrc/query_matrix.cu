@@ -348,7 +348,7 @@ extern "C" spq_status spq_query_matrix(spq_handle* h, const int32_t* sources, in
     handle_query_view(h, &ci, &cf, &f32store, &out_f32, &k);
     int32_t nbmax = 0;
     for (int32_t c = 0; c < k; ++c) nbmax = std::max(nbmax, h->h_nb[c]);
-    // (a component with more than about 6,000 boundary vertices)
+    // (a component with more than 6,400 boundary vertices)
     if ((size_t)(8 * (((nbmax > 0 ? nbmax : 1) + 31) & ~31)) * 4 > 200 * 1024) return SPQ_EUNSUPPORTED;
     std::vector<void*> tmp;
     auto alloc = [&](void** p, size_t bytes) {
@@ -380,16 +380,21 @@ extern "C" spq_status spq_query_matrix(spq_handle* h, const int32_t* sources, in
     }
     // the targets sorted by component, their tiles, t of a batch of sources
     const int64_t ldt = round_up(h->nbg + 3 * (int64_t)k, 4) + 4;
-    const int64_t rows = std::min(round_up(ns, MS), std::max<int64_t>(MS, kTElems / ldt / MS * MS));
+    int64_t rows = std::min(round_up(ns, MS), std::max<int64_t>(MS, kTElems / ldt / MS * MS));
     const int64_t max_tiles = (nt + MT - 1) / MT + k + 1;
     uint32_t *buf, *cnt;
     MTile* tiles;
     void* t;
     if ((e = alloc((void**)&buf, (size_t)(4 * nt + radix_hist_words(nt)) * 4)) != cudaSuccess ||
         (e = alloc((void**)&cnt, ((size_t)k + 2) * 4)) != cudaSuccess ||
-        (e = alloc((void**)&tiles, (size_t)max_tiles * sizeof(MTile))) != cudaSuccess ||
-        (e = alloc(&t, (size_t)(rows * ldt) * 4)) != cudaSuccess)
+        (e = alloc((void**)&tiles, (size_t)max_tiles * sizeof(MTile))) != cudaSuccess)
         return fail(e);
+    // (fewer sources at a time where t of that many does not fit)
+    while ((e = alloc(&t, (size_t)(rows * ldt) * 4)) == cudaErrorMemoryAllocation && rows > 1) {
+        cudaGetLastError();
+        rows = (rows + 1) / 2;
+    }
+    if (e != cudaSuccess) return fail(e);
     uint32_t* ntiles = cnt + k + 1;
     k_comp_keys<<<(unsigned)((nt + 255) / 256), 256, 0, st>>>(d_t, nt, h->n, h->comp, (uint32_t)k, buf, buf + nt);
     int bits = 0;
