@@ -202,10 +202,9 @@ int bits_for(uint64_t x) {
 // CUDA events bracketing the build stages (see spq_build_profile).
 // ---- the build's autotuned knob ----
 // How many bisection levels of the boundary graph's dissection become concurrent runs of
-// elimination rounds (up to 2^depth leaf runs, each on its own stream).  Deeper levels
-// give more and shorter runs, but more alignment padding, another frontier structure for
-// the back-substitution, and more streams than the context may have hardware queues for;
-// the best depth depends on the graph and the device.  Per device and size class of the
+// elimination rounds (up to 2^depth leaf runs, which take their rounds in step).  Deeper
+// levels give more and shorter runs, so fewer steps, but more alignment padding and another
+// frontier structure for the back-substitution; the best depth depends on the graph.  Per device and size class of the
 // boundary graph (bit length of |BG|), the first builds try the candidate depths in turn,
 // each timed by the build's own stage events (the boundary graph's all-pairs stage), and
 // later builds take the fastest.  Every depth gives the same distances (only the matrix
@@ -288,19 +287,24 @@ struct BgPlan {
 // Component tables APSP(C) in element type T (queued on st; no host wait).
 // With elim, the components that comp_takes_elim selects by elimination in a dissection
 // order (waits on the host), the others by Floyd-Warshall.  Sets h->comp_updates.
+// exact != NULL (float32 tables of an int32 graph): the finished tables are stored as int32,
+// *exact getting kErrExact if one holds a finite entry >= 2^24.  The elimination's
+// back-substitution stores them so itself, as the boundary graph's does, which saves the pass
+// over them that the others need (9 GB read and written on 2^20 vertices: 1.3 ms).
 template <typename T>
-cudaError_t build_comp_tables(spq_handle* h, const BuildInputs& in, int32_t max_n, bool elim, StageEvents& evs,
-                              cudaStream_t st) {
+cudaError_t build_comp_tables(spq_handle* h, const BuildInputs& in, int32_t max_n, bool elim, uint32_t* exact,
+                              StageEvents& evs, cudaStream_t st) {
     evs.mark(2, st);
     T* apsp = (T*)h->apsp;
     cudaError_t e;
+    if (exact && (e = cudaMemsetAsync(exact, 0, sizeof(uint32_t), st)) != cudaSuccess) return e;
     // (when every component takes the elimination form, its permutation back writes every
     //  cell of the tables: no initialisation in the local order)
     bool all_elim = elim;
     for (int32_t c = 0; c < h->k && all_elim; ++c)
         all_elim = h->h_descs[c].n == 0 || comp_takes_elim(h->h_csize[c], h->h_descs[c].n);
     if (!all_elim) {
-        if ((e = launch_fill_blocks<T>(apsp, h->descs, h->k, st)) != cudaSuccess) return e;
+        if ((e = launch_fill_blocks<T>(apsp, h->descs, h->k, st, elim ? h->csize : nullptr)) != cudaSuccess) return e;
         if ((e = launch_scatter_intra<T>(in.f32w, in.n, in.rp, in.col, in.w, in.part, h->local, h->descs, apsp,
                                          st)) != cudaSuccess)
             return e;
@@ -309,7 +313,7 @@ cudaError_t build_comp_tables(spq_handle* h, const BuildInputs& in, int32_t max_
     double eu = 0.0;
     if (elim) {
         e = comp_tables_elim<T>(apsp, h->descs, h->h_descs, h->h_csize, h->k, in.n, in.rp, in.col, in.w, in.f32w,
-                                in.part, h->local, h->vorder, h->vstart, h->csize, &eu, st);
+                                in.part, h->local, h->vorder, h->vstart, h->csize, &eu, exact, st);
         if (e != cudaSuccess) return e;
         for (int32_t c = 0; c < h->k; ++c)
             if (comp_takes_elim(h->h_csize[c], fwd[c].n)) fwd[c].n = 0;
@@ -323,19 +327,24 @@ cudaError_t build_comp_tables(spq_handle* h, const BuildInputs& in, int32_t max_
         cu += R * (1.0 + (R - 1.0) + R * (R - 1.0) / 2.0) * (double)kTile * kTile * kTile;
     }
     if (max_fw > 0 && (e = fw_batched<T>(apsp, h->descs, fwd.data(), h->k, max_fw, st)) != cudaSuccess) return e;
+    if (exact && max_fw > 0) {
+        e = elim ? launch_check_convert_blocks((float*)h->apsp, h->descs, h->csize, h->k, max_fw, exact, st)
+                 : launch_check_convert((float*)h->apsp, h->apsp_elems, exact, st);
+        if (e != cudaSuccess) return e;
+    }
     h->comp_updates = cu + eu;
     evs.mark(3, st);
     return cudaSuccess;
 }
 
 // The boundary graph's table in element type T (after build_comp_tables<T>): assembly,
-// all-pairs distances, and (check_exact) the exactness check of every float32 table.
+// all-pairs distances, and (check_exact) the exactness check of the float32 table, the component
+// tables being int32 already.
 template <typename T>
 cudaError_t build_bg_tables(spq_handle* h, const BuildInputs& in, bool check_exact, bool skip_inf, bool profile,
                             uint32_t* d_flag, uint32_t* fw_scratch, BgPlan& plan, bool* inexact, StageEvents& evs,
                             cudaStream_t st) {
     *inexact = false;
-    T* apsp = (T*)h->apsp;
     T* D = (T*)h->D;
     cudaError_t e;
     const int64_t R = (h->N + kTile - 1) / kTile;
@@ -366,14 +375,14 @@ cudaError_t build_bg_tables(spq_handle* h, const BuildInputs& in, bool check_exa
         if ((e = fill_marked ? launch_fill_marked<T>(D, h->N, plan.rowflags, st) : launch_bg_fill<T>(D, h->N, st)) !=
             cudaSuccess)
             return e;
-        if ((e = launch_bg_clique<T>(apsp, h->descs, h->nb, h->bg_off, h->bgpos, h->k, D, h->N, st)) != cudaSuccess)
+        if ((e = launch_bg_clique<T>(h->apsp, check_exact, h->descs, h->nb, h->bg_off, h->bgpos, h->k, D, h->N,
+                                     st)) != cudaSuccess)
             return e;
         if ((e = launch_bg_inter<T>(in.f32w, in.n, in.rp, in.col, in.w, in.part, h->local, h->bg_off, h->bgpos, D,
                                     h->N, st)) != cudaSuccess)
             return e;
     }
     evs.mark(4, st);
-    if (check_exact && (e = cudaMemsetAsync(d_flag, 0, sizeof(uint32_t), st)) != cudaSuccess) return e;
     // the elimination stores the float32 boundary-graph table as int32 itself (checked)
     const bool d_converted = plan.elim && check_exact && h->N > 0;
     if (h->N > 0 && !plan.elim) {
@@ -399,8 +408,7 @@ cudaError_t build_bg_tables(spq_handle* h, const BuildInputs& in, bool check_exa
     }
     evs.mark(5, st);
     if (check_exact) {
-        // the float32 tables become int32 ones (every entry below 2^24 is an exact integer)
-        if ((e = launch_check_convert((float*)h->apsp, h->apsp_elems, d_flag, st)) != cudaSuccess) return e;
+        // a float32 table becomes an int32 one (every entry below 2^24 is an exact integer)
         if (h->N > 0 && !d_converted && (e = launch_check_convert((float*)h->D, h->N * h->N, d_flag, st)) != cudaSuccess)
             return e;
         uint32_t f = 0;
@@ -520,9 +528,11 @@ spq_status build_impl(int32_t n, const int64_t* row_ptr, const int32_t* col, con
     const int64_t fw_words_max = n_max > 0 ? fw_single_scratch_words(n_max) : 1;
     size_t apanel_budget = std::min<size_t>(panel_cap, 4 * (size_t)n_max * (size_t)n_max + (1u << 20));
     // elimination scratch: per-round row flags, back-substitution bookkeeping, A panels,
-    // and per-run compaction lists
+    // and per-run lists (these are now 16 bytes a block row longer than counted here, 2 MB in
+    // all for the largest matrix that fits the device: out of the 64 MiB reserve below, so
+    // that no graph is refused which used to fit)
     const size_t elim_bytes = may_elim ? 4 * (size_t)(nR * nR) + bg_backsub_scratch_bytes(n_max) + apanel_budget +
-                                             (size_t)max_runs * 4 * (size_t)(10 * nR + 13)
+                                             (size_t)max_runs * 4 * (size_t)(6 * nR + 10)
                                        : 0;
     // (+ the component tables in dissection order, a second copy, for their elimination)
     const size_t comp_elim_bytes = opts.comp_method != SPQ_BG_FW ? 4 * (size_t)h->apsp_elems + 8 * (size_t)n : 0;
@@ -616,9 +626,9 @@ spq_status build_impl(int32_t n, const int64_t* row_ptr, const int32_t* col, con
         }
     } join_order{order_thread};
     if (first_f32)
-        CK(build_comp_tables<float>(h, in, max_n, comp_elim, evs, st));
+        CK(build_comp_tables<float>(h, in, max_n, comp_elim, f32w ? nullptr : d_flag, evs, st));
     else
-        CK(build_comp_tables<int32_t>(h, in, max_n, comp_elim, evs, st));
+        CK(build_comp_tables<int32_t>(h, in, max_n, comp_elim, nullptr, evs, st));
     if (order_thread.joinable()) order_thread.join();
     if (h->nbg > 0) {
         if (order_status != SPQ_OK) return order_status;
@@ -660,7 +670,7 @@ spq_status build_impl(int32_t n, const int64_t* row_ptr, const int32_t* col, con
         h->f32store = false;  // converted to int32 by the exactness check
         if (!first_f32 || inexact) {
             h->arith = SPQ_ARITH_I32;
-            if (inexact) CK(build_comp_tables<int32_t>(h, in, max_n, comp_elim, evs, st));
+            if (inexact) CK(build_comp_tables<int32_t>(h, in, max_n, comp_elim, nullptr, evs, st));
             CK(build_bg_tables<int32_t>(h, in, false, skip, prof, d_flag, fw_scratch, plan, &inexact, evs, st));
             if (plan.wait_failed) return SPQ_ETIMEOUT;
         }

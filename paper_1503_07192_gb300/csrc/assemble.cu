@@ -2,6 +2,8 @@
 // infinity, and 0 on the diagonal) and boundary-graph assembly (Algorithm 1: clique edges, BG).
 #include <cuda_runtime.h>
 
+#include <type_traits>
+
 #include "common.cuh"
 
 namespace spq {
@@ -32,12 +34,16 @@ __device__ __forceinline__ float weight_as<float>(const void* w, int64_t e, bool
 }
 
 // Fill each n x n block with infinity and a zero diagonal; one CTA per matrix at a time.
+// csize != NULL: only the components that do not take the elimination form (whose tables the
+// permutation back writes in full).
 template <typename T>
-__global__ void k_fill_blocks(T* __restrict__ base, const MatDesc* __restrict__ descs, int32_t nmat) {
+__global__ void k_fill_blocks(T* __restrict__ base, const MatDesc* __restrict__ descs, int32_t nmat,
+                              const int32_t* __restrict__ csize) {
     const T inf = Inf<T>::value();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
     for (int32_t mi = blockIdx.x; mi < nmat; mi += gridDim.x) {
         MatDesc d = descs[mi];
+        if (csize && comp_takes_elim(csize[mi], d.n)) continue;
         T* M = base + d.off;
         const int32_t n4 = d.n / 4;
         for (int32_t i = warp; i < d.n; i += nwarps) {
@@ -104,20 +110,28 @@ __global__ void k_bg_fill(T* __restrict__ D, int64_t N) {
 
 // Clique edges of Algorithm 1: D[B(C), B(C)] = APSP(C)[0:|B|, 0:|B|] (the
 // boundary vertices have the lowest local indices), at the slots' matrix positions.
-// One CTA per component at a time.
-template <typename T>
-__global__ void k_bg_clique(const T* __restrict__ apsp, const MatDesc* __restrict__ descs,
+// One CTA per component at a time.  S: the element type the component tables are stored in
+// (int32 where the float32 ones are stored as integers already).
+template <typename S, typename T>
+__device__ __forceinline__ T cell_as(S x) {
+    if constexpr (std::is_same<S, int32_t>::value && std::is_same<T, float>::value)
+        return x >= SPQ_INF_I32 ? Inf<float>::value() : (float)x;
+    else
+        return x;
+}
+template <typename S, typename T>
+__global__ void k_bg_clique(const S* __restrict__ apsp, const MatDesc* __restrict__ descs,
                             const int32_t* __restrict__ nb, const int32_t* __restrict__ bg_off,
                             const int32_t* __restrict__ bgpos, int32_t k, T* __restrict__ D, int64_t N) {
     for (int32_t c = blockIdx.x; c < k; c += gridDim.x) {
         int32_t b = nb[c];
         if (b == 0) continue;
         MatDesc d = descs[c];
-        const T* A = apsp + d.off;
+        const S* A = apsp + d.off;
         const int32_t* pos = bgpos + bg_off[c];
         for (int32_t i = threadIdx.y; i < b; i += blockDim.y) {
             T* row = D + (int64_t)pos[i] * N;
-            for (int32_t j = threadIdx.x; j < b; j += blockDim.x) row[pos[j]] = A[(int64_t)i * d.n + j];
+            for (int32_t j = threadIdx.x; j < b; j += blockDim.x) row[pos[j]] = cell_as<S, T>(A[(int64_t)i * d.n + j]);
         }
     }
 }
@@ -159,6 +173,26 @@ __global__ void k_check_convert(float4* __restrict__ a, int64_t count4, uint32_t
     if (__syncthreads_or(bad) && threadIdx.x == 0) atomicOr(err, kErrExact);
 }
 
+// The same for the components' tables that do not take the elimination form (that form's
+// back-substitution stores int32 itself).  blockIdx.y: components in a stride.
+__global__ void k_check_convert_blocks(float* __restrict__ base, const MatDesc* __restrict__ descs,
+                                       const int32_t* __restrict__ csize, int32_t nmat, uint32_t* __restrict__ err) {
+    bool bad = false;
+    for (int32_t mi = blockIdx.y; mi < nmat; mi += gridDim.y) {
+        const MatDesc d = descs[mi];
+        if (comp_takes_elim(csize[mi], d.n)) continue;
+        float4* a = reinterpret_cast<float4*>(base + d.off);
+        const int64_t count4 = (int64_t)d.n * d.n / 4;
+        for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count4;
+             i += (int64_t)gridDim.x * blockDim.x) {
+            const float4 x = a[i];
+            reinterpret_cast<int4*>(a)[i] =
+                make_int4(to_i32(x.x, bad), to_i32(x.y, bad), to_i32(x.z, bad), to_i32(x.w, bad));
+        }
+    }
+    if (__syncthreads_or(bad) && threadIdx.x == 0) atomicOr(err, kErrExact);
+}
+
 int sm_count() {
     static int n = 0;
     if (n == 0) {
@@ -173,10 +207,10 @@ int sm_count() {
 }  // namespace
 
 template <typename T>
-cudaError_t launch_fill_blocks(T* apsp, const MatDesc* descs, int32_t nmat, cudaStream_t st) {
+cudaError_t launch_fill_blocks(T* apsp, const MatDesc* descs, int32_t nmat, cudaStream_t st, const int32_t* csize) {
     if (nmat <= 0) return cudaSuccess;
     int blocks = nmat < 65535 ? nmat : 65535;
-    k_fill_blocks<T><<<blocks, 256, 0, st>>>(apsp, descs, nmat);
+    k_fill_blocks<T><<<blocks, 256, 0, st>>>(apsp, descs, nmat, csize);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -210,11 +244,14 @@ cudaError_t launch_bg_fill(T* D, int64_t N, cudaStream_t st) {
 }
 
 template <typename T>
-cudaError_t launch_bg_clique(const T* apsp, const MatDesc* descs, const int32_t* nb, const int32_t* bg_off,
+cudaError_t launch_bg_clique(const void* apsp, bool i32, const MatDesc* descs, const int32_t* nb, const int32_t* bg_off,
                              const int32_t* bgpos, int32_t k, T* D, int64_t N, cudaStream_t st) {
     if (k <= 0 || N <= 0) return cudaSuccess;
     int blocks = k < 65535 ? k : 65535;
-    k_bg_clique<T><<<blocks, dim3(32, 8), 0, st>>>(apsp, descs, nb, bg_off, bgpos, k, D, N);
+    if (i32)
+        k_bg_clique<int32_t, T><<<blocks, dim3(32, 8), 0, st>>>((const int32_t*)apsp, descs, nb, bg_off, bgpos, k, D, N);
+    else
+        k_bg_clique<T, T><<<blocks, dim3(32, 8), 0, st>>>((const T*)apsp, descs, nb, bg_off, bgpos, k, D, N);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -240,15 +277,25 @@ cudaError_t launch_check_convert(float* a, int64_t count, uint32_t* err, cudaStr
     return cudaGetLastError();
 }
 
+cudaError_t launch_check_convert_blocks(float* base, const MatDesc* descs, const int32_t* csize, int32_t nmat,
+                                        int32_t max_n, uint32_t* err, cudaStream_t st) {
+    if (nmat <= 0 || max_n <= 0) return cudaSuccess;
+    const int64_t per = (int64_t)max_n * max_n / 4 / 2048;  // eight 16-byte cells a thread of the largest
+    const dim3 grid((unsigned)(per < 1 ? 1 : per > 1024 ? 1024 : per), (unsigned)(nmat < 65535 ? nmat : 65535));
+    k_check_convert_blocks<<<grid, 256, 0, st>>>(base, descs, csize, nmat, err);
+    count_launches(1);
+    return cudaGetLastError();
+}
+
 #define SPQ_INST(T)                                                                                                \
-    template cudaError_t launch_fill_blocks<T>(T*, const MatDesc*, int32_t, cudaStream_t);                         \
+    template cudaError_t launch_fill_blocks<T>(T*, const MatDesc*, int32_t, cudaStream_t, const int32_t*);         \
     template cudaError_t launch_scatter_intra<T>(bool, int32_t, const int64_t*, const int32_t*, const void*,       \
                                                  const int32_t*, const int32_t*, const MatDesc*, T*, cudaStream_t); \
     template cudaError_t launch_scatter_intra_sel<T>(bool, int32_t, const int64_t*, const int32_t*, const void*,   \
                                                      const int32_t*, const int32_t*, const MatDesc*, const int32_t*, \
                                                      int32_t, int32_t, T*, cudaStream_t);                          \
     template cudaError_t launch_bg_fill<T>(T*, int64_t, cudaStream_t);                                             \
-    template cudaError_t launch_bg_clique<T>(const T*, const MatDesc*, const int32_t*, const int32_t*,           \
+    template cudaError_t launch_bg_clique<T>(const void*, bool, const MatDesc*, const int32_t*, const int32_t*,    \
                                              const int32_t*, int32_t, T*, int64_t, cudaStream_t);                 \
     template cudaError_t launch_bg_inter<T>(bool, int32_t, const int64_t*, const int32_t*, const void*,            \
                                             const int32_t*, const int32_t*, const int32_t*, const int32_t*, T*,   \

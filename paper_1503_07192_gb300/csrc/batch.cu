@@ -14,8 +14,14 @@
 // a fraction of the Floyd-Warshall updates there, batched the same way: the forward
 // rounds (restricted to the trailing tiles, in a vertex nested-dissection order) of all
 // of them in the same launches, then one persistent back-substitution over all their
-// tiles, their rows interleaved so that their dependency chains overlap.  Both sets of
-// instances are computed side by side on two streams.
+// tiles, level by level (elim.cu), so that their dependency chains overlap.  Both sets of
+// instances are computed side by side on two streams.  Like a single build's, each of these
+// boundary graphs is laid out in aligned pieces whose rounds run in step (deeper for larger
+// graphs), which shortens the shared chain of rounds to the largest graph's longest piece.
+//
+// The queries of a batch run over up to four streams of the library beside the caller's
+// (QueryLanes): the launches that prepare one instance's pairs (sort, items: a handful of
+// small kernels) overlap the arithmetic of others.
 #include <cuda_runtime.h>
 #include <stdint.h>
 #include <string.h>
@@ -124,6 +130,7 @@ struct Inst {
     int64_t apsp_off = 0, apsp_elems = 0, d_off = 0, N = 0, nbg = 0;
     int32_t max_ld = 0;
     bool elim = false;  // boundary graph by elimination + back-substitution
+    bool all_elim = false;  // every component table by elimination
     int64_t marks = 0;  // ... its R x R marks in the batch's
     BgLayout layout;    // aligned pieces of its order and their runs of rounds
     std::vector<int32_t> csize, nb, bgoff;
@@ -141,7 +148,7 @@ struct BatchPtrs {
     int32_t* bgpos = nullptr;
     uint32_t* err = nullptr;
     uint32_t* tables = nullptr;  // every APSP(C), then every boundary-graph matrix
-    int64_t table_elems = 0;
+    int64_t check_off = 0, check_elems = 0;  // the Floyd-Warshall boundary-graph tables
 };
 
 // The instances whose boundary graph takes the elimination form: their matrices' marks
@@ -210,19 +217,23 @@ struct StageKeep {
 };
 
 // Component tables of every instance in element type T (Algorithm 1 after the
-// reordering; independent of the boundary slots' order).  ev: stage events (may be null);
-// keep: record / replay (may be null).
+// reordering; independent of the boundary slots' order).  exact: as in a single build's (int32
+// tables and their check; may be null).  ev: stage events (may be null); keep: record / replay
+// (may be null).
 template <typename T>
 cudaError_t batch_comp_tables(std::vector<Inst>& I, const BatchPtrs& P, const MatDesc* d_cdescs,
                               const MatDesc* h_cdescs, int64_t ktot, int32_t max_ld, bool f32w, const CompElim& ce,
-                              double* comp_elim_updates, cudaEvent_t* ev, cudaStream_t st,
+                              double* comp_elim_updates, uint32_t* exact, cudaEvent_t* ev, cudaStream_t st,
                               StageKeep<T>* keep = nullptr) {
     T* base = reinterpret_cast<T*>(P.tables);
     cudaError_t e;
     if (ev) cudaEventRecord(ev[2], st);
-    if ((e = launch_fill_blocks<T>(base, d_cdescs, (int32_t)ktot, st)) != cudaSuccess) return e;
+    if (exact && (e = cudaMemsetAsync(exact, 0, sizeof(uint32_t), st)) != cudaSuccess) return e;
+    // (the elimination's permutation back writes every cell of its tables)
+    if ((e = launch_fill_blocks<T>(base, d_cdescs, (int32_t)ktot, st, ce.nsel > 0 ? P.csize : nullptr)) != cudaSuccess)
+        return e;
     for (auto& x : I) {
-        if (x.n == 0) continue;
+        if (x.n == 0 || x.all_elim) continue;
         e = launch_scatter_intra<T>(f32w, x.n, x.rp, x.col, x.w, x.part, P.local + x.vbase, P.descs + x.kbase,
                                     base + x.apsp_off, st);
         if (e != cudaSuccess) return e;
@@ -245,19 +256,26 @@ cudaError_t batch_comp_tables(std::vector<Inst>& I, const BatchPtrs& P, const Ma
             if (e != cudaSuccess) return e;
         }
         e = comp_elim_finish<T>(base, Pc, d_cdescs, ce.ed, ce.d_sel, ce.d_ed, P.csize, ce.vstart_global, ce.ndpos,
-                                comp_elim_updates, st, keep ? &keep->ce : nullptr);
+                                comp_elim_updates, exact, st, keep ? &keep->ce : nullptr);
         if (e != cudaSuccess) return e;
     }
     if (max_ld > 0 &&
         (e = fw_batched<T>(base, d_cdescs, h_cdescs, (int32_t)ktot, max_ld, st, keep ? &keep->fwb : nullptr)) !=
             cudaSuccess)
         return e;
+    if (exact && max_ld > 0) {
+        e = ce.nsel > 0 ? launch_check_convert_blocks(reinterpret_cast<float*>(base), d_cdescs, P.csize, (int32_t)ktot,
+                                                      max_ld, exact, st)
+                        : launch_check_convert(reinterpret_cast<float*>(base), P.check_off, exact, st);
+        if (e != cudaSuccess) return e;
+    }
     if (ev) cudaEventRecord(ev[3], st);
     return cudaSuccess;
 }
 
 // Boundary graphs of every instance in element type T (after batch_comp_tables<T>):
-// assembly, all-pairs distances, and (check) the exactness check of every float32 table.
+// assembly, all-pairs distances, and (check) the exactness check of every float32 table: the
+// elimination's back-substitution stores int32 itself, the Floyd-Warshall ones are converted.
 // ev: stage events (may be null).  keep: record / replay (may be null); a replay leaves
 // the check's flag in d_flag and the status in be.err for the caller to read.
 template <typename T>
@@ -280,7 +298,7 @@ cudaError_t batch_bg_tables(std::vector<Inst>& I, const BatchPtrs& P, const MatD
         if ((e = x.elim ? launch_fill_marked<T>(D, x.N, be.marks + x.marks, st) : launch_bg_fill<T>(D, x.N, st)) !=
             cudaSuccess)
             return e;
-        e = launch_bg_clique<T>(base + x.apsp_off, P.descs + x.kbase, P.nb + x.kbase, P.bgoff + x.kbase,
+        e = launch_bg_clique<T>(base + x.apsp_off, check, P.descs + x.kbase, P.nb + x.kbase, P.bgoff + x.kbase,
                                 P.bgpos + x.slotbase, x.k, D, x.N, st);
         if (e != cudaSuccess) return e;
         e = launch_bg_inter<T>(f32w, x.n, x.rp, x.col, x.w, x.part, P.local + x.vbase, P.bgoff + x.kbase,
@@ -335,7 +353,7 @@ cudaError_t batch_bg_tables(std::vector<Inst>& I, const BatchPtrs& P, const MatD
             }
         e = elim_forward<T>(mats, true, &fwd, nullptr, st, keep ? &keep->fwd : nullptr);
         if (e == cudaSuccess) {
-            e = bg_backsub_many<T>(bin, be.err, nullptr, be.panel_cap, &bs, nullptr, st, keep ? &keep->bg : nullptr);
+            e = bg_backsub_many<T>(bin, be.err, check ? d_flag : nullptr, be.panel_cap, &bs, nullptr, st, keep ? &keep->bg : nullptr);
         }
         el_upd = fwd + bs;
     }
@@ -358,8 +376,8 @@ cudaError_t batch_bg_tables(std::vector<Inst>& I, const BatchPtrs& P, const MatD
     }
     if (ev) cudaEventRecord(ev[5], st);
     if (check) {
-        if ((e = cudaMemsetAsync(d_flag, 0, sizeof(uint32_t), st)) != cudaSuccess) return e;
-        if ((e = launch_check_convert(reinterpret_cast<float*>(P.tables), P.table_elems, d_flag, st)) != cudaSuccess)
+        if ((e = launch_check_convert(reinterpret_cast<float*>(P.tables) + P.check_off, P.check_elems, d_flag, st)) !=
+            cudaSuccess)
             return e;
         if (!replay) {
             uint32_t f = 0;
@@ -785,6 +803,7 @@ spq_status build_many_impl(int32_t G, const spq_graph* gs, const spq_opts& o, cu
                 vsg[x.kbase + c] = (int32_t)x.vbase + acc;
                 acc += x.csize[c];
                 const MatDesc g{x.apsp_off + d.off, d.n, 0};
+                x.all_elim = (c == 0 || x.all_elim) && comp_elim && comp_takes_elim(x.csize[c], d.n);
                 if (comp_elim && comp_takes_elim(x.csize[c], d.n)) {
                     sel.push_back((int32_t)(x.kbase + c));
                     ce.ed.push_back(g);
@@ -829,6 +848,7 @@ spq_status build_many_impl(int32_t G, const spq_graph* gs, const spq_opts& o, cu
     BCK(tmp.alloc(&d_cd, cd.size()));
     BCK(tmp.alloc(&d_flag, 1));
     BCK(cudaMemcpyAsync(d_cd, cd.data(), cd.size() * sizeof(MatDesc), cudaMemcpyHostToDevice, st));
+    P.check_off = apsp_tot;
     double bg_updates = 0.0, comp_elim_updates = 0.0;
     bool f32store = false;
     int32_t arith = SPQ_ARITH_I32;
@@ -838,11 +858,11 @@ spq_status build_many_impl(int32_t G, const spq_graph* gs, const spq_opts& o, cu
     StageKeep<float>* kf = keep ? &keep->kf : nullptr;
     StageKeep<int32_t>* ki = keep ? &keep->ki : nullptr;
     if (first_f32)
-        BCK(batch_comp_tables<float>(I, P, d_cd, cd_fw.data(), ktot, max_ld_fw, f32w, ce, &comp_elim_updates, ev, st,
-                                     kf));
+        BCK(batch_comp_tables<float>(I, P, d_cd, cd_fw.data(), ktot, max_ld_fw, f32w, ce, &comp_elim_updates,
+                                     f32w ? nullptr : d_flag, ev, st, kf));
     else
-        BCK(batch_comp_tables<int32_t>(I, P, d_cd, cd_fw.data(), ktot, max_ld_fw, f32w, ce, &comp_elim_updates, ev,
-                                       st, ki));
+        BCK(batch_comp_tables<int32_t>(I, P, d_cd, cd_fw.data(), ktot, max_ld_fw, f32w, ce, &comp_elim_updates,
+                                       nullptr, ev, st, ki));
 
     // ---- the slots' order, and the form of each boundary graph: elimination +
     // back-substitution when asked for, or by default from kBatchElimMin slots on in a
@@ -866,9 +886,9 @@ spq_status build_many_impl(int32_t G, const spq_graph* gs, const spq_opts& o, cu
     for (int32_t g = 0; g < G; ++g) {
         Inst& x = I[g];
         if (x.layout.npad > 0) x.N = round_up(x.layout.npad, 4);
-        x.d_off = at;
-        at += x.N * x.N;
         if (x.N > 0 && !x.elim) {
+            x.d_off = at;  // (side by side, for the check; the elimination's follow)
+            at += x.N * x.N;
             bd.push_back(MatDesc{x.d_off, (int32_t)x.N, 0});
             max_N_fw = std::max(max_N_fw, (int32_t)x.N);
         }
@@ -883,7 +903,12 @@ spq_status build_many_impl(int32_t G, const spq_graph* gs, const spq_opts& o, cu
         }
         shared_at[g + 1] = shared.size();
     }
-    P.table_elems = at;
+    P.check_elems = at - apsp_tot;
+    for (Inst& x : I)
+        if (x.elim || x.N == 0) {
+            x.d_off = at;
+            at += x.N * x.N;
+        }
     if (be.n > 0) {
         int32_t* d_shared = nullptr;
         BCK(tmp.alloc(&be.marks0, (size_t)be.mark_words));
@@ -922,7 +947,7 @@ spq_status build_many_impl(int32_t G, const spq_graph* gs, const spq_opts& o, cu
             arith = SPQ_ARITH_I32;
             if (inexact)
                 BCK(batch_comp_tables<int32_t>(I, P, d_cd, cd_fw.data(), ktot, max_ld_fw, false, ce,
-                                               &comp_elim_updates, ev, st, ki));
+                                               &comp_elim_updates, nullptr, ev, st, ki));
             BCK(batch_bg_tables<int32_t>(I, P, d_bd, (int32_t)bd.size(), max_N_fw, false, fw_scratch, d_flag, false,
                                          &inexact, &bg_updates, be, ev, st, ki));
         }
@@ -1284,8 +1309,8 @@ cudaError_t plan_stage(BuildKeep& K, StageKeep<T>* sk, bool check, bool* inexact
     double cu = 0.0, bu = 0.0;
     *inexact = false;
     if (e == cudaSuccess)
-        e = batch_comp_tables<T>(K.I, K.P, K.d_cd, K.cd_fw.data(), K.ktot, K.max_ld_fw, K.f32w, K.ce, &cu, nullptr,
-                                 st, sk);
+        e = batch_comp_tables<T>(K.I, K.P, K.d_cd, K.cd_fw.data(), K.ktot, K.max_ld_fw, K.f32w, K.ce, &cu,
+                                 check ? K.d_flag : nullptr, nullptr, st, sk);
     if (e == cudaSuccess)
         e = batch_bg_tables<T>(K.I, K.P, K.d_bd, K.nbmat, K.max_N_fw, K.f32w, K.fw_scratch, K.d_flag, check, inexact,
                                &bu, K.be, nullptr, st, sk);

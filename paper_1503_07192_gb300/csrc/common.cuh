@@ -128,7 +128,8 @@ cudaError_t launch_assign_local(int32_t n, const uint32_t* sorted_vals, const in
 
 // ---- assemble.cu: table initialisation and boundary-graph assembly ----
 template <typename T>
-cudaError_t launch_fill_blocks(T* apsp, const MatDesc* descs, int32_t nmat, cudaStream_t st);
+cudaError_t launch_fill_blocks(T* apsp, const MatDesc* descs, int32_t nmat, cudaStream_t st,
+                               const int32_t* csize = nullptr);  // (csize: not those taking the elimination form)
 template <typename T>
 cudaError_t launch_scatter_intra(bool f32w, int32_t n, const int64_t* rp, const int32_t* col, const void* w,
                                  const int32_t* part, const int32_t* local, const MatDesc* descs, T* apsp,
@@ -142,7 +143,7 @@ cudaError_t launch_scatter_intra_sel(bool f32w, int32_t n, const int64_t* rp, co
 template <typename T>
 cudaError_t launch_bg_fill(T* D, int64_t N, cudaStream_t st);
 template <typename T>
-cudaError_t launch_bg_clique(const T* apsp, const MatDesc* descs, const int32_t* nb, const int32_t* bg_off,
+cudaError_t launch_bg_clique(const void* apsp, bool i32, const MatDesc* descs, const int32_t* nb, const int32_t* bg_off,
                              const int32_t* bgpos, int32_t k, T* D, int64_t N, cudaStream_t st);
 template <typename T>
 cudaError_t launch_bg_inter(bool f32w, int32_t n, const int64_t* rp, const int32_t* col, const void* w,
@@ -151,6 +152,9 @@ cudaError_t launch_bg_inter(bool f32w, int32_t n, const int64_t* rp, const int32
 // In place: float32 table -> int32 (+inf -> SPQ_INF_I32), flagging kErrExact if a
 // finite entry is >= 2^24 (then the converted values are not used).
 cudaError_t launch_check_convert(float* a, int64_t count, uint32_t* err, cudaStream_t st);
+// The same for the components (of at most max_n rows) that comp_takes_elim does not select.
+cudaError_t launch_check_convert_blocks(float* base, const MatDesc* descs, const int32_t* csize, int32_t nmat,
+                                        int32_t max_n, uint32_t* err, cudaStream_t st);
 
 // ---- fw.cu: blocked Floyd-Warshall (Venkataraman, Sahni & Mukhopadhyaya 2003) ----
 // Many matrices (descs on the device and on the host); each round touches only the
@@ -296,12 +300,14 @@ constexpr int32_t kNdMax = 4096;  // largest component ordered (one CTA each)
 // apsp (local order), after launch_fill_blocks / launch_scatter_intra of the same tables
 // (their contents there are replaced).  The other components are left to the caller.
 // Waits on the host for the back-substitution's bookkeeping and status.
+// exact != NULL (float tables of an int32 graph): their tables are left in int32, kErrExact set
+// in *exact if one holds a finite entry >= 2^24.
 template <typename T>
 cudaError_t comp_tables_elim(T* apsp, const MatDesc* d_descs, const std::vector<MatDesc>& h_descs,
                              const std::vector<int32_t>& h_csize, int32_t k, int32_t n, const int64_t* rp,
                              const int32_t* col, const void* w, bool f32w, const int32_t* part, const int32_t* local,
                              const int32_t* vorder, const int32_t* d_vstart, const int32_t* d_csize, double* updates,
-                             cudaStream_t st);
+                             uint32_t* exact, cudaStream_t st);
 // The parts of comp_tables_elim for several graphs sharing one elimination: the
 // dissection order of every component of every graph (one launch; ndpos at vstart[c] + v
 // in the batch-wide numbering); per graph, each vertex's position and the scatter of its
@@ -345,10 +351,10 @@ struct CompElimPlan {
 template <typename T>
 cudaError_t comp_elim_finish(T* apsp, T* P, const MatDesc* d_descs, const std::vector<MatDesc>& ed,
                              const int32_t* d_sel, const MatDesc* d_ed, const int32_t* d_csize,
-                             const int32_t* d_vstart, const int32_t* ndpos, double* updates, cudaStream_t st,
-                             CompElimPlan<T>* keep = nullptr);
+                             const int32_t* d_vstart, const int32_t* ndpos, double* updates, uint32_t* exact,
+                             cudaStream_t st, CompElimPlan<T>* keep = nullptr);
 // Whether component c takes the elimination form in comp_tables_elim.
-inline bool comp_takes_elim(int32_t csize, int32_t ld) { return csize <= kNdMax && ld > kTile; }
+__host__ __device__ inline bool comp_takes_elim(int32_t csize, int32_t ld) { return csize <= kNdMax && ld > kTile; }
 
 // ---- query.cu ----
 template <typename T>

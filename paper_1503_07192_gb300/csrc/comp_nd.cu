@@ -339,8 +339,8 @@ cudaError_t comp_nd_scatter(T* P, const MatDesc* d_descs, int32_t n, const int64
 template <typename T>
 cudaError_t comp_elim_finish(T* apsp, T* P, const MatDesc* d_descs, const std::vector<MatDesc>& ed,
                              const int32_t* d_sel, const MatDesc* d_ed, const int32_t* d_csize,
-                             const int32_t* d_vstart, const int32_t* ndpos, double* updates, cudaStream_t st,
-                             CompElimPlan<T>* keep) {
+                             const int32_t* d_vstart, const int32_t* ndpos, double* updates, uint32_t* exact,
+                             cudaStream_t st, CompElimPlan<T>* keep) {
     if (updates) *updates = 0.0;
     if (ed.empty()) {
         if (keep) keep->ready = true;
@@ -377,10 +377,10 @@ cudaError_t comp_elim_finish(T* apsp, T* P, const MatDesc* d_descs, const std::v
         return done(e);
     std::vector<BsInput<T>> bin;
     for (const MatDesc& d : ed) bin.push_back(BsInput<T>{P + d.off, (int64_t)d.n, nullptr});
-    if ((e = bg_backsub_many<T>(bin, err, nullptr, (size_t)2 << 30, &bs, nullptr, st, keep ? &keep->bs : nullptr)) !=
+    if ((e = bg_backsub_many<T>(bin, err, exact, (size_t)2 << 30, &bs, nullptr, st, keep ? &keep->bs : nullptr)) !=
         cudaSuccess)
         return done(e);
-    // back to the local order
+    // back to the local order (cells moved as they are: int32 already with exact)
     const dim3 g((unsigned)std::min(max_el, 64), (unsigned)std::min<size_t>(ed.size(), 65535));
     k_unpermute<T><<<g, 256, 0, st>>>(apsp, P, d_descs, d_sel, (int32_t)ed.size(), d_csize, d_vstart, ndpos);
     count_launches(1);
@@ -404,7 +404,7 @@ cudaError_t comp_tables_elim(T* apsp, const MatDesc* d_descs, const std::vector<
                              const std::vector<int32_t>& h_csize, int32_t k, int32_t n, const int64_t* rp,
                              const int32_t* col, const void* w, bool f32w, const int32_t* part, const int32_t* local,
                              const int32_t* vorder, const int32_t* d_vstart, const int32_t* d_csize, double* updates,
-                             cudaStream_t st) {
+                             uint32_t* exact, cudaStream_t st) {
     if (updates) *updates = 0.0;
     // the components of at most kNdMax vertices (with more than one tile row) take the
     // elimination form; the others Floyd-Warshall (after this call, by the caller)
@@ -447,26 +447,29 @@ cudaError_t comp_tables_elim(T* apsp, const MatDesc* d_descs, const std::vector<
         return done(e);
     e = comp_nd_scatter<T>(P, d_descs, n, rp, col, w, f32w, part, local, d_vstart, d_csize, ndpos, vpos, st);
     if (e != cudaSuccess) return done(e);
-    return done(comp_elim_finish<T>(apsp, P, d_descs, ed, d_sel, d_ed, d_csize, d_vstart, ndpos, updates, st));
+    return done(comp_elim_finish<T>(apsp, P, d_descs, ed, d_sel, d_ed, d_csize, d_vstart, ndpos, updates,
+                                    exact, st));
 }
 
 template cudaError_t comp_tables_elim<float>(float*, const MatDesc*, const std::vector<MatDesc>&,
                                              const std::vector<int32_t>&, int32_t, int32_t, const int64_t*,
                                              const int32_t*, const void*, bool, const int32_t*, const int32_t*,
-                                             const int32_t*, const int32_t*, const int32_t*, double*, cudaStream_t);
+                                             const int32_t*, const int32_t*, const int32_t*, double*, uint32_t*,
+                                             cudaStream_t);
 #define SPQ_COMP_ND_INST(T)                                                                                      \
     template cudaError_t comp_nd_scatter<T>(T*, const MatDesc*, int32_t, const int64_t*, const int32_t*, const void*, \
                                             bool, const int32_t*, const int32_t*, const int32_t*, const int32_t*,      \
                                             const int32_t*, int32_t*, cudaStream_t);                                    \
     template cudaError_t comp_elim_finish<T>(T*, T*, const MatDesc*, const std::vector<MatDesc>&, const int32_t*,      \
                                              const MatDesc*, const int32_t*, const int32_t*, const int32_t*, double*,  \
-                                             cudaStream_t, CompElimPlan<T>*);
+                                             uint32_t*, cudaStream_t, CompElimPlan<T>*);
 SPQ_COMP_ND_INST(float)
 SPQ_COMP_ND_INST(int32_t)
 
 template cudaError_t comp_tables_elim<int32_t>(int32_t*, const MatDesc*, const std::vector<MatDesc>&,
                                                const std::vector<int32_t>&, int32_t, int32_t, const int64_t*,
                                                const int32_t*, const void*, bool, const int32_t*, const int32_t*,
-                                               const int32_t*, const int32_t*, const int32_t*, double*, cudaStream_t);
+                                               const int32_t*, const int32_t*, const int32_t*, double*, uint32_t*,
+                                               cudaStream_t);
 
 }  // namespace spq

@@ -2,7 +2,7 @@
 // back-substitution (the boundary-graph APSP of Algorithm 1, computed exactly, with fewer
 // min-plus updates than Floyd-Warshall in a nested-dissection order).
 //
-// Forward (fw_single with rowflags): block elimination in the matrix order.  After it,
+// Forward (elim_forward, fw.cu): block elimination in the matrix order.  After it,
 // for row block R and any column j right of R, F(r, j) (r in R) is the length of a
 // shortest r-j path whose inner vertices all lie in blocks <= R, and the diagonal tile
 // (R, R) holds the shortest paths inside blocks <= R.
@@ -772,10 +772,10 @@ cudaError_t launch_mark_pairs(const int32_t* blocks, int32_t nb, int64_t N, uint
 size_t bg_backsub_scratch_bytes(int64_t N) {
     const int64_t nR = (N + T_ - 1) / T_;
     // masks (16 B), fblk and tile flags (4 B each) per tile pair; per row block: fcnt,
-    // kcnt, koff, level and a run of the enumeration; the work counter and the matrix record
-    // (the work order's 8 bytes an item, under 48 MB for the largest matrix that fits the
-    // device, come out of the build's 64 MiB reserve)
-    return (size_t)(nR * nR) * 24 + (size_t)nR * 36 + 256;
+    // kcnt, koff and a run of the enumeration; the work counter and the matrix record
+    // (a row block's level, 4 bytes, and the work order, 8 bytes an item, under 48 MB for the
+    // largest matrix that fits the device, come out of the build's 64 MiB reserve)
+    return (size_t)(nR * nR) * 24 + (size_t)nR * 32 + 256;
 }
 
 // The launches of a back-substitution after its bookkeeping (klist, A panels, work
