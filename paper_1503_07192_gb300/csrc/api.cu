@@ -290,10 +290,11 @@ struct BgPlan {
 // exact != NULL (float32 tables of an int32 graph): the finished tables are stored as int32,
 // *exact getting kErrExact if one holds a finite entry >= 2^24.  The elimination's
 // back-substitution stores them so itself, as the boundary graph's does, which saves the pass
-// over them that the others need (9 GB read and written on 2^20 vertices: 1.3 ms).
+// over them that the others need (9 GB read and written on 2^20 vertices: 1.3 ms).  *inexact
+// (host) is set if one of its tables is already found so; exact[1] is used as well.
 template <typename T>
 cudaError_t build_comp_tables(spq_handle* h, const BuildInputs& in, int32_t max_n, bool elim, uint32_t* exact,
-                              StageEvents& evs, cudaStream_t st) {
+                              bool* inexact, StageEvents& evs, cudaStream_t st) {
     evs.mark(2, st);
     T* apsp = (T*)h->apsp;
     cudaError_t e;
@@ -313,7 +314,7 @@ cudaError_t build_comp_tables(spq_handle* h, const BuildInputs& in, int32_t max_
     double eu = 0.0;
     if (elim) {
         e = comp_tables_elim<T>(apsp, h->descs, h->h_descs, h->h_csize, h->k, in.n, in.rp, in.col, in.w, in.f32w,
-                                in.part, h->local, h->vorder, h->vstart, h->csize, &eu, exact, st);
+                                in.part, h->local, h->vorder, h->vstart, h->csize, &eu, exact, inexact, st);
         if (e != cudaSuccess) return e;
         for (int32_t c = 0; c < h->k; ++c)
             if (comp_takes_elim(h->h_csize[c], fwd[c].n)) fwd[c].n = 0;
@@ -339,11 +340,12 @@ cudaError_t build_comp_tables(spq_handle* h, const BuildInputs& in, int32_t max_
 
 // The boundary graph's table in element type T (after build_comp_tables<T>): assembly,
 // all-pairs distances, and (check_exact) the exactness check of the float32 table, the component
-// tables being int32 already.
+// tables being int32 already.  d_flag[0] is its flag, d_flag[1] the component tables' (where
+// that is set the table is computed no further than the back-substitution: it is made again).
 template <typename T>
 cudaError_t build_bg_tables(spq_handle* h, const BuildInputs& in, bool check_exact, bool skip_inf, bool profile,
-                            uint32_t* d_flag, uint32_t* fw_scratch, BgPlan& plan, bool* inexact, StageEvents& evs,
-                            cudaStream_t st) {
+                            uint32_t* d_flag, uint32_t* fw_scratch, BgPlan& plan, bool* inexact, bool* comp_inexact,
+                            StageEvents& evs, cudaStream_t st) {
     *inexact = false;
     T* D = (T*)h->D;
     cudaError_t e;
@@ -383,6 +385,7 @@ cudaError_t build_bg_tables(spq_handle* h, const BuildInputs& in, bool check_exa
             return e;
     }
     evs.mark(4, st);
+    if (check_exact && (e = cudaMemcpyAsync(d_flag, d_flag + 1, 4, cudaMemcpyDeviceToDevice, st)) != cudaSuccess) return e;
     // the elimination stores the float32 boundary-graph table as int32 itself (checked)
     const bool d_converted = plan.elim && check_exact && h->N > 0;
     if (h->N > 0 && !plan.elim) {
@@ -411,10 +414,11 @@ cudaError_t build_bg_tables(spq_handle* h, const BuildInputs& in, bool check_exa
         // a float32 table becomes an int32 one (every entry below 2^24 is an exact integer)
         if (h->N > 0 && !d_converted && (e = launch_check_convert((float*)h->D, h->N * h->N, d_flag, st)) != cudaSuccess)
             return e;
-        uint32_t f = 0;
-        if ((e = cudaMemcpyAsync(&f, d_flag, sizeof(f), cudaMemcpyDeviceToHost, st)) != cudaSuccess) return e;
+        uint32_t f[2] = {0, 0};
+        if ((e = cudaMemcpyAsync(f, d_flag, sizeof(f), cudaMemcpyDeviceToHost, st)) != cudaSuccess) return e;
         if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return e;
-        *inexact = (f & kErrExact) != 0;
+        *inexact = (f[0] & kErrExact) != 0;
+        *comp_inexact = (f[1] & kErrExact) != 0;
     }
     evs.mark(6, st);
     return cudaSuccess;
@@ -476,7 +480,7 @@ spq_status build_impl(int32_t n, const int64_t* row_ptr, const int32_t* col, con
     uint32_t* d_flag;
     CK(tmp.alloc(&d_bflag, (size_t)n));
     CK(tmp.alloc(&d_cnt, 2 * (size_t)k));
-    CK(tmp.alloc(&d_flag, 1));
+    CK(tmp.alloc(&d_flag, 3));  // boundary graph, components, status of the components' elimination
     CK(cudaMemsetAsync(d_cnt, 0, 2 * (size_t)k * sizeof(int32_t), st));
     CK(cudaMemsetAsync(d_flag, 0, sizeof(uint32_t), st));
     CK(launch_validate(f32w, n, m, d_rp, d_col, d_w, d_part, k, d_bflag, d_cnt, d_cnt + k, d_flag, st));
@@ -625,10 +629,11 @@ spq_status build_impl(int32_t n, const int64_t* row_ptr, const int32_t* col, con
             if (t.joinable()) t.join();
         }
     } join_order{order_thread};
+    bool comp_inexact = false;
     if (first_f32)
-        CK(build_comp_tables<float>(h, in, max_n, comp_elim, f32w ? nullptr : d_flag, evs, st));
+        CK(build_comp_tables<float>(h, in, max_n, comp_elim, f32w ? nullptr : d_flag + 1, &comp_inexact, evs, st));
     else
-        CK(build_comp_tables<int32_t>(h, in, max_n, comp_elim, nullptr, evs, st));
+        CK(build_comp_tables<int32_t>(h, in, max_n, comp_elim, nullptr, nullptr, evs, st));
     if (order_thread.joinable()) order_thread.join();
     if (h->nbg > 0) {
         if (order_status != SPQ_OK) return order_status;
@@ -657,21 +662,24 @@ spq_status build_impl(int32_t n, const int64_t* row_ptr, const int32_t* col, con
         h->f32store = true;
         h->arith = SPQ_ARITH_F32;
         bool inexact = false;
-        CK(build_bg_tables<float>(h, in, false, skip, prof, d_flag, fw_scratch, plan, &inexact, evs, st));
+        CK(build_bg_tables<float>(h, in, false, skip, prof, d_flag, fw_scratch, plan, &inexact, &comp_inexact, evs, st));
         if (plan.wait_failed) return SPQ_ETIMEOUT;
     } else {
-        bool inexact = false;
-        if (first_f32) {
+        // (where a component is found inexact the float32 boundary graph is not tried; an int32
+        //  rebuild keeps component tables that passed the check: they are int32 already)
+        bool inexact = comp_inexact;
+        if (first_f32 && !inexact) {
             h->f32store = true;
             h->arith = SPQ_ARITH_F32;
-            CK(build_bg_tables<float>(h, in, true, skip, prof, d_flag, fw_scratch, plan, &inexact, evs, st));
+            CK(build_bg_tables<float>(h, in, true, skip, prof, d_flag, fw_scratch, plan, &inexact, &comp_inexact, evs,
+                                      st));
             if (plan.wait_failed) return SPQ_ETIMEOUT;
         }
         h->f32store = false;  // converted to int32 by the exactness check
         if (!first_f32 || inexact) {
             h->arith = SPQ_ARITH_I32;
-            if (inexact) CK(build_comp_tables<int32_t>(h, in, max_n, comp_elim, nullptr, evs, st));
-            CK(build_bg_tables<int32_t>(h, in, false, skip, prof, d_flag, fw_scratch, plan, &inexact, evs, st));
+            if (comp_inexact) CK(build_comp_tables<int32_t>(h, in, max_n, comp_elim, nullptr, nullptr, evs, st));
+            CK(build_bg_tables<int32_t>(h, in, false, skip, prof, d_flag, fw_scratch, plan, &inexact, nullptr, evs, st));
             if (plan.wait_failed) return SPQ_ETIMEOUT;
         }
     }

@@ -224,7 +224,7 @@ template <typename T>
 cudaError_t batch_comp_tables(std::vector<Inst>& I, const BatchPtrs& P, const MatDesc* d_cdescs,
                               const MatDesc* h_cdescs, int64_t ktot, int32_t max_ld, bool f32w, const CompElim& ce,
                               double* comp_elim_updates, uint32_t* exact, cudaEvent_t* ev, cudaStream_t st,
-                              StageKeep<T>* keep = nullptr) {
+                              StageKeep<T>* keep = nullptr, bool* inexact = nullptr) {
     T* base = reinterpret_cast<T*>(P.tables);
     cudaError_t e;
     if (ev) cudaEventRecord(ev[2], st);
@@ -256,7 +256,7 @@ cudaError_t batch_comp_tables(std::vector<Inst>& I, const BatchPtrs& P, const Ma
             if (e != cudaSuccess) return e;
         }
         e = comp_elim_finish<T>(base, Pc, d_cdescs, ce.ed, ce.d_sel, ce.d_ed, P.csize, ce.vstart_global, ce.ndpos,
-                                comp_elim_updates, exact, st, keep ? &keep->ce : nullptr);
+                                comp_elim_updates, exact, st, keep ? &keep->ce : nullptr, inexact);
         if (e != cudaSuccess) return e;
     }
     if (max_ld > 0 &&
@@ -276,13 +276,14 @@ cudaError_t batch_comp_tables(std::vector<Inst>& I, const BatchPtrs& P, const Ma
 // Boundary graphs of every instance in element type T (after batch_comp_tables<T>):
 // assembly, all-pairs distances, and (check) the exactness check of every float32 table: the
 // elimination's back-substitution stores int32 itself, the Floyd-Warshall ones are converted.
-// ev: stage events (may be null).  keep: record / replay (may be null); a replay leaves
-// the check's flag in d_flag and the status in be.err for the caller to read.
+// d_flag[0] is its flag, d_flag[1] the component tables'; ev: stage events (may be null).
+// keep: record / replay (may be null); a replay leaves the check's flag in d_flag and the
+// status in be.err for the caller to read.
 template <typename T>
 cudaError_t batch_bg_tables(std::vector<Inst>& I, const BatchPtrs& P, const MatDesc* d_bdescs, int32_t nbmat,
                             int32_t max_N, bool f32w, uint32_t* fw_scratch, uint32_t* d_flag, bool check,
                             bool* inexact, double* bg_updates, const BatchElim& be, cudaEvent_t* ev, cudaStream_t st,
-                            StageKeep<T>* keep = nullptr) {
+                            StageKeep<T>* keep = nullptr, bool* comp_inexact = nullptr) {
     *inexact = false;
     const bool replay = keep && keep->ready;
     T* base = reinterpret_cast<T*>(P.tables);
@@ -306,6 +307,7 @@ cudaError_t batch_bg_tables(std::vector<Inst>& I, const BatchPtrs& P, const MatD
         if (e != cudaSuccess) return e;
     }
     if (ev) cudaEventRecord(ev[4], st);
+    if (check && (e = cudaMemcpyAsync(d_flag, d_flag + 1, 4, cudaMemcpyDeviceToDevice, st)) != cudaSuccess) return e;
     // The Floyd-Warshall instances' rounds on a second stream, the elimination instances'
     // forward rounds and back-substitution here: both sets of launches side by side.  A
     // build waits on the host for the first set on a helper thread; a replay forks and
@@ -353,7 +355,8 @@ cudaError_t batch_bg_tables(std::vector<Inst>& I, const BatchPtrs& P, const MatD
             }
         e = elim_forward<T>(mats, true, &fwd, nullptr, st, keep ? &keep->fwd : nullptr);
         if (e == cudaSuccess) {
-            e = bg_backsub_many<T>(bin, be.err, check ? d_flag : nullptr, be.panel_cap, &bs, nullptr, st, keep ? &keep->bg : nullptr);
+            e = bg_backsub_many<T>(bin, be.err, check ? d_flag : nullptr, be.panel_cap, &bs, nullptr, st,
+                                   keep ? &keep->bg : nullptr, true);
         }
         el_upd = fwd + bs;
     }
@@ -380,10 +383,11 @@ cudaError_t batch_bg_tables(std::vector<Inst>& I, const BatchPtrs& P, const MatD
             cudaSuccess)
             return e;
         if (!replay) {
-            uint32_t f = 0;
-            if ((e = cudaMemcpyAsync(&f, d_flag, sizeof(f), cudaMemcpyDeviceToHost, st)) != cudaSuccess) return e;
+            uint32_t f[2] = {0, 0};
+            if ((e = cudaMemcpyAsync(f, d_flag, sizeof(f), cudaMemcpyDeviceToHost, st)) != cudaSuccess) return e;
             if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return e;
-            *inexact = (f & kErrExact) != 0;
+            *inexact = (f[0] & kErrExact) != 0;
+            if (comp_inexact) *comp_inexact = (f[1] & kErrExact) != 0;
         }
     }
     if (ev) cudaEventRecord(ev[6], st);
@@ -846,20 +850,20 @@ spq_status build_many_impl(int32_t G, const spq_graph* gs, const spq_opts& o, cu
     MatDesc *d_cd, *d_bd;
     uint32_t *fw_scratch, *d_flag;
     BCK(tmp.alloc(&d_cd, cd.size()));
-    BCK(tmp.alloc(&d_flag, 1));
+    BCK(tmp.alloc(&d_flag, 3));  // boundary graphs, components, status of their elimination
     BCK(cudaMemcpyAsync(d_cd, cd.data(), cd.size() * sizeof(MatDesc), cudaMemcpyHostToDevice, st));
     P.check_off = apsp_tot;
     double bg_updates = 0.0, comp_elim_updates = 0.0;
     bool f32store = false;
     int32_t arith = SPQ_ARITH_I32;
-    bool inexact = false;
+    bool inexact = false, comp_inexact = false;
     // float32 first (exact below 2^24, checked), int32 if asked or if the check fails
     const bool first_f32 = f32w || o.arith != SPQ_ARITH_I32;
     StageKeep<float>* kf = keep ? &keep->kf : nullptr;
     StageKeep<int32_t>* ki = keep ? &keep->ki : nullptr;
     if (first_f32)
         BCK(batch_comp_tables<float>(I, P, d_cd, cd_fw.data(), ktot, max_ld_fw, f32w, ce, &comp_elim_updates,
-                                     f32w ? nullptr : d_flag, ev, st, kf));
+                                     f32w ? nullptr : d_flag + 1, ev, st, kf, &comp_inexact));
     else
         BCK(batch_comp_tables<int32_t>(I, P, d_cd, cd_fw.data(), ktot, max_ld_fw, f32w, ce, &comp_elim_updates,
                                        nullptr, ev, st, ki));
@@ -938,14 +942,16 @@ spq_status build_many_impl(int32_t G, const spq_graph* gs, const spq_opts& o, cu
         BCK(batch_bg_tables<float>(I, P, d_bd, (int32_t)bd.size(), max_N_fw, true, fw_scratch, d_flag, false, &inexact,
                                    &bg_updates, be, ev, st, kf));
     } else {
-        if (first_f32) {
+        // (as in a single build: components found inexact, or int32 already)
+        inexact = comp_inexact;
+        if (first_f32 && !inexact) {
             arith = SPQ_ARITH_F32;
             BCK(batch_bg_tables<float>(I, P, d_bd, (int32_t)bd.size(), max_N_fw, false, fw_scratch, d_flag, true,
-                                       &inexact, &bg_updates, be, ev, st, kf));
+                                       &inexact, &bg_updates, be, ev, st, kf, &comp_inexact));
         }
         if (!first_f32 || inexact) {
             arith = SPQ_ARITH_I32;
-            if (inexact)
+            if (comp_inexact || (inexact && keep))  // (a plan records the int32 launches)
                 BCK(batch_comp_tables<int32_t>(I, P, d_cd, cd_fw.data(), ktot, max_ld_fw, false, ce,
                                                &comp_elim_updates, nullptr, ev, st, ki));
             BCK(batch_bg_tables<int32_t>(I, P, d_bd, (int32_t)bd.size(), max_N_fw, false, fw_scratch, d_flag, false,
@@ -1310,7 +1316,7 @@ cudaError_t plan_stage(BuildKeep& K, StageKeep<T>* sk, bool check, bool* inexact
     *inexact = false;
     if (e == cudaSuccess)
         e = batch_comp_tables<T>(K.I, K.P, K.d_cd, K.cd_fw.data(), K.ktot, K.max_ld_fw, K.f32w, K.ce, &cu,
-                                 check ? K.d_flag : nullptr, nullptr, st, sk);
+                                 check ? K.d_flag + 1 : nullptr, nullptr, st, sk);
     if (e == cudaSuccess)
         e = batch_bg_tables<T>(K.I, K.P, K.d_bd, K.nbmat, K.max_N_fw, K.f32w, K.fw_scratch, K.d_flag, check, inexact,
                                &bu, K.be, nullptr, st, sk);

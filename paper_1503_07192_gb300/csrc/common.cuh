@@ -272,7 +272,8 @@ struct BsPlan {
 };
 template <typename T>
 cudaError_t bg_backsub_many(const std::vector<BsInput<T>>& in, uint32_t* err, uint32_t* exact, size_t apanel_budget,
-                            double* updates, FwProfile* prof, cudaStream_t st, BsPlan<T>* keep = nullptr);
+                            double* updates, FwProfile* prof, cudaStream_t st, BsPlan<T>* keep = nullptr,
+                            bool bail = false);  // bail: stop, tables incomplete, once *exact is set
 // Marks of every pair of the nb given tiles (device list).
 cudaError_t launch_mark_pairs(const int32_t* blocks, int32_t nb, int64_t N, uint32_t* flags, cudaStream_t st);
 // Infinity (0 on the diagonal) in the marked tiles, their mirrors and the diagonal tiles.
@@ -301,13 +302,14 @@ constexpr int32_t kNdMax = 4096;  // largest component ordered (one CTA each)
 // (their contents there are replaced).  The other components are left to the caller.
 // Waits on the host for the back-substitution's bookkeeping and status.
 // exact != NULL (float tables of an int32 graph): their tables are left in int32, kErrExact set
-// in *exact if one holds a finite entry >= 2^24.
+// in *exact if one holds a finite entry >= 2^24, and *inexact (host) set then; exact[1] is used
+// as well.
 template <typename T>
 cudaError_t comp_tables_elim(T* apsp, const MatDesc* d_descs, const std::vector<MatDesc>& h_descs,
                              const std::vector<int32_t>& h_csize, int32_t k, int32_t n, const int64_t* rp,
                              const int32_t* col, const void* w, bool f32w, const int32_t* part, const int32_t* local,
                              const int32_t* vorder, const int32_t* d_vstart, const int32_t* d_csize, double* updates,
-                             uint32_t* exact, cudaStream_t st);
+                             uint32_t* exact, bool* inexact, cudaStream_t st);
 // The parts of comp_tables_elim for several graphs sharing one elimination: the
 // dissection order of every component of every graph (one launch; ndpos at vstart[c] + v
 // in the batch-wide numbering); per graph, each vertex's position and the scatter of its
@@ -352,7 +354,7 @@ template <typename T>
 cudaError_t comp_elim_finish(T* apsp, T* P, const MatDesc* d_descs, const std::vector<MatDesc>& ed,
                              const int32_t* d_sel, const MatDesc* d_ed, const int32_t* d_csize,
                              const int32_t* d_vstart, const int32_t* ndpos, double* updates, uint32_t* exact,
-                             cudaStream_t st, CompElimPlan<T>* keep = nullptr);
+                             cudaStream_t st, CompElimPlan<T>* keep = nullptr, bool* inexact = nullptr);
 // Whether component c takes the elimination form in comp_tables_elim.
 __host__ __device__ inline bool comp_takes_elim(int32_t csize, int32_t ld) { return csize <= kNdMax && ld > kTile; }
 

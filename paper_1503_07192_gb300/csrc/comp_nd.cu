@@ -340,8 +340,10 @@ template <typename T>
 cudaError_t comp_elim_finish(T* apsp, T* P, const MatDesc* d_descs, const std::vector<MatDesc>& ed,
                              const int32_t* d_sel, const MatDesc* d_ed, const int32_t* d_csize,
                              const int32_t* d_vstart, const int32_t* ndpos, double* updates, uint32_t* exact,
-                             cudaStream_t st, CompElimPlan<T>* keep) {
+                             cudaStream_t st, CompElimPlan<T>* keep, bool* inexact) {
     if (updates) *updates = 0.0;
+    if (inexact) *inexact = false;
+    const bool shared = exact != nullptr && keep == nullptr;  // the status word beside the flag: one read of both
     if (ed.empty()) {
         if (keep) keep->ready = true;
         return cudaSuccess;
@@ -349,11 +351,11 @@ cudaError_t comp_elim_finish(T* apsp, T* P, const MatDesc* d_descs, const std::v
     const bool replay = keep && keep->ready;
     int32_t max_el = 0;
     for (const MatDesc& d : ed) max_el = std::max(max_el, d.n);
-    uint32_t *scratch = replay ? keep->scratch : nullptr, *err = replay ? keep->err : nullptr;
+    uint32_t *scratch = replay ? keep->scratch : nullptr, *err = replay ? keep->err : shared ? exact + 1 : nullptr;
     cudaError_t e = cudaSuccess;
     if (!replay) {
         e = scratch_alloc((void**)&scratch, (size_t)fw_many_scratch_words((int32_t)ed.size(), max_el) * 4, st);
-        if (e == cudaSuccess) e = scratch_alloc((void**)&err, 4, st);
+        if (e == cudaSuccess && !shared) e = scratch_alloc((void**)&err, 4, st);
     }
     auto done = [&](cudaError_t r) {
         if (keep && !replay && r == cudaSuccess) {
@@ -366,7 +368,7 @@ cudaError_t comp_elim_finish(T* apsp, T* P, const MatDesc* d_descs, const std::v
         if (replay) return r;
         if (keep) keep->bs.release(st);
         if (scratch) cudaFreeAsync(scratch, st);
-        if (err) cudaFreeAsync(err, st);
+        if (err && !shared) cudaFreeAsync(err, st);
         return r;
     };
     if (e != cudaSuccess) return done(e);
@@ -390,10 +392,13 @@ cudaError_t comp_elim_finish(T* apsp, T* P, const MatDesc* d_descs, const std::v
         if (updates) *updates = keep->updates;
         return done(cudaSuccess);
     }
-    uint32_t f = 0;
-    if ((e = cudaMemcpyAsync(&f, err, 4, cudaMemcpyDeviceToHost, st)) != cudaSuccess) return done(e);
+    uint32_t f[2] = {0, 0};  // flag (with shared), status
+    if ((e = cudaMemcpyAsync(shared ? f : f + 1, shared ? exact : err, shared ? 8 : 4, cudaMemcpyDeviceToHost, st)) !=
+        cudaSuccess)
+        return done(e);
     if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return done(e);
-    if (f & kErrWait) return done(kWaitGaveUp);
+    if (f[1] & kErrWait) return done(kWaitGaveUp);
+    if (inexact) *inexact = (f[0] & kErrExact) != 0;
     if (updates) *updates = fwd + bs;
     if (keep) keep->updates = fwd + bs;
     return done(cudaSuccess);
@@ -404,8 +409,9 @@ cudaError_t comp_tables_elim(T* apsp, const MatDesc* d_descs, const std::vector<
                              const std::vector<int32_t>& h_csize, int32_t k, int32_t n, const int64_t* rp,
                              const int32_t* col, const void* w, bool f32w, const int32_t* part, const int32_t* local,
                              const int32_t* vorder, const int32_t* d_vstart, const int32_t* d_csize, double* updates,
-                             uint32_t* exact, cudaStream_t st) {
+                             uint32_t* exact, bool* inexact, cudaStream_t st) {
     if (updates) *updates = 0.0;
+    if (inexact) *inexact = false;
     // the components of at most kNdMax vertices (with more than one tile row) take the
     // elimination form; the others Floyd-Warshall (after this call, by the caller)
     std::vector<int32_t> sel;
@@ -448,21 +454,21 @@ cudaError_t comp_tables_elim(T* apsp, const MatDesc* d_descs, const std::vector<
     e = comp_nd_scatter<T>(P, d_descs, n, rp, col, w, f32w, part, local, d_vstart, d_csize, ndpos, vpos, st);
     if (e != cudaSuccess) return done(e);
     return done(comp_elim_finish<T>(apsp, P, d_descs, ed, d_sel, d_ed, d_csize, d_vstart, ndpos, updates,
-                                    exact, st));
+                                    exact, st, nullptr, inexact));
 }
 
 template cudaError_t comp_tables_elim<float>(float*, const MatDesc*, const std::vector<MatDesc>&,
                                              const std::vector<int32_t>&, int32_t, int32_t, const int64_t*,
                                              const int32_t*, const void*, bool, const int32_t*, const int32_t*,
                                              const int32_t*, const int32_t*, const int32_t*, double*, uint32_t*,
-                                             cudaStream_t);
+                                             bool*, cudaStream_t);
 #define SPQ_COMP_ND_INST(T)                                                                                      \
     template cudaError_t comp_nd_scatter<T>(T*, const MatDesc*, int32_t, const int64_t*, const int32_t*, const void*, \
                                             bool, const int32_t*, const int32_t*, const int32_t*, const int32_t*,      \
                                             const int32_t*, int32_t*, cudaStream_t);                                    \
     template cudaError_t comp_elim_finish<T>(T*, T*, const MatDesc*, const std::vector<MatDesc>&, const int32_t*,      \
                                              const MatDesc*, const int32_t*, const int32_t*, const int32_t*, double*,  \
-                                             uint32_t*, cudaStream_t, CompElimPlan<T>*);
+                                             uint32_t*, cudaStream_t, CompElimPlan<T>*, bool*);
 SPQ_COMP_ND_INST(float)
 SPQ_COMP_ND_INST(int32_t)
 
@@ -470,6 +476,6 @@ template cudaError_t comp_tables_elim<int32_t>(int32_t*, const MatDesc*, const s
                                                const std::vector<int32_t>&, int32_t, int32_t, const int64_t*,
                                                const int32_t*, const void*, bool, const int32_t*, const int32_t*,
                                                const int32_t*, const int32_t*, const int32_t*, double*, uint32_t*,
-                                               cudaStream_t);
+                                               bool*, cudaStream_t);
 
 }  // namespace spq

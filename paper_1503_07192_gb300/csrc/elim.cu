@@ -575,7 +575,10 @@ __device__ __forceinline__ void backsub_strip(T* __restrict__ M, int64_t N, int6
 // CONV (float tables of an int32 graph): every tile is stored as int32 (the final table
 // type) as soon as it is final, and the arithmetic runs on the integer encoding above
 // (tiles read as rows of d need no conversion); a finite value >= 2^24 sets kErrExact.
-// One launch may hold the tiles of several independent matrices, level by level.
+// With bail, the launch stops once that is set: the caller builds again in int32, so the other
+// tiles would be thrown away (the first tiles are the last row blocks', whose distances are
+// among the longest).  One launch may hold the tiles of several independent matrices, level by
+// level.
 template <typename T, bool CONV>
 __global__ void __launch_bounds__(NTH, SPQ_FW_MIN_CTAS)
     k_backsub(const BsMat<T>* __restrict__ mats, const BsItem* __restrict__ items,
@@ -584,7 +587,7 @@ __global__ void __launch_bounds__(NTH, SPQ_FW_MIN_CTAS)
               const T* __restrict__ A, int64_t aoff0, const int32_t* __restrict__ fblk,
               const int32_t* __restrict__ fcnt, uint32_t* __restrict__ tflags,
               unsigned long long* __restrict__ counter, uint32_t* __restrict__ err, uint32_t* __restrict__ exact,
-              unsigned long long wait_ns, int withhold) {
+              unsigned long long wait_ns, int withhold, int bail) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     PanelSmem<T>& sm = *reinterpret_cast<PanelSmem<T>*>(smem_raw);
     __shared__ int64_t s_item;
@@ -596,6 +599,8 @@ __global__ void __launch_bounds__(NTH, SPQ_FW_MIN_CTAS)
         if (tid == 0) {
             int64_t t = (int64_t)atomicAdd(counter, 1ull);
             if (*reinterpret_cast<volatile uint32_t*>(err) & kErrWait) t = nitems;
+            if constexpr (CONV)
+                if (bail && (*reinterpret_cast<volatile uint32_t*>(exact) & kErrExact)) t = nitems;
             s_item = t;
             s_fail = 0;
             if (t < nitems) s_it = items[t];
@@ -630,6 +635,11 @@ __global__ void __launch_bounds__(NTH, SPQ_FW_MIN_CTAS)
                                 s_fail = 1;
                                 break;
                             }
+                            if constexpr (CONV)
+                                if (bail && (*reinterpret_cast<volatile uint32_t*>(exact) & kErrExact)) {
+                                    s_fail = 1;
+                                    break;
+                                }
                             if (global_ns() - t0 > wait_ns) {
                                 atomicOr(err, kErrWait);
                                 s_fail = 1;
@@ -782,7 +792,7 @@ size_t bg_backsub_scratch_bytes(int64_t N) {
 // order): the k lists, then per launch its A panels and the persistent kernel.
 template <typename T>
 cudaError_t bs_enqueue(const BsPlan<T>& p, uint32_t* err, uint32_t* exact, std::vector<cudaEvent_t>* ev,
-                       cudaStream_t st) {
+                       bool bail, cudaStream_t st) {
     const bool conv = std::is_same<T, float>::value && exact != nullptr;
     auto kern = conv ? k_backsub<T, std::is_same<T, float>::value> : k_backsub<T, false>;
     const BsMat<T>* mats = static_cast<const BsMat<T>*>(p.mats);
@@ -834,7 +844,7 @@ cudaError_t bs_enqueue(const BsPlan<T>& p, uint32_t* err, uint32_t* exact, std::
         if (ev) cudaEventRecord((*ev)[2 * l], st);
         kern<<<grid, NTH, psm, st>>>(mats, items, nout, p.koff, p.kcnt, p.klist,
                                      p.A, L.aoff0, p.fblk, p.fcnt, p.tflags, p.counter, err, exact, g_wait_ns.load(),
-                                     g_withhold.load());
+                                     g_withhold.load(), bail ? 1 : 0);
         if (ev) cudaEventRecord((*ev)[2 * l + 1], st);
         count_launches(2);
         e = cudaGetLastError();
@@ -846,7 +856,7 @@ cudaError_t bs_enqueue(const BsPlan<T>& p, uint32_t* err, uint32_t* exact, std::
 // not): frontier marks afresh, checked against the recorded |K(R)|, then the same
 // launches; no host step, no allocation.
 template <typename T>
-cudaError_t bs_replay(const BsPlan<T>& p, uint32_t* err, uint32_t* exact, cudaStream_t st) {
+cudaError_t bs_replay(const BsPlan<T>& p, uint32_t* err, uint32_t* exact, bool bail, cudaStream_t st) {
     if (p.nmat == 0) return cudaSuccess;
     cudaError_t e = cudaMemsetAsync(p.tflags, 0, (size_t)p.P2 * 4, st);
     if (e != cudaSuccess) return e;
@@ -855,15 +865,15 @@ cudaError_t bs_replay(const BsPlan<T>& p, uint32_t* err, uint32_t* exact, cudaSt
                                                         err);
     count_launches(1);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    return bs_enqueue<T>(p, err, exact, nullptr, st);
+    return bs_enqueue<T>(p, err, exact, nullptr, bail, st);
 }
 
 template <typename T>
 cudaError_t bg_backsub_many(const std::vector<BsInput<T>>& in, uint32_t* err, uint32_t* exact, size_t apanel_budget,
-                            double* updates, FwProfile* prof, cudaStream_t st, BsPlan<T>* keep) {
+                            double* updates, FwProfile* prof, cudaStream_t st, BsPlan<T>* keep, bool bail) {
     if (keep && keep->ready) {
         if (updates) *updates = keep->updates;
-        return bs_replay<T>(*keep, err, exact, st);
+        return bs_replay<T>(*keep, err, exact, bail, st);
     }
     if (updates) *updates = 0.0;
     BsPlan<T> p;
@@ -1030,7 +1040,7 @@ cudaError_t bg_backsub_many(const std::vector<BsInput<T>>& in, uint32_t* err, ui
         for (auto& x : ev)
             if ((e = cudaEventCreate(&x)) != cudaSuccess) return done(e);
     }
-    e = bs_enqueue<T>(p, err, exact, prof ? &ev : nullptr, st);
+    e = bs_enqueue<T>(p, err, exact, prof ? &ev : nullptr, bail, st);
     if (prof && e == cudaSuccess && !ev.empty() && (e = cudaEventSynchronize(ev.back())) == cudaSuccess) {
         prof->bs_ms = 0.0;
         prof->bs_launches = 0;
@@ -1050,7 +1060,7 @@ template <typename T>
 cudaError_t bg_backsub(T* M, int64_t N, const uint32_t* rowflags, uint32_t* err, uint32_t* exact, size_t apanel_budget,
                        double* updates, FwProfile* prof, cudaStream_t st) {
     return bg_backsub_many<T>(std::vector<BsInput<T>>{BsInput<T>{M, N, rowflags}}, err, exact, apanel_budget, updates,
-                              prof, st, nullptr);
+                              prof, st, nullptr, true);
 }
 
 template cudaError_t bg_backsub<float>(float*, int64_t, const uint32_t*, uint32_t*, uint32_t*, size_t, double*,
@@ -1058,9 +1068,9 @@ template cudaError_t bg_backsub<float>(float*, int64_t, const uint32_t*, uint32_
 template cudaError_t bg_backsub<int32_t>(int32_t*, int64_t, const uint32_t*, uint32_t*, uint32_t*, size_t, double*,
                                          FwProfile*, cudaStream_t);
 template cudaError_t bg_backsub_many<float>(const std::vector<BsInput<float>>&, uint32_t*, uint32_t*, size_t, double*,
-                                            FwProfile*, cudaStream_t, BsPlan<float>*);
+                                            FwProfile*, cudaStream_t, BsPlan<float>*, bool);
 template cudaError_t bg_backsub_many<int32_t>(const std::vector<BsInput<int32_t>>&, uint32_t*, uint32_t*, size_t,
-                                              double*, FwProfile*, cudaStream_t, BsPlan<int32_t>*);
+                                              double*, FwProfile*, cudaStream_t, BsPlan<int32_t>*, bool);
 
 template cudaError_t launch_fill_marked<float>(float*, int64_t, const uint32_t*, cudaStream_t);
 template cudaError_t launch_fill_marked<int32_t>(int32_t*, int64_t, const uint32_t*, cudaStream_t);
