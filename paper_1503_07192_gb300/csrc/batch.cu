@@ -148,6 +148,10 @@ struct BatchPtrs {
     int32_t* bgpos = nullptr;
     uint32_t* err = nullptr;
     uint32_t* tables = nullptr;  // every APSP(C), then every boundary-graph matrix
+    const MatDesc* cdescs = nullptr;  // every component's table in `tables`, its graph, the graphs' matrices
+    const int32_t* cgraph = nullptr;
+    const CliqueGraph* cliques = nullptr;
+    int64_t ktot = 0;
     int64_t check_off = 0, check_elems = 0;  // the Floyd-Warshall boundary-graph tables
 };
 
@@ -299,9 +303,13 @@ cudaError_t batch_bg_tables(std::vector<Inst>& I, const BatchPtrs& P, const MatD
         if ((e = x.elim ? launch_fill_marked<T>(D, x.N, be.marks + x.marks, st) : launch_bg_fill<T>(D, x.N, st)) !=
             cudaSuccess)
             return e;
-        e = launch_bg_clique<T>(base + x.apsp_off, check, P.descs + x.kbase, P.nb + x.kbase, P.bgoff + x.kbase,
-                                P.bgpos + x.slotbase, x.k, D, x.N, st);
-        if (e != cudaSuccess) return e;
+    }
+    if ((e = launch_bg_clique_many<T>(base, check, P.cdescs, P.nb, P.bgoff, P.bgpos, P.cgraph, P.cliques,
+                                      (int32_t)P.ktot, st)) != cudaSuccess)
+        return e;
+    for (auto& x : I) {
+        if (x.N == 0) continue;
+        T* D = base + x.d_off;
         e = launch_bg_inter<T>(f32w, x.n, x.rp, x.col, x.w, x.part, P.local + x.vbase, P.bgoff + x.kbase,
                                P.bgpos + x.slotbase, D, x.N, st);
         if (e != cudaSuccess) return e;
@@ -932,6 +940,25 @@ spq_status build_many_impl(int32_t G, const spq_graph* gs, const spq_opts& o, cu
             BCK(launch_mark_pairs(d_shared + shared_at[g], (int32_t)(shared_at[g + 1] - shared_at[g]), x.N,
                                   be.marks0 + x.marks, st));
         }
+    }
+    {
+        std::vector<int32_t> cgraph(ktot);
+        std::vector<CliqueGraph> cq;
+        for (int32_t g = 0; g < G; ++g) {
+            cq.push_back(CliqueGraph{I[g].d_off, I[g].N, I[g].slotbase});
+            std::fill_n(cgraph.begin() + I[g].kbase, I[g].k, g);
+        }
+        int32_t* d_cgraph = nullptr;
+        CliqueGraph* d_cq = nullptr;
+        BCK(tmp.alloc(&d_cgraph, (size_t)ktot));
+        BCK(tmp.alloc(&d_cq, cq.size()));
+        // (pageable uploads: staged before they return)
+        BCK(cudaMemcpyAsync(d_cgraph, cgraph.data(), (size_t)ktot * 4, cudaMemcpyHostToDevice, st));
+        BCK(cudaMemcpyAsync(d_cq, cq.data(), cq.size() * sizeof(CliqueGraph), cudaMemcpyHostToDevice, st));
+        P.cdescs = d_cd;
+        P.cgraph = d_cgraph;
+        P.cliques = d_cq;
+        P.ktot = ktot;
     }
     BCK(tmp.alloc(&d_bd, bd.size()));
     BCK(tmp.alloc(&fw_scratch, (size_t)fw_words));

@@ -145,6 +145,14 @@ cudaError_t launch_bg_fill(T* D, int64_t N, cudaStream_t st);
 template <typename T>
 cudaError_t launch_bg_clique(const void* apsp, bool i32, const MatDesc* descs, const int32_t* nb, const int32_t* bg_off,
                              const int32_t* bgpos, int32_t k, T* D, int64_t N, cudaStream_t st);
+// The same for every component (descs: offsets in `tables`) of several graphs.
+struct CliqueGraph {
+    int64_t d_off, N, slotbase;  // its matrix in `tables`, the matrix's order, its slots in bgpos
+};
+template <typename T>
+cudaError_t launch_bg_clique_many(T* tables, bool i32, const MatDesc* descs, const int32_t* nb, const int32_t* bg_off,
+                                  const int32_t* bgpos, const int32_t* cgraph, const CliqueGraph* graphs, int32_t ktot,
+                                  cudaStream_t st);
 template <typename T>
 cudaError_t launch_bg_inter(bool f32w, int32_t n, const int64_t* rp, const int32_t* col, const void* w,
                             const int32_t* part, const int32_t* local, const int32_t* bg_off, const int32_t* bgpos, T* D,
