@@ -377,8 +377,10 @@ __global__ void __launch_bounds__(GTH) k_backward_flow(const View<T> V, const Wa
         if (W.foff[mid] <= i) lo = mid; else hi = mid;
     }
     const int32_t nb = V.nb[lo], vs = V.vstart[lo];
-    const int32_t r = (int32_t)(i - W.foff[lo]);
-    const bool ok = walk_hops<T, 1>(V, W, lo, r / nb, r % nb, (int64_t)V.n + 1, 0, 1u << (threadIdx.x & 31),
+    // (64 bits: |B|^2 passes 2^31 from 46,341 boundary vertices on)
+    const int64_t r = i - W.foff[lo], b = r / nb;
+    const bool ok = walk_hops<T, 1>(V, W, lo, (int32_t)b, (int32_t)(r - b * nb), (int64_t)V.n + 1, 0,
+                                    1u << (threadIdx.x & 31),
                                     [&](int32_t from, int32_t slot, int32_t) {
                                         atomicAdd(grad + W.vrange[vs + from].x + slot, g);
                                     });
