@@ -634,6 +634,7 @@ __global__ void __launch_bounds__(NTH, SPQ_FW_MIN_CTAS) k_elim_phase2(const Elim
             if (__ldcg(f) == 2u) *f = 1u;
         }
     }
+    __syncthreads();  // (a tile of row r marked there may be unmarked here)
     for (uint32_t ci = tid; ci < c; ci += blockDim.x) {
         const int64_t J = sc.cand[1 + ci];
         uint4* ka = reinterpret_cast<uint4*>(sc.kacc + J * 4);
