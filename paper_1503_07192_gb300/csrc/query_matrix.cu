@@ -16,8 +16,10 @@
 // targets' rows of APSP(C2) are read once per 64 sources and in whole lines (one target per
 // lane, walking its own row, read a sector per value: 1.39 ms for 64 x 2^18 where the two
 // stages take 0.4); the tile goes out through shared memory, so that runs of neighbouring
-// targets are written together.  The targets are sorted by component; the tiles are listed
-// on the device, and nothing waits on the host.
+// targets are written together.  The targets are sorted by component; the tiles, and the
+// components that have targets (the only ones t is computed and has columns for: 20,000
+// sources x 1 target 2.4 ms with columns for all 256 components, 512 sources at a time, 0.40
+// with one component's), are listed on the device, and nothing waits on the host.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -45,12 +47,6 @@ __device__ __forceinline__ T tmin2(T a, T b) {
 __device__ __forceinline__ int32_t add_min(int32_t a, int32_t b, int32_t t) { return __viaddmin_s32(a, b, t); }
 __device__ __forceinline__ float add_min(float a, float b, float t) { return fminf(t, a + b); }
 
-// Column of t where component c's values start: a multiple of 4, the components apart
-// (f(x) = x rounded up to 4 is at most x + 3).
-__device__ __forceinline__ int64_t t_off(const int32_t* __restrict__ bg_off, int32_t c) {
-    return ((int64_t)bg_off[c] + 3 * (int64_t)c + 3) & ~(int64_t)3;
-}
-
 // key = component of the vertex (k for an id out of range: sorted last), val = position
 __global__ void k_comp_keys(const int32_t* __restrict__ ids, int64_t n, int32_t nv, const int32_t* __restrict__ comp,
                             uint32_t k, uint32_t* __restrict__ keys, uint32_t* __restrict__ vals) {
@@ -62,15 +58,23 @@ __global__ void k_comp_keys(const int32_t* __restrict__ ids, int64_t n, int32_t 
 }
 
 // A tile of the sorted targets: positions [start, start + count) of component c (k: ids out
-// of range).
+// of range), whose values of t start at column toff (a multiple of 4).
 struct MTile {
-    uint32_t c, start, count, pad_;
+    uint32_t c, start, count, toff;
+};
+
+// What the targets need on the device: the number of tiles, of components with targets, and
+// of columns of t (only those components have any: a row of t over every component would leave
+// room for few sources at a time where the targets are few).
+struct MCount {
+    uint32_t ntiles, ncomp, width, pad_;
 };
 
 // The tiles of every component (thread c): its run of the sorted keys by two binary
-// searches, cut into pieces of MT; cnt[c] = the run's length.
+// searches, cut into pieces of MT; comps: the components with a run and their columns of t.
 __global__ void k_matrix_tiles(const uint32_t* __restrict__ keys, int64_t n, uint32_t k, MTile* __restrict__ tiles,
-                               uint32_t* __restrict__ ntiles, uint32_t* __restrict__ cnt) {
+                               MCount* __restrict__ count, uint2* __restrict__ comps,
+                               const int32_t* __restrict__ nb) {
     const uint32_t c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c > k) return;
     auto lower = [&](uint32_t x) {  // first position with keys >= x
@@ -82,26 +86,33 @@ __global__ void k_matrix_tiles(const uint32_t* __restrict__ keys, int64_t n, uin
         return lo;
     };
     const int64_t a = lower(c), b = lower(c + 1);
-    cnt[c] = (uint32_t)(b - a);
     if (a == b) return;
-    const uint32_t m = (uint32_t)((b - a + MT - 1) / MT), at = atomicAdd(ntiles, m);
+    uint32_t toff = 0;
+    if (c < k) {
+        toff = atomicAdd(&count->width, (uint32_t)(nb[c] + 3) & ~3u);
+        comps[atomicAdd(&count->ncomp, 1u)] = make_uint2(c, toff);
+    }
+    const uint32_t m = (uint32_t)((b - a + MT - 1) / MT), at = atomicAdd(&count->ntiles, m);
     for (uint32_t i = 0; i < m; ++i)
-        tiles[at + i] = MTile{c, (uint32_t)(a + (int64_t)i * MT), (uint32_t)std::min<int64_t>(MT, b - a - (int64_t)i * MT), 0u};
+        tiles[at + i] = MTile{c, (uint32_t)(a + (int64_t)i * MT), (uint32_t)std::min<int64_t>(MT, b - a - (int64_t)i * MT), toff};
 }
 
 // Stage 1: t of the sources sid[s0 .. s0 + ns) for the components with targets, a warp per
-// (source, component); values past |B2| up to a multiple of 4 are infinite.
+// (source, component); values past |B2| up to a multiple of 4 are infinite.  Only components
+// with targets are enumerated: over all k of them, a grid whose warps are a multiple of k gives
+// each warp one component for good, so that with few targets most warps had nothing to do.
 template <typename T>
-__global__ void __launch_bounds__(MTH) k_matrix_t(const QueryCtx<T> ctx, uint32_t k, const int32_t* __restrict__ sid,
-                                                  int64_t s0, int64_t ns, const uint32_t* __restrict__ cnt,
-                                                  int64_t ldt, T* __restrict__ t) {
+__global__ void __launch_bounds__(MTH) k_matrix_t(const QueryCtx<T> ctx, const int32_t* __restrict__ sid,
+                                                  int64_t s0, int64_t ns, const MCount* __restrict__ count,
+                                                  const uint2* __restrict__ comps, int64_t ldt,
+                                                  T* __restrict__ t) {
     const int lane = threadIdx.x & 31;
     const T inf = Inf<T>::value();
-    const int64_t nw = ((int64_t)gridDim.x * MTH) >> 5;
-    for (int64_t x = ((int64_t)blockIdx.x * MTH + threadIdx.x) >> 5; x < ns * k; x += nw) {
-        const int64_t s = x / k;
-        const int32_t c2 = (int32_t)(x - s * k);
-        if (cnt[c2] == 0) continue;
+    const int64_t nw = ((int64_t)gridDim.x * MTH) >> 5, nc = count->ncomp;
+    for (int64_t x = ((int64_t)blockIdx.x * MTH + threadIdx.x) >> 5; x < ns * nc; x += nw) {
+        const int64_t s = x / nc;
+        const uint2 ct = comps[x - s * nc];
+        const int32_t c2 = (int32_t)ct.x;
         const int32_t v1 = sid[s0 + s];
         if (v1 < 0 || v1 >= ctx.n) continue;
         const int32_t c1 = ctx.comp[v1];
@@ -110,7 +121,7 @@ __global__ void __launch_bounds__(MTH) k_matrix_t(const QueryCtx<T> ctx, uint32_
         const int32_t* pos1 = ctx.bgpos + ctx.bg_off[c1];
         const int32_t* pos2 = ctx.bgpos + ctx.bg_off[c2];
         const T* a1 = ctx.apsp + d1.off + (int64_t)ctx.local[v1] * d1.n;
-        T* tr = t + s * ldt + t_off(ctx.bg_off, c2);
+        T* tr = t + s * ldt + ct.y;
         for (int32_t jb = 0; jb < nb4; jb += 128) {
             int32_t col[4];
             T y[4];
@@ -162,13 +173,13 @@ template <typename T, bool OUT_F32>
 __global__ void __launch_bounds__(MTH, 2)
     k_matrix_out(const QueryCtx<T> ctx, uint32_t k, const int32_t* __restrict__ sid, int64_t s0, int64_t ns,
                  const int32_t* __restrict__ tid_, const uint32_t* __restrict__ tval, const MTile* __restrict__ tiles,
-                 const uint32_t* __restrict__ ntiles_p, int64_t nt, int64_t ldt, const T* __restrict__ t,
+                 const MCount* __restrict__ count, int64_t nt, int64_t ldt, const T* __restrict__ t,
                  void* __restrict__ out) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     MSmem<T>& sm = *reinterpret_cast<MSmem<T>*>(smem_raw);
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
     const T inf = Inf<T>::value();
-    const int64_t ntiles = *ntiles_p, nsg = (ns + MS - 1) / MS;
+    const int64_t ntiles = count->ntiles, nsg = (ns + MS - 1) / MS;
     for (int64_t item = blockIdx.x; item < ntiles * nsg; item += gridDim.x) {
         const MTile tl = tiles[item % ntiles];
         const int64_t sb = (item / ntiles) * MS;
@@ -181,7 +192,7 @@ __global__ void __launch_bounds__(MTH, 2)
         if (valid) {
             d2 = ctx.descs[tl.c];
             nb4 = (ctx.nb[tl.c] + 3) & ~3;
-            to = t_off(ctx.bg_off, (int32_t)tl.c);
+            to = tl.toff;
         }
         if (tid < MT) {
             const uint32_t p = tid < nt_ ? tval[tl.start + tid] : 0u;
@@ -299,19 +310,19 @@ constexpr int64_t kTElems = 1 << 24;  // most values of t at a time (64 MB), at 
 
 template <typename T, bool OUT_F32>
 cudaError_t matrix_launch(const QueryCtx<T>& ctx, uint32_t k, const int32_t* src, int64_t ns,
-                          const int32_t* tgt, const uint32_t* tval, const MTile* tiles, const uint32_t* ntiles,
-                          const uint32_t* cnt, int64_t nt, int64_t ldt, int64_t rows, T* t, void* out,
+                          const int32_t* tgt, const uint32_t* tval, const MTile* tiles, const MCount* count,
+                          const uint2* comps, int64_t nt, int64_t ldt, int64_t rows, T* t, void* out,
                           cudaStream_t st) {
     auto kern = k_matrix_out<T, OUT_F32>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(MSmem<T>));
     for (int64_t s0 = 0; s0 < ns && e == cudaSuccess; s0 += rows) {
         const int64_t n = std::min(rows, ns - s0);
-        const int64_t warps = n * (int64_t)k;
+        const int64_t warps = n * std::min<int64_t>(k, nt);  // at most
         k_matrix_t<T><<<(unsigned)std::min<int64_t>((warps + 7) / 8, (int64_t)msms() * 32), MTH, 0, st>>>(
-            ctx, k, src, s0, n, cnt, ldt, t);
+            ctx, src, s0, n, count, comps, ldt, t);
         const int64_t items = ((nt + MT - 1) / MT + k + 1) * ((n + MS - 1) / MS);
         kern<<<(unsigned)std::min<int64_t>(items, (int64_t)msms() * 2), MTH, sizeof(MSmem<T>), st>>>(
-            ctx, k, src, s0, n, tgt, tval, tiles, ntiles, nt, ldt, t, out);
+            ctx, k, src, s0, n, tgt, tval, tiles, count, nt, ldt, t, out);
         count_launches(2);
         e = cudaGetLastError();
     }
@@ -379,14 +390,16 @@ extern "C" spq_status spq_query_matrix(spq_handle* h, const int32_t* sources, in
         d_out = p3;
     }
     // the targets sorted by component, their tiles, t of a batch of sources
-    const int64_t ldt = round_up(h->nbg + 3 * (int64_t)k, 4) + 4;
+    // (its rows: the components with targets, at most nt of them)
+    const int64_t ldt = std::min(round_up(h->nbg + 3 * (int64_t)k, 4), std::min<int64_t>(nt, k) * round_up(nbmax, 4)) + 4;
     int64_t rows = std::min(round_up(ns, MS), std::max<int64_t>(MS, kTElems / ldt / MS * MS));
     const int64_t max_tiles = (nt + MT - 1) / MT + k + 1;
-    uint32_t *buf, *cnt;
+    uint32_t* buf;
+    MCount* count;  // then the components with targets
     MTile* tiles;
     void* t;
     if ((e = alloc((void**)&buf, (size_t)(4 * nt + radix_hist_words(nt)) * 4)) != cudaSuccess ||
-        (e = alloc((void**)&cnt, ((size_t)k + 2) * 4)) != cudaSuccess ||
+        (e = alloc((void**)&count, sizeof(MCount) + (size_t)k * sizeof(uint2))) != cudaSuccess ||
         (e = alloc((void**)&tiles, (size_t)max_tiles * sizeof(MTile))) != cudaSuccess)
         return fail(e);
     // (fewer sources at a time where t of that many does not fit)
@@ -395,28 +408,28 @@ extern "C" spq_status spq_query_matrix(spq_handle* h, const int32_t* sources, in
         rows = (rows + 1) / 2;
     }
     if (e != cudaSuccess) return fail(e);
-    uint32_t* ntiles = cnt + k + 1;
+    uint2* comps = reinterpret_cast<uint2*>(count + 1);
     k_comp_keys<<<(unsigned)((nt + 255) / 256), 256, 0, st>>>(d_t, nt, h->n, h->comp, (uint32_t)k, buf, buf + nt);
     int bits = 0;
     while (bits < 32 && ((uint64_t)k >> bits)) ++bits;
     bool in_k1 = false;
     if ((e = radix_sort_pairs(buf, buf + nt, buf + 2 * nt, buf + 3 * nt, buf + 4 * nt, nt, bits, &in_k1, st)) !=
             cudaSuccess ||
-        (e = cudaMemsetAsync(ntiles, 0, 4, st)) != cudaSuccess)
+        (e = cudaMemsetAsync(count, 0, sizeof(MCount), st)) != cudaSuccess)
         return fail(e);
     k_matrix_tiles<<<(unsigned)((k + 1 + 127) / 128), 128, 0, st>>>(in_k1 ? buf + 2 * nt : buf, nt, (uint32_t)k, tiles,
-                                                                    ntiles, cnt);
+                                                                    count, comps, h->nb);
     count_launches(2);
     const uint32_t* tval = in_k1 ? buf + 3 * nt : buf + nt;
     if (f32store)
-        e = out_f32 ? matrix_launch<float, true>(cf, (uint32_t)k, d_s, ns, d_t, tval, tiles, ntiles, cnt, nt,
+        e = out_f32 ? matrix_launch<float, true>(cf, (uint32_t)k, d_s, ns, d_t, tval, tiles, count, comps, nt,
                                                  ldt, rows, (float*)t, d_out, st)
-                    : matrix_launch<float, false>(cf, (uint32_t)k, d_s, ns, d_t, tval, tiles, ntiles, cnt, nt,
+                    : matrix_launch<float, false>(cf, (uint32_t)k, d_s, ns, d_t, tval, tiles, count, comps, nt,
                                                   ldt, rows, (float*)t, d_out, st);
     else
-        e = out_f32 ? matrix_launch<int32_t, true>(ci, (uint32_t)k, d_s, ns, d_t, tval, tiles, ntiles, cnt, nt,
+        e = out_f32 ? matrix_launch<int32_t, true>(ci, (uint32_t)k, d_s, ns, d_t, tval, tiles, count, comps, nt,
                                                    ldt, rows, (int32_t*)t, d_out, st)
-                    : matrix_launch<int32_t, false>(ci, (uint32_t)k, d_s, ns, d_t, tval, tiles, ntiles, cnt,
+                    : matrix_launch<int32_t, false>(ci, (uint32_t)k, d_s, ns, d_t, tval, tiles, count, comps,
                                                     nt, ldt, rows, (int32_t*)t, d_out, st);
     if (e != cudaSuccess) return fail(e);
     if (!ds) {
