@@ -500,6 +500,21 @@ __global__ void __launch_bounds__(GTH, 4) k_paths_hops(const View<T> V, const Wa
 
 constexpr int64_t kSavedSlice = 1 << 22;
 
+// Whether q pairs are answered with their witnesses in groups: what a group's block, a pair in
+// a group and a pair on its own take, in ns of the whole GPU, as functions of the mean |B(C)| =
+// nb that fit measurements of random pairs (at nb 28, 56, 118 and 235: a block 10, 16, 31 and
+// 108 ns, a pair on its own 2.1, 7.3, 29 and 97), and 60 us of launches for the sort.  Random
+// pairs make k^2 (1 - e^(-q / k^2)) groups.  0.95: many tying columns cost a few ns a pair.
+// (256 components with nb 118: 20,000 pairs 645 us a warp per pair and 644 grouped, 40,000 1,220
+// and 1,035, a million 28,400 and 4,240; 1,024 components with nb 28: a million 2,060 and 7,800.)
+bool saved_groups(const spq_handle* h, int64_t q) {
+    if (q < 4096 || h->k > 65535 || h->max_nb > query_blocks_max_nb()) return false;
+    const double n = (double)q, k2 = (double)h->k * h->k, nb = (double)h->nbg / h->k;
+    const double groups = k2 * -expm1(-n / k2);
+    return groups * std::max(4.0 + 0.225 * nb, 0.00195 * nb * nb) + n * (0.5 + 0.014 * nb) + 6e4 <
+           0.95 * n * (0.035 * nb + 0.00176 * nb * nb);
+}
+
 bool capturing(cudaStream_t st) {
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(st, &cap) == cudaSuccess) return cap != cudaStreamCaptureStatusNone;
@@ -678,13 +693,10 @@ spq_status spq_query_saved(spq_handle* h, const int32_t* pairs, int64_t q, void*
     if (((uintptr_t)pairs & 7u) || ((uintptr_t)saved & 7u) || ((uintptr_t)dist_out & 3u)) return SPQ_EINVAL;
     cudaStream_t st = (cudaStream_t)stream;
     // Large batches grouped by component pair, each block of the boundary matrix read once per
-    // group (1M pairs on 2^18 vertices: a warp per pair 29.5 ms, most of it the block's rows
-    // from DRAM again for every pair).  From 4,096 pairs, as spq_query, and 9e7 updates (the
-    // sort's launches take about 60 us, in which a warp per pair does that many); at most
-    // kSavedSlice pairs at a time (39 words of scratch a pair).  Not inside a stream capture: a
-    // captured call allocates nothing.
-    const double nb_mean = (double)h->nbg / h->k;
-    if (q >= 4096 && (double)q * nb_mean * nb_mean >= 9e7 && h->k <= 65535 && h->max_nb <= query_blocks_max_nb() && !capturing(st)) {
+    // group (1M pairs on 2^18 vertices: a warp per pair 28.3 ms, most of it the block's rows
+    // from DRAM again for every pair; grouped 4.2 ms); at most kSavedSlice pairs at a time (39
+    // words of scratch a pair).  Not inside a stream capture: a captured call allocates nothing.
+    if (saved_groups(h, q) && !capturing(st)) {
         uint32_t* scratch = nullptr;
         const int64_t slice = std::min(q, kSavedSlice);
         if (scratch_alloc((void**)&scratch, (size_t)query_saved_scratch_words(slice) * 4, st) == cudaSuccess) {
