@@ -566,9 +566,9 @@ __global__ void __launch_bounds__(256) k_qb_fallback(const QueryCtx<int32_t> ctx
 }
 
 // The witness form's last step, a warp per sorted position: of the columns attaining the
-// minimum, each with its first row b1 that attains t(b2) (read again from the matrix: a few
-// of the block's columns), the smallest (b1, b2); then the same-component distance, equal
-// and out-of-range pairs, as k_query_saved answers them.
+// minimum, each with its first row b1 that attains t(b2) (read again from the matrix: few
+// columns one by one, many together row by row), the smallest (b1, b2); then the
+// same-component distance, equal and out-of-range pairs, as k_query_saved answers them.
 template <typename T>
 __global__ void __launch_bounds__(256) k_qb_witness(const QueryCtx<T> ctx, const int2* __restrict__ pairs,
                                                     const uint32_t* __restrict__ keys,
@@ -609,30 +609,76 @@ __global__ void __launch_bounds__(256) k_qb_witness(const QueryCtx<T> ctx, const
             best = b < inf ? b : inf;
         }
         if (best < inf) {
-            const int32_t nw = (nb2 + 31) >> 5;
+            const int32_t bb = enc_min<T>(best), nw = (nb2 + 31) >> 5;
+            const T* A2 = ctx.apsp + ctx.descs[c2].off + (int64_t)ctx.local[pr.y] * ctx.descs[c2].n;
             const uint32_t mw = lane < nw ? masks[p * QB_MW + lane] : 0u;
+            // column j's first row attaining t(b2), and the smallest so far
+            auto column = [&](int32_t j) {
+                const int64_t cp = pos2[j];
+                const T* drow = ctx.D + cp * ctx.N;
+                T t = inf;
+                uint32_t ti = 0xffffffffu;
+                for (int32_t i = lane; i < nb1; i += 32) {
+                    // (D is symmetric bit for bit outside its diagonal tiles: read along
+                    //  row b2 there)
+                    const int64_t rp = pos1[i];
+                    const T cand = A1[i] + ((rp / kTile == cp / kTile) ? ctx.D[rp * ctx.N + cp] : drow[rp]);
+                    if (cand < t) {
+                        t = cand;
+                        ti = (uint32_t)i;
+                    }
+                }
+                const int32_t tb = enc_min<T>(t);
+                const int32_t mt = __reduce_min_sync(0xffffffffu, tb);
+                const uint32_t mi = __reduce_min_sync(0xffffffffu, tb == mt ? ti : 0xffffffffu);
+                const unsigned long long x = ((unsigned long long)mi << 32) | (uint32_t)j;
+                if (x < sel) sel = x;
+            };
             for (int32_t w = 0; w < nw; ++w) {
-                for (uint32_t bits = __shfl_sync(0xffffffffu, mw, w); bits; bits &= bits - 1u) {
-                    const int32_t j = 32 * w + __ffs(bits) - 1;
-                    const int64_t cp = pos2[j];
-                    const T* drow = ctx.D + cp * ctx.N;
-                    T t = inf;
-                    uint32_t ti = 0xffffffffu;
-                    for (int32_t i = lane; i < nb1; i += 32) {
-                        // (D is symmetric bit for bit outside its diagonal tiles: read along
-                        //  row b2 there)
-                        const int64_t rp = pos1[i];
-                        const T cand = A1[i] + ((rp / kTile == cp / kTile) ? ctx.D[rp * ctx.N + cp] : drow[rp]);
-                        if (cand < t) {
-                            t = cand;
-                            ti = (uint32_t)i;
+                uint32_t bits = __shfl_sync(0xffffffffu, mw, w);
+                if (bits == 0u) continue;
+                const uint32_t most = (uint32_t)(sel >> 32);  // (rows past it decide nothing)
+                const int32_t rows = most < (uint32_t)nb1 ? (int32_t)most + 1 : nb1;
+                if (rows > 8 * __popc(bits)) {
+                    for (; bits; bits &= bits - 1u) column(32 * w + __ffs(bits) - 1);
+                    continue;
+                }
+                // Many columns tie (unit weights: every second one): the rows from the first,
+                // a column a lane, until one attains the minimum.  In integers that row attains
+                // its column's t; float sums that round to the minimum may not, so that
+                // column's own first row is looked up.
+                const int32_t j = 32 * w + lane;
+                const bool mine = (bits >> lane) & 1u;
+                const int32_t col = pos2[mine ? j : 0];
+                const T c = mine ? A2[j] : inf;
+                for (int32_t i0 = 0; i0 < rows && bits; i0 += 4) {
+                    T d[4];
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        const int32_t i = i0 + q < rows ? i0 + q : rows - 1;
+                        d[q] = A1[i] + ctx.D[(int64_t)pos1[i] * ctx.N + col];
+                    }
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        if (i0 + q >= rows) break;
+                        uint32_t hit = __ballot_sync(0xffffffffu, ((bits >> lane) & 1u) && enc_min<T>(d[q] + c) == bb);
+                        if constexpr (std::is_same<T, int32_t>::value) {
+                            if (hit) {
+                                const unsigned long long x =
+                                    ((unsigned long long)(i0 + q) << 32) | (uint32_t)(32 * w + __ffs(hit) - 1);
+                                if (x < sel) sel = x;
+                                bits = 0u;  // (every other column's first row is no earlier)
+                            }
+                        } else {
+                            for (; hit; hit &= hit - 1u) {
+                                const int b = __ffs(hit) - 1;
+                                if ((((unsigned long long)(i0 + q) << 32) | (uint32_t)(32 * w + b)) >= sel) break;
+                                bits &= ~(1u << b);
+                                column(32 * w + b);
+                            }
+                            if ((uint32_t)(i0 + q) >= (uint32_t)(sel >> 32)) bits = 0u;
                         }
                     }
-                    const int32_t tb = enc_min<T>(t);
-                    const int32_t mt = __reduce_min_sync(0xffffffffu, tb);
-                    const uint32_t mi = __reduce_min_sync(0xffffffffu, tb == mt ? ti : 0xffffffffu);
-                    const unsigned long long x = ((unsigned long long)mi << 32) | (uint32_t)j;
-                    if (x < sel) sel = x;
                 }
             }
         }
