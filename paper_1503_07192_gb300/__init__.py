@@ -178,7 +178,7 @@ def spq_build(n: int, row_ptr, col, w, part, k: int, opts: SpqOpts | None = None
 def spq_build_many(graphs, opts: SpqOpts | None = None, stream=None) -> list:
     """Build many independent graphs at once.  graphs: sequence of (n, row_ptr, col, w,
     part, k) tuples (numpy arrays or tensors, host or device, one weight type for all).
-    Returns one SpqHandle per graph (they share one device allocation)."""
+    Returns one SpqHandle per graph (they share their device allocations)."""
     lib = _lib.load()
     keep = []
     arr = (_lib.SpqGraph * len(graphs))()

@@ -139,8 +139,7 @@ size_t pool_cached_bytes(int dev) {
 void free_handle_memory(spq_handle* h) {
     if (h->arena) {
         if (h->arena->refs.fetch_sub(1) == 1) {
-            cudaFreeAsync(h->arena->base, 0);  // back to the pool
-            cudaStreamSynchronize(0);
+            h->arena->release();
             delete h->arena;
         }
         h->arena = nullptr;

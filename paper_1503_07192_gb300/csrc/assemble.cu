@@ -143,14 +143,14 @@ template <typename S, typename T>
 __global__ void k_bg_clique_many(const S* base, const MatDesc* __restrict__ descs,
                                  const int32_t* __restrict__ nb, const int32_t* __restrict__ bg_off,
                                  const int32_t* __restrict__ bgpos, const int32_t* __restrict__ cgraph,
-                                 const CliqueGraph* __restrict__ graphs, int32_t ktot, T* tables) {
+                                 const CliqueGraph* __restrict__ graphs, int32_t ktot, T* mats) {
     for (int32_t c = blockIdx.x; c < ktot; c += gridDim.x) {
         const int32_t b = nb[c];
         if (b == 0) continue;
         const MatDesc d = descs[c];
         const CliqueGraph g = graphs[cgraph[c]];
         const S* A = base + d.off;
-        T* D = tables + g.d_off;
+        T* D = mats + g.d_off;
         const int32_t* pos = bgpos + g.slotbase + bg_off[c];
         for (int32_t i = threadIdx.y; i < b; i += blockDim.y) {
             T* row = D + (int64_t)pos[i] * g.N;
@@ -284,17 +284,17 @@ cudaError_t launch_bg_clique(const void* apsp, bool i32, const MatDesc* descs, c
 }
 
 template <typename T>
-cudaError_t launch_bg_clique_many(T* tables, bool i32, const MatDesc* descs, const int32_t* nb, const int32_t* bg_off,
-                                  const int32_t* bgpos, const int32_t* cgraph, const CliqueGraph* graphs, int32_t ktot,
-                                  cudaStream_t st) {
+cudaError_t launch_bg_clique_many(const void* apsp, T* mats, bool i32, const MatDesc* descs, const int32_t* nb,
+                                  const int32_t* bg_off, const int32_t* bgpos, const int32_t* cgraph,
+                                  const CliqueGraph* graphs, int32_t ktot, cudaStream_t st) {
     if (ktot <= 0) return cudaSuccess;
     const int blocks = ktot < 65535 ? ktot : 65535;
     if (i32)
-        k_bg_clique_many<int32_t, T><<<blocks, dim3(32, 8), 0, st>>>((const int32_t*)tables, descs, nb, bg_off, bgpos,
-                                                                     cgraph, graphs, ktot, tables);
+        k_bg_clique_many<int32_t, T><<<blocks, dim3(32, 8), 0, st>>>((const int32_t*)apsp, descs, nb, bg_off, bgpos,
+                                                                     cgraph, graphs, ktot, mats);
     else
-        k_bg_clique_many<T, T><<<blocks, dim3(32, 8), 0, st>>>(tables, descs, nb, bg_off, bgpos, cgraph, graphs, ktot,
-                                                               tables);
+        k_bg_clique_many<T, T><<<blocks, dim3(32, 8), 0, st>>>((const T*)apsp, descs, nb, bg_off, bgpos, cgraph, graphs,
+                                                               ktot, mats);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -340,7 +340,7 @@ cudaError_t launch_check_convert_blocks(float* base, const MatDesc* descs, const
     template cudaError_t launch_bg_fill<T>(T*, int64_t, cudaStream_t);                                             \
     template cudaError_t launch_bg_clique<T>(const void*, bool, const MatDesc*, const int32_t*, const int32_t*,    \
                                              const int32_t*, int32_t, T*, int64_t, cudaStream_t);                 \
-    template cudaError_t launch_bg_clique_many<T>(T*, bool, const MatDesc*, const int32_t*, const int32_t*,       \
+    template cudaError_t launch_bg_clique_many<T>(const void*, T*, bool, const MatDesc*, const int32_t*, const int32_t*,       \
                                                   const int32_t*, const int32_t*, const CliqueGraph*, int32_t,     \
                                                   cudaStream_t);                                                   \
     template cudaError_t launch_bg_inter<T>(bool, int32_t, const int64_t*, const int32_t*, const void*,            \

@@ -2,9 +2,9 @@
 // instances) and spq_query_many (Algorithm 2 for a query stream per instance).
 //
 // The instances share every launch where the work allows: one validation readback, one
-// device arena for all tables, one stable sort over every instance's vertices, one
-// readback of every instance's component adjacency (the host orders the instances'
-// boundary vertices in parallel threads), the component Floyd-Warshall of all
+// device allocation for the component tables and one for the boundary graphs' matrices, one
+// stable sort over every instance's vertices, one readback of every instance's component
+// adjacency (the host orders the instances' boundary vertices in parallel threads), the component Floyd-Warshall of all
 // components of all instances in the same launches, and the boundary-graph
 // Floyd-Warshall of all instances round by round in the same launches (each instance
 // with its own list of tiles with a finite pivot panel).  The per-instance work left is
@@ -137,7 +137,7 @@ struct Inst {
     std::vector<MatDesc> descs;  // relative to the instance's own APSP base
 };
 
-// Batch-wide device arrays (all inside the arena).
+// Batch-wide device arrays (all inside the arena's allocations).
 struct BatchPtrs {
     int32_t* comp = nullptr;
     int32_t* local = nullptr;
@@ -147,12 +147,13 @@ struct BatchPtrs {
     int32_t* csize = nullptr;
     int32_t* bgpos = nullptr;
     uint32_t* err = nullptr;
-    uint32_t* tables = nullptr;  // every APSP(C), then every boundary-graph matrix
+    uint32_t* tables = nullptr;  // every APSP(C)
+    uint32_t* mats = nullptr;    // every boundary-graph matrix
     const MatDesc* cdescs = nullptr;  // every component's table in `tables`, its graph, the graphs' matrices
     const int32_t* cgraph = nullptr;
     const CliqueGraph* cliques = nullptr;
     int64_t ktot = 0;
-    int64_t check_off = 0, check_elems = 0;  // the Floyd-Warshall boundary-graph tables
+    int64_t apsp_elems = 0, check_elems = 0;  // every APSP(C); the Floyd-Warshall matrices (the first ones)
 };
 
 // The instances whose boundary graph takes the elimination form: their matrices' marks
@@ -270,7 +271,7 @@ cudaError_t batch_comp_tables(std::vector<Inst>& I, const BatchPtrs& P, const Ma
     if (exact && max_ld > 0) {
         e = ce.nsel > 0 ? launch_check_convert_blocks(reinterpret_cast<float*>(base), d_cdescs, P.csize, (int32_t)ktot,
                                                       max_ld, exact, st)
-                        : launch_check_convert(reinterpret_cast<float*>(base), P.check_off, exact, st);
+                        : launch_check_convert(reinterpret_cast<float*>(base), P.apsp_elems, exact, st);
         if (e != cudaSuccess) return e;
     }
     if (ev) cudaEventRecord(ev[3], st);
@@ -290,7 +291,7 @@ cudaError_t batch_bg_tables(std::vector<Inst>& I, const BatchPtrs& P, const MatD
                             StageKeep<T>* keep = nullptr, bool* comp_inexact = nullptr) {
     *inexact = false;
     const bool replay = keep && keep->ready;
-    T* base = reinterpret_cast<T*>(P.tables);
+    T* base = reinterpret_cast<T*>(P.mats);
     cudaError_t e;
     if (be.n > 0 && (e = cudaMemcpyAsync(be.marks, be.marks0, (size_t)be.mark_words * 4, cudaMemcpyDeviceToDevice,
                                          st)) != cudaSuccess)
@@ -304,7 +305,7 @@ cudaError_t batch_bg_tables(std::vector<Inst>& I, const BatchPtrs& P, const MatD
             cudaSuccess)
             return e;
     }
-    if ((e = launch_bg_clique_many<T>(base, check, P.cdescs, P.nb, P.bgoff, P.bgpos, P.cgraph, P.cliques,
+    if ((e = launch_bg_clique_many<T>(P.tables, base, check, P.cdescs, P.nb, P.bgoff, P.bgpos, P.cgraph, P.cliques,
                                       (int32_t)P.ktot, st)) != cudaSuccess)
         return e;
     for (auto& x : I) {
@@ -387,8 +388,7 @@ cudaError_t batch_bg_tables(std::vector<Inst>& I, const BatchPtrs& P, const MatD
     }
     if (ev) cudaEventRecord(ev[5], st);
     if (check) {
-        if ((e = launch_check_convert(reinterpret_cast<float*>(P.tables) + P.check_off, P.check_elems, d_flag, st)) !=
-            cudaSuccess)
+        if ((e = launch_check_convert(reinterpret_cast<float*>(P.mats), P.check_elems, d_flag, st)) != cudaSuccess)
             return e;
         if (!replay) {
             uint32_t f[2] = {0, 0};
@@ -588,8 +588,8 @@ spq_status build_many_impl(int32_t G, const spq_graph* gs, const spq_opts& o, cu
     // The elimination's matrices may be ordered in aligned pieces whose rounds run side by
     // side (a matrix of 146 row blocks alone was 146 rounds one after another, two fifths of a
     // batch of 48): as many levels as leave pieces of 16 row blocks, each boundary padded to
-    // the tile edge.  Sized here for the most padding, placed once the order is known; without
-    // the pieces where that does not fit.
+    // the tile edge.  They are allocated once the order, and so the padding, is known; without
+    // the pieces where the most padding would not fit.
     auto run_depth = [](int64_t nbg) {
         int d = 0;
         while (d < kMaxRunDepth && (nbg >> (d + 1)) >= 16 * kTile) ++d;
@@ -605,7 +605,7 @@ spq_status build_many_impl(int32_t G, const spq_graph* gs, const spq_opts& o, cu
         return tot;
     };
     int64_t d_tot = reserve(true);
-    // arena: metadata arrays, then the tables (16-byte aligned)
+    // arena: metadata arrays, then the component tables (16-byte aligned)
     size_t off = 0;
     auto take = [&](size_t bytes) {
         size_t o2 = off;
@@ -617,7 +617,7 @@ spq_status build_many_impl(int32_t G, const spq_graph* gs, const spq_opts& o, cu
     const size_t o_bgoff = take(4 * (size_t)ktot), o_csize = take(4 * (size_t)ktot);
     const size_t o_bgpos = take(4 * (size_t)slot_tot), o_err = take(16 * (size_t)G);
     const size_t o_tables = off;
-    size_t arena_bytes = align256(o_tables + 4 * (size_t)(apsp_tot + d_tot));
+    const size_t arena_bytes = align256(o_tables + 4 * (size_t)apsp_tot);
     const int64_t fw_words = nbmat > 0 ? fw_many_scratch_words(nbmat, max_N) : 1;
     const bool comp_elim = o.comp_method != SPQ_BG_FW;
     const size_t temp_bytes = 16 * (size_t)ntot + 4 * (size_t)radix_hist_words(ntot) + 12 * (size_t)mtot +
@@ -626,28 +626,20 @@ spq_status build_many_impl(int32_t G, const spq_graph* gs, const spq_opts& o, cu
     size_t free_b = 0, total_b = 0;
     BCK(cudaMemGetInfo(&free_b, &total_b));
     free_b += pool_cached_bytes_current();
-    if (arena_bytes + temp_bytes > free_b) {
-        d_tot = reserve(false);
-        arena_bytes = align256(o_tables + 4 * (size_t)(apsp_tot + d_tot));
-    }
-    if (arena_bytes + temp_bytes > free_b) return SPQ_ENOMEM;
-    void* arena_base = nullptr;
-    {
-        // (from the library's pool: a batch's tens of gigabytes are kept mapped for the next)
-        cudaError_t e = scratch_alloc(&arena_base, arena_bytes, st);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-        if (e != cudaSuccess) return e == cudaErrorMemoryAllocation ? SPQ_ENOMEM : batch_cuda_fail(e);
-    }
+    if (arena_bytes + 4 * (size_t)d_tot + temp_bytes > free_b) d_tot = reserve(false);
+    if (arena_bytes + 4 * (size_t)d_tot + temp_bytes > free_b) return SPQ_ENOMEM;
     struct ArenaGuard {
-        void* p;
-        ~ArenaGuard() {
-            if (p) {
-                cudaFreeAsync(p, 0);
-                cudaStreamSynchronize(0);
-            }
-        }
-    } aguard{arena_base};
-    char* ab = static_cast<char*>(arena_base);
+        Arena a;
+        ~ArenaGuard() { a.release(); }
+    } aguard;
+    // (from the library's pool: a batch's tens of gigabytes are kept mapped for the next)
+    auto arena_alloc = [&](void** p, size_t bytes) {
+        const cudaError_t e = scratch_alloc(p, bytes, st);
+        return e == cudaSuccess ? SPQ_OK : e == cudaErrorMemoryAllocation ? SPQ_ENOMEM : batch_cuda_fail(e);
+    };
+    if (const spq_status s = arena_alloc(&aguard.a.base, arena_bytes)) return s;
+    BCK(cudaStreamSynchronize(st));
+    char* ab = static_cast<char*>(aguard.a.base);
     BatchPtrs P;
     P.comp = reinterpret_cast<int32_t*>(ab + o_comp);
     P.local = reinterpret_cast<int32_t*>(ab + o_local);
@@ -860,7 +852,7 @@ spq_status build_many_impl(int32_t G, const spq_graph* gs, const spq_opts& o, cu
     BCK(tmp.alloc(&d_cd, cd.size()));
     BCK(tmp.alloc(&d_flag, 3));  // boundary graphs, components, status of their elimination
     BCK(cudaMemcpyAsync(d_cd, cd.data(), cd.size() * sizeof(MatDesc), cudaMemcpyHostToDevice, st));
-    P.check_off = apsp_tot;
+    P.apsp_elems = apsp_tot;
     double bg_updates = 0.0, comp_elim_updates = 0.0;
     bool f32store = false;
     int32_t arith = SPQ_ARITH_I32;
@@ -891,7 +883,7 @@ spq_status build_many_impl(int32_t G, const spq_graph* gs, const spq_opts& o, cu
     BatchElim be;
     BCK(cudaGetDevice(&be.dev));
     be.panel_cap = o.bg_panel_mib > 0 ? ((size_t)o.bg_panel_mib << 20) : ((size_t)2 << 30);
-    int64_t at = apsp_tot;
+    int64_t at = 0;
     int32_t max_N_fw = 0;
     std::vector<int32_t> shared;  // the separators' blocks of every matrix (see launch_mark_pairs)
     std::vector<size_t> shared_at(G + 1, 0);
@@ -915,12 +907,16 @@ spq_status build_many_impl(int32_t G, const spq_graph* gs, const spq_opts& o, cu
         }
         shared_at[g + 1] = shared.size();
     }
-    P.check_elems = at - apsp_tot;
+    P.check_elems = at;
     for (Inst& x : I)
         if (x.elim || x.N == 0) {
             x.d_off = at;
             at += x.N * x.N;
         }
+    if (at > 0) {
+        if (const spq_status s = arena_alloc(&aguard.a.mats, 4 * (size_t)at)) return s;
+        P.mats = static_cast<uint32_t*>(aguard.a.mats);
+    }
     if (be.n > 0) {
         int32_t* d_shared = nullptr;
         BCK(tmp.alloc(&be.marks0, (size_t)be.mark_words));
@@ -1030,17 +1026,17 @@ spq_status build_many_impl(int32_t G, const spq_graph* gs, const spq_opts& o, cu
     BCK(cudaGetDevice(&dev));
     Arena* ar = new (std::nothrow) Arena();
     if (!ar) return SPQ_ENOMEM;
-    ar->base = arena_base;
+    ar->base = aguard.a.base;
+    ar->mats = aguard.a.mats;
     ar->refs = G;
-    aguard.p = nullptr;  // owned by the handles from here on
+    aguard.a.base = aguard.a.mats = nullptr;  // owned by the handles from here on
     out->resize(G, nullptr);
     for (int32_t g = 0; g < G; ++g) {
         const Inst& x = I[g];
         spq_handle* h = new (std::nothrow) spq_handle();
         if (!h) {  // nothing was handed out yet: release everything
             for (int32_t j = 0; j < g; ++j) delete (*out)[j];
-            cudaFreeAsync(ar->base, 0);
-            cudaStreamSynchronize(0);
+            ar->release();
             delete ar;
             out->clear();
             return SPQ_ENOMEM;
@@ -1065,7 +1061,7 @@ spq_status build_many_impl(int32_t G, const spq_graph* gs, const spq_opts& o, cu
         h->bgpos = P.bgpos + x.slotbase;
         h->err = P.err + 4 * (int64_t)g;
         h->apsp = P.tables + x.apsp_off;
-        h->D = x.N > 0 ? (void*)(P.tables + x.d_off) : nullptr;
+        h->D = x.N > 0 ? (void*)(P.mats + x.d_off) : nullptr;
         h->N = x.N;
         h->nbg = x.nbg;
         h->apsp_elems = x.apsp_elems;

@@ -145,12 +145,12 @@ cudaError_t launch_bg_fill(T* D, int64_t N, cudaStream_t st);
 template <typename T>
 cudaError_t launch_bg_clique(const void* apsp, bool i32, const MatDesc* descs, const int32_t* nb, const int32_t* bg_off,
                              const int32_t* bgpos, int32_t k, T* D, int64_t N, cudaStream_t st);
-// The same for every component (descs: offsets in `tables`) of several graphs.
+// The same for every component (descs: offsets in `apsp`) of several graphs.
 struct CliqueGraph {
-    int64_t d_off, N, slotbase;  // its matrix in `tables`, the matrix's order, its slots in bgpos
+    int64_t d_off, N, slotbase;  // its matrix in `mats`, the matrix's order, its slots in bgpos
 };
 template <typename T>
-cudaError_t launch_bg_clique_many(T* tables, bool i32, const MatDesc* descs, const int32_t* nb, const int32_t* bg_off,
+cudaError_t launch_bg_clique_many(const void* apsp, T* mats, bool i32, const MatDesc* descs, const int32_t* nb, const int32_t* bg_off,
                                   const int32_t* bgpos, const int32_t* cgraph, const CliqueGraph* graphs, int32_t ktot,
                                   cudaStream_t st);
 template <typename T>

@@ -11,11 +11,20 @@
 
 namespace spq {
 
-// One device allocation shared by the handles of a batch (spq_build_many); freed with
-// the last of them.
+// The device allocations shared by the handles of a batch (spq_build_many); freed with the
+// last of them.  The boundary graphs' matrices have one of their own: their size is known
+// only after the components' tables are under way.
 struct Arena {
-    void* base = nullptr;
+    void* base = nullptr;  // everything else
+    void* mats = nullptr;
     std::atomic<int> refs{0};
+    void release() {  // back to the pool
+        if (!base && !mats) return;
+        if (base) cudaFreeAsync(base, 0);
+        if (mats) cudaFreeAsync(mats, 0);
+        cudaStreamSynchronize(0);
+        base = mats = nullptr;
+    }
 };
 
 }  // namespace spq
