@@ -1148,9 +1148,14 @@ cudaError_t issue_queries(int32_t count, spq_handle* const* hs, const int32_t* c
     return e != cudaSuccess ? e : j;
 }
 
-// Scratch words of one lane, and the lanes' scratch (fewer lanes where it does not fit).
+// Scratch words of one lane, and the lanes' scratch: fewer lanes where it does not fit or
+// would pass kLaneBytes, which a query plan holds for its life (four lanes up to 700,000 pairs
+// an instance; beyond, one instance nearly fills the GPU: 8 x 1M pairs 10.4 ms on one lane, 9.6
+// on four, 8 x 50,000 pairs 1.18 and 0.85).
+constexpr int64_t kLaneBytes = (int64_t)256 << 20;
 int64_t lane_words(int64_t qmax) { return round_up(query_scratch_words(std::max<int64_t>(qmax, 1)), 4); }
 cudaError_t lane_scratch(uint32_t** p, int64_t words, QueryLanes& lanes, cudaStream_t st) {
+    lanes.n = (int)std::max<int64_t>(1, std::min<int64_t>(lanes.n, kLaneBytes / (words * 4)));
     cudaError_t e = scratch_alloc((void**)p, (size_t)(words * lanes.n) * 4, st);
     if (e != cudaSuccess && lanes.n > 1) {
         cudaGetLastError();

@@ -45,3 +45,23 @@ def test_handles_hold_their_footprints(bg):
     for h in hs:
         h.free()
     assert _used() == before
+
+
+@pytest.mark.parametrize("q", [50_000, 3_000_000])
+def test_a_query_plan_holds_bounded_scratch(q):
+    """Four instances in flight take four scratches (about 92 bytes a pair of the largest
+    instance), together at most 256 MiB; a larger instance takes one, as it needs anyway."""
+    m = spq()
+    torch, dev = torch_dev()
+    hs = m.spq_build_many(_graphs([(40, 60)] * 4))
+    pairs = [torch.randint(0, 1600, (q, 2), dtype=torch.int32, device=dev) for _ in hs]
+    ref = [m.spq_query(h, p) for h, p in zip(hs, pairs)]
+    before = _used()
+    plan = m.spq_query_plan(hs, pairs)
+    assert _used() - before <= max(256 << 20, 96 * q) + (8 << 20)
+    for out, r in zip(plan.run(), ref):
+        assert torch.equal(out, r)
+    plan.free()
+    assert _used() == before
+    for h in hs:
+        h.free()
