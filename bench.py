@@ -578,7 +578,9 @@ def run_grad(args, rank, local_rank):
     1,024, 1,000,000 pairs with upstream gradients N(0, 1).  One step = forward (build +
     distances with the minimising boundary pairs) + backward (path walks, gradient
     scatter onto the 1.5M CSR slots).  A seeded sample of 2,000 pairs is checked against
-    the CPU reference gradient (the oracle's Dijkstra paths, FP64)."""
+    the CPU reference gradient (the oracle's Dijkstra paths, FP64); of the last timed step,
+    the sample's distances and witnesses, and the whole gradient against the sum over the
+    same pairs in batches of 2,000 (which search every hop instead of the records)."""
     import numpy as np
     import torch
 
@@ -616,13 +618,16 @@ def run_grad(args, rank, local_rank):
         torch.cuda.synchronize()
         spq.spq_query_status(h)
         h.free()
-        return [e[i].elapsed_time(e[i + 1]) for i in range(3)]
+        return [e[i].elapsed_time(e[i + 1]) for i in range(3)], dist, saved
 
     clocks = ClockSampler(local_rank).started()
     for _ in range(args.warmup):
         step()
     clocks.mark()
-    times = [step() for _ in range(args.steps)]
+    times = []
+    for _ in range(args.steps):
+        t, dist, saved = step()
+        times.append(t)
     clk = clocks.stop()
     build_ms, fwd_ms, bwd_ms = (statistics.mean(t[i] for t in times) for i in range(3))
     # correctness on a sample of pairs: GPU gradient of the sample vs the CPU reference
@@ -632,8 +637,16 @@ def run_grad(args, rank, local_rank):
     dist_s, saved_s = spq.spq_query_saved(h, T(sp))
     gs = torch.zeros(g.m, dtype=torch.float32, device=dev)
     spq.spq_query_backward(h, T(sp), saved_s, T(su.astype(np.float32)), gs)
+    d_idx = T(idx)
+    timed_equal = bool(torch.equal(dist[d_idx], dist_s) and torch.equal(saved[d_idx], saved_s))
+    small = torch.zeros(g.m, dtype=torch.float32, device=dev)
+    for a in range(0, w.pairs.shape[0], 2000):
+        p, u = d_pairs[a : a + 2000].contiguous(), d_up[a : a + 2000].contiguous()
+        spq.spq_query_backward(h, p, saved[a : a + 2000].contiguous(), u, small)
     torch.cuda.synchronize()
+    spq.spq_query_status(h)
     h.free()
+    gerr = float((grad - small).abs().max() / small.abs().max().clamp(min=1.0))
     ref_d, ref_g = oracle.pairs_dist_f64(g.row_ptr, g.col, g.w.astype(np.float64), sp, g=su)
     src = np.repeat(np.arange(g.n), np.diff(g.row_ptr))
     key = np.minimum(src, g.col).astype(np.int64) * g.n + np.maximum(src, g.col)
@@ -651,7 +664,10 @@ def run_grad(args, rank, local_rank):
                        "weights": "float32 length x lognormal(0, 0.25)"},
             "build_ms": build_ms, "forward_query_ms": fwd_ms, "backward_ms": bwd_ms,
             "sample_check": {"pairs": 2000, "dist_max_rel_err_vs_fp64": derr,
-                             "grad_max_err_vs_cpu_reference_rel_to_max": float(err), "pass": bool(err <= 1e-4)},
+                             "grad_max_err_vs_cpu_reference_rel_to_max": float(err),
+                         "timed_step_equal_on_sample": timed_equal,
+                         "timed_grad_max_err_vs_small_batches_rel_to_max": gerr,
+                         "pass": bool(err <= 1e-4 and timed_equal and gerr <= 1e-4)},
             "clocks": clk}
     print(json.dumps(line), flush=True)
     return 0
@@ -757,15 +773,23 @@ def main():
     bs_ms = sum(pf.get("bs_ms", 0.0) for _, pf, _ in per)
     bs_launches = sum(pf.get("bs_launches", 0.0) for _, pf, _ in per)
     bs_updates = sum(pf.get("bs_updates", 0.0) for _, pf, _ in per)
-    sms = torch.cuda.get_device_properties(dev).multi_processor_count
-    # updates per clock and SM of the kernels' inner loop alone (packed adds and three-input
-    # mins, operands from shared memory; measured), at the maximum SM clock.  (The 64 that one
-    # add and one min on 128 lanes would give is no bound: the two run on different pipes.)
-    peak_gops = sms * 74 * 2070e6 / 1e9
+    # measured issue rates of the update (same process, after the timed region): mode 6 is the
+    # tile kernels' inner loop alone, its operands in shared memory: their peak.  (The 64 updates
+    # a clock that one add and one min on 128 lanes would give is no bound: the two run on
+    # different pipes.)
+    ups, pms = ctypes.c_double(), ctypes.c_double()
+    micro = {}
+    for mode, iters, ctas in ((1, 20000, 8), (2, 20000, 8), (3, 20000, 8), (6, 2000, 2)):
+        if lib.spq_peak_minplus(mode, iters, ctas, ctypes.byref(ups), ctypes.byref(pms)) != 0:
+            raise RuntimeError(f"spq_peak_minplus mode {mode} failed")
+        micro[str(mode)] = round(ups.value / 1e9, 1)
+    peak_gops = micro["6"]
+    elim = int(per[0][1].get("bg_method", 1)) == 2
     kern = {
-        "k_phase3_list": {"what": "k_phase3_list (boundary-graph elimination / Floyd-Warshall, phase 3)",
-                          "ms": p3_ms, "launches": p3_launches, "updates": p3_updates, "traffic": None,
-                          "traffic_note": "not captured for the elimination rounds"},
+        "phase 3": {"what": "k_elim_phase3 (boundary-graph elimination rounds, phase 3)" if elim else
+                            "k_phase3_list (boundary-graph Floyd-Warshall, phase 3)",
+                    "ms": p3_ms, "launches": p3_launches, "updates": p3_updates, "traffic": None,
+                    "traffic_note": "not captured"},
         "k_backsub": {"what": "k_backsub (boundary-graph back-substitution, persistent)",
                       "ms": bs_ms, "launches": bs_launches, "updates": bs_updates, "traffic": None,
                       "traffic_note": BACKSUB_TRAFFIC_NOTE},
@@ -801,13 +825,6 @@ def main():
                                                        "4*(roundup4(|B1|) + roundup4(|B2|)) + 16"},
             "traffic": None}
 
-    # measured issue peak of the update (same process, after the timed region)
-    ups, pms = ctypes.c_double(), ctypes.c_double()
-    micro = {}
-    for mode in (1, 2, 3):
-        if lib.spq_peak_minplus(mode, 20000, 8, ctypes.byref(ups), ctypes.byref(pms)) == 0:
-            micro[str(mode)] = round(ups.value / 1e9, 1)
-
     line = {
         "metric": METRIC,
         "value": whole_job_rate(K * q, world, elapsed_ms * 1e-3),
@@ -834,8 +851,8 @@ def main():
         "query_qps": q / (statistics.mean(query_ms) * 1e-3),
         "build_stage_ms": {k: round(statistics.mean(pf[k] for _, pf, _ in per), 2)
                            for k in ("validate", "reorder", "comp_fw", "bg_assemble", "bg_fw", "check")},
-        "roofline": dict(roof(top), peak_basis=f"{sms} SMs x 74 min-plus updates per clock (measured: packed adds + "
-                                                 "three-input mins from shared memory) x 2070 MHz",
+        "roofline": dict(roof(top), peak_basis="the tile kernels' inner loop alone, measured in this process "
+                                                 "(spq_peak_minplus mode 6)",
                          microbench_gops=micro),
         "roofline_other": [roof(x) for x in other] + ([roof_query] if roof_query else []),
         "gpu_launches": int(launches),

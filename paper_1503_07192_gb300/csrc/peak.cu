@@ -1,11 +1,15 @@
 // Throughput micro-benchmark of the min-plus update c = min(c, a + b) on the ALU/FMA
 // pipes, for the roofline of the Floyd-Warshall kernels (which are bound by it: min-plus
-// has no tensor-core form).  Every operand is a register; each thread keeps 16
+// has no tensor-core form).  In modes 0 to 5 every operand is a register; each thread keeps 16
 // independent accumulators and feeds them back as the next step's operands, so nothing
-// is loop-invariant and no memory traffic is involved.
+// is loop-invariant and no memory traffic is involved.  Mode 6 is the tile kernels' own inner
+// loop (compute_chunk) over panels that stay in shared memory: what those kernels could reach
+// without global memory, waits and tile boundaries.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "common.cuh"
+#include "fw_tile.cuh"
 #include "spq_bench.h"
 
 namespace {
@@ -113,6 +117,40 @@ __global__ void __launch_bounds__(256) k_peak(const float* __restrict__ in, floa
     out[blockIdx.x * blockDim.x + threadIdx.x] = s;
 }
 
+__global__ void __launch_bounds__(spq::NTH, SPQ_FW_MIN_CTAS) k_peak_chunk(const float* __restrict__ in,
+                                                                         float* __restrict__ out, int iters) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    spq::PanelSmem<float>& sm = *reinterpret_cast<spq::PanelSmem<float>*>(smem_raw);
+    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+    for (int i = tid; i < spq::KC * spq::T_; i += spq::NTH)
+        for (int s = 0; s < 2; ++s) {
+            sm.a[s][i / spq::T_][i % spq::T_] = in[(i + 7 * s) & 63];
+            sm.b[s][i / spq::T_][i % spq::T_] = in[(i + 11 * s + 3) & 63];
+        }
+    __syncthreads();
+    float acc[8][8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+#pragma unroll
+        for (int j = 0; j < 8; ++j) acc[i][j] = 1e9f;
+#pragma unroll 1
+    for (int it = 0; it < iters; ++it) spq::compute_chunk<float>(acc, sm, it & 1, tx, ty);
+    float s = 0.f;
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+#pragma unroll
+        for (int j = 0; j < 8; ++j) s += acc[i][j];
+    out[blockIdx.x * blockDim.x + tid] = s;
+}
+
+cudaError_t run_chunk(int blocks, const float* in, float* out, int iters, cudaStream_t st) {
+    const int smem = (int)sizeof(spq::PanelSmem<float>);
+    const cudaError_t e = cudaFuncSetAttribute(k_peak_chunk, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess) return e;
+    k_peak_chunk<<<blocks, spq::NTH, smem, st>>>(in, out, iters);
+    return cudaGetLastError();
+}
+
 template <int MODE>
 cudaError_t run(int blocks, const float* in, float* out, int iters, cudaStream_t st) {
     k_peak<MODE><<<blocks, 256, 0, st>>>(in, out, iters);
@@ -122,7 +160,7 @@ cudaError_t run(int blocks, const float* in, float* out, int iters, cudaStream_t
 }  // namespace
 
 extern "C" int spq_peak_minplus(int mode, int iters, int blocks_per_sm, double* updates_per_s, double* ms) {
-    if (mode < 0 || mode > 5 || iters <= 0 || blocks_per_sm <= 0) return (int)cudaErrorInvalidValue;
+    if (mode < 0 || mode > 6 || iters <= 0 || blocks_per_sm <= 0) return (int)cudaErrorInvalidValue;
     int dev = 0, sms = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -148,7 +186,8 @@ extern "C" int spq_peak_minplus(int mode, int iters, int blocks_per_sm, double* 
             case 2: e = run<2>(blocks, in, out, iters, st); break;
             case 3: e = run<3>(blocks, in, out, iters, st); break;
             case 4: e = run<4>(blocks, in, out, iters, st); break;
-            default: e = run<5>(blocks, in, out, iters, st); break;
+            case 5: e = run<5>(blocks, in, out, iters, st); break;
+            default: e = run_chunk(blocks, in, out, iters, st); break;
         }
         if (e != cudaSuccess) goto done;
         cudaEventRecord(e1, st);
@@ -157,7 +196,7 @@ extern "C" int spq_peak_minplus(int mode, int iters, int blocks_per_sm, double* 
     {
         float t = 0.f;
         cudaEventElapsedTime(&t, e0, e1);
-        const double per_iter = (mode == 0 || mode == 3 || mode == 4) ? 16.0 : 32.0;
+        const double per_iter = mode == 6 ? 64.0 * spq::KC : (mode == 0 || mode == 3 || mode == 4) ? 16.0 : 32.0;
         const double upd = (double)blocks * 256.0 * iters * per_iter;
         if (ms) *ms = t;
         if (updates_per_s) *updates_per_s = upd / (t * 1e-3);
