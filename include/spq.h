@@ -278,8 +278,9 @@ void spq_build_plan_free(spq_build_plan* plan);
  * in dist_out[i].  All buffers host memory (synchronous; SPQ_EINVAL if any pair was out of
  * range) or all device memory (queued; spq_query_status per handle).  One scratch
  * allocation serves every instance; the instances run over up to four streams of the library
- * that fork from `stream` and join it again (over `stream` alone while it is being captured,
- * or where the scratch of four does not fit).
+ * that fork from `stream` and join it again (over `stream` alone while it is being captured;
+ * over fewer where their scratch, about 90 bytes a pair of the largest instance for each,
+ * would pass 256 MiB or does not fit).
  */
 spq_status spq_query_many(int32_t count, spq_handle* const* hs, const int32_t* const* pairs, const int64_t* q,
                           void* const* dist_out, void* stream);
@@ -317,7 +318,8 @@ void spq_query_plan_free(spq_query_plan* plan);
  * 2^31 - 1; SPQ_EUNSUPPORTED for handles of spq_build_many or a component with more than
  * 6,400 boundary vertices.
  * Scratch (stream-ordered): 16 bytes per target for their sort, and t of a batch of sources
- * (at most about 64 MB or 64 sources' worth; fewer sources at a time where that does not fit).
+ * for the components with targets (at most about 64 MB or 64 sources' worth; fewer sources at
+ * a time where that does not fit).
  */
 spq_status spq_query_matrix(spq_handle* h, const int32_t* sources, int64_t ns, const int32_t* targets, int64_t nt,
                             void* dist_out, void* stream);
@@ -337,9 +339,12 @@ spq_status spq_query_matrix(spq_handle* h, const int32_t* sources, int64_t ns, c
  * hop = the neighbour minimising edge weight + table distance to the target).  Where the
  * path is unique this is the derivative of sum_i grad_dist[i] * dist_i with respect to the
  * slot weights (an undirected edge's derivative is the sum over its two slots).
- * Scratch (stream-ordered): for large batches the pairs' sort and the walks' records (per CSR
- * slot, boundary vertex and component's boundary pairs); where it does not fit, or while the
- * stream is being captured, the pairs are answered and walked one by one without it.
+ * Scratch (stream-ordered), for large batches: the grouped forward's (156 bytes a pair, at
+ * most 4,194,304 pairs at a time); the walks' records: 8 bytes per CSR slot and per vertex, 132
+ * per boundary vertex, 4 per vertex and boundary vertex of its component (the sum of
+ * |C| x |B(C)|), for the backward another 4 per boundary pair of a component (the sum of
+ * |B(C)|^2), and 16 bytes a pair for their sort.  Where it does not fit, or while the stream is
+ * being captured, the pairs are answered and walked one by one without it.
  * pairs and saved must be those of the forward call on the same handle.  A walk that
  * cannot reach its target (zero-length cycles) sets a mark reported by spq_query_status.
  * Handles from spq_build_many return SPQ_EUNSUPPORTED.

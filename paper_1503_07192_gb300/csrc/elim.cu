@@ -1078,11 +1078,6 @@ template cudaError_t launch_fill_marked<int32_t>(int32_t*, int64_t, const uint32
 
 }  // namespace spq
 
-namespace spq {
-unsigned long long wait_bound_ns() { return g_wait_ns.load(); }
-int wait_withhold() { return g_withhold.load(); }
-}  // namespace spq
-
 extern "C" void spq_test_backsub_wait(unsigned long long limit_ns, int32_t withhold) {
     spq::g_wait_ns.store(limit_ns > 0 ? limit_ns : spq::kWaitNs);
     spq::g_withhold.store(withhold != 0 ? 1 : 0);

@@ -232,27 +232,6 @@ __device__ __forceinline__ void phase3_tile(T* __restrict__ M, int64_t n, int64_
     if (I != J) store_c_transposed<T>(acc, M, n, ci, cj, tx, ty);
 }
 
-// ---------------- phase 3, batched form: tiles (I, J), I <= J, I, J != r ----------------
-template <typename T>
-__global__ void __launch_bounds__(NTH, SPQ_FW_MIN_CTAS) k_phase3_batched(T* __restrict__ base, const MatDesc* __restrict__ descs,
-                                                           int32_t nmat, int32_t r) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    PanelSmem<T>& sm = *reinterpret_cast<PanelSmem<T>*>(smem_raw);
-    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-    for (int32_t mi = blockIdx.y; mi < nmat; mi += gridDim.y) {
-        const MatDesc d = descs[mi];
-        const int64_t n = d.n;
-        const int32_t R = (int32_t)((n + T_ - 1) / T_);
-        const int64_t Rm = R - 1;
-        if (r >= R || (int64_t)blockIdx.x >= Rm * (Rm + 1) / 2) continue;
-        int64_t I, J;
-        tri_pair((int64_t)blockIdx.x, Rm, I, J);
-        I += (I >= r);
-        J += (J >= r);
-        phase3_tile<T>(base + d.off, n, (int64_t)r * T_, I, J, sm, tid, tx, ty);
-    }
-}
-
 // ---------------- phase 3 over the matrices active in round r ----------------
 // sel[0..nsel) = matrices with more than r + 1 tile rows; p3off[0..nsel] = exclusive
 // prefix of their task counts Rm(Rm + 1)/2 (Rm = tiles per side minus the pivot).
@@ -559,7 +538,8 @@ __global__ void __launch_bounds__(1024, 1) k_elim_phase1(const ElimEnt<T>* __res
     }
 }
 
-// A step's tiles are split into strips when fewer than this many would be at work.
+// A step's tiles are split into strips when fewer than this many would be at work: one per SM
+// of a GB300 (a strip takes a quarter of a tile's time, so up to there the split shortens the step).
 constexpr int64_t kStripTiles = 152;
 
 // Phase 2: the candidate row tiles (r, J) <- D*(r, r) (x) D(r, J) and their transposes.  A
@@ -770,9 +750,6 @@ cudaError_t set_smem_attrs() {
     e = cudaFuncSetAttribute(k_elim_phase1<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, T_ * T_ * (int)sizeof(T));
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(k_phase2<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(PanelSmem<T>));
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_phase3_batched<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)sizeof(PanelSmem<T>));
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(k_phase3_list<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(PanelSmem<T>));
     if (e != cudaSuccess) return e;

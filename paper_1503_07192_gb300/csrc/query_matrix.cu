@@ -306,6 +306,9 @@ int msms() {
     return g_msms;
 }
 
+// Most boundary vertices of a component: the entry point's documented limit.  (It dates from a
+// kernel that kept t of eight sources in shared memory; the kernels here need no such buffer.)
+constexpr int32_t kMatrixMaxNb = 6400;
 constexpr int64_t kTElems = 1 << 24;  // most values of t at a time (64 MB), at least MS rows
 
 template <typename T, bool OUT_F32>
@@ -357,10 +360,7 @@ extern "C" spq_status spq_query_matrix(spq_handle* h, const int32_t* sources, in
     bool f32store = false, out_f32 = false;
     int32_t k = 0;
     handle_query_view(h, &ci, &cf, &f32store, &out_f32, &k);
-    int32_t nbmax = 0;
-    for (int32_t c = 0; c < k; ++c) nbmax = std::max(nbmax, h->h_nb[c]);
-    // (a component with more than 6,400 boundary vertices)
-    if ((size_t)(8 * (((nbmax > 0 ? nbmax : 1) + 31) & ~31)) * 4 > 200 * 1024) return SPQ_EUNSUPPORTED;
+    if (h->max_nb > kMatrixMaxNb) return SPQ_EUNSUPPORTED;
     std::vector<void*> tmp;
     auto alloc = [&](void** p, size_t bytes) {
         cudaError_t e = scratch_alloc(p, bytes ? bytes : 4, st);
@@ -391,7 +391,7 @@ extern "C" spq_status spq_query_matrix(spq_handle* h, const int32_t* sources, in
     }
     // the targets sorted by component, their tiles, t of a batch of sources
     // (its rows: the components with targets, at most nt of them)
-    const int64_t ldt = std::min(round_up(h->nbg + 3 * (int64_t)k, 4), std::min<int64_t>(nt, k) * round_up(nbmax, 4)) + 4;
+    const int64_t ldt = std::min(round_up(h->nbg + 3 * (int64_t)k, 4), std::min<int64_t>(nt, k) * round_up(h->max_nb, 4)) + 4;
     int64_t rows = std::min(round_up(ns, MS), std::max<int64_t>(MS, kTElems / ldt / MS * MS));
     const int64_t max_tiles = (nt + MT - 1) / MT + k + 1;
     uint32_t* buf;

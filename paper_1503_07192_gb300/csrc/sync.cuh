@@ -1,6 +1,5 @@
 // Device-side flag synchronisation between CTAs of one launch (the back-substitution's
-// tile flags, the elimination rounds' task flags): release stores, acquire loads and the
-// global timer that bounds every wait.
+// tile flags): release stores, acquire loads and the global timer that bounds every wait.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -21,10 +20,5 @@ __device__ __forceinline__ uint32_t ld_acquire(const uint32_t* p) {
 __device__ __forceinline__ void st_release(uint32_t* p, uint32_t v) {
     asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
-
-// Bound of one device-side dependency wait in ns, and whether launches withhold their
-// releases (both from the test hook spq_test_backsub_wait; elim.cu).
-unsigned long long wait_bound_ns();
-int wait_withhold();
 
 }  // namespace spq

@@ -49,7 +49,7 @@ def test_handles_hold_their_footprints(bg):
 
 @pytest.mark.parametrize("q", [50_000, 3_000_000])
 def test_a_query_plan_holds_bounded_scratch(q):
-    """Four instances in flight take four scratches (about 92 bytes a pair of the largest
+    """Four instances in flight take four scratches (about 90 bytes a pair of the largest
     instance), together at most 256 MiB; a larger instance takes one, as it needs anyway."""
     m = spq()
     torch, dev = torch_dev()
