@@ -123,15 +123,14 @@ __device__ __forceinline__ int32_t best_slot(const View<T>& V, const WalkCtx<T>&
                                              int32_t vs, int32_t& x, int32_t t, int g, unsigned mask) {
     const int2 er = W.vrange[vs + x];
     T best = Inf<T>::value();
-    int32_t be = INT32_MAX, to = -1;  // (slots are numbered below INT32_MAX)
-    // (unsigned: with up to 2^31 - 1 slots the last step may go past INT32_MAX)
-    for (uint32_t e = (uint32_t)er.x + (uint32_t)g; e < (uint32_t)er.y; e += SUB) {
+    int32_t be = INT32_MAX, to = -1;  // (a graph has fewer than INT32_MAX slots)
+    for (int32_t e = er.x + g; e < er.y; e += SUB) {
         const int32_t u = W.slots[e].x;
         if (u < 0) continue;
         const T cand = V.w[e] + A[(int64_t)u * ld + t];
         if (less_lex(cand, e, best, be)) {
             best = cand;
-            be = (int32_t)e;
+            be = e;
             to = u;
         }
     }
@@ -288,13 +287,13 @@ __device__ __forceinline__ bool walk_bg(const View<T>& V, const WalkCtx<T>& W, i
         const bool many = __any_sync(0xffffffffu, oa.z == -2);
         if (many) {
             const int2 er = W.vrange[vs + l];
-            for (uint32_t e = (uint32_t)er.x + (uint32_t)lane; e < (uint32_t)er.y; e += 32) {
+            for (int32_t e = er.x + lane; e < er.y; e += 32) {
                 const int2 s = W.slots[e];
                 if (s.x >= 0 || s.x == INT32_MIN) continue;
                 const uint32_t k = word_of((T)(V.w[e] + (dist(s.y) + T(0))));
                 if (k < ek) {
                     ek = k;
-                    ei = (int32_t)e;
+                    ei = e;
                 }
             }
         }
