@@ -634,7 +634,8 @@ __global__ void __launch_bounds__(256) k_qb_witness(const QueryCtx<T> ctx, const
                 const unsigned long long x = ((unsigned long long)mi << 32) | (uint32_t)j;
                 if (x < sel) sel = x;
             };
-            for (int32_t w = 0; w < nw; ++w) {
+            const uint32_t ws = __ballot_sync(0xffffffffu, mw != 0u);
+            for (int32_t w = __ffs(ws) - 1; w < nw && (ws >> w); ++w) {
                 uint32_t bits = __shfl_sync(0xffffffffu, mw, w);
                 if (bits == 0u) continue;
                 const uint32_t most = (uint32_t)(sel >> 32);  // (rows past it decide nothing)
