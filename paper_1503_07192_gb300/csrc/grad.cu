@@ -550,10 +550,12 @@ bool on_device(const void* p) {
 }
 
 // The records of walk.cuh for handle h, in one stream-ordered allocation (freed by the caller
-// with cudaFreeAsync(*mem)); false if it does not fit (the caller walks without them).
+// with cudaFreeAsync(*mem)); false if it does not fit, or if a walk's loop over slots, in 32
+// bits and steps of up to 32, could pass INT32_MAX (the caller walks without them).
 template <typename T>
 bool walk_records(const spq_handle* h, bool want_flow, cudaStream_t st, WalkCtx<T>* W, void** mem, int64_t* nflow) {
     const int32_t k = h->k;
+    if (h->m > INT32_MAX - 32) return false;
     std::vector<int64_t> off;
     try {
         off.assign(2 * ((size_t)k + 1), 0);
