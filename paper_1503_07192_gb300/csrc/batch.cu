@@ -629,9 +629,13 @@ spq_status build_many_impl(int32_t G, const spq_graph* gs, const spq_opts& o, cu
     if (arena_bytes + 4 * (size_t)d_tot + temp_bytes > free_b) d_tot = reserve(false);
     if (arena_bytes + 4 * (size_t)d_tot + temp_bytes > free_b) return SPQ_ENOMEM;
     struct ArenaGuard {
+        cudaStream_t st;
         Arena a;
-        ~ArenaGuard() { a.release(); }
-    } aguard;
+        ~ArenaGuard() {
+            if (a.base) cudaStreamSynchronize(st);  // (a build that fails half-way has work queued)
+            a.release();
+        }
+    } aguard{st, {}};
     // (from the library's pool: a batch's tens of gigabytes are kept mapped for the next)
     auto arena_alloc = [&](void** p, size_t bytes) {
         const cudaError_t e = scratch_alloc(p, bytes, st);
